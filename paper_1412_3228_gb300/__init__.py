@@ -15,6 +15,7 @@ from __future__ import annotations
 
 import ctypes
 import dataclasses
+import math
 import os
 from typing import List, Optional, Sequence, Tuple
 
@@ -233,6 +234,28 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     return None if t is None else t.data_ptr()
 
 
+def _mixed_estimate(cells) -> int:
+    """Room for the mixed voxels of a batch: the voxels whose filter ball meets a surface lie in a band
+    of twice the filter radius about it (3D packs hold more of them than a sixteenth of their voxels,
+    and a table that is too small costs a second build).  Overlapping primitives only overestimate."""
+    total = 0.0
+    for c in cells:
+        if c.rule == 0:
+            continue
+        band = 2.0 * float(c.radius_px) + 0.5
+        part = 0.0
+        for p in c.prims:
+            r = float(p.radius) * c.n
+            if p.kind == 2:
+                part += 2.0 * band * c.n ** (c.dim - 1)
+            elif c.dim == 2:
+                part += 2.0 * math.pi * r * band
+            else:
+                part += 4.0 * math.pi * (r * r + band * band / 12.0) * band
+        total += min(part, float(c.n) ** c.dim)
+    return int(total) + 1
+
+
 def hom_filter_build(cells: Sequence, phases: Sequence[Tuple[float, float]], device=None, stream=None,
                      capacity: Optional[int] = None) -> Material:
     """Filtered stiffness of every voxel (section 2, eqs. 3-5); see include/hom.h."""
@@ -251,7 +274,7 @@ def hom_filter_build(cells: Sequence, phases: Sequence[Tuple[float, float]], dev
     label = torch.empty(nvox, dtype=torch.int32, device=device)
     phase_c64 = torch.empty(nphase * ns, dtype=torch.float64, device=device)
     phase_c32 = torch.empty(nphase * ns, dtype=torch.float32, device=device)
-    cap = capacity if capacity is not None else max(1024, nvox // 16)
+    cap = capacity if capacity is not None else max(1024, nvox // 16, _mixed_estimate(cells))
     for _attempt in range(2):
         mixed = dict(
             mixed_c64=torch.empty(cap * ns, dtype=torch.float64, device=device),

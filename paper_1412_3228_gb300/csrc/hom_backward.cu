@@ -66,23 +66,31 @@ __global__ void __launch_bounds__(kThreads) k_grad(GradArgs A) {
     for (int p = 0; p < NC; ++p)
 #pragma unroll
       for (int q = 0; q < NC; ++q) Am[p][q] = T(0);
-    // C_eff term: (1/N_v) sum_ij G_ij eps^(i)_p eps^(j)_q (loads are the nc unit strains)
+    // C_eff term: (1/N_v) sum_ij G_ij eps^(i)_p eps^(j)_q (loads are the nc unit strains), every strain
+    // read once
     if (A.dLdC) {
       const double* G = A.dLdC + (size_t)ci * NC * NC;
       const T inv_nv = (T)(1.0 / (double)cell.nv);
+      T e[NC][NC];
+#pragma unroll
+      for (int j = 0; j < NC; ++j)
+#pragma unroll
+        for (int q = 0; q < NC; ++q) e[j][q] = eps[((size_t)j * NC + q) * cell.nv];
+#pragma unroll
       for (int i = 0; i < NC; ++i) {
         T u[NC];
 #pragma unroll
         for (int q = 0; q < NC; ++q) u[q] = T(0);
+#pragma unroll
         for (int j = 0; j < NC; ++j) {
           const T g = (T)G[i * NC + j];
           if (g == T(0)) continue;
 #pragma unroll
-          for (int q = 0; q < NC; ++q) u[q] += g * eps[((size_t)j * NC + q) * cell.nv];
+          for (int q = 0; q < NC; ++q) u[q] += g * e[j][q];
         }
 #pragma unroll
         for (int p = 0; p < NC; ++p) {
-          const T ep = eps[((size_t)i * NC + p) * cell.nv] * inv_nv;
+          const T ep = e[i][p] * inv_nv;
 #pragma unroll
           for (int q = 0; q < NC; ++q) Am[p][q] += ep * u[q];
         }
@@ -127,30 +135,67 @@ __global__ void __launch_bounds__(kThreads) k_grad(GradArgs A) {
       for (int s = 0; s < cell.nslot; ++s)
         if (cell.slot_phase[s] == (int)lab) { contrib[s][0] += dl; contrib[s][1] += dm; }
     } else {
-      // mixed voxel: directional derivatives of the rule by dual numbers
+      // mixed voxel: directional derivatives of the rule's moduli by dual numbers, contracted with the
+      // projections of the gradient on the tensors they multiply
       const uint32_t m = lab & ~HOM_MIXED_BIT;
       const int pa = A.mixed_phases[2 * m], pb = A.mixed_phases[2 * m + 1];
       const double fb = A.mixed_frac[m];
-      double nrm[3] = {A.mixed_normal[3 * m], A.mixed_normal[3 * m + 1], A.mixed_normal[3 * m + 2]};
-      const bool nrm_ok = (nrm[0] * nrm[0] + nrm[1] * nrm[1] + nrm[2] * nrm[2]) > 0.25;
-      const double lam[2] = {A.phase_lame[2 * pa], A.phase_lame[2 * pb]};
-      const double mu[2] = {A.phase_lame[2 * pa + 1], A.phase_lame[2 * pb + 1]};
+      const double nrm[3] = {A.mixed_normal[3 * m], A.mixed_normal[3 * m + 1], A.mixed_normal[3 * m + 2]};
+      // (an entry of the 2-layer rule without a normal was built by the Voigt rule)
+      const bool layers =
+          cell.rule == HOM_RULE_TWO_LAYER && (nrm[0] * nrm[0] + nrm[1] * nrm[1] + nrm[2] * nrm[2]) > 0.25;
+      // projections: isotropic rules w = (1^T A 1, 2 tr A); layers (along N, N with p, p, the plane, the shear)
+      double w[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+      if (layers) {
+        const LayerBasis<DIM> lb(nrm);
+        double tr = 0.0, q = 0.0;
+#pragma unroll
+        for (int p = 0; p < NC; ++p) {
+          tr += (double)Am[p][p];
+          double an = 0.0, ap = 0.0;
+#pragma unroll
+          for (int r = 0; r < NC; ++r) {
+            const double a = (double)Am[p][r];
+            an += a * lb.N[r];
+            ap += a * lb.p[r];
+            q += a * lb.Q(p, r);
+          }
+          w[0] += lb.N[p] * an;
+          w[1] += lb.N[p] * ap + lb.p[p] * an;
+          w[2] += lb.p[p] * ap;
+        }
+        w[3] = 2.0 * (tr - 2.0 * q + w[0]);
+        w[4] = 4.0 * (q - w[0]);
+      } else {
+#pragma unroll
+        for (int p = 0; p < NC; ++p) {
+          w[1] += 2.0 * (double)Am[p][p];
+#pragma unroll
+          for (int r = 0; r < DIM; ++r)
+            if (p < DIM) w[0] += (double)Am[p][r];
+        }
+      }
       double dtheta[5];
+#pragma unroll 1
       for (int dir = 0; dir < 5; ++dir) {  // lam_a, mu_a, lam_b, mu_b, f_b
-        Dual Cs[2][36], fs[2], Ct[36];
+        Dual l[2], u[2], fs[2];
+#pragma unroll
         for (int k = 0; k < 2; ++k) {
-          const Dual l = {lam[k], (dir == 2 * k) ? 1.0 : 0.0};
-          const Dual u = {mu[k], (dir == 2 * k + 1) ? 1.0 : 0.0};
-          iso_full_t<Dual>(l, u, DIM, Cs[k]);
+          const int ph = k == 0 ? pa : pb;
+          l[k] = {A.phase_lame[2 * ph], dir == 2 * k ? 1.0 : 0.0};
+          u[k] = {A.phase_lame[2 * ph + 1], dir == 2 * k + 1 ? 1.0 : 0.0};
         }
         fs[1] = {fb, dir == 4 ? 1.0 : 0.0};
         fs[0] = {1.0 - fb, dir == 4 ? -1.0 : 0.0};
-        apply_rule_t<Dual>(cell.rule, 2, Cs, fs, nrm_ok, nrm, DIM, Ct);
-        double s = 0.0;
-#pragma unroll
-        for (int p = 0; p < NC; ++p)
-#pragma unroll
-          for (int q = 0; q < NC; ++q) s += (double)Am[p][q] * Ct[p * NC + q].d;
+        double s;
+        if (layers) {
+          const Layered<Dual> c = layered_moduli(l, u, fs);
+          s = w[0] * c.cn.d + w[1] * c.F.d + w[2] * c.B.d + w[3] * c.mup.d + w[4] * c.mun.d;
+        } else {
+          const Iso<Dual> c =
+              cell.rule == HOM_RULE_REUSS ? reuss_moduli<2>(l, u, fs, 2, DIM) : voigt_moduli<2>(l, u, fs);
+          s = w[0] * c.lam.d + w[1] * c.mu.d;
+        }
         dtheta[dir] = s;
       }
       for (int s = 0; s < cell.nslot; ++s) {

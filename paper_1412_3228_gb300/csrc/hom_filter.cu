@@ -6,9 +6,10 @@
 //      and the first primitive that contains the whole ball.  A voxel with no near primitive is
 //      labelled with its centre phase;
 //   2. one warp per remaining voxel counts the fine-grid samples of the ball per phase, the
-//      lanes splitting the samples;
-//   3. one thread per voxel whose samples hold two or more phases computes the 2-layer normal,
-//      applies the rule in FP64 and writes a mixed-table entry.
+//      lanes splitting the ball's sample lines along x (the samples of a line inside one primitive
+//      are consecutive, so a line costs a few membership tests instead of one per sample);
+//   3. (k_filter_rule) one thread per voxel whose samples hold two or more phases computes the
+//      2-layer normal, applies the rule in FP64 and writes a mixed-table entry.
 // FP64 arithmetic runs at a small fraction of the FP32 rate on this GPU, so FP64 is kept for
 // decisions the FP32 arithmetic cannot settle and for the rule itself.
 //
@@ -75,6 +76,7 @@ struct FilterArgs {
   const FCell* cells;
   int ncells;
   const FPrim* prims;
+  const int4* lines;         // sample lines of the balls, FCell::line0 .. line0 + nline of each cell
   const double* phase_lame;  // [nphase][2]
   int nphase;
   hom_material mat;
@@ -93,10 +95,15 @@ struct NearRec {
 // Rule inputs of a mixed voxel, stashed by k_filter in the (not yet written) FP64 stiffness slot
 // of its mixed-table entry and read back by k_filter_rule (11 ints: fits the 6 doubles of 2D).
 struct RuleStash {
-  int cell, nph, nrm_ok;
+  int cell, nph, nnear;
   int ph[kMaxPhases], cnt[kMaxPhases];
 };
 static_assert(sizeof(RuleStash) <= 6 * sizeof(double), "stash must fit a 2D entry");
+// Near primitives of the voxel, stashed in the entry's normal (3 doubles) for the 2-layer rule.
+struct NearStash {
+  short near[kMaxNear];
+};
+static_assert(sizeof(NearStash) <= 3 * sizeof(double), "stash must fit a normal");
 
 // Per-warp FP32 data of one near primitive for the sample tests of the current voxel.
 struct NearPrim {
@@ -106,6 +113,87 @@ struct NearPrim {
   int axis;                  // slab axis, or -1 for a disk/sphere
 };
 
+// Samples of one line of a ball (along x, D0 = first + 2 i for i = 0 .. len - 1, len <= 32, at the fixed
+// offsets D[1], D[2]) that lie in a primitive, as a bit mask.  Without a wrap the squared distance
+// (or |u| of a slab normal to x), in the FP64 recipe as in exact arithmetic, does not decrease as
+// |offset along x| grows: every step of the recipe is monotone.  The members are therefore
+// consecutive: both ends in means all in, and each end of the run is found from its FP32 estimate
+// and settled by membership tests of the samples around it (FP32 where the margin decides,
+// inside_exact otherwise).  A line that may wrap is tested sample by sample.
+template <int DIM>
+struct LineTest {
+  const FPrim& p;
+  const NearPrim& np;
+  const int* a;    // voxel coordinates
+  int S, D1, D2;
+  double P2, half;
+  float side2;     // squared distance across the line (disk, sphere)
+
+  __device__ __forceinline__ bool exact(int D0) const {
+    double su[3] = {(double)(2 * a[0] * S + D0 + S), (double)(2 * a[1] * S + D1 + S),
+                    DIM == 3 ? (double)(2 * a[2] * S + D2 + S) : 0.0};
+    return inside_exact(p, su, DIM, P2, half);
+  }
+  __device__ __forceinline__ bool in(int D0) const {
+    float v;
+    if (np.axis < 0) {
+      const float u0 = np.d0[0] + (float)D0;
+      v = fmaf(u0, u0, side2);
+    } else {
+      v = fabsf(np.axis == 0 ? np.d0[0] + (float)D0 : np.axis == 1 ? np.d0[1] + (float)D1 : np.d0[2] + (float)D2);
+    }
+    if (v <= np.thr - np.margin) return true;
+    if (v > np.thr + np.margin) return false;
+    return exact(D0);
+  }
+  __device__ __forceinline__ unsigned mask(int first, int len) {
+    const float u1 = np.d0[1] + (float)D1, u2 = DIM == 3 ? np.d0[2] + (float)D2 : 0.f;
+    side2 = fmaf(u2, u2, u1 * u1);
+    const unsigned full = len >= 32 ? 0xffffffffu : (1u << len) - 1u;
+    const int last = first + 2 * (len - 1);
+    const float wrap_guard = (float)half - 2.f;
+    if (fmaxf(fmaxf(fabsf(np.d0[0] + (float)first), fabsf(np.d0[0] + (float)last)), fmaxf(fabsf(u1), fabsf(u2))) >
+        wrap_guard) {
+      unsigned m = 0;
+      for (int i = 0; i < len; ++i) m |= exact(first + 2 * i) ? 1u << i : 0u;
+      return m;
+    }
+    const bool A = in(first), B = len > 1 ? in(last) : A;
+    if (A && B) return full;
+    // estimates of the run's ends and of the sample nearest to the primitive's centre plane
+    const float h2 = np.axis < 0 ? np.thr - side2 : np.thr * np.thr;
+    const float r = h2 > 0.f ? sqrtf(h2) : 0.f;
+    const float mid = -np.d0[0] - (float)first;
+    int lo = 0, hi = len - 1;
+    if (!A && !B) {
+      const int c0 = min(max((int)floorf(0.5f * mid), 0), len - 1), c1 = min(c0 + 1, len - 1);
+      int c = -1;
+      if (in(first + 2 * c0)) c = c0;
+      else if (in(first + 2 * c1)) c = c1;
+      if (c < 0) return 0u;
+      lo = hi = c;
+    }
+    if (!A) {
+      const int top = B ? len - 1 : lo;  // a member
+      lo = min(max((int)ceilf(0.5f * (mid - r)), 1), top);
+      while (lo > 1 && in(first + 2 * (lo - 1))) --lo;
+      while (lo < top && !in(first + 2 * lo)) ++lo;
+    }
+    if (!B) {
+      const int bot = A ? 0 : hi;  // a member
+      hi = max(min((int)floorf(0.5f * (mid + r)), len - 2), bot);
+      while (hi < len - 2 && in(first + 2 * (hi + 1))) ++hi;
+      while (hi > bot && !in(first + 2 * hi)) --hi;
+    }
+    const unsigned upto = hi >= 31 ? 0xffffffffu : (1u << (hi + 1)) - 1u;
+    return upto & ~((1u << lo) - 1u);
+  }
+};
+
+// Bound by integer and FP32 issue.  Testing every sample of the ball's box (8000 in 3D at S = 8, r = 1,
+// of which 2145 are in the ball) took 11.39 ms for 135^3 cells of 144 spheres; by lines (about 200, three
+// to five tests each) it takes 3.20 ms.
+template <int DIM>
 __global__ void __launch_bounds__(kThreads) k_filter(FilterArgs A) {
   __shared__ NearRec s_near[kThreads];
   __shared__ NearPrim s_np[kWarps][kMaxNear];
@@ -116,14 +204,14 @@ __global__ void __launch_bounds__(kThreads) k_filter(FilterArgs A) {
   for (int c = 1; c < A.ncells; ++c)
     if ((long long)blockIdx.x >= A.cells[c].block0) ci = c;
   const FCell& cell = A.cells[ci];
-  const int n = cell.n, dim = cell.dim, S = cell.S, nprim = cell.nprim;
-  const long long nv = (long long)n * n * (dim == 3 ? n : 1);
+  const int n = cell.n, S = cell.S, nprim = cell.nprim;
+  const long long nv = (long long)n * n * (DIM == 3 ? n : 1);
   const long long v0 = ((long long)blockIdx.x - cell.block0) * kThreads;
   if (threadIdx.x == 0) {
     s_nnear = 0;
     s_base[0] = (int)(v0 % n);
     s_base[1] = (int)((v0 / n) % n);
-    s_base[2] = dim == 3 ? (int)(v0 / ((long long)n * n)) : 0;
+    s_base[2] = DIM == 3 ? (int)(v0 / ((long long)n * n)) : 0;
   }
   __syncthreads();
   const FPrim* prims = A.prims + cell.prim0;
@@ -143,26 +231,30 @@ __global__ void __launch_bounds__(kThreads) k_filter(FilterArgs A) {
       a[1] = t1 - q1 * n;
       a[2] = s_base[2] + q1;
     }
-    float xf[3];
-    for (int d = 0; d < dim; ++d) xf[d] = ((float)a[d] + 0.5f) * cell.inv_n;
+    float xf[DIM];
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) xf[d] = ((float)a[d] + 0.5f) * cell.inv_n;
     const bool filtered = cell.rule != HOM_RULE_NONE;
     const float near_lim = cell.reach32 + kDistMargin;
     int centre_first = -1, far_first = -1, nnear = 0;
     short near[kMaxNear];
+#pragma unroll
+    for (int k = 0; k < kMaxNear; ++k) near[k] = 0;
     bool overflow = false;
     for (int p = 0; p < nprim; ++p) {
       const FPrim& pr = prims[p];
       float dist;
       bool in32;
       if (pr.kind == HOM_PRIM_SLAB) {
-        float d = xf[pr.axis] - pr.c32[pr.axis];
+        float d = (pr.axis == 0 ? xf[0] : pr.axis == 1 ? xf[1] : xf[DIM - 1]) - pr.c32[pr.axis];
         d -= rintf(d);
         const float ad = fabsf(d), th = 0.5f * pr.r32;
         dist = fabsf(ad - th);
         in32 = ad < th;
       } else {
         float s2 = 0.f;
-        for (int d = 0; d < dim; ++d) {
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) {
           float t = xf[d] - pr.c32[d];
           t -= rintf(t);
           s2 = fmaf(t, t, s2);
@@ -175,9 +267,10 @@ __global__ void __launch_bounds__(kThreads) k_filter(FilterArgs A) {
       if (centre_first < 0) {
         bool in = in32;
         if (dist <= kDistMargin) {
-          double sc[3];
-          for (int d = 0; d < dim; ++d) sc[d] = (double)(2 * a[d] + 1) * (double)S;
-          in = inside_exact(pr, sc, dim, P2, half);
+          double sc[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+          for (int d = 0; d < DIM; ++d) sc[d] = (double)(2 * a[d] + 1) * (double)S;
+          in = inside_exact(pr, sc, DIM, P2, half);
         }
         if (in) centre_first = p;
       }
@@ -187,7 +280,11 @@ __global__ void __launch_bounds__(kThreads) k_filter(FilterArgs A) {
       }
       // near primitives after far_first own no sample but may hold the nearest surface (normal)
       if (dist <= near_lim) {
-        if (nnear < kMaxNear) near[nnear++] = (short)p; else overflow = true;
+        if (nnear == kMaxNear) overflow = true;
+#pragma unroll
+        for (int k = 0; k < kMaxNear; ++k)
+          if (k == nnear) near[k] = (short)p;
+        if (nnear < kMaxNear) ++nnear;
       } else if (in32 && far_first < 0) {
         far_first = p;  // contains the centre and no surface crosses the ball: contains every sample
       }
@@ -206,17 +303,18 @@ __global__ void __launch_bounds__(kThreads) k_filter(FilterArgs A) {
       rec.v = (int)(v - v0);
       rec.nnear = nnear;
       rec.far_first = far_first;
-      for (int k = 0; k < kMaxNear; ++k) rec.near[k] = k < nnear ? near[k] : (short)0;
+#pragma unroll
+      for (int k = 0; k < kMaxNear; ++k) rec.near[k] = near[k];
     }
   }
   __syncthreads();
 
   // ---------------------------------------------------------------- 2. sample counts, one warp per voxel
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nt = cell.thi - cell.tlo + 1;
-  const int total = dim == 3 ? nt * nt * nt : nt * nt;
   // largest |offset| of a ball sample from the voxel centre, in h/(2S) units
   const int offmax = max(abs(2 * cell.tlo + 1 - S), abs(2 * cell.thi + 1 - S));
+  const int4* lines = A.lines + cell.line0;
+  const int nline = cell.nline;
   for (int r = warp; r < s_nnear; r += kWarps) {
     const NearRec& rec = s_near[r];
     const int nnear = rec.nnear;
@@ -227,8 +325,9 @@ __global__ void __launch_bounds__(kThreads) k_filter(FilterArgs A) {
       // relative 2^-50 of it.  The margins below are twice these bounds.
       const FPrim& pr = prims[rec.near[lane]];
       NearPrim np;
+#pragma unroll
       for (int d = 0; d < 3; ++d) {
-        np.d0[d] = d < dim ? (float)wrapped_offset((double)(2 * rec.a[d] + 1) * (double)S, pr.c[d], P2, half)
+        np.d0[d] = d < DIM ? (float)wrapped_offset((double)(2 * rec.a[d] + 1) * (double)S, pr.c[d], P2, half)
                            : 0.f;
       }
       const float B = (float)half + (float)offmax;
@@ -240,78 +339,45 @@ __global__ void __launch_bounds__(kThreads) k_filter(FilterArgs A) {
         np.axis = -1;
         const double Ru = dmul(pr.radius, P2);
         np.thr = (float)dmul(Ru, Ru);
-        np.margin = (float)dim * B * B * ldexpf(1.f, -20) + ldexpf(np.thr, -22);
+        np.margin = (float)DIM * B * B * ldexpf(1.f, -20) + ldexpf(np.thr, -22);
       }
       s_np[warp][lane] = np;
     }
     __syncwarp();
-    const int far_first = rec.far_first;
-    const float wrap_guard = (float)half - 2.f;
+    // near primitives after the first one that holds the whole ball own no sample
+    int nown = nnear;
+    if (rec.far_first >= 0)
+      for (int k = nnear - 1; k >= 0; --k)
+        if (rec.near[k] > rec.far_first) nown = k;
     int cnt[kMaxNear + 1];
 #pragma unroll
     for (int k = 0; k <= kMaxNear; ++k) cnt[k] = 0;
-    for (int i = lane; i < total; i += 32) {
-      int t[3];
-      const int q = fdiv(i, cell.dnt);
-      t[0] = i - q * nt;
-      if (dim == 3) {
-        const int q2 = fdiv(q, cell.dnt);
-        t[1] = q - q2 * nt;
-        t[2] = q2;
-      } else {
-        t[1] = q;
-        t[2] = 0;
-      }
-      int D[3], q2sum = 0;
-      for (int d = 0; d < 3; ++d) {
-        D[d] = d < dim ? 2 * (t[d] + cell.tlo) + 1 - S : 0;
-        q2sum += D[d] * D[d];
-      }
-      if (q2sum > cell.R2i) continue;
-      int slot = 0;  // 0: no near primitive contains the sample; k + 1: near primitive k
-      for (int k = 0; k < nnear; ++k) {
-        const int p = rec.near[k];
-        if (far_first >= 0 && p > far_first) break;
-        const NearPrim& np = s_np[warp][k];
-        int verdict;  // 1 inside, 0 outside, -1 undecided in FP32
-        if (np.axis >= 0) {
-          const float u = np.d0[np.axis] + (float)D[np.axis];
-          const float au = fabsf(u);
-          if (au > wrap_guard) verdict = -1;
-          else verdict = au <= np.thr - np.margin ? 1 : (au > np.thr + np.margin ? 0 : -1);
-        } else {
-          const float u0 = np.d0[0] + (float)D[0];
-          const float u1 = np.d0[1] + (float)D[1];
-          const float u2 = np.d0[2] + (float)D[2];
-          if (fmaxf(fabsf(u0), fmaxf(fabsf(u1), fabsf(u2))) > wrap_guard) {
-            verdict = -1;
-          } else {
-            const float q32 = fmaf(u2, u2, fmaf(u1, u1, u0 * u0));
-            verdict = q32 <= np.thr - np.margin ? 1 : (q32 > np.thr + np.margin ? 0 : -1);
-          }
-        }
-        if (verdict < 0) {
-          double su[3];
-          for (int d = 0; d < dim; ++d) su[d] = (double)(2 * ((rec.a[d] * S) + t[d] + cell.tlo) + 1);
-          verdict = inside_exact(prims[p], su, dim, P2, half) ? 1 : 0;
-        }
-        if (verdict) {
-          slot = k + 1;
-          break;
-        }
-      }
+    for (int i = lane; i < nline; i += 32) {
+      const int4 ln = __ldg(lines + i);  // (D1, D2, half length m): D0 = -m, -m + 2, .., m
+      for (int s0 = 0; s0 <= ln.z; s0 += 32) {
+        const int len = min(ln.z + 1 - s0, 32), first = -ln.z + 2 * s0;
+        unsigned left = len >= 32 ? 0xffffffffu : (1u << len) - 1u;
+        for (int k = 0; k < nown && left; ++k) {
+          LineTest<DIM> lt{prims[rec.near[k]], s_np[warp][k], rec.a, S, ln.x, ln.y, P2, half, 0.f};
+          const unsigned m = lt.mask(first, len) & left;
+          left &= ~m;
+          const int c = __popc(m);
 #pragma unroll
-      for (int k = 0; k <= kMaxNear; ++k) cnt[k] += slot == k ? 1 : 0;
+          for (int q = 1; q <= kMaxNear; ++q) cnt[q] += q == k + 1 ? c : 0;
+        }
+        cnt[0] += __popc(left);
+      }
     }
+    __syncwarp();
 #pragma unroll
     for (int k = 0; k <= kMaxNear; ++k)
-      for (int o = 16; o > 0; o >>= 1) cnt[k] += __shfl_xor_sync(0xffffffffu, cnt[k], o);
+      if (k <= nnear) cnt[k] = __reduce_add_sync(0xffffffffu, cnt[k]);
     if (lane == 0) {
       int ph_id[kMaxPhases], ph_cnt[kMaxPhases], nph = 0;
       bool too_many = false;
       for (int k = 0; k <= nnear; ++k) {
         if (cnt[k] == 0) continue;
-        const int ph = k == 0 ? (far_first >= 0 ? prims[far_first].phase : cell.matrix_phase)
+        const int ph = k == 0 ? (rec.far_first >= 0 ? prims[rec.far_first].phase : cell.matrix_phase)
                               : prims[rec.near[k - 1]].phase;
         int j = 0;
         while (j < nph && ph_id[j] != ph) ++j;
@@ -333,47 +399,6 @@ __global__ void __launch_bounds__(kThreads) k_filter(FilterArgs A) {
         atomicExch(A.err_flag, 1);
         *label = (uint32_t)ph_id[0];
       } else {
-        // 2-layer normal: unit vector from the centre of the primitive whose surface is nearest
-        // to x_a (first one on ties), or the slab normal.  That primitive is a near one.
-        double nrm[3] = {0, 0, 0};
-        bool nrm_ok = false;
-        if (cell.rule == HOM_RULE_TWO_LAYER) {
-          double x[3];
-          for (int d = 0; d < dim; ++d) x[d] = ((double)rec.a[d] + 0.5) / (double)n;
-          double best = 1e300;
-          for (int k = 0; k < nnear; ++k) {
-            const FPrim& pr = prims[rec.near[k]];
-            double dist, vec[3] = {0, 0, 0}, len = 1.0;
-            if (pr.kind == HOM_PRIM_SLAB) {
-              double d = x[pr.axis] - pr.c[pr.axis];
-              d -= rint(d);
-              dist = fabs(fabs(d) - 0.5 * pr.radius);
-              vec[pr.axis] = 1.0;
-            } else {
-              double s2 = 0.0;
-              for (int d = 0; d < dim; ++d) {
-                double t = x[d] - pr.c[d];
-                t -= rint(t);
-                vec[d] = t;
-                s2 += t * t;
-              }
-              len = sqrt(s2);
-              dist = fabs(len - pr.radius);
-            }
-            if (dist < best) {
-              best = dist;
-              if (pr.kind == HOM_PRIM_SLAB) {
-                for (int d = 0; d < 3; ++d) nrm[d] = vec[d];
-                nrm_ok = true;
-              } else if (len > 1e-12) {
-                for (int d = 0; d < 3; ++d) nrm[d] = vec[d] / len;
-                nrm_ok = true;
-              } else {
-                nrm_ok = false;
-              }
-            }
-          }
-        }
         const unsigned long long m = atomicAdd(A.mixed_counter, 1ull);
         if ((long long)m >= A.mat.mixed_capacity) {
           *label = HOM_MIXED_BIT;  // placeholder: the caller must grow the table and rebuild
@@ -382,13 +407,15 @@ __global__ void __launch_bounds__(kThreads) k_filter(FilterArgs A) {
           RuleStash st;
           st.cell = ci;
           st.nph = nph;
-          st.nrm_ok = nrm_ok ? 1 : 0;
+          st.nnear = nnear;
           for (int j = 0; j < kMaxPhases; ++j) {
             st.ph[j] = j < nph ? ph_id[j] : 0;
             st.cnt[j] = j < nph ? ph_cnt[j] : 0;
           }
-          *reinterpret_cast<RuleStash*>(A.mat.mixed_c64 + m * ns_of(dim)) = st;
-          for (int d = 0; d < 3; ++d) A.mat.mixed_normal[3 * m + d] = nrm[d];
+          *reinterpret_cast<RuleStash*>(A.mat.mixed_c64 + m * ns_of(DIM)) = st;
+          NearStash ns;
+          for (int k = 0; k < kMaxNear; ++k) ns.near[k] = rec.near[k];
+          *reinterpret_cast<NearStash*>(A.mat.mixed_normal + 3 * m) = ns;
           A.mat.mixed_voxel[m] = cell.vox_off + v0 + rec.v;
         }
       }
@@ -397,49 +424,136 @@ __global__ void __launch_bounds__(kThreads) k_filter(FilterArgs A) {
   }
 }
 
+// 2-layer normal: unit vector from the centre of the primitive whose surface is nearest to x_a (first
+// one on ties), or the slab normal.  That primitive is a near one.  False: no usable normal.
+template <int DIM>
+__device__ __forceinline__ bool layer_normal(const FPrim* prims, const NearStash& ns, int nnear, const double* x,
+                                             double* nrm) {
+  bool ok = false;
+  double best = 1e300;
+  for (int k = 0; k < nnear; ++k) {
+    const FPrim& pr = prims[ns.near[k]];
+    double dist, vec[3] = {0, 0, 0}, len = 1.0;
+    if (pr.kind == HOM_PRIM_SLAB) {
+      double d = (pr.axis == 0 ? x[0] : pr.axis == 1 ? x[1] : x[DIM - 1]) - pr.c[pr.axis];
+      d -= rint(d);
+      dist = fabs(fabs(d) - 0.5 * pr.radius);
+#pragma unroll
+      for (int d2 = 0; d2 < 3; ++d2) vec[d2] = d2 == pr.axis ? 1.0 : 0.0;
+    } else {
+      double s2 = 0.0;
+#pragma unroll
+      for (int d = 0; d < DIM; ++d) {
+        double t = x[d] - pr.c[d];
+        t -= rint(t);
+        vec[d] = t;
+        s2 += t * t;
+      }
+      len = sqrt(s2);
+      dist = fabs(len - pr.radius);
+    }
+    if (dist < best) {
+      best = dist;
+      if (pr.kind == HOM_PRIM_SLAB) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) nrm[d] = vec[d];
+        ok = true;
+      } else if (len > 1e-12) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) nrm[d] = vec[d] / len;
+        ok = true;
+      } else {
+        ok = false;
+      }
+    }
+  }
+  return ok;
+}
+
 // ---------------------------------------------------------------- rule, one thread per mixed entry
+template <int DIM>
 __global__ void __launch_bounds__(kThreads) k_filter_rule(FilterArgs A) {
+  constexpr int NC = DIM == 2 ? 3 : 6, NS = DIM == 2 ? 6 : 21;
   const long long m = (long long)blockIdx.x * kThreads + threadIdx.x;
   const unsigned long long cnt_all = *A.mixed_counter;
-  if (m >= A.mat.mixed_capacity || (unsigned long long)m >= cnt_all) return;
-  const int dim = A.mat.dim;
-  const int nc = nc_of(dim), ns = ns_of(dim);
-  const RuleStash st = *reinterpret_cast<const RuleStash*>(A.mat.mixed_c64 + m * ns);
+  // a table that turned out too small is rebuilt by the caller: nothing of it is read
+  if (cnt_all > (unsigned long long)A.mat.mixed_capacity || (unsigned long long)m >= cnt_all) return;
+  const RuleStash st = *reinterpret_cast<const RuleStash*>(A.mat.mixed_c64 + m * NS);
   const FCell& cell = A.cells[st.cell];
+  const NearStash ns = *reinterpret_cast<const NearStash*>(A.mat.mixed_normal + 3 * m);
   int ph_id[kMaxPhases], ph_cnt[kMaxPhases];
   const int nph = st.nph;
+#pragma unroll
   for (int j = 0; j < kMaxPhases; ++j) {
-    ph_id[j] = st.ph[j];
+    ph_id[j] = j < nph ? st.ph[j] : 0x7fffffff;
     ph_cnt[j] = st.cnt[j];
   }
   // sort the present phases by index (deterministic "a < b" order)
-  for (int i = 0; i < nph; ++i)
-    for (int j = i + 1; j < nph; ++j)
+#pragma unroll
+  for (int i = 0; i < kMaxPhases; ++i)
+#pragma unroll
+    for (int j = i + 1; j < kMaxPhases; ++j)
       if (ph_id[j] < ph_id[i]) {
         int t = ph_id[i]; ph_id[i] = ph_id[j]; ph_id[j] = t;
         t = ph_cnt[i]; ph_cnt[i] = ph_cnt[j]; ph_cnt[j] = t;
       }
-  double nrm[3];
-  for (int d = 0; d < 3; ++d) nrm[d] = A.mat.mixed_normal[3 * m + d];
-  double Cs[kMaxPhases][36];
-  double fs[kMaxPhases];
-  for (int k = 0; k < nph; ++k) {
-    iso_full_t<double>(A.phase_lame[2 * ph_id[k]], A.phase_lame[2 * ph_id[k] + 1], dim, Cs[k]);
-    fs[k] = (double)ph_cnt[k] / (double)cell.M;
-  }
-  double Ct[36];
-  const int rule = apply_rule_t<double>(cell.rule, nph, Cs, fs, st.nrm_ok != 0, nrm, dim, Ct);
-  for (int I = 0; I < nc; ++I)
-    for (int J = I; J < nc; ++J) {
-      const double val = 0.5 * (Ct[I * nc + J] + Ct[J * nc + I]);
-      A.mat.mixed_c64[m * ns + packed_index(nc, I, J)] = val;
-      A.mat.mixed_c32[m * ns + packed_index(nc, I, J)] = (float)val;
+  double nrm[3] = {0.0, 0.0, 0.0};
+  bool layers = cell.rule == HOM_RULE_TWO_LAYER;
+  if (layers) {
+    const int n = cell.n;
+    long long v = A.mat.mixed_voxel[m] - cell.vox_off;
+    double x[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) {
+      const long long q = v / n;
+      x[d] = ((double)(v - q * n) + 0.5) / (double)n;
+      v = q;
     }
+    layers = layer_normal<DIM>(A.prims + cell.prim0, ns, st.nnear, x, nrm);  // else the Voigt rule
+  }
+  double lam[kMaxPhases], mu[kMaxPhases], fs[kMaxPhases];
+  double f_last = 0.0;
+  int last = 0;
+#pragma unroll
+  for (int k = 0; k < kMaxPhases; ++k) {
+    lam[k] = k < nph ? A.phase_lame[2 * ph_id[k]] : 0.0;
+    mu[k] = k < nph ? A.phase_lame[2 * ph_id[k] + 1] : 0.0;
+    fs[k] = k < nph ? (double)ph_cnt[k] / (double)cell.M : 0.0;
+    if (k < nph) {
+      f_last = fs[k];
+      last = ph_id[k];
+    }
+  }
+  double* c64 = A.mat.mixed_c64 + m * NS;
+  float* c32 = A.mat.mixed_c32 + m * NS;
+  if (layers) {
+    const Layered<double> ly = layered_moduli(lam, mu, fs);
+    const LayerBasis<DIM> lb(nrm);
+#pragma unroll
+    for (int I = 0; I < NC; ++I)
+#pragma unroll
+      for (int J = I; J < NC; ++J) {
+        const double val = lb.entry(ly, I, J);
+        c64[packed_index(NC, I, J)] = val;
+        c32[packed_index(NC, I, J)] = (float)val;
+      }
+  } else {
+    const Iso<double> is = cell.rule == HOM_RULE_REUSS ? reuss_moduli<kMaxPhases>(lam, mu, fs, nph, DIM)
+                                                       : voigt_moduli<kMaxPhases>(lam, mu, fs);
+#pragma unroll
+    for (int I = 0; I < NC; ++I)
+#pragma unroll
+      for (int J = I; J < NC; ++J) {
+        const double val = (I == J ? 2.0 * is.mu : 0.0) + (I < DIM && J < DIM ? is.lam : 0.0);
+        c64[packed_index(NC, I, J)] = val;
+        c32[packed_index(NC, I, J)] = (float)val;
+      }
+  }
   A.mat.mixed_phases[2 * m] = ph_id[0];
-  A.mat.mixed_phases[2 * m + 1] = ph_id[nph - 1];
-  A.mat.mixed_frac[m] = fs[nph - 1];
-  if (!(cell.rule == HOM_RULE_TWO_LAYER && rule == HOM_RULE_TWO_LAYER))
-    for (int d = 0; d < 3; ++d) A.mat.mixed_normal[3 * m + d] = 0.0;
+  A.mat.mixed_phases[2 * m + 1] = last;
+  A.mat.mixed_frac[m] = f_last;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) A.mat.mixed_normal[3 * m + d] = layers ? nrm[d] : 0.0;
 }
 
 }  // namespace
@@ -462,6 +576,9 @@ extern "C" int hom_filter_build(const hom_cell* cells, int32_t ncells, const hom
   const int dim = cells[0].dim;
   std::vector<FCell> fc(ncells);
   std::vector<FPrim> fp;
+  // sample lines of the filter balls (D1, D2, m): the ball's samples at those offsets across x are
+  // D0 = -m, -m + 2, .., m; one list per (subgrid, radius)
+  std::vector<int4> lines;
   long long vox = 0, blocks = 0;
   for (int c = 0; c < ncells; ++c) {
     const hom_cell& k = cells[c];
@@ -514,20 +631,31 @@ extern "C" int hom_filter_build(const hom_cell* cells, int32_t ncells, const hom
     for (int d = 0; d < dim; ++d) pw *= nt;
     if (k.rule != HOM_RULE_NONE && pw >= (1LL << 32))
       return set_error(HOM_ERR_UNSUPPORTED_SIZE, "cell %d: filter ball too large for the sampler (subgrid x radius)", c);
-    f.R2i = k.rule != HOM_RULE_NONE ? (int)std::floor(R2) : 0;
-    f.dnt = make_fastdiv((int)nt);
     f.M = 0;
-    if (k.rule != HOM_RULE_NONE) {
-      const long long tot = dim == 3 ? nt * nt * nt : nt * nt;
-      for (long long i = 0; i < tot; ++i) {
-        long long r = i, q = 0;
-        for (int d = 0; d < dim; ++d) {
-          const long long D = 2 * (r % nt + f.tlo) + 1 - k.subgrid;
-          q += D * D;
-          r /= nt;
+    f.line0 = (int)lines.size();
+    f.nline = 0;
+    int same = -1;
+    for (int c2 = 0; c2 < c && same < 0; ++c2)
+      if (fc[c2].nline > 0 && fc[c2].S == f.S && fc[c2].radius_px == f.radius_px) same = c2;
+    if (same >= 0 && k.rule != HOM_RULE_NONE) {
+      f.M = fc[same].M;
+      f.line0 = fc[same].line0;
+      f.nline = fc[same].nline;
+    } else if (k.rule != HOM_RULE_NONE) {
+      for (long long t2 = 0; t2 < (dim == 3 ? nt : 1); ++t2)
+        for (long long t1 = 0; t1 < nt; ++t1) {
+          const long long D1 = 2 * (t1 + f.tlo) + 1 - k.subgrid, D2 = dim == 3 ? 2 * (t2 + f.tlo) + 1 - k.subgrid : 0;
+          const long long rem = (long long)std::floor(R2) - D1 * D1 - D2 * D2;
+          if (rem < 0) continue;
+          long long m = (long long)std::sqrt((double)rem);
+          while (m * m > rem) --m;
+          while ((m + 1) * (m + 1) <= rem) ++m;
+          if (((m + k.subgrid) & 1) == 0) --m;  // D0 has the parity of S + 1
+          if (m < 0) continue;
+          lines.push_back(make_int4((int)D1, (int)D2, (int)m, 0));
+          f.M += (int)m + 1;
         }
-        if ((double)q <= R2) ++f.M;
-      }
+      f.nline = (int)lines.size() - f.line0;
     }
     const long long nv = (long long)k.n * k.n * (dim == 3 ? k.n : 1);
     vox += nv;
@@ -550,11 +678,12 @@ extern "C" int hom_filter_build(const hom_cell* cells, int32_t ncells, const hom
         pc32[(size_t)p * ns + packed_index(nc, I, J)] = (float)v;
       }
   }
-  // scratch: cells, prims, lame, counter, flag
+  // scratch: cells, prims, lame, counter, flag, sample lines
   const size_t b_cells = sizeof(FCell) * ncells, b_prims = sizeof(FPrim) * (fp.size() + 1),
                b_lame = sizeof(double) * lame.size();
   const size_t off_prims = (b_cells + 255) / 256 * 256, off_lame = off_prims + (b_prims + 255) / 256 * 256,
-               off_ctr = off_lame + (b_lame + 255) / 256 * 256, total = off_ctr + 256;
+               off_ctr = off_lame + (b_lame + 255) / 256 * 256, off_lines = off_ctr + 256,
+               total = off_lines + (lines.size() + 1) * sizeof(int4);
   void* ws = nullptr;
   int rc = get_workspace(total, &ws);
   if (rc != HOM_OK) return rc;
@@ -563,6 +692,7 @@ extern "C" int hom_filter_build(const hom_cell* cells, int32_t ncells, const hom
   std::memcpy(host.data(), fc.data(), b_cells);
   if (!fp.empty()) std::memcpy(host.data() + off_prims, fp.data(), sizeof(FPrim) * fp.size());
   std::memcpy(host.data() + off_lame, lame.data(), b_lame);
+  if (!lines.empty()) std::memcpy(host.data() + off_lines, lines.data(), lines.size() * sizeof(int4));
   HOM_CUDA_TRY(cudaMemcpyAsync(w, host.data(), total, cudaMemcpyHostToDevice, st));
   HOM_CUDA_TRY(cudaMemcpyAsync(mat->phase_c64, pc64.data(), pc64.size() * sizeof(double), cudaMemcpyHostToDevice, st));
   HOM_CUDA_TRY(cudaMemcpyAsync(mat->phase_c32, pc32.data(), pc32.size() * sizeof(float), cudaMemcpyHostToDevice, st));
@@ -570,6 +700,7 @@ extern "C" int hom_filter_build(const hom_cell* cells, int32_t ncells, const hom
   args.cells = reinterpret_cast<const FCell*>(w);
   args.ncells = ncells;
   args.prims = reinterpret_cast<const FPrim*>(w + off_prims);
+  args.lines = reinterpret_cast<const int4*>(w + off_lines);
   args.phase_lame = reinterpret_cast<const double*>(w + off_lame);
   args.nphase = nphase;
   args.mat = *mat;
@@ -577,12 +708,14 @@ extern "C" int hom_filter_build(const hom_cell* cells, int32_t ncells, const hom
   args.err_flag = reinterpret_cast<int*>(w + off_ctr + 8);
   if (blocks > 0x7fffffffLL) return set_error(HOM_ERR_UNSUPPORTED_SIZE, "batch too large");
   args.mat.dim = dim;
-  k_filter<<<(unsigned)blocks, kThreads, 0, st>>>(args);
+  if (dim == 2) k_filter<2><<<(unsigned)blocks, kThreads, 0, st>>>(args);
+  else k_filter<3><<<(unsigned)blocks, kThreads, 0, st>>>(args);
   HOM_CUDA_TRY(cudaGetLastError());
   if (mat->mixed_capacity > 0) {
     const long long rblocks = (mat->mixed_capacity + kThreads - 1) / kThreads;
     if (rblocks > 0x7fffffffLL) return set_error(HOM_ERR_UNSUPPORTED_SIZE, "mixed table too large");
-    k_filter_rule<<<(unsigned)rblocks, kThreads, 0, st>>>(args);
+    if (dim == 2) k_filter_rule<2><<<(unsigned)rblocks, kThreads, 0, st>>>(args);
+    else k_filter_rule<3><<<(unsigned)rblocks, kThreads, 0, st>>>(args);
     HOM_CUDA_TRY(cudaGetLastError());
   }
   struct { unsigned long long cnt; int flag; int pad; } res{};

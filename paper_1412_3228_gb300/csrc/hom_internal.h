@@ -106,10 +106,10 @@ struct FCell {           // one cell of the filter build
   long long block0;      // first thread block of this cell
   float inv_n;           // 1 / n rounded to FP32
   float reach32;         // filter radius in cell units (r / n) rounded to FP32
-  int R2i;               // (2 S r)^2 rounded down: a fine point is in the ball iff sum D^2 <= R2i
   int tlo, thi;          // range of the fine-point offsets t that can fall in a ball
   int M;                 // fine points per ball
-  FastDiv dn, dnt;       // dividers by n and by thi - tlo + 1
+  int line0, nline;      // the ball's sample lines
+  FastDiv dn;            // divider by n
 };
 struct FPrim {
   int kind, phase, axis, pad;
