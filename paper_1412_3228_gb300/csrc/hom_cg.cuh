@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(kCgCtlThreads) k_cg_control(SolveArgs A, CgArg
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
-    const unsigned prev = atomicAdd(A.done, 1u);
+    const unsigned prev = (unsigned)atomicAdd(A.done, 1ull);
     s_last = prev == gridDim.x - 1;
   }
   __syncthreads();
@@ -306,7 +306,7 @@ __global__ void __launch_bounds__(kCgCtlThreads) k_cg_control(SolveArgs A, CgArg
       for (int i = 0; i < (int)(blockDim.x >> 5); ++i) tot += s_cnt[i];
       *A.nactive = tot;
       *A.it_dev = it + 1;
-      *A.done = 0u;
+      *A.done = 0ull;
     }
   }
 }

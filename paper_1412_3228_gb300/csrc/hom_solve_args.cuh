@@ -45,7 +45,7 @@ struct SolveArgs {
   int* best_it;
   int* it_dev;
   int* nactive;
-  unsigned int* done;
+  unsigned long long* done;  // control kernel: arrivals (low half), active pairs (high half)
   unsigned long long* bytes;  // [HOM_NKERNEL]
   int L, criterion, max_iter, diverge_window, stall_window;
   int green;  // HOM_GREEN_CONTINUOUS or HOM_GREEN_ROTATED

@@ -661,131 +661,148 @@ __global__ void __launch_bounds__(kThreads) k_ypass(SolveArgs A) {
 // One CTA per (cell, load): FP64 sums of the pair's partials (per-task partials of the row pass
 // and of the Green pass, summed in a fixed order: deterministic), equilibrium errors, stopping
 // rule.  The last CTA to finish counts the active pairs and advances the iteration.
-constexpr int kCtlThreads = 128;
-__global__ void __launch_bounds__(kCtlThreads) k_control(SolveArgs A, int nc) {
-  __shared__ bool s_last;
-  __shared__ double s_red[kCtlThreads / 32][9];
-  __shared__ int s_cnt[kCtlThreads / 32];
+// Bound by latency: a chain of a few dependent loads, FP64 sums and FP64 divisions.  Each thread keeps
+// several tasks' loads in flight, the CTA grows with the pair's task count (ctl_threads: 4590 + 4590
+// tasks of a 135^3 pair on 128 threads took 56 us, on 1024 32 us), and the scalar FP64 chain
+// (square roots and divisions, hundreds of cycles each) runs side by side in the lanes of one warp
+// instead of one after the other in one thread (45^2, 3 pairs: 13.0 us, now 8.6 us).
+constexpr int kCtlMaxThreads = 1024;
+inline unsigned ctl_threads(int most_tasks) {
+  unsigned t = 128;
+  while (t < (unsigned)kCtlMaxThreads && (int)t * 4 < most_tasks) t *= 2;
+  return t;
+}
+template <int NC>
+__global__ void __launch_bounds__(kCtlMaxThreads) k_control(SolveArgs A) {
+  __shared__ double s_red[kCtlMaxThreads / 32][NC + 3];
   const int pair = blockIdx.x;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nthr = blockDim.x, nw = nthr >> 5;
   const int it = *A.it_dev;
+  int still = 0;  // thread 0: the pair stays active
   if (A.active[pair]) {
     const PairDev pr = A.pairs[pair];
-    const CellDev c = A.cells[pr.cell];
-    // v[0..nc): sigma sums, v[6]: residual sum, v[7]: normalised residual sum, v[8]: compatibility
-    // residual sum (Eyre-Milton scheme)
-    double v[9];
+    // v[0..NC): sigma sums, v[NC]: residual sum, v[NC + 1]: normalised residual sum, v[NC + 2]:
+    // compatibility residual sum (Eyre-Milton scheme)
+    double v[NC + 3];
 #pragma unroll
-    for (int k = 0; k < 9; ++k) v[k] = 0.0;
-    for (int tk = pr.rtask0 + (int)threadIdx.x; tk < pr.rtask1; tk += kCtlThreads) {
-      const double* p = A.partR + ((size_t)tk * A.L + pr.load) * nc;
-      for (int k = 0; k < nc; ++k) v[k] += p[k];
+    for (int k = 0; k < NC + 3; ++k) v[k] = 0.0;
+    const double* pR = A.partR + (size_t)pr.load * NC;
+    const size_t rs = (size_t)A.L * NC;
+#pragma unroll 4
+    for (int tk = pr.rtask0 + (int)threadIdx.x; tk < pr.rtask1; tk += nthr) {
+      const double* p = pR + (size_t)tk * rs;
+#pragma unroll
+      for (int k = 0; k < NC; ++k) v[k] += p[k];
     }
-    for (int tk = pr.ctask0 + (int)threadIdx.x; tk < pr.ctask1; tk += kCtlThreads) {
-      v[6] += A.partC[2 * (size_t)tk];
-      v[7] += A.partC[2 * (size_t)tk + 1];
-      if (A.partE) v[8] += A.partE[tk];
+    const double2* pC = reinterpret_cast<const double2*>(A.partC);
+    const bool em = A.partE != nullptr;
+#pragma unroll 4
+    for (int tk = pr.ctask0 + (int)threadIdx.x; tk < pr.ctask1; tk += nthr) {
+      const double2 q = pC[tk];
+      v[NC] += q.x;
+      v[NC + 1] += q.y;
+      if (em) v[NC + 2] += A.partE[tk];
     }
 #pragma unroll
-    for (int k = 0; k < 9; ++k)
-      for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
+    for (int k = 0; k < NC + 3; ++k)
+      if (k < NC + 2 || em)
+        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
     if (lane == 0)
 #pragma unroll
-      for (int k = 0; k < 9; ++k) s_red[wid][k] = v[k];
+      for (int k = 0; k < NC + 3; ++k) s_red[wid][k] = v[k];
     __syncthreads();
-    if (threadIdx.x == 0) {
-      double sum[9];
-      for (int k = 0; k < 9; ++k) {
-        sum[k] = 0.0;
-        for (int w = 0; w < kCtlThreads / 32; ++w) sum[k] += s_red[w][k];
+    if (wid == 0) {
+      const double nv = (double)A.cells[pr.cell].nv;
+      double sum = 0.0;  // lane k: total k
+      if (lane < NC + 3)
+        for (int w = 0; w < nw; ++w) sum += s_red[w][lane];
+      double den2 = 0.0, e2 = 0.0;
+#pragma unroll
+      for (int k = 0; k < NC; ++k) {
+        const double x = __shfl_sync(0xffffffffu, sum, k);
+        den2 += x * x;
       }
-      double den2 = 0.0;
-      for (int k = 0; k < nc; ++k) {
-        A.mean_sigma[(size_t)pair * nc + k] = sum[k] / (double)c.nv;
-        den2 += sum[k] * sum[k];
+      if (em && lane == NC + 2) {
+        const double* Ep = A.E + (size_t)pair * NC;
+        for (int k = 0; k < NC; ++k) e2 += Ep[k] * Ep[k];
       }
-      const double r2 = sum[6], rn2 = sum[7];
-      double e, en;
-      if (A.res0) {  // adjoint: relative to the first iterate's residual
-        if (it == 0) {
-          A.res0[2 * pair] = r2;
-          A.res0[2 * pair + 1] = rn2;
+      // lanes 0 .. NC - 1: the mean stress; NC and NC + 1: e and e_n; NC + 2: e_c
+      double num = sum, den = nv;
+      if (lane >= NC && lane < NC + 3) {
+        if (A.res0 && lane < NC + 2) {  // adjoint: relative to the first iterate's residual
+          double* r0 = A.res0 + 2 * pair + (lane - NC);
+          if (it == 0) *r0 = sum;
+          den = *r0;
+          num = den > 0.0 ? sum / den : 0.0;
+          den = 1.0;
+        } else if (lane < NC + 2) {
+          den = den2;
+        } else {
+          den = e2;
         }
-        const double d0 = A.res0[2 * pair], d1 = A.res0[2 * pair + 1];
-        e = d0 > 0.0 ? sqrt(r2 / d0) : 0.0;
-        en = d1 > 0.0 ? sqrt(rn2 / d1) : 0.0;
-      } else {
-        const double den = sqrt(den2);
-        e = sqrt(r2) / den;
-        en = sqrt(rn2) / den;
+        num = sqrt(num);
+        den = sqrt(den) * (lane == NC + 2 ? nv : 1.0);
       }
-      A.err[pair] = e;
-      A.errn[pair] = en;
-      double crit = A.criterion == HOM_CRIT_E ? e : en;
-      if (A.partE) {  // Eyre-Milton: e_c = |eps_hat - P eps_hat| / (N_v |E|) must pass too
-        const double* Ep = A.E + (size_t)pair * nc;
-        double e2 = 0.0;
-        for (int k = 0; k < nc; ++k) e2 += Ep[k] * Ep[k];
-        const double ec = sqrt(sum[8]) / ((double)c.nv * sqrt(e2));
-        A.errc[pair] = ec;
-        crit = fmax(crit, ec);
-        if (!isfinite(ec)) crit = ec;
-      }
-      int st = -1;
-      const bool skip = A.warm && it == 0;  // warm start: g of the caller's field is unknown
-      if (A.hist && !A.inner && it <= A.max_iter)
-        A.hist[(size_t)pair * (A.max_iter + 1) + it] = skip ? (double)NAN : crit;
-      if (A.inner) {  // defect-correction inner solve: a fixed number of iterations, no error test
-        if (it >= A.kinner[pair]) st = HOM_STATUS_MAX_ITER;
-      } else if (skip) {
-        if (it >= A.max_iter) st = HOM_STATUS_MAX_ITER;
-      } else if (!isfinite(crit)) st = HOM_STATUS_DIVERGED;
-      else if (crit < A.tol) st = HOM_STATUS_CONVERGED;
-      else if (it >= A.max_iter) st = HOM_STATUS_MAX_ITER;
-      else {
-        if (A.diverge_window > 0) {
-          int gcount = crit > A.last_err[pair] ? A.grow[pair] + 1 : 0;
-          A.grow[pair] = gcount;
-          if (gcount >= A.diverge_window) st = HOM_STATUS_DIVERGED;
+      const double q = num / den;
+      if (lane < NC) A.mean_sigma[(size_t)pair * NC + lane] = q;
+      const double e = __shfl_sync(0xffffffffu, q, NC), en = __shfl_sync(0xffffffffu, q, NC + 1),
+                   ec = __shfl_sync(0xffffffffu, q, NC + 2);
+      if (lane == 0) {
+        A.err[pair] = e;
+        A.errn[pair] = en;
+        double crit = A.criterion == HOM_CRIT_E ? e : en;
+        if (em) {  // Eyre-Milton: e_c = |eps_hat - P eps_hat| / (N_v |E|) must pass too
+          A.errc[pair] = ec;
+          crit = fmax(crit, ec);
+          if (!isfinite(ec)) crit = ec;
         }
-        // stagnation: no new smallest error for stall_window iterations (the FP32 floor)
-        if (st < 0 && A.stall_window > 0) {
-          if (crit < A.best_err[pair]) {
-            A.best_err[pair] = crit;
-            A.best_it[pair] = it;
-          } else if (it - A.best_it[pair] >= A.stall_window) {
-            st = HOM_STATUS_STALLED;
+        int st = -1;
+        const bool skip = A.warm && it == 0;  // warm start: g of the caller's field is unknown
+        if (A.hist && !A.inner && it <= A.max_iter)
+          A.hist[(size_t)pair * (A.max_iter + 1) + it] = skip ? (double)NAN : crit;
+        if (A.inner) {  // defect-correction inner solve: a fixed number of iterations, no error test
+          if (it >= A.kinner[pair]) st = HOM_STATUS_MAX_ITER;
+        } else if (skip) {
+          if (it >= A.max_iter) st = HOM_STATUS_MAX_ITER;
+        } else if (!isfinite(crit)) st = HOM_STATUS_DIVERGED;
+        else if (crit < A.tol) st = HOM_STATUS_CONVERGED;
+        else if (it >= A.max_iter) st = HOM_STATUS_MAX_ITER;
+        else {
+          if (A.diverge_window > 0) {
+            int gcount = crit > A.last_err[pair] ? A.grow[pair] + 1 : 0;
+            A.grow[pair] = gcount;
+            if (gcount >= A.diverge_window) st = HOM_STATUS_DIVERGED;
+          }
+          // stagnation: no new smallest error for stall_window iterations (the FP32 floor)
+          if (st < 0 && A.stall_window > 0) {
+            if (crit < A.best_err[pair]) {
+              A.best_err[pair] = crit;
+              A.best_it[pair] = it;
+            } else if (it - A.best_it[pair] >= A.stall_window) {
+              st = HOM_STATUS_STALLED;
+            }
           }
         }
-      }
-      if (!skip) A.last_err[pair] = crit;
-      if (st >= 0) {
-        A.status[pair] = st;
-        A.iters[pair] = it;
-        A.active[pair] = 0;
+        if (!skip) A.last_err[pair] = crit;
+        if (st >= 0) {
+          A.status[pair] = st;
+          A.iters[pair] = it;
+          A.active[pair] = 0;
+        } else {
+          still = 1;
+        }
       }
     }
   }
-  __syncthreads();
   if (threadIdx.x == 0) {
-    __threadfence();
-    const unsigned prev = atomicAdd(A.done, 1u);
-    s_last = prev == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (s_last) {
-    __threadfence();
-    int cnt = 0;
-    for (int p = threadIdx.x; p < A.npairs; p += blockDim.x) cnt += ((volatile int*)A.active)[p] ? 1 : 0;
-    for (int o = 16; o > 0; o >>= 1) cnt += __shfl_down_sync(0xffffffffu, cnt, o);
-    if (lane == 0) s_cnt[wid] = cnt;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int tot = 0;
-      for (int i = 0; i < (int)(blockDim.x >> 5); ++i) tot += s_cnt[i];
+    // arrivals in the low half, active pairs in the high half: the last CTA has both
+    const unsigned long long mine = 1ull + ((unsigned long long)still << 32);
+    const unsigned long long all = atomicAdd(A.done, mine) + mine;
+    if ((unsigned)all == gridDim.x) {
+      const int tot = (int)(all >> 32);
       *A.nactive = tot;
       *A.it_dev = it + 1;
-      *A.done = 0u;
+      *A.done = 0ull;
       // whole-solve graph: run another iteration while a pair is active and the budget allows
       // (the host loop's bound: at most max_iter + 1 iterations)
       if (A.use_cond) cudaGraphSetConditional(A.cond, (tot > 0 && it + 1 <= A.max_iter) ? 1u : 0u);
@@ -1046,7 +1063,7 @@ __global__ void k_init_pairs_masked(SolveArgs A, const int* mask) {
     for (int q = 0; q < A.npairs; ++q) cnt += mask[q] ? 1 : 0;
     *A.it_dev = 0;
     *A.nactive = cnt;
-    *A.done = 0u;
+    *A.done = 0ull;
   }
 }
 
@@ -1064,7 +1081,7 @@ __global__ void k_init_pairs(SolveArgs A) {
   if (p == 0) {
     *A.it_dev = 0;
     *A.nactive = A.npairs;
-    *A.done = 0u;
+    *A.done = 0ull;
   }
 }
 
@@ -1101,6 +1118,20 @@ struct Layout {
 };
 
 
+// The control kernel's arrival word: 64 bits after the pair bookkeeping of npairs pairs at `ib`.
+unsigned long long* done_word(int* ib, int npairs) {
+  return reinterpret_cast<unsigned long long*>((reinterpret_cast<uintptr_t>(ib + 5 * npairs + 2) + 7) & ~(uintptr_t)7);
+}
+
+// Most tasks of one pair in one pass (sizes the control kernel's CTAs).
+int most_tasks(const Layout& lay) {
+  int m = 1;
+  for (const PairDev& p : lay.pairs) m = std::max(m, std::max(p.rtask1 - p.rtask0, p.ctask1 - p.ctask0));
+  return m;
+}
+
+template <int DIM> constexpr int nc_of_dim() { return DIM == 2 ? 3 : 6; }
+
 long long vox_total(const Layout& lay) {
   long long v = 0;
   for (const CellDev& c : lay.cells) v += c.nv;
@@ -1126,6 +1157,18 @@ TaskL make_task(int cell, int load, int kx0, int ntk, int fixed, int nc, int dim
 constexpr size_t kGreenBudget = (size_t)110 * 1024;
 constexpr size_t kRowBudget = (size_t)96 * 1024;
 
+// A batch of few or small cells leaves most of the chip idle when every CTA takes as much as its
+// shared memory holds: below kFewTasks tasks in a pass (four per SM) the tasks are made smaller, down
+// to one row (two where they pair up) or one kx column, or one load per row task on the specialised
+// passes.  Measured (us per launch): the 61 cells of an FP64 convergence study: row 142 -> 111, Green 170
+// -> 146; 45^2 FP32 on the specialised passes: row 18.7 -> 13.8.
+constexpr size_t kFewTasks = 4 * 152;
+// Rows (or columns) per task, at most `fit`, that bring the pass's tasks (total at `fit`) near kFewTasks.
+int spread(int fit, size_t total) {
+  if (total >= kFewTasks || fit <= 1) return fit;
+  return (int)std::max<size_t>(1, fit * total / kFewTasks);
+}
+
 int build_layout(const hom_cell* cells, int ncells, int L, int dim, size_t vsize, int max_radix, const double* c0,
                  bool external, Layout& lay, bool em = false) {
   const int nc = nc_of(dim);
@@ -1139,6 +1182,30 @@ int build_layout(const hom_cell* cells, int ncells, int L, int dim, size_t vsize
   }
   long long vox = 0;
   std::vector<int> plan_n;
+  // rows per row task and kx columns per Green/y task that fit on chip, and the passes' tasks with them
+  auto row_lines = [&](int rows) { return (size_t)((rows * L * nc + 1) / 2) + 1; };
+  auto rows_fit = [&](int n) {
+    const int nrows = dim == 2 ? n : n * n;
+    const size_t line_bytes = (size_t)n * vsize;  // one line; the twiddle table is one more
+    int r = 1;
+    while (r < nrows &&
+           row_lines(r + 1) * line_bytes + (size_t)(r + 1) * L * nc * (sizeof(long long) + vsize) <= budget)
+      ++r;
+    return lay.fast ? std::min(kFastRows, nrows) : r;
+  };
+  auto cols_fit = [&](int n) {
+    const size_t line_bytes = (size_t)n * vsize, gbudget = kGreenBudget;
+    int ntk = (int)std::max<size_t>(1, (gbudget - std::min(gbudget, 2 * line_bytes)) / ((size_t)nc * line_bytes));
+    return std::min(lay.fast ? kFastCols : ntk, n / 2 + 1);
+  };
+  std::vector<int> task_rows, task_cols;
+  size_t row_total = 0, col_total = 0;
+  for (int ci = 0; ci < ncells; ++ci) {
+    const int n = cells[ci].n, r = rows_fit(n), q = cols_fit(n);
+    row_total += ((size_t)(dim == 2 ? n : n * n) + r - 1) / r;
+    col_total += (size_t)(n / 2 + q) / q * L * (dim == 2 ? 1 : n);
+  }
+  const bool split_loads = lay.fast && L > 1 && row_total < kFewTasks;
   for (int ci = 0; ci < ncells; ++ci) {
     const hom_cell& k = cells[ci];
     CellDev c{};
@@ -1218,48 +1285,69 @@ int build_layout(const hom_cell* cells, int ncells, int L, int dim, size_t vsize
     lay.ws_elems += (size_t)L * c.nrows * c.Hp * nc;
     lay.g_elems += (size_t)L * c.nrows * c.Hp * (em ? nc : dim);  // EM: u_hat (nc) instead of g (dim)
     // row-pass tasks: as many rows as fit in the shared-memory budget with every load active
-    const size_t line_bytes = (size_t)k.n * vsize;  // one line; the twiddle table is one more
-    auto row_lines = [&](int rows) { return (size_t)((rows * L * nc + 1) / 2) + 1; };
-    int r = 1;
-    while (r < c.nrows &&
-           row_lines(r + 1) * line_bytes + (size_t)(r + 1) * L * nc * (sizeof(long long) + vsize) <= budget)
-      ++r;
-    if (lay.fast) r = std::min(kFastRows, c.nrows);
+    const size_t line_bytes = (size_t)k.n * vsize;
+    int r = rows_fit(k.n);
+    if (!lay.fast) {
+      const int fit = r;
+      r = spread(fit, row_total);
+      // an odd number of real rows leaves half of a complex line empty (405^2 FP64, 3 loads: tasks of one
+      // row, 9 real rows, took 329 us, tasks of 3 rows 288)
+      if (r < fit && (r & 1) && (L * nc & 1)) ++r;
+    }
     const size_t need_r = row_lines(r) * line_bytes + (size_t)r * L * nc * (sizeof(long long) + 2 * vsize / 2);
     if (need_r > kMaxSmem) return set_error(HOM_ERR_UNSUPPORTED_SIZE, "row of n = %d with %d loads does not fit on chip", k.n, L);
     lay.smem_row = std::max(lay.smem_row, need_r);
-    // row tasks: every load per task (one load per task measured 3 % slower on the 2D sweep)
-    c.rtask0 = (int)lay.tR.size();
-    std::vector<int> rt0(L, c.rtask0), rt1(L, c.rtask0);
-    if (lay.fast && dim == 3) {  // groups of 4 rows (consecutive y) within each z plane, every load
-      for (int z = 0; z < k.n; ++z)
-        for (int y0 = 0; y0 < k.n; y0 += r) lay.tR.push_back(TaskR{ci, z * k.n + y0, std::min(r, k.n - y0), -1});
-    } else {  // every load per task: labels and twiddles are shared across the loads
-      for (int r0 = 0; r0 < c.nrows; r0 += r) lay.tR.push_back(TaskR{ci, r0, std::min(r, c.nrows - r0), -1});
-    }
-    for (int l = 0; l < L; ++l) rt1[l] = (int)lay.tR.size();
-    c.rtask1 = (int)lay.tR.size();
-    // Green-pass and y-pass tiles of kx
-    // Green/y tiles: ntk kx columns x nc lines, plus the twiddle table and the wave-number table
-    const size_t gbudget = kGreenBudget;
-    int ntk = (int)std::max<size_t>(1, (gbudget - std::min(gbudget, 2 * line_bytes)) / ((size_t)nc * line_bytes));
-    if (lay.fast) ntk = kFastCols;
-    ntk = std::min(ntk, c.H);
+    const int ntk = lay.fast ? cols_fit(k.n) : spread(cols_fit(k.n), col_total);
     const size_t need_l = ((size_t)ntk * nc + 2) * line_bytes;
     lay.smem_green = std::max(lay.smem_green, need_l);
     lay.smem_y = std::max(lay.smem_y, need_l);
+    task_rows.push_back(r);
+    task_cols.push_back(ntk);
+    lay.cells.push_back(c);
+  }
+  // tasks, largest grids first: the small cells' tasks fill the end of each launch
+  std::vector<int> order(ncells);
+  for (int ci = 0; ci < ncells; ++ci) order[ci] = ci;
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cells[a].n > cells[b].n; });
+  lay.pairs.resize((size_t)ncells * L);
+  for (int ci : order) {
+    const hom_cell& k = cells[ci];
+    CellDev& c = lay.cells[ci];
+    const int r = task_rows[ci], ntk = task_cols[ci];
+    // row tasks: every load per task (one load per task measured 3 % slower on the 2D sweep: labels and
+    // twiddles are shared across the loads), or one load per task where the batch has few (split_loads)
+    c.rtask0 = (int)lay.tR.size();
+    std::vector<int> rt0(L, c.rtask0), rt1(L, c.rtask0);
+    for (int l = 0; l < (split_loads ? L : 1); ++l) {
+      rt0[l] = (int)lay.tR.size();
+      const int load = split_loads ? l : -1;
+      if (lay.fast && dim == 3) {  // groups of 4 rows (consecutive y) within each z plane
+        for (int z = 0; z < k.n; ++z)
+          for (int y0 = 0; y0 < k.n; y0 += r) lay.tR.push_back(TaskR{ci, z * k.n + y0, std::min(r, k.n - y0), load});
+      } else {
+        for (int r0 = 0; r0 < c.nrows; r0 += r) lay.tR.push_back(TaskR{ci, r0, std::min(r, c.nrows - r0), load});
+      }
+      rt1[l] = (int)lay.tR.size();
+    }
+    if (!split_loads)
+      for (int l = 1; l < L; ++l) {
+        rt0[l] = rt0[0];
+        rt1[l] = rt1[0];
+      }
+    c.rtask1 = (int)lay.tR.size();
+    // Green-pass and y-pass tiles of kx: ntk kx columns x nc lines, plus the twiddle table and the
+    // wave-number table
     for (int l = 0; l < L; ++l) {
       PairDev pd{ci, l, (int)lay.tC.size(), 0, rt0[l], rt1[l]};
       const int nfix = dim == 2 ? 1 : k.n;
       for (int f = 0; f < nfix; ++f)
         for (int kx0 = 0; kx0 < c.H; kx0 += ntk) lay.tC.push_back(make_task(ci, l, kx0, std::min(ntk, c.H - kx0), f, nc, dim));
       pd.ctask1 = (int)lay.tC.size();
-      lay.pairs.push_back(pd);
+      lay.pairs[(size_t)ci * L + l] = pd;
       if (dim == 3)
         for (int z = 0; z < k.n; ++z)
           for (int kx0 = 0; kx0 < c.H; kx0 += ntk) lay.tY.push_back(make_task(ci, l, kx0, std::min(ntk, c.H - kx0), z, nc, dim));
     }
-    lay.cells.push_back(c);
   }
   return HOM_OK;
 }
@@ -1444,7 +1532,7 @@ int refine_solve(SolveArgs& A, unsigned char* ws, int npairs, int nc, const hom_
       X.best_it = ib + 4 * npairs;
       X.it_dev = ib + 5 * npairs;
       X.nactive = ib + 5 * npairs + 1;
-      X.done = reinterpret_cast<unsigned int*>(ib + 5 * npairs + 2);
+      X.done = done_word(ib, npairs);
       double* db = reinterpret_cast<double*>(ws + o_dbl2) + (size_t)which * npairs * (4 + nc);
       X.err = db;
       X.errn = db + npairs;
@@ -1485,19 +1573,20 @@ int refine_solve(SolveArgs& A, unsigned char* ws, int npairs, int nc, const hom_
       if ((rc = allow_smem(k_ypass<double, false, 15>, smem_y64)) != HOM_OK) return rc;
     }
     const unsigned nR = (unsigned)lay.tR.size(), nC = (unsigned)lay.tC.size(), nY = (unsigned)lay.tY.size();
+    const unsigned nctl = ctl_threads(most_tasks(lay));
     auto iter64 = [&]() {
       k_row<double, DIM, false, 15><<<nR, kThreads, smem_row64, st>>>(A64);
       if (DIM == 3) k_ypass<double, true, 15><<<nY, kThreads, smem_y64, st>>>(A64);
       k_green<double, DIM, 15><<<nC, kThreads, smem_green64, st>>>(A64);
       if (DIM == 3) k_ypass<double, false, 15><<<nY, kThreads, smem_y64, st>>>(A64);
-      k_control<<<(unsigned)npairs, kCtlThreads, 0, st>>>(A64, nc);
+      k_control<nc_of_dim<DIM>()><<<(unsigned)npairs, nctl, 0, st>>>(A64);
     };
     auto iter32 = [&]() {
       k_row<float, DIM, false, MAXR><<<nR, kThreads, lay.smem_row, st>>>(Ain);
       if (DIM == 3) k_ypass<float, true, MAXR><<<nY, kThreads, lay.smem_y, st>>>(Ain);
       k_green<float, DIM, MAXR><<<nC, kThreads, lay.smem_green, st>>>(Ain);
       if (DIM == 3) k_ypass<float, false, MAXR><<<nY, kThreads, lay.smem_y, st>>>(Ain);
-      k_control<<<(unsigned)npairs, kCtlThreads, 0, st>>>(Ain, nc);
+      k_control<nc_of_dim<DIM>()><<<(unsigned)npairs, nctl, 0, st>>>(Ain);
     };
     const dim3 eg(64, (unsigned)npairs);
     float2* e32a = static_cast<float2*>(A.eps[0]);
@@ -1798,7 +1887,7 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
   A.best_it = ib + 4 * npairs;
   A.it_dev = ib + 5 * npairs;
   A.nactive = ib + 5 * npairs + 1;
-  A.done = reinterpret_cast<unsigned int*>(ib + 5 * npairs + 2);
+  A.done = done_word(ib, npairs);
   double* db = reinterpret_cast<double*>(ws + o_dbl);
   A.err = db;
   A.errn = db + npairs;
@@ -1872,7 +1961,7 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
   Timer tm{out->stats, st, {}};
   const unsigned nR = (unsigned)lay.tR.size(), nC = (unsigned)lay.tC.size(), nY = (unsigned)lay.tY.size();
   NvtxRange nvtx_init_("hom_solve: initial state");
-  const unsigned nCtl = (unsigned)npairs;  // one control CTA per (cell, load)
+  const unsigned nCtl = (unsigned)npairs, nctl = ctl_threads(most_tasks(lay));  // one control CTA per (cell, load)
   tm.begin(HOM_K_INIT);
   k_init_pairs<<<(npairs + 255) / 256, 256, 0, st>>>(A);
   if (em) {
@@ -1938,7 +2027,7 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
       k_cg_control<kCgUpdate><<<nCtl, kCgCtlThreads, 0, st>>>(A, G, nc);
       k_cg_elems<T, DIM, kCgDir><<<cg_grid, kCgThreads, 0, st>>>(A, G);
     } else {
-      k_control<<<nCtl, kCtlThreads, 0, st>>>(A, nc);
+      k_control<nc_of_dim<DIM>()><<<nCtl, nctl, 0, st>>>(A);
     }
     tm.end();
   };
@@ -1966,7 +2055,7 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
     SolveArgs K = A;  // the output buffers are not used by the iterations: not part of the key
     K.out_eps = K.out_sig = nullptr;
     std::string key(reinterpret_cast<const char*>(&K), sizeof(K));
-    const size_t dims[] = {nR, nC, nY, nCtl, lay.smem_row, lay.smem_green, lay.smem_y, smem_frow, smem_fgreen,
+    const size_t dims[] = {nR, nC, nY, nCtl, nctl, lay.smem_row, lay.smem_green, lay.smem_y, smem_frow, smem_fgreen,
                            smem_fy, (size_t)lay.fast, (size_t)DIM, sizeof(T), (size_t)MAXR};
     key.append(reinterpret_cast<const char*>(dims), sizeof(dims));
     cudaGraphExec_t gexec = find_graph(dev, key);
