@@ -26,6 +26,7 @@
 #define HOM_FILE_ID 2
 #include <algorithm>
 #include <cstring>
+#include <functional>
 #include <mutex>
 #include <vector>
 
@@ -38,20 +39,8 @@
 namespace hom {
 namespace {
 
-#ifndef HOM_GREEN_TW2
-#define HOM_GREEN_TW2 1  // Green pass with a scalar twiddle table (three CTAs per SM)
-#endif
-#ifndef HOM_ROW_TW2
-#define HOM_ROW_TW2 1    // row pass with a scalar twiddle table (three CTAs per SM)
-#endif
-#ifndef HOM_ROW_LANDING
-#define HOM_ROW_LANDING 1  // row pass: rows land by cp.async in their line slots (0: register loads)
-#endif
 #ifndef HOM_ROW_PREFETCH
 #define HOM_ROW_PREFETCH 0  // row pass L2 prefetch: 1 = the next load, 2 = the next task (bit mask)
-#endif
-#ifndef HOM_GREEN_BULK
-#define HOM_GREEN_BULK 1  // Green pass: its contiguous tile in and out by one bulk copy each (TMA unit)
 #endif
 #ifndef HOM_GREEN_GPF
 #define HOM_GREEN_GPF 1  // Green pass: L2 prefetch of the task's own g (or u_hat) block before its forward FFT
@@ -74,11 +63,6 @@ __device__ __forceinline__ size_t tile_index(const CellDev& c, int n, int l, int
 constexpr uint32_t kLabel8Mixed = 255;  // one-byte label of a mixed voxel
 
 constexpr int kRowSpare = 2 * NP * kFastRows;  // float4 entries of the row pass's spare landing area
-template <int N>
-__device__ __forceinline__ float4* row_slot(float4* s, float4* spare, int p, int k, int r) {
-  return row_slot_p<N, NP, NP>(s, spare, p, k, r);
-}
-
 // ------------------------------------------------------------------ row pass
 // eps (stored x half-spectra) -> inverse x-DFT -> tau = sigma - c0 : eps -> forward x-DFT -> tau.
 // OUT: the final fields eps and sigma of the returned iterate (real, solver output layout).
@@ -92,11 +76,12 @@ struct RowShared {
 // (lam - lam0, 2 mu - 2 mu0)); a mixed group first solves eps = (c~ + c0)^-1 u per voxel and takes
 // tau = c~ : eps - c0 : eps; the output pass turns u into eps first; the row sums of sigma are
 // (tau + u) / 2.
-template <int N, bool OUT, bool SRC, bool EM = false>
-__device__ __forceinline__ void row_body(const SolveArgs& A, int task, const TaskR& t, const CellDev& c,
+template <bool OUT, bool SRC, bool EM, class PL>
+__device__ __forceinline__ void row_body(const PL& pl, const SolveArgs& A, int task, const TaskR& t, const CellDev& c,
                                          const FastPlanDev& fp, float4* s, RowShared& sh) {
-  constexpr int H = (N + 1) / 2;
-  constexpr int P = (H + 1) / 2;  // kx pairs holding data
+  const int N = pl.n;
+  const int H = N / 2 + 1;
+  const int P = (H + 1) / 2;  // kx pairs holding data
   int* s_al = sh.al;
   int& s_nal = sh.nal;
   auto& s_dc = sh.dc;
@@ -122,21 +107,15 @@ __device__ __forceinline__ void row_body(const SolveArgs& A, int task, const Tas
   const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
   // one-byte labels of the task's rows (transform order) and the twiddle table -> shared memory,
   // behind the first loads
-  constexpr int NL = (N + 15) / 16 * 16;  // label row stride (bytes)
-  uint8_t* slab = reinterpret_cast<uint8_t*>(s + N * NP);
+  const int NL = (N + 15) / 16 * 16;  // label row stride (bytes)
+  uint8_t* slab = reinterpret_cast<uint8_t*>(s + pl.tile);
   {
     const uint4* src = reinterpret_cast<const uint4*>(A.label8 + c.lp_off + (size_t)y0 * NL);
     for (int i = threadIdx.x; i < nr * NL / 16; i += kT) cp16(slab + 16 * i, src + i);
   }
-#if HOM_ROW_TW2
-  float2* tws = reinterpret_cast<float2*>(s + N * NP + kFastRows * NL / 16);
+  float2* tws = reinterpret_cast<float2*>(s + pl.tile + kFastRows * NL / 16);
   for (int i = threadIdx.x; i < (N + 1) / 2; i += kT) cp16(tws + 2 * i, fp.tw2 + 2 * i);
-  float4* spare = s + N * NP + kFastRows * NL / 16 + (N + 1) / 2;
-#else
-  float4* tws = s + N * NP + kFastRows * NL / 16;
-  for (int i = threadIdx.x; i < N; i += kT) cp16(tws + i, fp.tw4 + i);
-  float4* spare = s + N * NP + kFastRows * NL / 16 + N;
-#endif
+  float4* spare = s + pl.tile + kFastRows * NL / 16 + (N + 1) / 2;
   float2* sph = reinterpret_cast<float2*>(spare + kRowSpare);
   float2* sinv = sph + c.nph;  // EM: per local phase, (c + c0)^-1 as the pair (coefficient of tr(u) I, of u)
   cp_commit();
@@ -161,7 +140,6 @@ __device__ __forceinline__ void row_body(const SolveArgs& A, int task, const Tas
   for (int la = 0; la < nal; ++la) {
     const int l = s_al[la];
     const float4* ein = static_cast<const float4*>(A.eps[OUT ? (A.iters[t.cell * A.L + l] & 1) : (it & 1)]);
-#if HOM_ROW_LANDING
     // 1. four half-spectrum rows -> two Hermitian-extended complex lines per component.  Item
     // (p, k) = kx pair p, component k: its four row values (one 16-byte lane pair each) land, by
     // asynchronous copies all in flight at once, in the tile slots of the four line positions
@@ -172,7 +150,7 @@ __device__ __forceinline__ void row_body(const SolveArgs& A, int task, const Tas
       const float4* src = ein + tile_index(c, N, l, p, y0) + k;
 #pragma unroll
       for (int r = 0; r < kFastRows; ++r)
-        cp16z(row_slot<N>(s, spare, p, k, r), src + (size_t)(r < nr ? r : 0) * NP, r < nr ? 16u : 0u);
+        cp16z(row_slot_p<NP>(pl, s, spare, p, k, r), src + (size_t)(r < nr ? r : 0) * NP, r < nr ? 16u : 0u);
     }
     cp_commit();
     // the next active load's rows of every pair (192 contiguous bytes each) -> L2, so that its
@@ -188,7 +166,7 @@ __device__ __forceinline__ void row_body(const SolveArgs& A, int task, const Tas
       const int p = f / NP, k = f - p * NP;
       float4 v[kFastRows];
 #pragma unroll
-      for (int r = 0; r < kFastRows; ++r) v[r] = *row_slot<N>(s, spare, p, k, r);
+      for (int r = 0; r < kFastRows; ++r) v[r] = *row_slot_p<NP>(pl, s, spare, p, k, r);
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int kx = 2 * p + h;
@@ -199,9 +177,10 @@ __device__ __forceinline__ void row_body(const SolveArgs& A, int task, const Tas
         const float2 q2 = h ? make_float2(v[2].y, v[2].w) : make_float2(v[2].x, v[2].z);
         const float2 q3 = h ? make_float2(v[3].y, v[3].w) : make_float2(v[3].x, v[3].z);
         // A + iB at kx and conj(A) + i conj(B) at n - kx, for (A, B) = (row 0, row 1) and (row 2, row 3)
-        s[kx * NP + k] = make_float4(q0.x - q1.y, q2.x - q3.y, q0.y + q1.x, q2.y + q3.x);
+        s[pl.at(kx) + k] = make_float4(q0.x - q1.y, q2.x - q3.y, q0.y + q1.x, q2.y + q3.x);
         if (kx > 0) {
-          s[(N - kx) * NP + k] = make_float4(q0.x + q1.y, q2.x + q3.y, q1.x - q0.y, q3.x - q2.y);
+          if (2 * kx != N)  // the Nyquist column of an even grid is its own partner (real rows: q.y = 0)
+            s[pl.at(N - kx) + k] = make_float4(q0.x + q1.y, q2.x + q3.y, q1.x - q0.y, q3.x - q2.y);
         } else {
           s_dc[la][0][0][k] = q0.x;
           s_dc[la][0][1][k] = q1.x;
@@ -211,56 +190,13 @@ __device__ __forceinline__ void row_body(const SolveArgs& A, int task, const Tas
       }
     }
     __syncthreads();
-#else
-    // 1. four half-spectrum rows -> two Hermitian-extended complex lines per component; item
-    // (p, k) reads rows y0..y0+3 of pair p (U items per round: 4 U loads in flight per thread)
-    constexpr int U = 1;
-    for (int f0 = threadIdx.x; f0 < P * NP; f0 += U * kT) {
-      float4 v[U][kFastRows];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int f = f0 + u * kT;
-        const int p = f / NP, k = f - p * NP;
-        const size_t b = tile_index(c, N, l, p, y0) + k;
-#pragma unroll
-        for (int r = 0; r < kFastRows; ++r) v[u][r] = (f < P * NP && r < nr) ? ein[b + (size_t)r * NP] : z4;
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int f = f0 + u * kT;
-        if (f >= P * NP) continue;
-        const int p = f / NP, k = f - p * NP;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int kx = 2 * p + h;
-          if (kx >= H) break;
-          // row r at kx: (re, im) = lane h of v[u][r]
-          const float2 q0 = h ? make_float2(v[u][0].y, v[u][0].w) : make_float2(v[u][0].x, v[u][0].z);
-          const float2 q1 = h ? make_float2(v[u][1].y, v[u][1].w) : make_float2(v[u][1].x, v[u][1].z);
-          const float2 q2 = h ? make_float2(v[u][2].y, v[u][2].w) : make_float2(v[u][2].x, v[u][2].z);
-          const float2 q3 = h ? make_float2(v[u][3].y, v[u][3].w) : make_float2(v[u][3].x, v[u][3].z);
-          // A + iB at kx and conj(A) + i conj(B) at n - kx, for (A, B) = (row 0, row 1) and (row 2, row 3)
-          s[kx * NP + k] = make_float4(q0.x - q1.y, q2.x - q3.y, q0.y + q1.x, q2.y + q3.x);
-          if (kx > 0) {
-            s[(N - kx) * NP + k] = make_float4(q0.x + q1.y, q2.x + q3.y, q1.x - q0.y, q3.x - q2.y);
-          } else {
-            s_dc[la][0][0][k] = q0.x;
-            s_dc[la][0][1][k] = q1.x;
-            s_dc[la][0][2][k] = q2.x;
-            s_dc[la][0][3][k] = q3.x;
-          }
-        }
-      }
-    }
-    cp_wait_all();
-    __syncthreads();
-#endif
-    fft_dif_p<NP, N, false>(s, tws);  // inverse: eps at digit-reversed positions
+    fft_dif<NP, false, kT>(pl, s, tws);  // inverse: eps at digit-reversed positions
 
     // 2. constitutive update: lanes (x, y, z, w) of a float4 are rows (0, 2, 1, 3).  A one-byte
     // label is the local phase index of a pure voxel, or kLabel8Mixed (full label read from the
     // material, which also covers any voxel whose phase is not in the cell's list).
     for (int pos = threadIdx.x; pos < N; pos += kT) {
+      const int at = pl.at(pos);
       uint32_t lab[kFastRows];
       bool mixed = false;
 #pragma unroll
@@ -280,7 +216,7 @@ __device__ __forceinline__ void row_body(const SolveArgs& A, int task, const Tas
       }
       float4 e[NP];
 #pragma unroll
-      for (int k = 0; k < NP; ++k) e[k] = s[pos * NP + k];
+      for (int k = 0; k < NP; ++k) e[k] = s[at + k];
       if (EM && (OUT || mixed)) {
         // e holds u: eps = (c~ + c0)^-1 u, per voxel (mixed: the per-call table; pure: in closed form)
         float ev[NP][kFastRows];
@@ -405,12 +341,12 @@ __device__ __forceinline__ void row_body(const SolveArgs& A, int task, const Tas
         }
       } else {
 #pragma unroll
-        for (int k = 0; k < NP; ++k) s[pos * NP + k] = o[k];
+        for (int k = 0; k < NP; ++k) s[at + k] = o[k];
       }
     }
     __syncthreads();  // the tile is read above and rewritten below (or by the next load's fill)
     if (OUT) continue;
-    fft_dit_p<NP, N, true>(s, tws);  // forward: natural order
+    fft_dit<NP, true, kT>(pl, s, tws);  // forward: natural order
 
     // 3. split the two real rows of each line; store the half spectra of tau, pair by pair
     for (int f = threadIdx.x; f < P * NP; f += kT) {
@@ -422,8 +358,8 @@ __device__ __forceinline__ void row_body(const SolveArgs& A, int task, const Tas
       for (int h = 0; h < 2; ++h) {
         const int kx = 2 * p + h;
         if (kx >= H) break;
-        const float4 Z = s[kx * NP + k];
-        const float4 Zm = s[(kx == 0 ? 0 : N - kx) * NP + k];
+        const float4 Z = s[pl.at(kx) + k];
+        const float4 Zm = s[pl.at(kx == 0 ? 0 : N - kx) + k];
         // (Z[k] + conj Z[n-k]) / 2 -> first row of a line, (Z[k] - conj Z[n-k]) / 2i -> second row
         const float2 o0 = make_float2(0.5f * (Z.x + Zm.x), 0.5f * (Z.z - Zm.z));
         const float2 o1 = make_float2(0.5f * (Z.z + Zm.z), 0.5f * (Zm.x - Z.x));
@@ -496,8 +432,9 @@ __device__ __forceinline__ void prefetch_row_task(const SolveArgs& A, int task) 
 
 // One CTA per task.  `ahead` is the number of CTAs resident on the device at once: task b + ahead
 // is about the one that starts when this CTA ends, so CTA b prefetches its first load into L2.
-template <bool OUT, bool SRC, bool EM = false>
-__global__ void __launch_bounds__(kT, HOM_ROW_TW2 ? 3 : 2) k_row_f2d(SolveArgs A, int ntasks, int ahead) {
+// RUN: radices read from the plan (any size; see k_row_r2d).
+template <bool OUT, bool SRC, bool EM, bool RUN>
+__device__ __forceinline__ void row_task(const SolveArgs& A, int ntasks, int ahead) {
   HOM_DBG_POISON();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ RowShared sh;
@@ -510,16 +447,32 @@ __global__ void __launch_bounds__(kT, HOM_ROW_TW2 ? 3 : 2) k_row_f2d(SolveArgs A
   if (!HOM_CHECK(A, t.row0 >= 0 && t.nrows >= 1 && t.nrows <= kFastRows && t.row0 + t.nrows <= c.nrows &&
                         t.load < A.L, (size_t)task))
     return;
-  const FastPlanDev fp = A.fplans[c.fplan];
-  switch (c.n) {
-    case 45: row_body<45, OUT, SRC, EM>(A, task, t, c, fp, s, sh); break;
-    case 75: row_body<75, OUT, SRC, EM>(A, task, t, c, fp, s, sh); break;
-    case 135: row_body<135, OUT, SRC, EM>(A, task, t, c, fp, s, sh); break;
-    case 225: row_body<225, OUT, SRC, EM>(A, task, t, c, fp, s, sh); break;
-    case 405: row_body<405, OUT, SRC, EM>(A, task, t, c, fp, s, sh); break;
-    case 1215: row_body<1215, OUT, SRC, EM>(A, task, t, c, fp, s, sh); break;
-    default: break;
+  const FastPlanDev& fp = A.fplans[c.fplan];
+  if constexpr (RUN) {
+    row_body<OUT, SRC, EM>(RunN<NP>(fp.run), A, task, t, c, fp, s, sh);
+  } else {
+    switch (c.n) {
+      case 45: row_body<OUT, SRC, EM>(FixedN<45, NP>(), A, task, t, c, fp, s, sh); break;
+      case 75: row_body<OUT, SRC, EM>(FixedN<75, NP>(), A, task, t, c, fp, s, sh); break;
+      case 135: row_body<OUT, SRC, EM>(FixedN<135, NP>(), A, task, t, c, fp, s, sh); break;
+      case 225: row_body<OUT, SRC, EM>(FixedN<225, NP>(), A, task, t, c, fp, s, sh); break;
+      case 405: row_body<OUT, SRC, EM>(FixedN<405, NP>(), A, task, t, c, fp, s, sh); break;
+      case 1215: row_body<OUT, SRC, EM>(FixedN<1215, NP>(), A, task, t, c, fp, s, sh); break;
+      default: break;
+    }
   }
+}
+template <bool OUT, bool SRC, bool EM = false>
+__global__ void __launch_bounds__(kT, 3) k_row_f2d(SolveArgs A, int ntasks, int ahead) {
+  row_task<OUT, SRC, EM, false>(A, ntasks, ahead);
+}
+// The same pass with radices read from a plan, for batches that hold a size without compiled ones: the
+// largest radix (16 lane pairs) takes 128 registers, two CTAs per SM.  Measured against the generic
+// row pass, which keeps two real rows per complex line and scalar arithmetic: 2 cells of 512^2, 3 loads:
+// 55 us (72 us generic); 143^2: 20 us (43 us).
+template <bool OUT, bool SRC, bool EM = false>
+__global__ void __launch_bounds__(kT, 2) k_row_r2d(SolveArgs A, int ntasks, int ahead) {
+  row_task<OUT, SRC, EM, true>(A, ntasks, ahead);
 }
 
 // eps = E: the stored x-spectrum holds E at kx = 0 of every row (lane A of pair 0), zero elsewhere.
@@ -553,10 +506,13 @@ __global__ void k_init_f2d(SolveArgs A, int ncells) {
 // Eyre-Milton scheme: the positions of one thread, lane by lane through em_core (hom_em.cuh); the
 // private state is u_hat of the current iterate, [position][6 complex] = (kx0 components 0..2, kx0+1
 // components 0..2) as three float4, in place of g.  Returns the three compensated sums.
-template <int N>
-__device__ __forceinline__ void green_em(const SolveArgs& A, int kx0, bool hasB, const CellDev& c, const float* sx,
+template <class PL>
+__device__ __forceinline__ void green_em(const PL& pl, const SolveArgs& A, int kx0, bool hasB, const CellDev& c, const float* sx,
                                          const FastPlanDev& fp, float4* s, float4* ub, const double* Eld,
                                          Acc<float> (&acc)[3]) {
+  const int N = pl.n;
+  // Nyquist bins of an even grid (a wave number no odd grid has)
+  const float nyq = (N & 1) ? -1.f : __ldg(fp.xinat + N / 2);
   CellConst<float> cc;
   cell_const(c, cc);
   const float nvT = (float)c.nv, inv_nv = cc.inv_nv, lam0 = cc.lam0, mu2_0 = cc.mu2;
@@ -571,49 +527,59 @@ __device__ __forceinline__ void green_em(const SolveArgs& A, int kx0, bool hasB,
     float2 th[NP], uh[NP], un[NP];
 #pragma unroll
     for (int k = 0; k < NP; ++k) {
-      const float* T = sf + 4 * (pos * NP + k);  // (re A, re B, im A, im B)
+      const float* T = sf + 4 * (pl.at(pos) + k);  // (re A, re B, im A, im B)
       th[k] = make_float2(T[h], T[2 + h]);
       uh[k] = u2[6 * pos + 3 * h + k];
     }
     const float xi[2] = {X[h], sx[pos]};
-    em_core<float, 2>(th, uh, un, xi, h == 0 && kx0 == 0 && pos == 0, false, h == 0 && kx0 == 0, nvT, inv_nv, lam0,
-                      mu2_0, a0, inv_mu2_0, cc.inv_mu0, cc.ratio, Eld, acc[0], acc[1], acc[2]);
+    em_core<float, 2>(th, uh, un, xi, h == 0 && kx0 == 0 && pos == 0, xi[0] == nyq || xi[1] == nyq,
+                      (h == 0 && kx0 == 0) || xi[0] == nyq, nvT, inv_nv, lam0, mu2_0, a0, inv_mu2_0, cc.inv_mu0, cc.ratio, Eld, acc[0], acc[1], acc[2]);
 #pragma unroll
     for (int k = 0; k < NP; ++k) {
-      float* T = sf + 4 * (pos * NP + k);
+      float* T = sf + 4 * (pl.at(pos) + k);
       T[h] = un[k].x;
       T[2 + h] = un[k].y;
       u2[6 * pos + 3 * h + k] = un[k];
     }
   }
   if (!hasB)  // the missing lane B of the last pair stays zero
-    for (int i = threadIdx.x; i < N * NP; i += kT) {
+    for (int i = threadIdx.x; i < pl.tile; i += kT) {
       sf[4 * i + 1] = 0.f;
       sf[4 * i + 3] = 0.f;
     }
 }
 
+// Piece `i` of a tile that bulk copies move: the whole tile (contiguous in HBM and in shared memory), or,
+// padded, the positions between two paddings.
+template <class PL>
+__device__ __forceinline__ int tile_pieces(const PL& pl) {
+  if constexpr (PL::fixed) return 1;
+  else return pl.p.pad ? pl.n / pl.p.r[0] : 1;
+}
+template <class PL>
+__device__ __forceinline__ int piece_len(const PL& pl, int pieces) { return pl.n / pieces * NP; }
+
 // The finished tile (natural order after the inverse transform) -> the next eps buffer.
-template <int N>
-__device__ __forceinline__ void green_store(const SolveArgs& A, const float4* s, float4* out) {
-#if HOM_GREEN_BULK
+template <class PL>
+__device__ __forceinline__ void green_store(const PL& pl, const float4* s, float4* out) {
   fence_proxy_async();  // this thread's tile writes, visible to the bulk copy
   __syncthreads();
-  if (threadIdx.x == 0) {
-    bulk_store(out, s, (unsigned)(N * NP * sizeof(float4)));
-    bulk_store_wait_read();  // the CTA keeps its shared memory until the copy has read it
-  }
-#else
-  for (int f = threadIdx.x; f < N * NP; f += kT) out[f] = s[f];
-#endif
-  (void)A;
+  const int pieces = tile_pieces(pl), len = piece_len(pl, pieces);
+  for (int i = threadIdx.x; i < pieces; i += kT) bulk_store(out + i * len, s + i * (len + 1), (unsigned)(len * sizeof(float4)));
+  if (threadIdx.x < pieces) bulk_store_wait_read();  // the CTA keeps its shared memory until the copies have read it
+}
+
+// Positions per thread of a fixed-size Green task.
+template <class PL> __host__ __device__ constexpr int green_npos() {
+  if constexpr (PL::fixed) return (PL::n + kT - 1) / kT;
+  else return 1;
 }
 
 // tau (mixed domain) -> forward y-DFT -> Gamma0 and the residual on J (eq. 2) -> inverse y-DFT -> eps.
-template <int N, bool EM = false>
-__device__ __forceinline__ void green_body(const SolveArgs& A, int task, const TaskL& t, const CellDev& c,
+template <bool EM, class PL>
+__device__ __forceinline__ void green_body(const PL& pl, const SolveArgs& A, int task, const TaskL& t, const CellDev& c,
                                            const FastPlanDev& fp, float4* s) {
-  constexpr int H = (N + 1) / 2;
+  const int N = pl.n, H = N / 2 + 1;
   const int cl = t.cell * A.L + t.load;
   if (!A.active[cl]) return;
   const int it = *A.it_dev;
@@ -628,37 +594,28 @@ __device__ __forceinline__ void green_body(const SolveArgs& A, int task, const T
   float4* gb = static_cast<float4*>(A.g) +
                (c.g_off + ((size_t)t.load * (Hp / 2) + (size_t)(kx0 / 2)) * N * 4) / 2;
   // tile, twiddles and the wave numbers of the positions -> shared memory
-#if HOM_GREEN_TW2
-  float2* tws = reinterpret_cast<float2*>(s + N * NP);  // scalar twiddles: 3 CTAs per SM fit
-  float* sx = reinterpret_cast<float*>(s + N * NP + (N + 1) / 2);
+  float2* tws = reinterpret_cast<float2*>(s + pl.tile);  // scalar twiddles: 3 CTAs per SM fit
+  float* sx = reinterpret_cast<float*>(s + pl.tile + (N + 1) / 2);
   for (int i = threadIdx.x; i < (N + 1) / 2; i += kT) cp16(tws + 2 * i, fp.tw2 + 2 * i);
-#else
-  float4* tws = s + N * NP;
-  float* sx = reinterpret_cast<float*>(tws + N);
-  for (int i = threadIdx.x; i < N; i += kT) cp16(tws + i, fp.tw4 + i);
-#endif
-#if HOM_GREEN_BULK
-  // the tile (N NP float4, contiguous in HBM and in shared memory) by one bulk copy
+  // the tile (N NP float4, contiguous in HBM) by bulk copies
   __shared__ __align__(8) unsigned long long tile_bar;
-  fence_proxy_async();  // earlier generic writes to this shared memory are ordered before the copy's
+  const int pieces = tile_pieces(pl), len = piece_len(pl, pieces);
+  fence_proxy_async();  // earlier generic writes to this shared memory are ordered before the copies'
   __syncthreads();
   if (threadIdx.x == 0) {
     mbar_init(&tile_bar, 1);
-    bulk_load(s, in, (unsigned)(N * NP * sizeof(float4)), &tile_bar);
+    mbar_expect(&tile_bar, (unsigned)(N * NP * sizeof(float4)));
   }
-#else
-  for (int i = threadIdx.x; i < N * NP; i += kT) cp16(s + i, in + i);
-#endif
+  __syncthreads();
+  for (int i = threadIdx.x; i < pieces; i += kT)
+    bulk_load(s + i * (len + 1), in + i * len, (unsigned)(len * sizeof(float4)), &tile_bar);
   for (int i = threadIdx.x; i < (N + 3) / 4; i += kT) cp16(sx + 4 * i, fp.xipos + 4 * i);
   cp_commit();
   cp_wait_all();
-#if HOM_GREEN_BULK
-  __syncthreads();  // the barrier's initialisation is visible before anyone waits on it
   // bounded wait (a copy of 60 KB lands in microseconds); running out is recorded, never a hang
   if (!mbar_wait(&tile_bar, 0, 1 << 22) && A.dbg) atomicCAS(A.dbg, 0u, 0xFFFFFFFFu);
   __syncthreads();
   if (threadIdx.x == 0) mbar_inval(&tile_bar);
-#endif
   __syncthreads();
 #if HOM_GREEN_GPF
   // the private state of this column pair (contiguous: N positions x 2 or 3 float4) -> L2, so that
@@ -672,12 +629,12 @@ __device__ __forceinline__ void green_body(const SolveArgs& A, int task, const T
     for (unsigned o = threadIdx.x * kPiece; o < bytes; o += 32 * kPiece) prefetch_l2(gsrc + o, min(kPiece, bytes - o));
   }
 #endif
-  fft_dif_p<NP, N, true>(s, tws);  // forward: bin ky at position perm(ky)
+  fft_dif<NP, true, kT>(pl, s, tws);  // forward: bin ky at position perm(ky)
 
   if constexpr (EM) {
     float4* ub = static_cast<float4*>(A.g) + (c.g_off + ((size_t)t.load * (Hp / 2) + (size_t)(kx0 / 2)) * N * 6) / 2;
     Acc<float> acc[3];
-    green_em<N>(A, kx0, hasB, c, sx, fp, s, ub, A.E + (size_t)cl * NP, acc);
+    green_em(pl, A, kx0, hasB, c, sx, fp, s, ub, A.E + (size_t)cl * NP, acc);
     double tot[3];
     block_sum<float, 3, kT>(acc, tot);  // contains the barrier before the inverse transform
     if (threadIdx.x == 0) {
@@ -685,8 +642,8 @@ __device__ __forceinline__ void green_body(const SolveArgs& A, int task, const T
       A.partC[2 * (size_t)task + 1] = tot[1];
       A.partE[task] = tot[2];
     }
-    fft_dit_p<NP, N, false>(s, tws);  // inverse: natural order
-    green_store<N>(A, s, out);
+    fft_dit<NP, false, kT>(pl, s, tws);  // inverse: natural order
+    green_store(pl, s, out);
     if (threadIdx.x == 0) {
       const int ntk = hasB ? 2 : 1;
       atomicAdd(A.bytes + HOM_K_GREEN, (unsigned long long)(4 * (size_t)N * ntk * NP * sizeof(float2)));
@@ -701,27 +658,32 @@ __device__ __forceinline__ void green_body(const SolveArgs& A, int task, const T
   const float rs2 = 0.707106781186547524400844362105f;
   const float2 X = make_float2(__ldg(fp.xinat + kx0), hasB ? __ldg(fp.xinat + kx0 + 1) : 0.f);
   const float2 X2 = mul2(X, X);
-  const float2 wgt = make_float2(kx0 == 0 ? 1.f : 2.f, hasB ? 2.f : 0.f);
+  // even grids: a wave vector with a Nyquist component (n/2) has no conjugate partner in the spectrum
+  // of a real field; its strain is set to zero and it is left out of the residual
+  const bool even = !(N & 1);
+  const float nyq = even ? __ldg(fp.xinat + N / 2) : 0.f;
+  const bool deadA = even && 2 * kx0 == N, deadB = !hasB || (even && 2 * kx0 + 2 == N);
+  const float2 wgt = make_float2(deadA ? 0.f : kx0 == 0 ? 1.f : 2.f, deadB ? 0.f : 2.f);
   const double* Eld = A.E + (size_t)cl * NP;
   float2 r2s = z2, r2c = z2, rns = z2, rnc = z2;  // Kahan sums (value, lost low part) per lane
-  // g of every position of this thread, loaded at once
-  constexpr int NPOS = (N + kT - 1) / kT;
+  // g of every position of this thread, loaded at once where their number is known
+  constexpr int NPOS = green_npos<PL>();
   float4 gr[NPOS][2];
-#pragma unroll
-  for (int i = 0; i < NPOS; ++i) {
-    const int pos = threadIdx.x + i * kT;
+  auto load_g = [&](int pos, float4(&r)[2]) {
     if (pos < N) {
-      gr[i][0] = gb[2 * pos];
-      gr[i][1] = gb[2 * pos + 1];
+      r[0] = gb[2 * pos];
+      r[1] = gb[2 * pos + 1];
     }
-  }
+  };
+  if constexpr (PL::fixed) {
 #pragma unroll
-  for (int i = 0; i < NPOS; ++i) {
-    const int pos = threadIdx.x + i * kT;
-    if (pos >= N) break;
-    const float4 ga = gr[i][0], gbv = gr[i][1];
+    for (int i = 0; i < NPOS; ++i) load_g(threadIdx.x + i * kT, gr[i]);
+  }
+  auto point = [&](int pos, const float4(&gin)[2]) {
+    const float4 ga = gin[0], gbv = gin[1];
+    const int at = pl.at(pos);
     const float2 Y = f2(sx[pos]);
-    const P2 T0 = ldp(s[pos * NP]), T1 = ldp(s[pos * NP + 1]), T2 = ldp(s[pos * NP + 2]);
+    const P2 T0 = ldp(s[at]), T1 = ldp(s[at + 1]), T2 = ldp(s[at + 2]);
     const P2 G0{make_float2(ga.x, gbv.x), make_float2(ga.y, gbv.y)};
     const P2 G1{make_float2(ga.z, gbv.z), make_float2(ga.w, gbv.w)};
     // v = tau_hat . xi (tau_01 = T2 / sqrt 2)
@@ -741,7 +703,9 @@ __device__ __forceinline__ void green_body(const SolveArgs& A, int task, const T
     r2 = fma2(R1.re, R1.re, r2);
     r2 = fma2(R1.im, R1.im, r2);
     const bool k0 = kx0 == 0 && pos == 0;  // k = 0: eps_hat(0) = E, g = 0, no residual
-    const float2 iq = make_float2(k0 ? 0.f : __fdividef(1.f, q2.x), hasB ? __fdividef(1.f, q2.y) : 0.f);
+    const bool dead = even && Y.x == nyq;  // the last axis at Nyquist
+    const float2 iq = make_float2(k0 || deadA || dead ? 0.f : __fdividef(1.f, q2.x),
+                                  deadB || dead ? 0.f : __fdividef(1.f, q2.y));
     // g' = K0^-1 (tau_hat xi), eps_hat' = -sym(xi (x) g') / N_v
     const float2 imq = mul2(inv_mu0, iq);
     const float2 rq = mul2(ratio, iq);
@@ -755,7 +719,7 @@ __device__ __forceinline__ void green_body(const SolveArgs& A, int task, const T
     P2 E2{mul2(ns, fma2(X, W1.re, mul2(Y, W0.re))), mul2(ns, fma2(X, W1.im, mul2(Y, W0.im)))};
     float4 gna = make_float4(W0.re.x, W0.im.x, W1.re.x, W1.im.x);
     const float4 gnb = make_float4(W0.re.y, W0.im.y, W1.re.y, W1.im.y);
-    float2 wr = wgt;
+    float2 wr = dead ? z2 : wgt;
     if (k0) {
       E0.re.x = (float)Eld[0]; E0.im.x = 0.f;
       E1.re.x = (float)Eld[1]; E1.im.x = 0.f;
@@ -763,9 +727,9 @@ __device__ __forceinline__ void green_body(const SolveArgs& A, int task, const T
       gna = make_float4(0.f, 0.f, 0.f, 0.f);
       wr.x = 0.f;
     }
-    s[pos * NP] = stp(E0);
-    s[pos * NP + 1] = stp(E1);
-    s[pos * NP + 2] = stp(E2);
+    s[at] = stp(E0);
+    s[at + 1] = stp(E1);
+    s[at + 2] = stp(E2);
     gb[2 * pos] = gna;
     gb[2 * pos + 1] = gnb;
     // Kahan accumulation of wgt * r2 and wgt * r2 / q2, lane by lane
@@ -779,6 +743,22 @@ __device__ __forceinline__ void green_body(const SolveArgs& A, int task, const T
       const float2 yv = sub2(a2, rnc), tv = add2(rns, yv);
       rnc = sub2(sub2(tv, rns), yv);
       rns = tv;
+    }
+  };
+  if constexpr (PL::fixed) {
+#pragma unroll
+    for (int i = 0; i < NPOS; ++i) {
+      const int pos = threadIdx.x + i * kT;
+      if (pos < N) point(pos, gr[i]);
+    }
+  } else {
+    float4 nx[2];  // g of the thread's next position, loaded while this one is processed
+    load_g(threadIdx.x, nx);
+    for (int pos = threadIdx.x; pos < N; pos += kT) {
+      gr[0][0] = nx[0];
+      gr[0][1] = nx[1];
+      load_g(pos + kT, nx);
+      point(pos, gr[0]);
     }
   }
   {
@@ -799,8 +779,8 @@ __device__ __forceinline__ void green_body(const SolveArgs& A, int task, const T
       A.partC[2 * (size_t)task + 1] = tot[1];
     }
   }
-  fft_dit_p<NP, N, false>(s, tws);  // inverse: natural order
-  green_store<N>(A, s, out);
+  fft_dit<NP, false, kT>(pl, s, tws);  // inverse: natural order
+  green_store(pl, s, out);
   if (threadIdx.x == 0) {
     const int ntk = hasB ? 2 : 1;
     atomicAdd(A.bytes + HOM_K_GREEN,
@@ -827,8 +807,8 @@ __device__ __forceinline__ void prefetch_green_task(const SolveArgs& A, int task
 }
 
 // One CTA per task; CTA b prefetches task b + ahead into L2 (see k_row_f2d).
-template <bool EM = false>
-__global__ void __launch_bounds__(kT, HOM_GREEN_TW2 ? 3 : 2) k_green_f2d(SolveArgs A, int ntasks, int ahead) {
+template <bool EM, bool RUN>
+__device__ __forceinline__ void green_task(const SolveArgs& A, int ntasks, int ahead) {
   HOM_DBG_POISON();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float4* s = reinterpret_cast<float4*>(smem_raw);
@@ -839,16 +819,30 @@ __global__ void __launch_bounds__(kT, HOM_GREEN_TW2 ? 3 : 2) k_green_f2d(SolveAr
   // debug builds: an even kx pair start inside the half spectrum, a valid load
   if (!HOM_CHECK(A, t.kx0 >= 0 && (t.kx0 & 1) == 0 && t.kx0 < c.H && t.load >= 0 && t.load < A.L, (size_t)task))
     return;
-  const FastPlanDev fp = A.fplans[c.fplan];
-  switch (c.n) {
-    case 45: green_body<45, EM>(A, task, t, c, fp, s); break;
-    case 75: green_body<75, EM>(A, task, t, c, fp, s); break;
-    case 135: green_body<135, EM>(A, task, t, c, fp, s); break;
-    case 225: green_body<225, EM>(A, task, t, c, fp, s); break;
-    case 405: green_body<405, EM>(A, task, t, c, fp, s); break;
-    case 1215: green_body<1215, EM>(A, task, t, c, fp, s); break;
-    default: break;
+  const FastPlanDev& fp = A.fplans[c.fplan];
+  if constexpr (RUN) {
+    green_body<EM>(RunN<NP>(fp.run), A, task, t, c, fp, s);
+  } else {
+    switch (c.n) {
+      case 45: green_body<EM>(FixedN<45, NP>(), A, task, t, c, fp, s); break;
+      case 75: green_body<EM>(FixedN<75, NP>(), A, task, t, c, fp, s); break;
+      case 135: green_body<EM>(FixedN<135, NP>(), A, task, t, c, fp, s); break;
+      case 225: green_body<EM>(FixedN<225, NP>(), A, task, t, c, fp, s); break;
+      case 405: green_body<EM>(FixedN<405, NP>(), A, task, t, c, fp, s); break;
+      case 1215: green_body<EM>(FixedN<1215, NP>(), A, task, t, c, fp, s); break;
+      default: break;
+    }
   }
+}
+template <bool EM = false>
+__global__ void __launch_bounds__(kT, 3) k_green_f2d(SolveArgs A, int ntasks, int ahead) {
+  green_task<EM, false>(A, ntasks, ahead);
+}
+// Radices read from a plan (see k_row_r2d): 2 cells of 512^2, 3 loads: 45 us (103 us generic); 143^2:
+// 19 us (42 us).
+template <bool EM = false>
+__global__ void __launch_bounds__(kT, 2) k_green_r2d(SolveArgs A, int ntasks, int ahead) {
+  green_task<EM, true>(A, ntasks, ahead);
 }
 
 // ------------------------------------------------------------------ labels in transform order
@@ -879,6 +873,7 @@ __global__ void k_permute_labels(SolveArgs A, int ncells) {
 // ------------------------------------------------------------------ host side
 struct FastCacheEntry {
   int dev, n;
+  bool run;
   FastPlanDev p;
   void* mem;
 };
@@ -908,9 +903,56 @@ bool fast2d_size(int n) {
   return false;
 }
 
-int fast2d_plan_host(int n, std::vector<unsigned char>& h, FastPlanDev* out) {
+namespace {
+// Radices (DIT order) of the run-time plans: the fewest stages of radices up to 16, then the smallest
+// largest radix; even radices first (their stage is padded, and the spans that follow are then multiples
+// of 8 or 16 where the size allows, which keeps neighbouring butterflies on distinct banks).
+std::vector<int> run_radices(int n) {
+  static const int kR[] = {16, 15, 13, 11, 9, 8, 7, 5, 4, 3, 2};
+  std::vector<int> best, cur;
+  std::function<void(int)> search = [&](int rem) {
+    if (rem == 1) {
+      auto key = [](const std::vector<int>& v) { return std::make_pair(v.size(), *std::max_element(v.begin(), v.end())); };
+      if (best.empty() || key(cur) < key(best)) best = cur;
+      return;
+    }
+    if ((int)cur.size() >= kMaxRunStages || (!best.empty() && cur.size() + 1 > best.size())) return;
+    for (int r : kR) {
+      if (rem % r != 0 || (!cur.empty() && r > cur.back())) continue;
+      cur.push_back(r);
+      search(rem / r);
+      cur.pop_back();
+    }
+  };
+  search(n);
+  std::stable_sort(best.begin(), best.end(), [](int a, int b) { return (a & 1) < (b & 1); });
+  return best;
+}
+void fill_run_plan(const HostPlan& hp, RunPlan& r) {
+  r.n = hp.n;
+  r.m = (int)hp.radix.size();
+  r.pad = (hp.radix[0] & 1) ? 0 : 1;
+  int off = 0;
+  for (int st = 0; st < r.m; ++st) {
+    r.r[st] = hp.radix[st];
+    r.L[st] = hp.span[st];
+    r.tw[st] = off;
+    if (st > 0) off += r.L[st] * (r.r[st] - 1);
+    r.d_nb[st] = make_fastdiv(r.n / r.r[st]);
+    r.d_L[st] = make_fastdiv(r.L[st]);
+  }
+  r.d_r0 = make_fastdiv(r.r[0]);
+}
+}  // namespace
+
+bool run2d_size(int n) {  // the row pass's tile, twiddles and labels of 4 rows on chip, a few phases
+  return grid_supported(n) && fast2d_smem_row(n, 64) <= 200 * 1024;
+}
+
+int fast2d_plan_host(int n, bool run, std::vector<unsigned char>& h, FastPlanDev* out) {
   HostPlan hp;
-  if (radices_of(n).empty() || !build_host_plan_radices(n, radices_of(n), hp))
+  const std::vector<int> radix = run ? run_radices(n) : radices_of(n);
+  if (radix.empty() || !build_host_plan_radices(n, radix, hp))
     return set_error(HOM_ERR_UNSUPPORTED_SIZE, "no specialised plan for n = %d", n);
   auto up = [](size_t b) { return (b + 255) / 256 * 256; };
   const size_t b_tw = up((size_t)n * 16), b_ip = up((size_t)n * 2), b_xp = up((size_t)n * 4), b_xn = up((size_t)n * 4),
@@ -947,6 +989,7 @@ int fast2d_plan_host(int n, std::vector<unsigned char>& h, FastPlanDev* out) {
   p.xinat = reinterpret_cast<const float*>(b_tw + b_ip + b_xp);
   p.tw2 = reinterpret_cast<const float2*>(b_tw + b_ip + b_xp + b_xn);
   p.n = n;
+  fill_run_plan(hp, p.run);
   *out = p;
   return HOM_OK;
 }
@@ -960,24 +1003,24 @@ void fast2d_plan_rebase(FastPlanDev& p, const unsigned char* base) {
   p.tw2 = reinterpret_cast<const float2*>(at(p.tw2));
 }
 
-int fast2d_plan(int n, FastPlanDev* out) {
+int fast2d_plan(int n, bool run, FastPlanDev* out) {
   int dev = 0;
   HOM_CUDA_TRY(cudaGetDevice(&dev));
   std::lock_guard<std::mutex> lk(g_fast_mu);
   for (const auto& e : g_fast_cache)
-    if (e.dev == dev && e.n == n) {
+    if (e.dev == dev && e.n == n && e.run == run) {
       *out = e.p;
       return HOM_OK;
     }
   std::vector<unsigned char> h;
   FastPlanDev p{};
-  int rc = fast2d_plan_host(n, h, &p);
+  int rc = fast2d_plan_host(n, run, h, &p);
   if (rc != HOM_OK) return rc;
   void* mem = nullptr;
   HOM_CUDA_TRY(cudaMalloc(&mem, h.size()));
   HOM_CUDA_TRY(cudaMemcpy(mem, h.data(), h.size(), cudaMemcpyHostToDevice));
   fast2d_plan_rebase(p, static_cast<const unsigned char*>(mem));
-  g_fast_cache.push_back({dev, n, p, mem});
+  g_fast_cache.push_back({dev, n, run, p, mem});
   *out = p;
   return HOM_OK;
 }
@@ -996,15 +1039,17 @@ void fast2d_release() {
 
 // row: tile | one-byte labels of 4 rows | twiddles | spare landing slots | per-phase update constants
 // Green: tile | twiddles | wave numbers
+// (even sizes: the tile with its padding, at most one float4 for every two positions)
+namespace {
+size_t tile_bytes(int n) { return ((size_t)n * NP + ((n & 1) ? 0 : n / 2)) * sizeof(float4); }
+}  // namespace
 size_t fast2d_smem_row(int nmax, int nphase_cell) {
   const size_t labels = (size_t)kFastRows * ((nmax + 15) / 16 * 16);
-  const size_t tw = HOM_ROW_TW2 ? ((size_t)nmax + 1) / 2 * 16 : (size_t)nmax * sizeof(float4);
-  return (size_t)nmax * NP * sizeof(float4) + labels + tw + (size_t)kRowSpare * sizeof(float4) +
+  return tile_bytes(nmax) + labels + ((size_t)nmax + 1) / 2 * 16 + (size_t)kRowSpare * sizeof(float4) +
          ((size_t)nphase_cell * 16 + 15) / 16 * 16;  // two float2 per phase (the second for the Eyre-Milton scheme)
 }
 size_t fast2d_smem_green(int nmax) {
-  const size_t tw = HOM_GREEN_TW2 ? ((size_t)nmax + 1) / 2 * 16 : (size_t)nmax * sizeof(float4);
-  return (size_t)nmax * NP * sizeof(float4) + tw + ((size_t)nmax + 3) / 4 * 16;
+  return tile_bytes(nmax) + ((size_t)nmax + 1) / 2 * 16 + ((size_t)nmax + 3) / 4 * 16;
 }
 
 namespace {
@@ -1015,38 +1060,33 @@ int opt_in(K kernel, size_t bytes) {
 }
 }  // namespace
 
-int fast2d_row(const SolveArgs& A, unsigned ntasks, size_t smem, cudaStream_t st) {
-  if (A.scheme == HOM_SCHEME_EYRE_MILTON) {
-    int rc = opt_in(k_row_f2d<false, false, true>, smem);
-    if (rc != HOM_OK) return rc;
-    k_row_f2d<false, false, true><<<ntasks, kT, smem, st>>>(A, (int)ntasks,
-                                                            resident_ctas(k_row_f2d<false, false, true>, kT, smem));
-    return HOM_OK;
-  }
-  if (A.src) {  // adjoint solve: the constitutive step takes the source term
-    int rc = opt_in(k_row_f2d<false, true>, smem);
-    if (rc != HOM_OK) return rc;
-    k_row_f2d<false, true><<<ntasks, kT, smem, st>>>(A, (int)ntasks, resident_ctas(k_row_f2d<false, true>, kT, smem));
-    return HOM_OK;
-  }
-  int rc = opt_in(k_row_f2d<false, false>, smem);
+namespace {
+template <typename K>
+int launch_tasks(K kernel, const SolveArgs& A, unsigned ntasks, size_t smem, cudaStream_t st) {
+  int rc = opt_in(kernel, smem);
   if (rc != HOM_OK) return rc;
-  k_row_f2d<false, false><<<ntasks, kT, smem, st>>>(A, (int)ntasks, resident_ctas(k_row_f2d<false, false>, kT, smem));
+  kernel<<<ntasks, kT, smem, st>>>(A, (int)ntasks, resident_ctas(kernel, kT, smem));
   return HOM_OK;
 }
+}  // namespace
 
-int fast2d_out(const SolveArgs& A, unsigned ntasks, size_t smem, cudaStream_t st) {
-  if (A.scheme == HOM_SCHEME_EYRE_MILTON) {
-    int rc = opt_in(k_row_f2d<true, false, true>, smem);
-    if (rc != HOM_OK) return rc;
-    k_row_f2d<true, false, true><<<ntasks, kT, smem, st>>>(A, (int)ntasks,
-                                                           resident_ctas(k_row_f2d<true, false, true>, kT, smem));
-    return HOM_OK;
-  }
-  int rc = opt_in(k_row_f2d<true, false>, smem);
-  if (rc != HOM_OK) return rc;
-  k_row_f2d<true, false><<<ntasks, kT, smem, st>>>(A, (int)ntasks, resident_ctas(k_row_f2d<true, false>, kT, smem));
-  return HOM_OK;
+int fast2d_row(const SolveArgs& A, unsigned ntasks, size_t smem, bool run, cudaStream_t st) {
+  if (A.scheme == HOM_SCHEME_EYRE_MILTON)
+    return run ? launch_tasks(k_row_r2d<false, false, true>, A, ntasks, smem, st)
+               : launch_tasks(k_row_f2d<false, false, true>, A, ntasks, smem, st);
+  if (A.src)  // adjoint solve: the constitutive step takes the source term
+    return run ? launch_tasks(k_row_r2d<false, true>, A, ntasks, smem, st)
+               : launch_tasks(k_row_f2d<false, true>, A, ntasks, smem, st);
+  return run ? launch_tasks(k_row_r2d<false, false>, A, ntasks, smem, st)
+             : launch_tasks(k_row_f2d<false, false>, A, ntasks, smem, st);
+}
+
+int fast2d_out(const SolveArgs& A, unsigned ntasks, size_t smem, bool run, cudaStream_t st) {
+  if (A.scheme == HOM_SCHEME_EYRE_MILTON)
+    return run ? launch_tasks(k_row_r2d<true, false, true>, A, ntasks, smem, st)
+               : launch_tasks(k_row_f2d<true, false, true>, A, ntasks, smem, st);
+  return run ? launch_tasks(k_row_r2d<true, false>, A, ntasks, smem, st)
+             : launch_tasks(k_row_f2d<true, false>, A, ntasks, smem, st);
 }
 
 int fast2d_init(const SolveArgs& A, int ncells, cudaStream_t st) {
@@ -1056,17 +1096,10 @@ int fast2d_init(const SolveArgs& A, int ncells, cudaStream_t st) {
   return HOM_OK;
 }
 
-int fast2d_green(const SolveArgs& A, unsigned ntasks, size_t smem, cudaStream_t st) {
-  if (A.scheme == HOM_SCHEME_EYRE_MILTON) {
-    int rc = opt_in(k_green_f2d<true>, smem);
-    if (rc != HOM_OK) return rc;
-    k_green_f2d<true><<<ntasks, kT, smem, st>>>(A, (int)ntasks, resident_ctas(k_green_f2d<true>, kT, smem));
-    return HOM_OK;
-  }
-  int rc = opt_in(k_green_f2d<false>, smem);
-  if (rc != HOM_OK) return rc;
-  k_green_f2d<false><<<ntasks, kT, smem, st>>>(A, (int)ntasks, resident_ctas(k_green_f2d<false>, kT, smem));
-  return HOM_OK;
+int fast2d_green(const SolveArgs& A, unsigned ntasks, size_t smem, bool run, cudaStream_t st) {
+  if (A.scheme == HOM_SCHEME_EYRE_MILTON)
+    return run ? launch_tasks(k_green_r2d<true>, A, ntasks, smem, st) : launch_tasks(k_green_f2d<true>, A, ntasks, smem, st);
+  return run ? launch_tasks(k_green_r2d<false>, A, ntasks, smem, st) : launch_tasks(k_green_f2d<false>, A, ntasks, smem, st);
 }
 
 int fast2d_permute_labels(const SolveArgs& A, int ncells, long long max_nv, cudaStream_t st) {

@@ -9,9 +9,21 @@
 #include <cstdint>
 #include <vector>
 
+#include "hom_common.cuh"
+
 namespace hom {
 
 struct SolveArgs;
+
+// Stages of a transform whose length is known at run time only (RunN in hom_fastfft.cuh), DIT order.
+constexpr int kMaxRunStages = 5;
+struct RunPlan {
+  int n, m;              // length, stages
+  int pad;               // 1: one float4 of padding after every r[0] positions (even r[0])
+  int r[kMaxRunStages], L[kMaxRunStages];  // radix and span of each stage
+  int tw[kMaxRunStages];                   // offset of its twiddle table
+  FastDiv d_nb[kMaxRunStages], d_L[kMaxRunStages], d_r0;
+};
 
 // Device tables of one grid size n (plan with the radices compiled into the specialised passes).
 struct FastPlanDev {
@@ -21,31 +33,36 @@ struct FastPlanDev {
   const float* xinat;     // 2 pi a(k) in natural order
   const float2* tw2;      // the twiddle tables as (cos, -sin) pairs
   int n, pad;
+  RunPlan run;            // the same transform for the run-time-size passes
 };
 
 constexpr int kFastRows = 4;  // real rows per row-pass task (two complex lines, one lane pair)
 constexpr int kFastCols = 2;  // kx columns per Green-pass task (one lane pair)
 
-// True if n has specialised 2D / 3D passes.
+// True if n has specialised 2D / 3D passes with its radices compiled in, and if it fits the passes
+// whose radices are chosen at run time (every supported size up to what a tile can hold on chip).
 bool fast2d_size(int n);
 bool fast3d_size(int n);
-// Device tables of size n (built and uploaded on first use, kept until hom_release); every size
-// of fast2d_size or fast3d_size has one.
-int fast2d_plan(int n, FastPlanDev* out);
+bool run2d_size(int n);
+bool run3d_size(int n);
+// Device tables of size n (built and uploaded on first use, kept until hom_release).  `run`: for the
+// passes with run-time radices, whose digit order differs from the compiled ones'.
+int fast2d_plan(int n, bool run, FastPlanDev* out);
 // The same tables built on the host only (no device allocation): `h` receives them and `out` their
 // layout, with byte offsets from the start of `h` in place of the table pointers; after `h` is
 // copied to device memory at `base`, fast2d_plan_rebase turns the offsets into device pointers.
-int fast2d_plan_host(int n, std::vector<unsigned char>& h, FastPlanDev* out);
+int fast2d_plan_host(int n, bool run, std::vector<unsigned char>& h, FastPlanDev* out);
 void fast2d_plan_rebase(FastPlanDev& p, const unsigned char* base);
 // Dynamic shared memory of the row and Green passes for the largest grid size n of a call.
 size_t fast2d_smem_row(int nmax, int nphase_cell);
 size_t fast2d_smem_green(int nmax);
-// Launches (one CTA per task); `smem` from fast2d_smem_row / fast2d_smem_green.
-int fast2d_row(const SolveArgs& A, unsigned ntasks, size_t smem, cudaStream_t st);
-int fast2d_green(const SolveArgs& A, unsigned ntasks, size_t smem, cudaStream_t st);
+// Launches (one CTA per task); `smem` from fast2d_smem_row / fast2d_smem_green; `run`: radices read from
+// the plans.
+int fast2d_row(const SolveArgs& A, unsigned ntasks, size_t smem, bool run, cudaStream_t st);
+int fast2d_green(const SolveArgs& A, unsigned ntasks, size_t smem, bool run, cudaStream_t st);
 // Output pass (final eps and sigma fields) and the initial state eps = E, in the tiled layout of
 // the specialised passes (see hom_fast2d.cu).
-int fast2d_out(const SolveArgs& A, unsigned ntasks, size_t smem, cudaStream_t st);
+int fast2d_out(const SolveArgs& A, unsigned ntasks, size_t smem, bool run, cudaStream_t st);
 int fast2d_init(const SolveArgs& A, int ncells, cudaStream_t st);
 // label8[lp_off + y nl + pos] = index, in the cell's list of pure phases, of the phase of
 // label[vox_off + y n + iperm[pos]] (255 for a mixed voxel; nl = n rounded up to 16).
@@ -57,9 +74,9 @@ void fast2d_release();
 size_t fast3d_smem_row(int nmax, int nphase_cell);
 size_t fast3d_smem_y(int nmax);
 size_t fast3d_smem_green(int nmax);
-int fast3d_row(const SolveArgs& A, unsigned ntasks, size_t smem, bool out, cudaStream_t st);
-int fast3d_ypass(const SolveArgs& A, unsigned ntasks, size_t smem, bool fwd, cudaStream_t st);
-int fast3d_green(const SolveArgs& A, unsigned ntasks, size_t smem, cudaStream_t st);
+int fast3d_row(const SolveArgs& A, unsigned ntasks, size_t smem, bool out, bool run, cudaStream_t st);
+int fast3d_ypass(const SolveArgs& A, unsigned ntasks, size_t smem, bool fwd, bool run, cudaStream_t st);
+int fast3d_green(const SolveArgs& A, unsigned ntasks, size_t smem, bool run, cudaStream_t st);
 int fast3d_init(const SolveArgs& A, int ncells, cudaStream_t st);
 
 }  // namespace hom

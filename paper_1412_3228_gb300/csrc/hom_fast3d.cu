@@ -37,6 +37,7 @@ constexpr int kSizes3[] = {27, 45, 81, 135, 243};
 #endif
 constexpr int kT3 = HOM_FAST3D_THREADS;     // threads per CTA: the 3D lines (n <= 243) give few
                                             // butterflies per stage, so smaller CTAs idle less
+constexpr int kRunB3 = 512 / kT3;           // the same for the passes whose radices come from a plan
 constexpr int kMinB3 = 768 / kT3;           // resident CTAs per SM the register budget targets
 constexpr uint32_t kLabel8Mixed = 255;      // one-byte label of a mixed voxel
 
@@ -55,12 +56,13 @@ constexpr int kRowSpare3 = 2 * NP * kFastRows;  // float4 entries of the row pas
 // EM (Eyre-Milton scheme): as in the 2D row pass, the state is u = sigma + c0 : eps; pure voxels take
 // tau = W u with a per-phase isotropic W, mixed groups and the output pass solve eps = (c~ + c0)^-1 u
 // first, and the row sums of sigma are (tau + u) / 2.
-template <int N, bool OUT, bool SRC, bool EM = false>
-__device__ __forceinline__ void row3_body(const SolveArgs& A, int task, const TaskR& t, const CellDev& c,
+template <bool OUT, bool SRC, bool EM, class PL>
+__device__ __forceinline__ void row3_body(const PL& pl, const SolveArgs& A, int task, const TaskR& t, const CellDev& c,
                                           const FastPlanDev& fp, float4* s, RowShared3& sh) {
-  constexpr int H = (N + 1) / 2;
-  constexpr int P = (H + 1) / 2;
-  constexpr int NL = (N + 15) / 16 * 16;
+  const int N = pl.n;
+  const int H = N / 2 + 1;
+  const int P = (H + 1) / 2;
+  const int NL = (N + 15) / 16 * 16;
   const int it = *A.it_dev;
   if (threadIdx.x == 0) {
     int nal = 0;
@@ -77,14 +79,14 @@ __device__ __forceinline__ void row3_body(const SolveArgs& A, int task, const Ta
   const float lam0 = OUT ? 0.f : cc.lam0, mu2_0 = OUT ? 0.f : cc.mu2;
   float4* taub = static_cast<float4*>(A.tau);
   const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-  uint8_t* slab = reinterpret_cast<uint8_t*>(s + N * SP);
+  uint8_t* slab = reinterpret_cast<uint8_t*>(s + pl.tile);
   {
     const uint4* src = reinterpret_cast<const uint4*>(A.label8 + c.lp_off + (size_t)t.row0 * NL);
     for (int i = threadIdx.x; i < nr * NL / 16; i += kT3) cp16(slab + 16 * i, src + i);
   }
-  float2* tws = reinterpret_cast<float2*>(s + N * SP + kFastRows * NL / 16);
+  float2* tws = reinterpret_cast<float2*>(s + pl.tile + kFastRows * NL / 16);
   for (int i = threadIdx.x; i < (N + 1) / 2; i += kT3) cp16(tws + 2 * i, fp.tw2 + 2 * i);
-  float4* spare = s + N * SP + kFastRows * NL / 16 + (N + 1) / 2;
+  float4* spare = s + pl.tile + kFastRows * NL / 16 + (N + 1) / 2;
   float2* sph = reinterpret_cast<float2*>(spare + kRowSpare3);
   float2* sinv = sph + c.nph;  // EM: per local phase, (c + c0)^-1 as (coefficient of tr(u) I, of u)
   cp_commit();
@@ -116,7 +118,7 @@ __device__ __forceinline__ void row3_body(const SolveArgs& A, int task, const Ta
       const float4* src = ein + idx3(c, N, l, p, z, y0) + k;
 #pragma unroll
       for (int r = 0; r < kFastRows; ++r)
-        cp16z(row_slot_p<N, NP, SP>(s, spare, p, k, r), src + (size_t)(r < nr ? r : 0) * NP, r < nr ? 16u : 0u);
+        cp16z(row_slot_p<NP>(pl, s, spare, p, k, r), src + (size_t)(r < nr ? r : 0) * NP, r < nr ? 16u : 0u);
     }
     cp_commit();
     if (la + 1 < nal) {  // the next active load's rows -> L2
@@ -131,7 +133,7 @@ __device__ __forceinline__ void row3_body(const SolveArgs& A, int task, const Ta
       const int p = f / NP, k = f - p * NP;
       float4 v[kFastRows];
 #pragma unroll
-      for (int r = 0; r < kFastRows; ++r) v[r] = *row_slot_p<N, NP, SP>(s, spare, p, k, r);
+      for (int r = 0; r < kFastRows; ++r) v[r] = *row_slot_p<NP>(pl, s, spare, p, k, r);
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int kx = 2 * p + h;
@@ -140,9 +142,10 @@ __device__ __forceinline__ void row3_body(const SolveArgs& A, int task, const Ta
         const float2 q1 = h ? make_float2(v[1].y, v[1].w) : make_float2(v[1].x, v[1].z);
         const float2 q2 = h ? make_float2(v[2].y, v[2].w) : make_float2(v[2].x, v[2].z);
         const float2 q3 = h ? make_float2(v[3].y, v[3].w) : make_float2(v[3].x, v[3].z);
-        s[kx * SP + k] = make_float4(q0.x - q1.y, q2.x - q3.y, q0.y + q1.x, q2.y + q3.x);
+        s[pl.at(kx) + k] = make_float4(q0.x - q1.y, q2.x - q3.y, q0.y + q1.x, q2.y + q3.x);
         if (kx > 0) {
-          s[(N - kx) * SP + k] = make_float4(q0.x + q1.y, q2.x + q3.y, q1.x - q0.y, q3.x - q2.y);
+          if (2 * kx != N)  // the Nyquist column of an even grid is its own partner (real rows: q.y = 0)
+            s[pl.at(N - kx) + k] = make_float4(q0.x + q1.y, q2.x + q3.y, q1.x - q0.y, q3.x - q2.y);
         } else {
           sh.dc[la][0][0][k] = q0.x;
           sh.dc[la][0][1][k] = q1.x;
@@ -152,10 +155,11 @@ __device__ __forceinline__ void row3_body(const SolveArgs& A, int task, const Ta
       }
     }
     __syncthreads();
-    fft_dif_p<NP, N, false, float2, SP, kT3>(s, tws);  // inverse: eps at digit-reversed positions
+    fft_dif<NP, false, kT3>(pl, s, tws);  // inverse: eps at digit-reversed positions
 
     // 2. constitutive update; lanes (x, y, z, w) of a float4 are rows (0, 2, 1, 3)
     for (int pos = threadIdx.x; pos < N; pos += kT3) {
+      const int at = pl.at(pos);
       uint32_t lab[kFastRows];
       bool mixed = false;
 #pragma unroll
@@ -165,7 +169,7 @@ __device__ __forceinline__ void row3_body(const SolveArgs& A, int task, const Ta
       }
       float4 e[NP], o[NP];
 #pragma unroll
-      for (int k = 0; k < NP; ++k) e[k] = s[pos * SP + k];
+      for (int k = 0; k < NP; ++k) e[k] = s[at + k];
       if (EM && (OUT || mixed)) {
         // e holds u: eps = (c~ + c0)^-1 u per voxel (mixed: the per-call table; pure: closed form)
         const int x = __ldg(fp.iperm + pos);
@@ -300,12 +304,12 @@ __device__ __forceinline__ void row3_body(const SolveArgs& A, int task, const Ta
         }
       } else {
 #pragma unroll
-        for (int k = 0; k < NP; ++k) s[pos * SP + k] = o[k];
+        for (int k = 0; k < NP; ++k) s[at + k] = o[k];
       }
     }
     __syncthreads();  // the tile is read above and rewritten below (or by the next load's fill)
     if (OUT) continue;
-    fft_dit_p<NP, N, true, float2, SP, kT3>(s, tws);  // forward: natural order
+    fft_dit<NP, true, kT3>(pl, s, tws);  // forward: natural order
 
     // 3. split the two real rows of each line; store the half spectra of tau pair by pair
     for (int f = threadIdx.x; f < P * NP; f += kT3) {
@@ -317,8 +321,8 @@ __device__ __forceinline__ void row3_body(const SolveArgs& A, int task, const Ta
       for (int h = 0; h < 2; ++h) {
         const int kx = 2 * p + h;
         if (kx >= H) break;
-        const float4 Z = s[kx * SP + k];
-        const float4 Zm = s[(kx == 0 ? 0 : N - kx) * SP + k];
+        const float4 Z = s[pl.at(kx) + k];
+        const float4 Zm = s[pl.at(kx == 0 ? 0 : N - kx) + k];
         const float2 o0 = make_float2(0.5f * (Z.x + Zm.x), 0.5f * (Z.z - Zm.z));
         const float2 o1 = make_float2(0.5f * (Z.z + Zm.z), 0.5f * (Zm.x - Z.x));
         const float2 o2 = make_float2(0.5f * (Z.y + Zm.y), 0.5f * (Z.w - Zm.w));
@@ -388,9 +392,9 @@ __device__ __forceinline__ void prefetch_row3_task(const SolveArgs& A, int task)
 }
 
 // One CTA per task; CTA b prefetches the first load of task b + ahead (about the task that starts
-// when this CTA ends: `ahead` CTAs are resident at once) into L2.
-template <bool OUT, bool SRC, bool EM = false>
-__global__ void __launch_bounds__(kT3, kMinB3) k_row_f3d(SolveArgs A, int ntasks, int ahead) {
+// when this CTA ends: `ahead` CTAs are resident at once) into L2.  RUN: radices read from the plan.
+template <bool OUT, bool SRC, bool EM, bool RUN>
+__device__ __forceinline__ void row3_task(const SolveArgs& A, int ntasks, int ahead) {
   HOM_DBG_POISON();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ RowShared3 sh;
@@ -403,33 +407,41 @@ __global__ void __launch_bounds__(kT3, kMinB3) k_row_f3d(SolveArgs A, int ntasks
   if (!HOM_CHECK(A, t.row0 >= 0 && t.nrows >= 1 && t.row0 + t.nrows <= c.nrows &&
                         t.row0 / c.n == (t.row0 + t.nrows - 1) / c.n && t.load < A.L, (size_t)task))
     return;
-  const FastPlanDev fp = A.fplans[c.fplan];
-  switch (c.n) {
-    case 27: row3_body<27, OUT, SRC, EM>(A, task, t, c, fp, s, sh); break;
-    case 45: row3_body<45, OUT, SRC, EM>(A, task, t, c, fp, s, sh); break;
-    case 81: row3_body<81, OUT, SRC, EM>(A, task, t, c, fp, s, sh); break;
-    case 135: row3_body<135, OUT, SRC, EM>(A, task, t, c, fp, s, sh); break;
-    case 243: row3_body<243, OUT, SRC, EM>(A, task, t, c, fp, s, sh); break;
-    default: break;
+  const FastPlanDev& fp = A.fplans[c.fplan];
+  if constexpr (RUN) {
+    row3_body<OUT, SRC, EM>(RunN<SP>(fp.run), A, task, t, c, fp, s, sh);
+  } else {
+    switch (c.n) {
+      case 27: row3_body<OUT, SRC, EM>(FixedN<27, SP>(), A, task, t, c, fp, s, sh); break;
+      case 45: row3_body<OUT, SRC, EM>(FixedN<45, SP>(), A, task, t, c, fp, s, sh); break;
+      case 81: row3_body<OUT, SRC, EM>(FixedN<81, SP>(), A, task, t, c, fp, s, sh); break;
+      case 135: row3_body<OUT, SRC, EM>(FixedN<135, SP>(), A, task, t, c, fp, s, sh); break;
+      case 243: row3_body<OUT, SRC, EM>(FixedN<243, SP>(), A, task, t, c, fp, s, sh); break;
+      default: break;
+    }
   }
 }
+template <bool OUT, bool SRC, bool EM = false>
+__global__ void __launch_bounds__(kT3, kMinB3) k_row_f3d(SolveArgs A, int ntasks, int ahead) {
+  row3_task<OUT, SRC, EM, false>(A, ntasks, ahead);
+}
+// The same pass with radices read from a plan, for batches that hold a size without compiled ones (128
+// registers for radix 16).  Measured against the generic row pass at 64^3, 6 loads: 111 us (112 us).
+template <bool OUT, bool SRC, bool EM = false>
+__global__ void __launch_bounds__(kT3, kRunB3) k_row_r3d(SolveArgs A, int ntasks, int ahead) {
+  row3_task<OUT, SRC, EM, true>(A, ntasks, ahead);
+}
 
-#ifndef HOM_3D_BULK
-#define HOM_3D_BULK 1  // y passes: the tile in and out by bulk copies of one position each
-#endif
 #ifndef HOM_3D_GREEN_GPF
 #define HOM_3D_GREEN_GPF 1  // Green pass: L2 prefetch of the task's own g (or u_hat) block before its forward FFT
 #endif
-#ifndef HOM_3D_GREEN_BULK
-#define HOM_3D_GREEN_BULK 0  // the same for the Green pass, whose positions are a z plane apart in HBM
-#endif
-
 // Bulk copies of the N positions of a tile (NP float4 each, contiguous in HBM at stride gs float4,
 // at stride SP in shared memory) in or out; threads issue one position each in turn.  `load`
 // waits (bounded) for all of them on `bar`, initialised here; running out is recorded in A.dbg.
-template <int N>
-__device__ __forceinline__ void tile_bulk_load(const SolveArgs& A, float4* s, const float4* g, size_t gs,
+template <class PL>
+__device__ __forceinline__ void tile_bulk_load(const PL& pl, float4* s, const float4* g, size_t gs,
                                                unsigned long long* bar) {
+  const int N = pl.n;
   fence_proxy_async();
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -441,7 +453,7 @@ __device__ __forceinline__ void tile_bulk_load(const SolveArgs& A, float4* s, co
   __syncthreads();
   for (int p = threadIdx.x; p < N; p += kT3)
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_u32(s + (size_t)p * SP)),
+                     smem_u32(s + pl.at(p))),
                  "l"(g + (size_t)p * gs), "r"((unsigned)(NP * sizeof(float4))), "r"(smem_u32(bar))
                  : "memory");
 }
@@ -450,14 +462,14 @@ __device__ __forceinline__ void tile_bulk_wait(const SolveArgs& A, unsigned long
   __syncthreads();
   if (threadIdx.x == 0) mbar_inval(bar);
 }
-template <int N>
-__device__ __forceinline__ void tile_bulk_store(float4* g, size_t gs, const float4* s) {
+template <class PL>
+__device__ __forceinline__ void tile_bulk_store(const PL& pl, float4* g, size_t gs, const float4* s) {
   fence_proxy_async();
   __syncthreads();
   bool any = false;
-  for (int p = threadIdx.x; p < N; p += kT3) {
+  for (int p = threadIdx.x; p < pl.n; p += kT3) {
     asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(g + (size_t)p * gs),
-                 "r"(smem_u32(s + (size_t)p * SP)), "r"((unsigned)(NP * sizeof(float4)))
+                 "r"(smem_u32(s + pl.at(p))), "r"((unsigned)(NP * sizeof(float4)))
                  : "memory");
     any = true;
   }
@@ -470,43 +482,34 @@ __device__ __forceinline__ void tile_bulk_store(float4* g, size_t gs, const floa
 // ------------------------------------------------------------------ y passes
 // FWD: tau -> forward y-DFT -> tau (digit-reversed y positions).  Inverse: tau -> inverse y-DFT
 // -> the next eps buffer (natural order).  One contiguous tile per task: [y][component].
-template <int N, bool FWD>
-__device__ __forceinline__ void ypass3_body(const SolveArgs& A, const TaskL& t, const CellDev& c,
+template <bool FWD, class PL>
+__device__ __forceinline__ void ypass3_body(const PL& pl, const SolveArgs& A, const TaskL& t, const CellDev& c,
                                             const FastPlanDev& fp, float4* s) {
   if (!A.active[t.cell * A.L + t.load]) return;
+  const int N = pl.n;
   const int it = *A.it_dev;
   const size_t tb = idx3(c, N, t.load, t.kx0 / 2, t.fixed, 0);
   const float4* in = static_cast<const float4*>(A.tau) + tb;
   float4* out = static_cast<float4*>(FWD ? A.tau : A.eps[(it + 1) & 1]) + tb;
-  float2* tws = reinterpret_cast<float2*>(s + N * SP);
-#if HOM_3D_BULK
+  float2* tws = reinterpret_cast<float2*>(s + pl.tile);
   __shared__ __align__(8) unsigned long long ybar;
-  tile_bulk_load<N>(A, s, in, NP, &ybar);
-#else
-  for (int i = threadIdx.x; i < N * NP; i += kT3) cp16(s + (i / NP) * SP + i % NP, in + i);
-#endif
+  tile_bulk_load(pl, s, in, NP, &ybar);
   for (int i = threadIdx.x; i < (N + 1) / 2; i += kT3) cp16(tws + 2 * i, fp.tw2 + 2 * i);
   cp_commit();
   cp_wait_all();
-#if HOM_3D_BULK
   tile_bulk_wait(A, &ybar);
-#endif
   __syncthreads();
-  if (FWD) fft_dif_p<NP, N, true, float2, SP, kT3>(s, tws);
-  else fft_dit_p<NP, N, false, float2, SP, kT3>(s, tws);
-#if HOM_3D_BULK
-  tile_bulk_store<N>(out, NP, s);
-#else
-  for (int i = threadIdx.x; i < N * NP; i += kT3) out[i] = s[(i / NP) * SP + i % NP];
-#endif
+  if (FWD) fft_dif<NP, true, kT3>(pl, s, tws);
+  else fft_dit<NP, false, kT3>(pl, s, tws);
+  tile_bulk_store(pl, out, NP, s);
   if (threadIdx.x == 0) {
     const int ntk = t.kx0 + 1 < c.H ? 2 : 1;
     atomicAdd(A.bytes + (FWD ? HOM_K_YFWD : HOM_K_YINV), (unsigned long long)(2 * (size_t)N * ntk * NP * sizeof(float2)));
   }
 }
 
-template <bool FWD>
-__global__ void __launch_bounds__(kT3, 1024 / kT3) k_ypass_f3d(SolveArgs A) {
+template <bool FWD, bool RUN>
+__device__ __forceinline__ void ypass3_task(const SolveArgs& A) {
   HOM_DBG_POISON();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float4* s = reinterpret_cast<float4*>(smem_raw);
@@ -515,25 +518,41 @@ __global__ void __launch_bounds__(kT3, 1024 / kT3) k_ypass_f3d(SolveArgs A) {
   if (!HOM_CHECK(A, t.kx0 >= 0 && (t.kx0 & 1) == 0 && t.kx0 < c.H && t.fixed >= 0 && t.fixed < c.n &&
                         t.load >= 0 && t.load < A.L, (size_t)blockIdx.x))
     return;
-  const FastPlanDev fp = A.fplans[c.fplan];
-  switch (c.n) {
-    case 27: ypass3_body<27, FWD>(A, t, c, fp, s); break;
-    case 45: ypass3_body<45, FWD>(A, t, c, fp, s); break;
-    case 81: ypass3_body<81, FWD>(A, t, c, fp, s); break;
-    case 135: ypass3_body<135, FWD>(A, t, c, fp, s); break;
-    case 243: ypass3_body<243, FWD>(A, t, c, fp, s); break;
-    default: break;
+  const FastPlanDev& fp = A.fplans[c.fplan];
+  if constexpr (RUN) {
+    ypass3_body<FWD>(RunN<SP>(fp.run), A, t, c, fp, s);
+  } else {
+    switch (c.n) {
+      case 27: ypass3_body<FWD>(FixedN<27, SP>(), A, t, c, fp, s); break;
+      case 45: ypass3_body<FWD>(FixedN<45, SP>(), A, t, c, fp, s); break;
+      case 81: ypass3_body<FWD>(FixedN<81, SP>(), A, t, c, fp, s); break;
+      case 135: ypass3_body<FWD>(FixedN<135, SP>(), A, t, c, fp, s); break;
+      case 243: ypass3_body<FWD>(FixedN<243, SP>(), A, t, c, fp, s); break;
+      default: break;
+    }
   }
+}
+template <bool FWD>
+__global__ void __launch_bounds__(kT3, 1024 / kT3) k_ypass_f3d(SolveArgs A) {
+  ypass3_task<FWD, false>(A);
+}
+// radices read from a plan: 64^3, 6 loads: 58 us (115-120 us for the generic passes)
+template <bool FWD>
+__global__ void __launch_bounds__(kT3, kRunB3) k_ypass_r3d(SolveArgs A) {
+  ypass3_task<FWD, true>(A);
 }
 
 // ------------------------------------------------------------------ Green pass (z lines)
 // Eyre-Milton scheme: the positions of one thread, lane by lane through em_core (hom_em.cuh); the
 // private state is u_hat of the current iterate, [z position][6 components] as lane pairs (the
 // layout of the tile), in place of g.
-template <int N>
-__device__ __forceinline__ void green3_em(int kx0, bool hasB, int py, const CellDev& c, const float* sx,
+template <class PL>
+__device__ __forceinline__ void green3_em(const PL& pl, int kx0, bool hasB, int py, const CellDev& c, const float* sx,
                                           const FastPlanDev& fp, float4* s, float4* ub, const double* Eld,
                                           Acc<float> (&acc)[3]) {
+  const int N = pl.n;
+  // Nyquist bins of an even grid (a wave number no odd grid has)
+  const float nyq = (N & 1) ? -1.f : __ldg(fp.xinat + N / 2);
   CellConst<float> cc;
   cell_const(c, cc);
   const float nvT = (float)c.nv, inv_nv = cc.inv_nv, lam0 = cc.lam0, mu2_0 = cc.mu2;
@@ -548,17 +567,18 @@ __device__ __forceinline__ void green3_em(int kx0, bool hasB, int py, const Cell
     float2 th[NP], uh[NP], un[NP];
 #pragma unroll
     for (int k = 0; k < NP; ++k) {
-      const float* T = sf + 4 * (pos * SP + k);
+      const float* T = sf + 4 * (pl.at(pos) + k);
       const float* U = uf + 4 * (NP * pos + k);
       th[k] = make_float2(T[h], T[2 + h]);
       uh[k] = make_float2(U[h], U[2 + h]);
     }
     const float xi[3] = {X[h], Y, sx[pos]};
-    em_core<float, 3>(th, uh, un, xi, h == 0 && kx0 == 0 && py == 0 && pos == 0, false, h == 0 && kx0 == 0, nvT,
-                      inv_nv, lam0, mu2_0, a0, inv_mu2_0, cc.inv_mu0, cc.ratio, Eld, acc[0], acc[1], acc[2]);
+    em_core<float, 3>(th, uh, un, xi, h == 0 && kx0 == 0 && py == 0 && pos == 0,
+                      xi[0] == nyq || Y == nyq || xi[2] == nyq, (h == 0 && kx0 == 0) || xi[0] == nyq, nvT, inv_nv,
+                       lam0, mu2_0, a0, inv_mu2_0, cc.inv_mu0, cc.ratio, Eld, acc[0], acc[1], acc[2]);
 #pragma unroll
     for (int k = 0; k < NP; ++k) {
-      float* T = sf + 4 * (pos * SP + k);
+      float* T = sf + 4 * (pl.at(pos) + k);
       float* U = uf + 4 * (NP * pos + k);
       T[h] = un[k].x;
       T[2 + h] = un[k].y;
@@ -569,15 +589,15 @@ __device__ __forceinline__ void green3_em(int kx0, bool hasB, int py, const Cell
   if (!hasB)  // the missing lane B of the last pair stays zero
     for (int i = threadIdx.x; i < N * NP; i += kT3) {
       const int pos = i / NP, k = i - pos * NP;
-      sf[4 * (pos * SP + k) + 1] = 0.f;
-      sf[4 * (pos * SP + k) + 3] = 0.f;
+      sf[4 * (pl.at(pos) + k) + 1] = 0.f;
+      sf[4 * (pl.at(pos) + k) + 3] = 0.f;
     }
 }
 
-template <int N, bool EM = false>
-__device__ __forceinline__ void green3_body(const SolveArgs& A, const TaskL& t, const CellDev& c,
+template <bool EM, class PL>
+__device__ __forceinline__ void green3_body(const PL& pl, const SolveArgs& A, const TaskL& t, const CellDev& c,
                                             const FastPlanDev& fp, float4* s) {
-  constexpr int H = (N + 1) / 2;
+  const int N = pl.n, H = N / 2 + 1;
   const int cl = t.cell * A.L + t.load;
   if (!A.active[cl]) return;
   const int kx0 = t.kx0, py = t.fixed, p = kx0 / 2;
@@ -585,24 +605,17 @@ __device__ __forceinline__ void green3_body(const SolveArgs& A, const TaskL& t, 
   float4* st = static_cast<float4*>(A.tau);
   const size_t zs = (size_t)N * NP;  // float4 stride between z planes at fixed y
   const size_t b0 = idx3(c, N, t.load, p, 0, py);
-  float2* tws = reinterpret_cast<float2*>(s + N * SP);
-  float* sx = reinterpret_cast<float*>(s + N * SP + (N + 1) / 2);
-#if HOM_3D_GREEN_BULK
-  __shared__ __align__(8) unsigned long long gbar;
-  tile_bulk_load<N>(A, s, st + b0, zs, &gbar);
-#else
+  float2* tws = reinterpret_cast<float2*>(s + pl.tile);
+  float* sx = reinterpret_cast<float*>(s + pl.tile + (N + 1) / 2);
+  // (positions a z plane apart in HBM: 96-byte bulk copies measured 8 % slower than these)
   for (int i = threadIdx.x; i < N * NP; i += kT3) {
     const int zz = i / NP, k = i - zz * NP;
-    cp16(s + zz * SP + k, st + b0 + zz * zs + k);
+    cp16(s + pl.at(zz) + k, st + b0 + zz * zs + k);
   }
-#endif
   for (int i = threadIdx.x; i < (N + 1) / 2; i += kT3) cp16(tws + 2 * i, fp.tw2 + 2 * i);
   for (int i = threadIdx.x; i < (N + 3) / 4; i += kT3) cp16(sx + 4 * i, fp.xipos + 4 * i);
   cp_commit();
   cp_wait_all();
-#if HOM_3D_GREEN_BULK
-  tile_bulk_wait(A, &gbar);
-#endif
   __syncthreads();
 #if HOM_3D_GREEN_GPF
   // the private state of this (kx pair, ky) (contiguous: N positions x 3 or 6 float4) -> L2
@@ -615,13 +628,13 @@ __device__ __forceinline__ void green3_body(const SolveArgs& A, const TaskL& t, 
     for (unsigned o = threadIdx.x * kPiece; o < bytes; o += 32 * kPiece) prefetch_l2(gsrc + o, min(kPiece, bytes - o));
   }
 #endif
-  fft_dif_p<NP, N, true, float2, SP, kT3>(s, tws);  // forward: bin kz at position perm(kz)
+  fft_dif<NP, true, kT3>(pl, s, tws);  // forward: bin kz at position perm(kz)
 
   if constexpr (EM) {
     float4* ub = static_cast<float4*>(A.g) +
                  (c.g_off + (((size_t)t.load * (c.Hp / 2) + p) * N + py) * (size_t)N * 12) / 2;
     Acc<float> acc[3];
-    green3_em<N>(kx0, hasB, py, c, sx, fp, s, ub, A.E + (size_t)cl * NP, acc);
+    green3_em(pl, kx0, hasB, py, c, sx, fp, s, ub, A.E + (size_t)cl * NP, acc);
     double tot[3];
     block_sum<float, 3, kT3>(acc, tot);  // contains the barrier before the inverse transform
     if (threadIdx.x == 0) {
@@ -629,15 +642,11 @@ __device__ __forceinline__ void green3_body(const SolveArgs& A, const TaskL& t, 
       A.partC[2 * (size_t)blockIdx.x + 1] = tot[1];
       A.partE[blockIdx.x] = tot[2];
     }
-    fft_dit_p<NP, N, false, float2, SP, kT3>(s, tws);  // inverse: natural z order
-#if HOM_3D_GREEN_BULK
-    tile_bulk_store<N>(st + b0, zs, s);
-#else
+    fft_dit<NP, false, kT3>(pl, s, tws);  // inverse: natural z order
     for (int i = threadIdx.x; i < N * NP; i += kT3) {
       const int zz = i / NP, k = i - zz * NP;
-      st[b0 + zz * zs + k] = s[zz * SP + k];
+      st[b0 + zz * zs + k] = s[pl.at(zz) + k];
     }
-#endif
     if (threadIdx.x == 0) {
       const int ntk = hasB ? 2 : 1;
       atomicAdd(A.bytes + HOM_K_GREEN, (unsigned long long)(4 * (size_t)N * ntk * NP * sizeof(float2)));
@@ -653,17 +662,22 @@ __device__ __forceinline__ void green3_body(const SolveArgs& A, const TaskL& t, 
   const float2 X = make_float2(__ldg(fp.xinat + kx0), hasB ? __ldg(fp.xinat + kx0 + 1) : 0.f);
   const float2 Y = f2(sx[py]);
   const float2 XY2 = fma2(Y, Y, mul2(X, X));
-  const float2 wgt = make_float2(kx0 == 0 ? 1.f : 2.f, hasB ? 2.f : 0.f);
+  // even grids: wave vectors with a Nyquist component get zero strain and no residual (see the 2D pass)
+  const bool even = !(N & 1);
+  const float nyq = even ? __ldg(fp.xinat + N / 2) : 0.f;
+  const bool deadA = even && (2 * kx0 == N || Y.x == nyq), deadB = !hasB || (even && (2 * kx0 + 2 == N || Y.x == nyq));
+  const float2 wgt = make_float2(deadA ? 0.f : kx0 == 0 ? 1.f : 2.f, deadB ? 0.f : 2.f);
   // g of this (kx pair, y position): [z position][3 lane pairs]
   float4* gb = static_cast<float4*>(A.g) +
                (c.g_off + (((size_t)t.load * (c.Hp / 2) + p) * N + py) * (size_t)N * 6) / 2;
   const double* Eld = A.E + (size_t)cl * NP;
   float2 r2s = make_float2(0.f, 0.f), r2c = r2s, rns = r2s, rnc = r2s;
   for (int pos = threadIdx.x; pos < N; pos += kT3) {
+    const int at = pl.at(pos);
     const float2 Z = f2(sx[pos]);
     P2 T[NP];
 #pragma unroll
-    for (int k = 0; k < NP; ++k) T[k] = ldp(s[pos * SP + k]);
+    for (int k = 0; k < NP; ++k) T[k] = ldp(s[at + k]);
     P2 G[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) G[d] = ldp(gb[3 * pos + d]);
@@ -692,7 +706,9 @@ __device__ __forceinline__ void green3_body(const SolveArgs& A, const TaskL& t, 
     r2 = fma2(R2.re, R2.re, r2);
     r2 = fma2(R2.im, R2.im, r2);
     const bool k0 = kx0 == 0 && py == 0 && pos == 0;  // k = 0: eps_hat(0) = E, g = 0, no residual
-    const float2 iq = make_float2(k0 ? 0.f : __fdividef(1.f, q2.x), hasB ? __fdividef(1.f, q2.y) : 0.f);
+    const bool dead = even && Z.x == nyq;
+    const float2 iq = make_float2(k0 || deadA || dead ? 0.f : __fdividef(1.f, q2.x),
+                                  deadB || dead ? 0.f : __fdividef(1.f, q2.y));
     // g' = K0^-1 (tau_hat xi), eps_hat' = -sym(xi (x) g') / N_v
     const float2 imq = mul2(inv_mu0, iq);
     const float2 rq = mul2(ratio, iq);
@@ -714,7 +730,7 @@ __device__ __forceinline__ void green3_body(const SolveArgs& A, const TaskL& t, 
     E[4] = sym(W0, Z, W2, X);  // 13
     E[5] = sym(W0, Y, W1, X);  // 12
     P2 Gn[3] = {W0, W1, W2};
-    float2 wr = wgt;
+    float2 wr = dead ? make_float2(0.f, 0.f) : wgt;
     if (k0) {
 #pragma unroll
       for (int k = 0; k < NP; ++k) {
@@ -729,7 +745,7 @@ __device__ __forceinline__ void green3_body(const SolveArgs& A, const TaskL& t, 
       wr.x = 0.f;
     }
 #pragma unroll
-    for (int k = 0; k < NP; ++k) s[pos * SP + k] = stp(E[k]);
+    for (int k = 0; k < NP; ++k) s[at + k] = stp(E[k]);
 #pragma unroll
     for (int d = 0; d < 3; ++d) gb[3 * pos + d] = stp(Gn[d]);
     const float2 a1 = mul2(wr, r2), a2 = mul2(a1, iq);
@@ -761,15 +777,11 @@ __device__ __forceinline__ void green3_body(const SolveArgs& A, const TaskL& t, 
       A.partC[2 * (size_t)blockIdx.x + 1] = tot[1];
     }
   }
-  fft_dit_p<NP, N, false, float2, SP, kT3>(s, tws);  // inverse: natural z order
-#if HOM_3D_GREEN_BULK
-  tile_bulk_store<N>(st + b0, zs, s);
-#else
+  fft_dit<NP, false, kT3>(pl, s, tws);  // inverse: natural z order
   for (int i = threadIdx.x; i < N * NP; i += kT3) {
     const int zz = i / NP, k = i - zz * NP;
-    st[b0 + zz * zs + k] = s[zz * SP + k];
+    st[b0 + zz * zs + k] = s[pl.at(zz) + k];
   }
-#endif
   if (threadIdx.x == 0) {
     const int ntk = hasB ? 2 : 1;
     atomicAdd(A.bytes + HOM_K_GREEN,
@@ -777,8 +789,8 @@ __device__ __forceinline__ void green3_body(const SolveArgs& A, const TaskL& t, 
   }
 }
 
-template <bool EM = false>
-__global__ void __launch_bounds__(kT3, kMinB3) k_green_f3d(SolveArgs A) {
+template <bool EM, bool RUN>
+__device__ __forceinline__ void green3_task(const SolveArgs& A) {
   HOM_DBG_POISON();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float4* s = reinterpret_cast<float4*>(smem_raw);
@@ -787,15 +799,28 @@ __global__ void __launch_bounds__(kT3, kMinB3) k_green_f3d(SolveArgs A) {
   if (!HOM_CHECK(A, t.kx0 >= 0 && (t.kx0 & 1) == 0 && t.kx0 < c.H && t.fixed >= 0 && t.fixed < c.n &&
                         t.load >= 0 && t.load < A.L, (size_t)blockIdx.x))
     return;
-  const FastPlanDev fp = A.fplans[c.fplan];
-  switch (c.n) {
-    case 27: green3_body<27, EM>(A, t, c, fp, s); break;
-    case 45: green3_body<45, EM>(A, t, c, fp, s); break;
-    case 81: green3_body<81, EM>(A, t, c, fp, s); break;
-    case 135: green3_body<135, EM>(A, t, c, fp, s); break;
-    case 243: green3_body<243, EM>(A, t, c, fp, s); break;
-    default: break;
+  const FastPlanDev& fp = A.fplans[c.fplan];
+  if constexpr (RUN) {
+    green3_body<EM>(RunN<SP>(fp.run), A, t, c, fp, s);
+  } else {
+    switch (c.n) {
+      case 27: green3_body<EM>(FixedN<27, SP>(), A, t, c, fp, s); break;
+      case 45: green3_body<EM>(FixedN<45, SP>(), A, t, c, fp, s); break;
+      case 81: green3_body<EM>(FixedN<81, SP>(), A, t, c, fp, s); break;
+      case 135: green3_body<EM>(FixedN<135, SP>(), A, t, c, fp, s); break;
+      case 243: green3_body<EM>(FixedN<243, SP>(), A, t, c, fp, s); break;
+      default: break;
+    }
   }
+}
+template <bool EM = false>
+__global__ void __launch_bounds__(kT3, kMinB3) k_green_f3d(SolveArgs A) {
+  green3_task<EM, false>(A);
+}
+// radices read from a plan: 64^3, 6 loads: 81 us (179 us generic)
+template <bool EM = false>
+__global__ void __launch_bounds__(kT3, kRunB3) k_green_r3d(SolveArgs A) {
+  green3_task<EM, true>(A);
 }
 
 // eps = E: the stored x-spectrum holds E at kx = 0 (lane A of pair 0) of every row, zero elsewhere.
@@ -839,64 +864,70 @@ bool fast3d_size(int n) {
   return false;
 }
 
+bool run3d_size(int n) {  // the row pass's tile, twiddles and labels of 4 rows on chip, a few phases
+  return grid_supported(n) && fast3d_smem_row(n, 64) <= 200 * 1024;
+}
+
 // row: tile | one-byte labels of 4 rows | twiddles | spare landing slots | per-phase constants;
 // y: tile | twiddles;
 // Green: tile | twiddles | wave numbers
+// (even sizes: the tile with its padding, at most one float4 for every two positions)
+namespace {
+size_t tile_bytes3(int n) { return ((size_t)n * SP + ((n & 1) ? 0 : n / 2)) * sizeof(float4); }
+}  // namespace
 size_t fast3d_smem_row(int nmax, int nphase_cell) {
-  return (size_t)nmax * SP * sizeof(float4) + (size_t)kFastRows * ((nmax + 15) / 16 * 16) +
-         ((size_t)nmax + 1) / 2 * 16 + (size_t)kRowSpare3 * sizeof(float4) + ((size_t)nphase_cell * 16 + 15) / 16 * 16;
+  return tile_bytes3(nmax) + (size_t)kFastRows * ((nmax + 15) / 16 * 16) + ((size_t)nmax + 1) / 2 * 16 +
+         (size_t)kRowSpare3 * sizeof(float4) + ((size_t)nphase_cell * 16 + 15) / 16 * 16;
 }
-size_t fast3d_smem_y(int nmax) { return (size_t)nmax * SP * sizeof(float4) + ((size_t)nmax + 1) / 2 * 16; }
+size_t fast3d_smem_y(int nmax) { return tile_bytes3(nmax) + ((size_t)nmax + 1) / 2 * 16; }
 size_t fast3d_smem_green(int nmax) {
-  return (size_t)nmax * SP * sizeof(float4) + ((size_t)nmax + 1) / 2 * 16 + ((size_t)nmax + 3) / 4 * 16;
+  return tile_bytes3(nmax) + ((size_t)nmax + 1) / 2 * 16 + ((size_t)nmax + 3) / 4 * 16;
 }
 
-int fast3d_row(const SolveArgs& A, unsigned ntasks, size_t smem, bool out, cudaStream_t st) {
-  int rc;
-  if (A.scheme == HOM_SCHEME_EYRE_MILTON && out) {
-    if ((rc = opt_in3(k_row_f3d<true, false, true>, smem)) != HOM_OK) return rc;
-    k_row_f3d<true, false, true><<<ntasks, kT3, smem, st>>>(A, (int)ntasks,
-                                                            resident_ctas(k_row_f3d<true, false, true>, kT3, smem));
-  } else if (A.scheme == HOM_SCHEME_EYRE_MILTON) {
-    if ((rc = opt_in3(k_row_f3d<false, false, true>, smem)) != HOM_OK) return rc;
-    k_row_f3d<false, false, true><<<ntasks, kT3, smem, st>>>(A, (int)ntasks,
-                                                             resident_ctas(k_row_f3d<false, false, true>, kT3, smem));
-  } else if (out) {
-    if ((rc = opt_in3(k_row_f3d<true, false>, smem)) != HOM_OK) return rc;
-    k_row_f3d<true, false><<<ntasks, kT3, smem, st>>>(A, (int)ntasks, resident_ctas(k_row_f3d<true, false>, kT3, smem));
-  } else if (A.src) {  // adjoint solve: the constitutive step takes the source term
-    if ((rc = opt_in3(k_row_f3d<false, true>, smem)) != HOM_OK) return rc;
-    k_row_f3d<false, true><<<ntasks, kT3, smem, st>>>(A, (int)ntasks, resident_ctas(k_row_f3d<false, true>, kT3, smem));
-  } else {
-    if ((rc = opt_in3(k_row_f3d<false, false>, smem)) != HOM_OK) return rc;
-    k_row_f3d<false, false><<<ntasks, kT3, smem, st>>>(A, (int)ntasks, resident_ctas(k_row_f3d<false, false>, kT3, smem));
-  }
-  return HOM_OK;
-}
-
-int fast3d_ypass(const SolveArgs& A, unsigned ntasks, size_t smem, bool fwd, cudaStream_t st) {
-  int rc;
-  if (fwd) {
-    if ((rc = opt_in3(k_ypass_f3d<true>, smem)) != HOM_OK) return rc;
-    k_ypass_f3d<true><<<ntasks, kT3, smem, st>>>(A);
-  } else {
-    if ((rc = opt_in3(k_ypass_f3d<false>, smem)) != HOM_OK) return rc;
-    k_ypass_f3d<false><<<ntasks, kT3, smem, st>>>(A);
-  }
-  return HOM_OK;
-}
-
-int fast3d_green(const SolveArgs& A, unsigned ntasks, size_t smem, cudaStream_t st) {
-  if (A.scheme == HOM_SCHEME_EYRE_MILTON) {
-    int rc = opt_in3(k_green_f3d<true>, smem);
-    if (rc != HOM_OK) return rc;
-    k_green_f3d<true><<<ntasks, kT3, smem, st>>>(A);
-    return HOM_OK;
-  }
-  int rc = opt_in3(k_green_f3d<false>, smem);
+namespace {
+template <typename K>
+int launch_row3(K kernel, const SolveArgs& A, unsigned ntasks, size_t smem, cudaStream_t st) {
+  int rc = opt_in3(kernel, smem);
   if (rc != HOM_OK) return rc;
-  k_green_f3d<false><<<ntasks, kT3, smem, st>>>(A);
+  kernel<<<ntasks, kT3, smem, st>>>(A, (int)ntasks, resident_ctas(kernel, kT3, smem));
   return HOM_OK;
+}
+template <typename K>
+int launch_lines3(K kernel, const SolveArgs& A, unsigned ntasks, size_t smem, cudaStream_t st) {
+  int rc = opt_in3(kernel, smem);
+  if (rc != HOM_OK) return rc;
+  kernel<<<ntasks, kT3, smem, st>>>(A);
+  return HOM_OK;
+}
+}  // namespace
+
+int fast3d_row(const SolveArgs& A, unsigned ntasks, size_t smem, bool out, bool run, cudaStream_t st) {
+  if (A.scheme == HOM_SCHEME_EYRE_MILTON) {
+    if (out)
+      return run ? launch_row3(k_row_r3d<true, false, true>, A, ntasks, smem, st)
+                 : launch_row3(k_row_f3d<true, false, true>, A, ntasks, smem, st);
+    return run ? launch_row3(k_row_r3d<false, false, true>, A, ntasks, smem, st)
+               : launch_row3(k_row_f3d<false, false, true>, A, ntasks, smem, st);
+  }
+  if (out)
+    return run ? launch_row3(k_row_r3d<true, false>, A, ntasks, smem, st)
+               : launch_row3(k_row_f3d<true, false>, A, ntasks, smem, st);
+  if (A.src)  // adjoint solve: the constitutive step takes the source term
+    return run ? launch_row3(k_row_r3d<false, true>, A, ntasks, smem, st)
+               : launch_row3(k_row_f3d<false, true>, A, ntasks, smem, st);
+  return run ? launch_row3(k_row_r3d<false, false>, A, ntasks, smem, st)
+             : launch_row3(k_row_f3d<false, false>, A, ntasks, smem, st);
+}
+
+int fast3d_ypass(const SolveArgs& A, unsigned ntasks, size_t smem, bool fwd, bool run, cudaStream_t st) {
+  if (fwd) return run ? launch_lines3(k_ypass_r3d<true>, A, ntasks, smem, st) : launch_lines3(k_ypass_f3d<true>, A, ntasks, smem, st);
+  return run ? launch_lines3(k_ypass_r3d<false>, A, ntasks, smem, st) : launch_lines3(k_ypass_f3d<false>, A, ntasks, smem, st);
+}
+
+int fast3d_green(const SolveArgs& A, unsigned ntasks, size_t smem, bool run, cudaStream_t st) {
+  if (A.scheme == HOM_SCHEME_EYRE_MILTON)
+    return run ? launch_lines3(k_green_r3d<true>, A, ntasks, smem, st) : launch_lines3(k_green_f3d<true>, A, ntasks, smem, st);
+  return run ? launch_lines3(k_green_r3d<false>, A, ntasks, smem, st) : launch_lines3(k_green_f3d<false>, A, ntasks, smem, st);
 }
 
 int fast3d_init(const SolveArgs& A, int ncells, cudaStream_t st) {

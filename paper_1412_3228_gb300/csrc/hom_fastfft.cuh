@@ -82,8 +82,10 @@ __device__ __forceinline__ void mbar_init(unsigned long long* bar, unsigned coun
 __device__ __forceinline__ void mbar_inval(unsigned long long* bar) {
   asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-__device__ __forceinline__ void bulk_load(void* sdst, const void* gsrc, unsigned bytes, unsigned long long* bar) {
+__device__ __forceinline__ void mbar_expect(unsigned long long* bar, unsigned bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void bulk_load(void* sdst, const void* gsrc, unsigned bytes, unsigned long long* bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                    smem_u32(sdst)),
                "l"(gsrc), "r"(bytes), "r"(smem_u32(bar))
@@ -133,13 +135,14 @@ __device__ __forceinline__ void bulk_store_wait_read() { asm volatile("cp.async.
 // N - 1, and H - 1, H) are no other pair's landing slots.
 // (NC lane pairs per position, SP float4 between positions in shared memory; the spare area holds
 // 2 NC kFastRows float4.)
-template <int N, int NC, int SP>
-__device__ __forceinline__ float4* row_slot_p(float4* s, float4* spare, int p, int k, int r) {
-  constexpr int H = (N + 1) / 2, P = (H + 1) / 2;
+// On even N the last pair holds the Nyquist column N / 2, its own partner: it lands in the spare area too.
+template <int NC, class PL>
+__device__ __forceinline__ float4* row_slot_p(const PL& pl, float4* s, float4* spare, int p, int k, int r) {
+  const int N = pl.n, H = N / 2 + 1, P = (H + 1) / 2;
   if (p == 0) return spare + k * kFastRows + r;
-  if ((H & 1) && p == P - 1) return spare + (NC + k) * kFastRows + r;
+  if (p == P - 1 && ((H & 1) || !(N & 1))) return spare + (NC + k) * kFastRows + r;
   const int pos = r < 2 ? 2 * p + r : N - 2 * p - (3 - r);  // 2p, 2p + 1, N - 2p - 1, N - 2p
-  return s + pos * SP + k;
+  return s + pl.at(pos) + k;
 }
 
 // Two complex numbers, one per line: re = (re_A, re_B), im = (im_A, im_B).
@@ -175,17 +178,29 @@ constexpr float kH3 = 0.866025403784438646763723170753f;  // sin(2 pi / 3)
 constexpr float kC51 = 0.309016994374947424102293417183f, kC52 = -0.809016994374947424102293417183f;
 constexpr float kS51 = 0.951056516295153572116439333379f, kS52 = 0.587785252292473129168705954639f;
 enum { KMH = 0, KH3, KNH3, KC51, KC52, KS51, KS52, KNS51, KNS52, KTW9 };
-constexpr int kTw15 = KTW9 + 27;
-__constant__ float2 kP[kTw15 + 45] = {
+constexpr int kTw15 = KTW9 + 27, kTw7 = kTw15 + 45, kTw11 = kTw7 + 21, kTw13 = kTw11 + 33, kTw16 = kTw13 + 39;
+__constant__ float2 kP[kTw16 + 48] = {
     {-0.5f, -0.5f}, {kH3, kH3}, {-kH3, -kH3}, {kC51, kC51}, {kC52, kC52}, {kS51, kS51}, {kS52, kS52}, {-kS51, -kS51},
     {-kS52, -kS52},
     HOM_TWP(9, 0), HOM_TWP(9, 1), HOM_TWP(9, 2), HOM_TWP(9, 3), HOM_TWP(9, 4), HOM_TWP(9, 5), HOM_TWP(9, 6),
     HOM_TWP(9, 7), HOM_TWP(9, 8),
     HOM_TWP(15, 0), HOM_TWP(15, 1), HOM_TWP(15, 2), HOM_TWP(15, 3), HOM_TWP(15, 4), HOM_TWP(15, 5), HOM_TWP(15, 6),
     HOM_TWP(15, 7), HOM_TWP(15, 8), HOM_TWP(15, 9), HOM_TWP(15, 10), HOM_TWP(15, 11), HOM_TWP(15, 12),
-    HOM_TWP(15, 13), HOM_TWP(15, 14)};
+    HOM_TWP(15, 13), HOM_TWP(15, 14),
+    HOM_TWP(49, 0), HOM_TWP(49, 7), HOM_TWP(49, 14), HOM_TWP(49, 21), HOM_TWP(49, 28), HOM_TWP(49, 35), HOM_TWP(49, 42),
+    HOM_TWP(11, 0), HOM_TWP(11, 1), HOM_TWP(11, 2), HOM_TWP(11, 3), HOM_TWP(11, 4), HOM_TWP(11, 5), HOM_TWP(11, 6),
+    HOM_TWP(11, 7), HOM_TWP(11, 8), HOM_TWP(11, 9), HOM_TWP(11, 10),
+    HOM_TWP(13, 0), HOM_TWP(13, 1), HOM_TWP(13, 2), HOM_TWP(13, 3), HOM_TWP(13, 4), HOM_TWP(13, 5), HOM_TWP(13, 6),
+    HOM_TWP(13, 7), HOM_TWP(13, 8), HOM_TWP(13, 9), HOM_TWP(13, 10), HOM_TWP(13, 11), HOM_TWP(13, 12),
+    HOM_TWP(16, 0), HOM_TWP(16, 1), HOM_TWP(16, 2), HOM_TWP(16, 3), HOM_TWP(16, 4), HOM_TWP(16, 5), HOM_TWP(16, 6),
+    HOM_TWP(16, 7), HOM_TWP(16, 8), HOM_TWP(16, 9), HOM_TWP(16, 10), HOM_TWP(16, 11), HOM_TWP(16, 12),
+    HOM_TWP(16, 13), HOM_TWP(16, 14), HOM_TWP(16, 15)};
 #undef HOM_TWP
-template <int R> __device__ __forceinline__ constexpr int tw_base() { return R == 9 ? KTW9 : kTw15; }
+template <int R> __device__ __forceinline__ constexpr int tw_base() {
+  return R == 9 ? KTW9 : R == 7 ? kTw7 : R == 11 ? kTw11 : R == 13 ? kTw13 : R == 16 || R == 8 || R == 4 ? kTw16 : kTw15;
+}
+// entry step of radix R in its constant table (4 and 8 use the table of 16)
+template <int R> __device__ __forceinline__ constexpr int tw_step() { return R == 4 ? 4 : R == 8 ? 2 : 1; }
 
 // ------------------------------------------------------------------ register DFTs on lane pairs
 // Forward transforms use w = exp(-2 pi i / r), inverse ones conj(w); no scaling.  Composite sizes
@@ -241,7 +256,7 @@ __device__ __forceinline__ void dft_compositep(P2* v) {
         v[B * ka + nb] = x;
       } else {
         // x (cos + i sn), sn = -+sin(2 pi m / R)
-        const int b = tw_base<R>() + 3 * m;
+        const int b = tw_base<R>() + 3 * m * tw_step<R>();
         const float2 c = kP[b], sp = kP[b + 1], sm = kP[b + 2];
         const float2 sn = FWD ? sm : sp, nsn = FWD ? sp : sm;
         v[B * ka + nb] = P2{fma2(x.im, nsn, mul2(x.re, c)), fma2(x.im, c, mul2(x.re, sn))};
@@ -252,10 +267,57 @@ __device__ __forceinline__ void dft_compositep(P2* v) {
   for (int ka = 0; ka < A; ++ka) dftp<B, FWD>(v + B * ka);
 }
 
+__device__ __forceinline__ void dft2p(P2* v) {
+  const P2 t = v[0] - v[1];
+  v[0] = v[0] + v[1];
+  v[1] = t;
+}
+template <bool FWD>
+__device__ __forceinline__ void dft4p(P2* v) {  // X[k] left in v[out_pos<4>(k)] (order 0, 2, 1, 3)
+  const P2 a = v[0] + v[2], b = v[0] - v[2], c = v[1] + v[3], d = v[1] - v[3];
+  v[0] = a + c;
+  v[1] = a - c;
+  const P2 p{add2(b.re, d.im), sub2(b.im, d.re)}, m{sub2(b.re, d.im), add2(b.im, d.re)};  // b -/+ i d
+  v[2] = FWD ? p : m;
+  v[3] = FWD ? m : p;
+}
+// Prime sizes by symmetric pairs (dft_prime in hom_common.cuh)
+template <int R, bool FWD>
+__device__ __forceinline__ void dft_primep(P2* v) {
+  constexpr int H = (R - 1) / 2;
+  P2 a[H + 1], b[H + 1];
+#pragma unroll
+  for (int q = 1; q <= H; ++q) {
+    a[q] = v[q] + v[R - q];
+    b[q] = v[q] - v[R - q];
+  }
+  const P2 x0 = v[0];
+  P2 t = x0;
+#pragma unroll
+  for (int q = 1; q <= H; ++q) t = t + a[q];
+  v[0] = t;
+#pragma unroll
+  for (int p = 1; p <= H; ++p) {
+    P2 re = x0, im;
+#pragma unroll
+    for (int q = 1; q <= H; ++q) {
+      const int k = (p * q) % R;
+      const float2 c = kP[tw_base<R>() + 3 * k], s = kP[tw_base<R>() + 3 * k + (FWD ? 1 : 2)];
+      re = P2{fma2(a[q].re, c, re.re), fma2(a[q].im, c, re.im)};
+      im = q == 1 ? P2{mul2(b[q].re, s), mul2(b[q].im, s)} : P2{fma2(b[q].re, s, im.re), fma2(b[q].im, s, im.im)};
+    }
+    v[p] = P2{add2(re.re, im.im), sub2(re.im, im.re)};
+    v[R - p] = P2{sub2(re.re, im.im), add2(re.im, im.re)};
+  }
+}
+
 template <int R, bool FWD>
 __device__ __forceinline__ void dftp(P2* v) {
-  if constexpr (R == 3) dft3p<FWD>(v);
+  if constexpr (R == 2) dft2p(v);
+  else if constexpr (R == 3) dft3p<FWD>(v);
+  else if constexpr (R == 4) dft4p<FWD>(v);
   else if constexpr (R == 5) dft5p<FWD>(v);
+  else if constexpr (R == 7 || R == 11 || R == 13) dft_primep<R, FWD>(v);
   else dft_compositep<split_a<R>(), R / split_a<R>(), FWD>(v);
 }
 
@@ -374,6 +436,125 @@ __device__ __forceinline__ void fft_dif_p(float4* s, const TW* tw) {
   }
   stage_p<NP, N, P::r0, 1, FWD, false, TW, SP, NT>(s, tw);
   __syncthreads();
+}
+
+// ------------------------------------------------------------------ plan views of the pass bodies
+// FixedN: length and radices known at compile time (SP float4 between positions).
+template <int N_, int SP_> struct FixedN {
+  static constexpr int n = N_;
+  static constexpr bool fixed = true;
+  static constexpr int tile = N_ * SP_;  // float4 entries of a tile
+  __device__ __forceinline__ int at(int pos) const { return pos * SP_; }
+};
+// RunN: length and radices read from the plan.  With an even first radix r0 the lines of the span-1
+// stage would start a multiple of r0 SP float4 apart, on the same banks: one float4 of padding after
+// every r0 positions moves them apart, and every later span is a multiple of r0, so addresses stay linear.
+template <int SP_> struct RunN {
+  static constexpr bool fixed = false;
+  const RunPlan& p;
+  int n, tile;
+  __device__ __forceinline__ explicit RunN(const RunPlan& plan) : p(plan), n(plan.n) { tile = run_tile(plan.n, plan.pad, plan.r[0]); }
+  static __host__ __device__ __forceinline__ int run_tile(int n, int pad, int r0) { return n * SP_ + (pad ? n / r0 : 0); }
+  __device__ __forceinline__ int at(int pos) const { return pos * SP_ + (p.pad ? fdiv(pos, p.d_r0) : 0); }
+};
+
+// Twiddles w^q (q < R) of one butterfly: w and every fourth power come from the table, the others are
+// products of at most three factors, formed where they are used (few registers stay live).
+template <int R> struct TwPow {
+  float2 w1, w2, w3, w4, w8, w12;
+  __device__ __forceinline__ TwPow(const float2* tw, int L, int j) {
+    w1 = tw[j];
+    w2 = cmul1(w1, w1);
+    w3 = cmul1(w2, w1);
+    w4 = w8 = w12 = w1;
+    if constexpr (R > 4) w4 = tw[3 * L + j];
+    if constexpr (R > 8) w8 = R > 9 ? tw[7 * L + j] : cmul1(w4, w4);
+    if constexpr (R > 12) w12 = tw[11 * L + j];
+  }
+  __device__ __forceinline__ float2 operator()(int q) const {
+    const float2 hi = q < 8 ? w4 : q < 12 ? w8 : w12;
+    const int r = q & 3;
+    if (q < 4) return r == 1 ? w1 : r == 2 ? w2 : w3;
+    return r == 0 ? hi : cmul1(hi, r == 1 ? w1 : r == 2 ? w2 : w3);
+  }
+};
+
+// One stage with its span read from the plan (see stage_p).
+template <int NP, int R, bool FWD, bool DIT, int SP, int NT>
+__device__ __forceinline__ void stage_run(float4* s, const float2* tws, const RunPlan& p, int st) {
+  const int n = p.n, L = p.L[st], NB = n / R, pad = p.pad;
+  const float2* tw = tws + p.tw[st];
+  const int qs = L * SP + (pad && L > 1 ? fdiv(L, p.d_r0) : 0);  // L = 1: st = 0, a butterfly is one padded group
+  const FastDiv dnb = p.d_nb[st], dl = p.d_L[st];
+  for (int t = threadIdx.x; t < NB * NP; t += NT) {
+    const int cc = fdiv(t, dnb), b = t - cc * NB;
+    const int blk = fdiv(b, dl), j = b - blk * L;
+    const int p0 = blk * (L * R) + j;
+    float4* base = s + p0 * SP + (pad ? fdiv(p0, p.d_r0) : 0) + cc;
+    P2 v[R];
+    if (DIT) {
+      v[0] = ldp(base[0]);
+#pragma unroll
+      for (int q = 1; q < R; ++q) v[q] = ldp(base[q * qs]);
+      if (L > 1) {
+        const TwPow<R> w(tw, L, j);
+#pragma unroll
+        for (int q = 1; q < R; ++q) v[q] = twmul<FWD>(v[q], w(q));
+      }
+      dftp<R, FWD>(v);
+#pragma unroll
+      for (int q = 0; q < R; ++q) base[q * qs] = stp(v[out_pos<R>(q)]);
+    } else {
+#pragma unroll
+      for (int q = 0; q < R; ++q) v[q] = ldp(base[q * qs]);
+      dftp<R, FWD>(v);
+      base[0] = stp(v[0]);
+      if (L > 1) {
+        const TwPow<R> w(tw, L, j);
+#pragma unroll
+        for (int q = 1; q < R; ++q) base[q * qs] = stp(twmul<FWD>(v[out_pos<R>(q)], w(q)));
+      } else {
+#pragma unroll
+        for (int q = 1; q < R; ++q) base[q * qs] = stp(v[out_pos<R>(q)]);
+      }
+    }
+  }
+}
+template <int NP, bool FWD, bool DIT, int SP, int NT>
+__device__ __forceinline__ void stage_any(float4* s, const float2* tws, const RunPlan& p, int st) {
+  switch (p.r[st]) {
+    case 2: stage_run<NP, 2, FWD, DIT, SP, NT>(s, tws, p, st); break;
+    case 3: stage_run<NP, 3, FWD, DIT, SP, NT>(s, tws, p, st); break;
+    case 4: stage_run<NP, 4, FWD, DIT, SP, NT>(s, tws, p, st); break;
+    case 5: stage_run<NP, 5, FWD, DIT, SP, NT>(s, tws, p, st); break;
+    case 7: stage_run<NP, 7, FWD, DIT, SP, NT>(s, tws, p, st); break;
+    case 8: stage_run<NP, 8, FWD, DIT, SP, NT>(s, tws, p, st); break;
+    case 9: stage_run<NP, 9, FWD, DIT, SP, NT>(s, tws, p, st); break;
+    case 11: stage_run<NP, 11, FWD, DIT, SP, NT>(s, tws, p, st); break;
+    case 13: stage_run<NP, 13, FWD, DIT, SP, NT>(s, tws, p, st); break;
+    case 15: stage_run<NP, 15, FWD, DIT, SP, NT>(s, tws, p, st); break;
+    case 16: stage_run<NP, 16, FWD, DIT, SP, NT>(s, tws, p, st); break;
+    default: break;
+  }
+  __syncthreads();
+}
+
+// Whole transforms of the pass bodies, for either kind of plan.
+template <int NP, bool FWD, int NT, int N, int SP>
+__device__ __forceinline__ void fft_dif(const FixedN<N, SP>&, float4* s, const float2* tw) {
+  fft_dif_p<NP, N, FWD, float2, SP, NT>(s, tw);
+}
+template <int NP, bool FWD, int NT, int N, int SP>
+__device__ __forceinline__ void fft_dit(const FixedN<N, SP>&, float4* s, const float2* tw) {
+  fft_dit_p<NP, N, FWD, float2, SP, NT>(s, tw);
+}
+template <int NP, bool FWD, int NT, int SP>
+__device__ __forceinline__ void fft_dif(const RunN<SP>& pl, float4* s, const float2* tw) {
+  for (int st = pl.p.m - 1; st >= 0; --st) stage_any<NP, FWD, false, SP, NT>(s, tw, pl.p, st);
+}
+template <int NP, bool FWD, int NT, int SP>
+__device__ __forceinline__ void fft_dit(const RunN<SP>& pl, float4* s, const float2* tw) {
+  for (int st = 0; st < pl.p.m; ++st) stage_any<NP, FWD, true, SP, NT>(s, tw, pl.p, st);
 }
 
 }  // namespace

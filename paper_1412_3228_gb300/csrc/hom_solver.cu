@@ -1112,7 +1112,7 @@ struct Layout {
   std::vector<FastPlanDev> fplans;  // specialised FP32 passes: per-size tables
   std::vector<std::vector<unsigned char>> fplan_host;  // external workspace: their host copies
   bool fast = false;
-  int fast_nmax = 0;
+  bool run = false;  // fast, with radices read from the plans (a size without compiled ones)
   size_t ws_elems = 0, g_elems = 0, fld_elems = 0;
   size_t smem_row = 0, smem_green = 0, smem_y = 0;
 };
@@ -1176,22 +1176,40 @@ int build_layout(const hom_cell* cells, int ncells, int L, int dim, size_t vsize
   const size_t kMaxSmem = 227 * 1024;
   // The specialised passes take 4-row and 2-column tasks; the output pass (generic row kernel)
   // then needs 4 rows of every load on chip.
+  // The row radices are compiled in where every size of the batch has them, else read from plans (not
+  // for the no-allocation entry point, whose scratch rules are fixed by the sizes it documents).
   if (lay.fast) {
-    for (int ci = 0; ci < ncells; ++ci)
-      if (!(dim == 2 ? fast2d_size(cells[ci].n) : fast3d_size(cells[ci].n))) lay.fast = false;
+    for (int ci = 0; ci < ncells; ++ci) {
+      const int n = cells[ci].n;
+      if (!(dim == 2 ? fast2d_size(n) : fast3d_size(n))) lay.run = true;
+      if (external && lay.run) lay.fast = false;
+      if (!(dim == 2 ? run2d_size(n) : run3d_size(n))) lay.fast = false;
+    }
+    if (lay.run) {  // what the one-byte labels and their kernel cannot hold stays on the generic passes
+      if (ncells > 65535) lay.fast = false;
+      for (int ci = 0; ci < ncells && lay.fast; ++ci) {
+        std::vector<int> ph{cells[ci].matrix_phase};
+        for (int p = 0; p < cells[ci].nprim; ++p) ph.push_back(cells[ci].prims[p].phase);
+        std::sort(ph.begin(), ph.end());
+        if (std::unique(ph.begin(), ph.end()) - ph.begin() > 254) lay.fast = false;
+      }
+    }
+    lay.run = lay.run && lay.fast;
   }
   long long vox = 0;
   std::vector<int> plan_n;
   // rows per row task and kx columns per Green/y task that fit on chip, and the passes' tasks with them
   auto row_lines = [&](int rows) { return (size_t)((rows * L * nc + 1) / 2) + 1; };
+  // (compiled sizes: four rows of every load, also where the generic kernel would hold fewer)
   auto rows_fit = [&](int n) {
     const int nrows = dim == 2 ? n : n * n;
+    if (lay.fast && !lay.run) return std::min(kFastRows, nrows);
     const size_t line_bytes = (size_t)n * vsize;  // one line; the twiddle table is one more
     int r = 1;
     while (r < nrows &&
            row_lines(r + 1) * line_bytes + (size_t)(r + 1) * L * nc * (sizeof(long long) + vsize) <= budget)
       ++r;
-    return lay.fast ? std::min(kFastRows, nrows) : r;
+    return r;
   };
   auto cols_fit = [&](int n) {
     const size_t line_bytes = (size_t)n * vsize, gbudget = kGreenBudget;
@@ -1201,7 +1219,7 @@ int build_layout(const hom_cell* cells, int ncells, int L, int dim, size_t vsize
   std::vector<int> task_rows, task_cols;
   size_t row_total = 0, col_total = 0;
   for (int ci = 0; ci < ncells; ++ci) {
-    const int n = cells[ci].n, r = rows_fit(n), q = cols_fit(n);
+    const int n = cells[ci].n, r = lay.fast ? kFastRows : rows_fit(n), q = cols_fit(n);
     row_total += ((size_t)(dim == 2 ? n : n * n) + r - 1) / r;
     col_total += (size_t)(n / 2 + q) / q * L * (dim == 2 ? 1 : n);
   }
@@ -1251,16 +1269,15 @@ int build_layout(const hom_cell* cells, int ncells, int L, int dim, size_t vsize
         int rc;
         if (external) {  // host tables, uploaded into the caller's workspace with the call
           lay.fplan_host.emplace_back();
-          rc = fast2d_plan_host(k.n, lay.fplan_host.back(), &fp);
+          rc = fast2d_plan_host(k.n, lay.run, lay.fplan_host.back(), &fp);
         } else {
-          rc = fast2d_plan(k.n, &fp);
+          rc = fast2d_plan(k.n, lay.run, &fp);
         }
         if (rc != HOM_OK) return rc;
         lay.fplans.push_back(fp);
         idx = (int)lay.fplans.size() - 1;
       }
       c.fplan = idx;
-      lay.fast_nmax = std::max(lay.fast_nmax, k.n);
     }
     c.vox_off = vox;
     c.fld_off = (long long)lay.fld_elems;
@@ -1294,9 +1311,11 @@ int build_layout(const hom_cell* cells, int ncells, int L, int dim, size_t vsize
       // row, 9 real rows, took 329 us, tasks of 3 rows 288)
       if (r < fit && (r & 1) && (L * nc & 1)) ++r;
     }
+    // (passes with run-time radices refuse what the generic ones do, although they would hold it)
     const size_t need_r = row_lines(r) * line_bytes + (size_t)r * L * nc * (sizeof(long long) + 2 * vsize / 2);
     if (need_r > kMaxSmem) return set_error(HOM_ERR_UNSUPPORTED_SIZE, "row of n = %d with %d loads does not fit on chip", k.n, L);
     lay.smem_row = std::max(lay.smem_row, need_r);
+    if (lay.fast) r = std::min(kFastRows, c.nrows);
     const int ntk = lay.fast ? cols_fit(k.n) : spread(cols_fit(k.n), col_total);
     const size_t need_l = ((size_t)ntk * nc + 2) * line_bytes;
     lay.smem_green = std::max(lay.smem_green, need_l);
@@ -1936,11 +1955,12 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
     G.E = A.E;
     G.nchunk = cg_nchunk;
   }
-  const size_t smem_frow =
-      !lay.fast ? 0 : DIM == 2 ? fast2d_smem_row(lay.fast_nmax, nph_max) : fast3d_smem_row(lay.fast_nmax, nph_max);
-  const size_t smem_fgreen =
-      !lay.fast ? 0 : DIM == 2 ? fast2d_smem_green(lay.fast_nmax) : fast3d_smem_green(lay.fast_nmax);
-  const size_t smem_fy = lay.fast && DIM == 3 ? fast3d_smem_y(lay.fast_nmax) : 0;
+  size_t smem_frow = 0, smem_fgreen = 0, smem_fy = 0;  // the largest over the batch's sizes
+  for (const FastPlanDev& fp : lay.fplans) {
+    smem_frow = std::max(smem_frow, DIM == 2 ? fast2d_smem_row(fp.n, nph_max) : fast3d_smem_row(fp.n, nph_max));
+    smem_fgreen = std::max(smem_fgreen, DIM == 2 ? fast2d_smem_green(fp.n) : fast3d_smem_green(fp.n));
+    if (DIM == 3) smem_fy = std::max(smem_fy, fast3d_smem_y(fp.n));
+  }
   if (lay.fast && (rc = fast2d_permute_labels(A, ncells, nv_max, st)) != HOM_OK) return rc;
 
   if (warm && (rc = allow_smem(k_state_in<T, DIM, MAXR>, lay.smem_row)) != HOM_OK) return rc;
@@ -1993,26 +2013,26 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
   auto one_pass = [&]() {
     NvtxRange r_("hom_solve: passes");
     tm.begin(HOM_K_ROW);
-    if (lay.fast && DIM == 3) fast3d_row(A, nR, smem_frow, false, st);
-    else if (lay.fast) fast2d_row(A, nR, smem_frow, st);
+    if (lay.fast && DIM == 3) fast3d_row(A, nR, smem_frow, false, lay.run, st);
+    else if (lay.fast) fast2d_row(A, nR, smem_frow, lay.run, st);
     else if (em) k_row<T, DIM, false, MAXR, true><<<nR, kThreads, lay.smem_row, st>>>(A);
     else k_row<T, DIM, false, MAXR><<<nR, kThreads, lay.smem_row, st>>>(A);
     tm.end();
     if (DIM == 3) {
       tm.begin(HOM_K_YFWD);
-      if (lay.fast) fast3d_ypass(A, nY, smem_fy, true, st);
+      if (lay.fast) fast3d_ypass(A, nY, smem_fy, true, lay.run, st);
       else k_ypass<T, true, MAXR><<<nY, kThreads, lay.smem_y, st>>>(A);
       tm.end();
     }
     tm.begin(HOM_K_GREEN);
-    if (lay.fast && DIM == 3) fast3d_green(A, nC, smem_fgreen, st);
-    else if (lay.fast) fast2d_green(A, nC, smem_fgreen, st);
+    if (lay.fast && DIM == 3) fast3d_green(A, nC, smem_fgreen, lay.run, st);
+    else if (lay.fast) fast2d_green(A, nC, smem_fgreen, lay.run, st);
     else if (em) k_green<T, DIM, MAXR, true><<<nC, kThreads, lay.smem_green, st>>>(A);
     else k_green<T, DIM, MAXR><<<nC, kThreads, lay.smem_green, st>>>(A);
     tm.end();
     if (DIM == 3) {
       tm.begin(HOM_K_YINV);
-      if (lay.fast) fast3d_ypass(A, nY, smem_fy, false, st);
+      if (lay.fast) fast3d_ypass(A, nY, smem_fy, false, lay.run, st);
       else k_ypass<T, false, MAXR><<<nY, kThreads, lay.smem_y, st>>>(A);
       tm.end();
     }
@@ -2056,7 +2076,7 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
     K.out_eps = K.out_sig = nullptr;
     std::string key(reinterpret_cast<const char*>(&K), sizeof(K));
     const size_t dims[] = {nR, nC, nY, nCtl, nctl, lay.smem_row, lay.smem_green, lay.smem_y, smem_frow, smem_fgreen,
-                           smem_fy, (size_t)lay.fast, (size_t)DIM, sizeof(T), (size_t)MAXR};
+                           smem_fy, (size_t)lay.fast, (size_t)lay.run, (size_t)DIM, sizeof(T), (size_t)MAXR};
     key.append(reinterpret_cast<const char*>(dims), sizeof(dims));
     cudaGraphExec_t gexec = find_graph(dev, key);
     if (!gexec) {
@@ -2132,8 +2152,8 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
   if (want_fields) {
     NvtxRange r_("hom_solve: output fields");
     tm.begin(HOM_K_OUTPUT);
-    if (lay.fast && DIM == 3) fast3d_row(A, nR, smem_frow, true, st);
-    else if (lay.fast) fast2d_out(A, nR, smem_frow, st);
+    if (lay.fast && DIM == 3) fast3d_row(A, nR, smem_frow, true, lay.run, st);
+    else if (lay.fast) fast2d_out(A, nR, smem_frow, lay.run, st);
     else if (em) k_row<T, DIM, true, MAXR, true><<<nR, kThreads, lay.smem_row, st>>>(A);
     else k_row<T, DIM, true, MAXR><<<nR, kThreads, lay.smem_row, st>>>(A);
     tm.end();
