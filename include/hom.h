@@ -407,8 +407,8 @@ int hom_effective_stiffness(int32_t ncells, int32_t dim, const double* E, const 
 /* The autotuner's record.  The first FP32 hom_solve of a batch shape (device, dimension, load count,
  * Green operator, multiset of grid sizes) with opts->tune = 1 (passes = AUTO, max_radix = 0) times
  * four candidate plans on that batch -- the specialised passes and the generic passes with register
- * radices up to 15, 27 and 45 -- over 4 fixed iterations each (after one untimed call), and every
- * later solve of the shape runs the fastest.  Writes one line per shape, "shape: timings -> choice",
+ * radices up to 15, 27 and 45 -- by the difference of calls of 16 and of 4 fixed iterations (after one
+ * untimed call), and every later solve of the shape runs the fastest.  Writes one line per shape, "shape: timings -> choice",
  * into buf (at most len bytes, NUL-terminated) and returns the full length.  The choice depends on
  * measured times, so two processes may pick different plans (results then differ by FP32 rounding). */
 int32_t hom_autotune_report(char* buf, int32_t len);

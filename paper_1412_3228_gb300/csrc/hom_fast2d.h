@@ -69,6 +69,13 @@ int fast2d_init(const SolveArgs& A, int ncells, cudaStream_t st);
 int fast2d_permute_labels(const SolveArgs& A, int ncells, long long max_nv, cudaStream_t st);
 void fast2d_release();
 
+// On-chip solver of the small grids of a batch (hom_resident2d.cu): runs every pair whose grid fits a
+// thread-block cluster to its stopping point and leaves it inactive, its iterate where the output pass
+// reads it.  `list` holds room for every pair; *count receives the number of pairs taken.
+struct CellDev;
+int resident2d_solve(const SolveArgs& A, const std::vector<CellDev>& cells, int L, int* list, int nphase_cell,
+                     cudaStream_t st, int* count);
+
 // Specialised 3D passes (hom_fast3d.cu): row, y forward / inverse, Green (z lines), the initial
 // state eps = E and the output pass, on the kx-pair tiled state of those passes.
 size_t fast3d_smem_row(int nmax, int nphase_cell);

@@ -480,17 +480,18 @@ template <int R> struct TwPow {
 };
 
 // One stage with its span read from the plan (see stage_p).
-template <int NP, int R, bool FWD, bool DIT, int SP, int NT>
-__device__ __forceinline__ void stage_run(float4* s, const float2* tws, const RunPlan& p, int st) {
+// MULTI: over nl lines, NP of each tile of `tile` float4, instead of the NP lines of one.
+template <int NP, int R, bool FWD, bool DIT, int SP, int NT, bool MULTI = false>
+__device__ __forceinline__ void stage_run(float4* s, const float2* tws, const RunPlan& p, int st, int nl = NP, int tile = 0) {
   const int n = p.n, L = p.L[st], NB = n / R, pad = p.pad;
   const float2* tw = tws + p.tw[st];
   const int qs = L * SP + (pad && L > 1 ? fdiv(L, p.d_r0) : 0);  // L = 1: st = 0, a butterfly is one padded group
   const FastDiv dnb = p.d_nb[st], dl = p.d_L[st];
-  for (int t = threadIdx.x; t < NB * NP; t += NT) {
+  for (int t = threadIdx.x; t < NB * nl; t += NT) {
     const int cc = fdiv(t, dnb), b = t - cc * NB;
     const int blk = fdiv(b, dl), j = b - blk * L;
     const int p0 = blk * (L * R) + j;
-    float4* base = s + p0 * SP + (pad ? fdiv(p0, p.d_r0) : 0) + cc;
+    float4* base = s + p0 * SP + (pad ? fdiv(p0, p.d_r0) : 0) + (MULTI ? (cc / NP) * tile + cc % NP : cc);
     P2 v[R];
     if (DIT) {
       v[0] = ldp(base[0]);
@@ -520,22 +521,15 @@ __device__ __forceinline__ void stage_run(float4* s, const float2* tws, const Ru
     }
   }
 }
-template <int NP, bool FWD, bool DIT, int SP, int NT>
-__device__ __forceinline__ void stage_any(float4* s, const float2* tws, const RunPlan& p, int st) {
+template <int NP, bool FWD, bool DIT, int SP, int NT, bool MULTI = false>
+__device__ __forceinline__ void stage_any(float4* s, const float2* tws, const RunPlan& p, int st, int nl = NP, int tile = 0) {
+#define HOM_STAGE(R) case R: stage_run<NP, R, FWD, DIT, SP, NT, MULTI>(s, tws, p, st, nl, tile); break
   switch (p.r[st]) {
-    case 2: stage_run<NP, 2, FWD, DIT, SP, NT>(s, tws, p, st); break;
-    case 3: stage_run<NP, 3, FWD, DIT, SP, NT>(s, tws, p, st); break;
-    case 4: stage_run<NP, 4, FWD, DIT, SP, NT>(s, tws, p, st); break;
-    case 5: stage_run<NP, 5, FWD, DIT, SP, NT>(s, tws, p, st); break;
-    case 7: stage_run<NP, 7, FWD, DIT, SP, NT>(s, tws, p, st); break;
-    case 8: stage_run<NP, 8, FWD, DIT, SP, NT>(s, tws, p, st); break;
-    case 9: stage_run<NP, 9, FWD, DIT, SP, NT>(s, tws, p, st); break;
-    case 11: stage_run<NP, 11, FWD, DIT, SP, NT>(s, tws, p, st); break;
-    case 13: stage_run<NP, 13, FWD, DIT, SP, NT>(s, tws, p, st); break;
-    case 15: stage_run<NP, 15, FWD, DIT, SP, NT>(s, tws, p, st); break;
-    case 16: stage_run<NP, 16, FWD, DIT, SP, NT>(s, tws, p, st); break;
+    HOM_STAGE(2); HOM_STAGE(3); HOM_STAGE(4); HOM_STAGE(5); HOM_STAGE(7); HOM_STAGE(8); HOM_STAGE(9); HOM_STAGE(11);
+    HOM_STAGE(13); HOM_STAGE(15); HOM_STAGE(16);
     default: break;
   }
+#undef HOM_STAGE
   __syncthreads();
 }
 

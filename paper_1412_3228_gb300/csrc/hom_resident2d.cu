@@ -1,0 +1,396 @@
+// On-chip solver of small 2D grids (FP32, section 2, eqs. 1-a, 1-b, 2, or the Eyre-Milton scheme): one
+// thread-block cluster runs a (cell, load) pair from its initial state to its stopping point.
+//
+// Why.  The passes of hom_fast2d.cu take three launches per iteration, and on a small grid each is a chain
+// of a few short stages: at 45^2 (one cell, three loads) an iteration took 33 us for about 2 us of work.
+// Here the half-spectrum state stays in the shared memory of the cluster's CTAs.  CTA r owns a block of
+// row groups (4 real rows each) and a block of kx pairs; both kinds of tile have the layout of the passes
+// (n positions of three float4 lane pairs):
+//   rows    : pull the four rows of every kx pair of the group from the CTAs that own the pairs (distributed
+//             shared memory), inverse x-DFT, constitutive update, forward x-DFT, push the rows of tau back;
+//   columns : forward y-DFT, Green operator and residual, inverse y-DFT, in place;
+//   control : the FP64 partial sums go to rank 0, whose first warp applies the stopping rule while the
+//             others start the next rows; the flag comes back with the barrier after the pull.
+// Three cluster barriers an iteration, no launch and no trip through HBM.  The Green step's private state
+// (g, or u_hat of the Eyre-Milton scheme) has two buffers used in turn, in shared memory where they fit (n up
+// to about 190) and in the workspace otherwise: when iterate `it` passes, its own spectrum is rebuilt from the state it was made with, and its rows are left where
+// the output pass reads them.  The steps are those of the passes, so the iterates are too.
+//
+// Measured, 40 iterations, 3 loads (whole call): 45^2, one cell: 1.72 ms in passes, 0.69 ms here; 143^2, two
+// cells: 3.67 ms (generic passes), 1.10 ms.
+#define HOM_FILE_ID 4
+#include <cooperative_groups.h>
+
+#include <algorithm>
+#include <cstring>
+#include <vector>
+
+#include "hom_control.cuh"
+#include "hom_fast2d.h"
+#include "hom_point2d.cuh"
+
+namespace hom {
+namespace {
+
+namespace cg = cooperative_groups;
+
+constexpr int kTR = 256;         // threads per CTA
+constexpr int kMaxCluster = 8;   // portable cluster size
+constexpr int kSums = 6;         // per-rank totals: three stress sums, three residual sums
+constexpr size_t kResSmem = 200 * 1024;  // dynamic shared memory a CTA may take
+
+struct ResShape {  // how a pair of grid size n is spread over C CTAs
+  int gpc, ppc;    // row groups and kx pairs per CTA
+  size_t bytes;    // dynamic shared memory of a CTA, without and
+  size_t priv;     // for the Green step's private state
+};
+__host__ __device__ inline int res_tile(int n, int pad, int r0) { return n * NP + (pad ? n / r0 : 0); }
+ResShape res_shape(int n, int C, int nph, int tile, bool em) {
+  const int G = (n + kFastRows - 1) / kFastRows, P = (n / 2 + 2) / 2;
+  ResShape s;
+  s.gpc = (G + C - 1) / C;
+  s.ppc = (P + C - 1) / C;
+  s.bytes = (size_t)(s.gpc + s.ppc) * tile * sizeof(float4) + ((size_t)n + 1) / 2 * 16 + ((size_t)n + 3) / 4 * 16 +
+            (size_t)s.gpc * kFastRows * ((n + 15) / 16 * 16) + (size_t)s.gpc * 2 * kFastRows * NP * sizeof(float) + 2 * NP * sizeof(double) +
+            ((size_t)nph * 16 + 15) / 16 * 16 + (size_t)kMaxCluster * kSums * sizeof(double) + 64;
+  s.priv = 2 * (size_t)s.ppc * n * (em ? 3 : 2) * sizeof(float4);
+  return s;
+}
+
+template <bool EM>
+__global__ void __launch_bounds__(kTR, 2) k_resident2d(SolveArgs A, const int* list, int priv_on_chip) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ RunPlan sp;
+  __shared__ double s_mine[kSums];
+  __shared__ int s_stop;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  const int pair = list[blockIdx.x / C];
+  const PairDev pr = A.pairs[pair];
+  const CellDev c = A.cells[pr.cell];
+  const FastPlanDev& fp = A.fplans[c.fplan];
+  for (int i = threadIdx.x; i < (int)(sizeof(RunPlan) / sizeof(int)); i += kTR)
+    reinterpret_cast<int*>(&sp)[i] = reinterpret_cast<const int*>(&fp.run)[i];
+  if (threadIdx.x == 0) s_stop = 0;
+  __syncthreads();
+  const RunN<NP> pl(sp);
+  const int N = pl.n, tile = pl.tile, H = N / 2 + 1, P = (H + 1) / 2, G = (N + kFastRows - 1) / kFastRows;
+  const int NL = (N + 15) / 16 * 16;
+  const int gpc = (G + C - 1) / C, ppc = (P + C - 1) / C;
+  const int g0 = min(rank * gpc, G), ng = min(gpc, G - g0), p0 = min(rank * ppc, P), np = min(ppc, P - p0);
+  const int l = pr.load;
+
+  // shared memory: row tiles | column tiles | twiddles | wave numbers | labels | row sums | phase constants
+  float4* rows = reinterpret_cast<float4*>(smem_raw);
+  float4* cols = rows + (size_t)gpc * tile;
+  float2* tws = reinterpret_cast<float2*>(cols + (size_t)ppc * tile);
+  float* sx = reinterpret_cast<float*>(reinterpret_cast<float4*>(tws) + (N + 1) / 2);
+  uint8_t* slab = reinterpret_cast<uint8_t*>(reinterpret_cast<float4*>(sx) + (N + 3) / 4);
+  double* s_part = reinterpret_cast<double*>(slab + (size_t)gpc * kFastRows * NL);  // [rank][kSums], filled by every rank
+  double* s_rs = s_part + kMaxCluster * kSums;                                      // [eps, tau][component]
+  float* s_dc = reinterpret_cast<float*>(s_rs + 2 * NP);                            // [group][eps, tau][row][component]
+  float2* sph = reinterpret_cast<float2*>(s_dc + (size_t)gpc * 2 * kFastRows * NP);
+  float2* sinv = sph + c.nph;
+  constexpr int GP = EM ? 3 : 2;  // float4 per position of the Green step's private state
+  float4* s_priv = reinterpret_cast<float4*>(sph + 2 * c.nph);  // [buffer][pair][position][GP]
+
+  CellConst<float> cc;
+  cell_const(c, cc);
+  phase_constants<false, EM>(A, c, cc, sph, sinv, kTR);
+  for (int i = threadIdx.x; i < (N + 1) / 2; i += kTR) cp16(tws + 2 * i, fp.tw2 + 2 * i);
+  for (int i = threadIdx.x; i < (N + 3) / 4; i += kTR) cp16(sx + 4 * i, fp.xipos + 4 * i);
+  const int myrows = max(0, min(ng * kFastRows, N - g0 * kFastRows));
+  {
+    const uint4* src = reinterpret_cast<const uint4*>(A.label8 + c.lp_off + (size_t)g0 * kFastRows * NL);
+    for (int i = threadIdx.x; i < myrows * NL / 16; i += kTR) cp16(slab + 16 * i, src + i);
+  }
+  // the initial state of the owned pairs
+  const float4* e0 = static_cast<const float4*>(A.eps[0]);
+  for (int i = threadIdx.x; i < np * N * NP; i += kTR) {
+    const int pp = i / (N * NP), r = i - pp * (N * NP), y = r / NP, k = r - y * NP;
+    cp16(cols + (size_t)pp * tile + pl.at(y) + k, e0 + tile_index(c, N, l, p0 + pp, y) + k);
+  }
+  cp_commit();
+  cp_wait_all();
+  // the Green step's private state of an owned pair: iterate `it` was made with buffer it & 1 (in the
+  // workspace: g's own array, then the pair's tile of the tau array, which these pairs do not use)
+  auto priv_ws = [&](int pp, int which) -> float4* {
+    const int p = p0 + pp;
+    return which ? static_cast<float4*>(A.tau) + tile_index(c, N, l, p, 0)
+                 : static_cast<float4*>(A.g) + (c.g_off + ((size_t)l * (c.Hp / 2) + p) * N * 2 * GP) / 2;
+  };
+  auto priv = [&](int pp, int which) -> float4* {
+    return priv_on_chip ? s_priv + (size_t)(which * ppc + pp) * N * GP : priv_ws(pp, which);
+  };
+  if (priv_on_chip)
+    for (int i = threadIdx.x; i < np * N * GP; i += kTR) {
+      const int pp = i / (N * GP), r = i - pp * (N * GP);
+      priv(pp, 0)[r] = priv_ws(pp, 0)[r];
+    }
+  const double* Eld = A.E + (size_t)pair * NP;
+  const int nrl = ng * NP, ncl = np * NP;  // owned lines of lane pairs
+  cluster.sync();
+
+  int it = 0;
+  for (;; ++it) {
+    // stopping rule of the last iterate: rank 0's first warp, beside the pull below
+    if (it > 0 && rank == 0 && threadIdx.x < 32) {
+      double sum = 0.0;
+      if (threadIdx.x < kSums)
+        for (int r = 0; r < C; ++r) sum += s_part[r * kSums + threadIdx.x];
+      const int still = control_pair<NP>(A, pair, (double)c.nv, sum, it - 1);
+      if (threadIdx.x == 0 && !still)
+        for (int r = 0; r < C; ++r) *cluster.map_shared_rank(&s_stop, r) = 1;
+    }
+    // rows: four half-spectrum rows -> two Hermitian-extended complex lines per component (see k_row_f2d)
+    for (int f = threadIdx.x; f < ng * P * NP; f += kTR) {
+      const int gl = f / (P * NP), q = f - gl * (P * NP), p = q / NP, k = q - p * NP;
+      const int owner = p / ppc, y0 = (g0 + gl) * kFastRows;
+      const float4* src = cluster.map_shared_rank(cols, owner) + (size_t)(p - owner * ppc) * tile + k;
+      float4 v[kFastRows];
+#pragma unroll
+      for (int r = 0; r < kFastRows; ++r)
+        v[r] = y0 + r < N ? src[pl.at(y0 + r)] : make_float4(0.f, 0.f, 0.f, 0.f);
+      float4* s = rows + (size_t)gl * tile + k;
+      float* dc = s_dc + (size_t)gl * 2 * kFastRows * NP + k;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int kx = 2 * p + h;
+        if (kx >= H) break;
+        const float2 q0 = h ? make_float2(v[0].y, v[0].w) : make_float2(v[0].x, v[0].z);
+        const float2 q1 = h ? make_float2(v[1].y, v[1].w) : make_float2(v[1].x, v[1].z);
+        const float2 q2 = h ? make_float2(v[2].y, v[2].w) : make_float2(v[2].x, v[2].z);
+        const float2 q3 = h ? make_float2(v[3].y, v[3].w) : make_float2(v[3].x, v[3].z);
+        s[pl.at(kx)] = make_float4(q0.x - q1.y, q2.x - q3.y, q0.y + q1.x, q2.y + q3.x);
+        if (kx > 0) {
+          if (2 * kx != N) s[pl.at(N - kx)] = make_float4(q0.x + q1.y, q2.x + q3.y, q1.x - q0.y, q3.x - q2.y);
+        } else {
+          dc[0] = q0.x;
+          dc[NP] = q1.x;
+          dc[2 * NP] = q2.x;
+          dc[3 * NP] = q3.x;
+        }
+      }
+    }
+    cg::cluster_group::arrival_token tok = cluster.barrier_arrive();  // the columns may be overwritten once all have read
+    __syncthreads();
+    for (int st = sp.m - 1; st >= 0; --st) stage_any<NP, false, false, NP, kTR, true>(rows, tws, sp, st, nrl, tile);
+    for (int i = threadIdx.x; i < ng * N; i += kTR) {
+      const int gl = i / N, pos = i - gl * N, y0 = (g0 + gl) * kFastRows, nr = min(kFastRows, N - y0);
+      float4* s = rows + (size_t)gl * tile + pl.at(pos);
+      uint32_t lab[kFastRows];
+#pragma unroll
+      for (int r = 0; r < kFastRows; ++r) lab[r] = r < nr ? (uint32_t)slab[(size_t)(gl * kFastRows + r) * NL + pos] : 0u;
+      float4 e[NP], o[NP];
+#pragma unroll
+      for (int k = 0; k < NP; ++k) e[k] = s[k];
+      tau_point<false, false, EM>(A, c, fp, sph, sinv, cc, nr, y0, l, pos, lab, e, o);
+#pragma unroll
+      for (int k = 0; k < NP; ++k) s[k] = o[k];
+    }
+    __syncthreads();
+    for (int st = 0; st < sp.m; ++st) stage_any<NP, true, true, NP, kTR, true>(rows, tws, sp, st, nrl, tile);
+    cluster.barrier_wait(std::move(tok));
+    if (s_stop) break;
+    // split the two real rows of each line and push the half spectra of tau to the owners of their columns
+    for (int f = threadIdx.x; f < ng * P * NP; f += kTR) {
+      const int gl = f / (P * NP), q = f - gl * (P * NP), p = q / NP, k = q - p * NP;
+      const int owner = p / ppc, y0 = (g0 + gl) * kFastRows;
+      const float4* s = rows + (size_t)gl * tile + k;
+      float* dc = s_dc + (size_t)gl * 2 * kFastRows * NP + kFastRows * NP + k;
+      float4 w[kFastRows];
+#pragma unroll
+      for (int r = 0; r < kFastRows; ++r) w[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int kx = 2 * p + h;
+        if (kx >= H) break;
+        const float4 Z = s[pl.at(kx)];
+        const float4 Zm = s[pl.at(kx == 0 ? 0 : N - kx)];
+        const float2 o0 = make_float2(0.5f * (Z.x + Zm.x), 0.5f * (Z.z - Zm.z));
+        const float2 o1 = make_float2(0.5f * (Z.z + Zm.z), 0.5f * (Zm.x - Z.x));
+        const float2 o2 = make_float2(0.5f * (Z.y + Zm.y), 0.5f * (Z.w - Zm.w));
+        const float2 o3 = make_float2(0.5f * (Z.w + Zm.w), 0.5f * (Zm.y - Z.y));
+        if (h == 0) {
+          w[0].x = o0.x; w[0].z = o0.y; w[1].x = o1.x; w[1].z = o1.y;
+          w[2].x = o2.x; w[2].z = o2.y; w[3].x = o3.x; w[3].z = o3.y;
+          if (kx == 0) {
+            dc[0] = o0.x;
+            dc[NP] = o1.x;
+            dc[2 * NP] = o2.x;
+            dc[3 * NP] = o3.x;
+          }
+        } else {
+          w[0].y = o0.x; w[0].w = o0.y; w[1].y = o1.x; w[1].w = o1.y;
+          w[2].y = o2.x; w[2].w = o2.y; w[3].y = o3.x; w[3].w = o3.y;
+        }
+      }
+      float4* dst = cluster.map_shared_rank(cols, owner) + (size_t)(p - owner * ppc) * tile + k;
+#pragma unroll
+      for (int r = 0; r < kFastRows; ++r)
+        if (y0 + r < N) dst[pl.at(y0 + r)] = w[r];
+    }
+    cluster.sync();
+    // sum of sigma over the owned rows (see the row pass), FP64: warp q sums row values q = (eps or tau,
+    // component) over the rows, and c0 is applied to the sums
+    if (threadIdx.x < 2 * NP * 32) {
+      const int q = threadIdx.x >> 5, lane = threadIdx.x & 31, which = q / NP, k = q - which * NP;
+      double x = 0.0;
+      for (int r = lane; r < myrows; r += 32)
+        x += (double)s_dc[((size_t)(r / kFastRows) * 2 + which) * kFastRows * NP + (r % kFastRows) * NP + k];
+      for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+      if (lane == 0) s_rs[q] = x;
+    }
+    // columns
+    for (int st = sp.m - 1; st >= 0; --st) stage_any<NP, true, false, NP, kTR, true>(cols, tws, sp, st, ncl, tile);
+    Acc<float> acc[EM ? 3 : 2];
+    if constexpr (EM) {
+      GreenPairEm gp(A, c, fp, 0, Eld);
+      for (int i = threadIdx.x; i < np * 2 * N; i += kTR) {
+        const int pp = i / (2 * N), q = i - pp * (2 * N), pos = q >> 1, h = q & 1, kx0 = 2 * (p0 + pp);
+        float* T = reinterpret_cast<float*>(cols + (size_t)pp * tile + pl.at(pos));
+        if (h && kx0 + 1 >= H) {  // the missing lane B of the last pair stays zero
+#pragma unroll
+          for (int k = 0; k < NP; ++k) T[4 * k + 1] = T[4 * k + 3] = 0.f;
+          continue;
+        }
+        gp.set_pair(N, fp, kx0);
+        const float2* uin = reinterpret_cast<const float2*>(priv(pp, it & 1)) + 6 * pos + 3 * h;
+        float2* uout = reinterpret_cast<float2*>(priv(pp, (it + 1) & 1)) + 6 * pos + 3 * h;
+        gp.point(T, h, sx[pos], pos == 0, uin, uout, acc);
+      }
+    } else {
+      GreenPair gp(A, c, fp, 0, pair);
+      for (int i = threadIdx.x; i < np * N; i += kTR) {
+        const int pp = i / N, pos = i - pp * N;
+        gp.set_pair(N, fp, 2 * (p0 + pp));
+        const float4* gin = priv(pp, it & 1) + 2 * pos;
+        const float4 g[2] = {gin[0], gin[1]};
+        gp.point(cols + (size_t)pp * tile + pl.at(pos), sx[pos], pos == 0, g, priv(pp, (it + 1) & 1) + 2 * pos);
+      }
+      gp.sums(acc);
+    }
+    double tot[EM ? 3 : 2];
+    block_sum<float, EM ? 3 : 2, kTR>(acc, tot);  // contains the barrier before the inverse transform
+    if (threadIdx.x == 0) {
+#pragma unroll
+      for (int q = 0; q < 3; ++q) s_mine[NP + q] = q < (EM ? 3 : 2) ? tot[q] : 0.0;
+    }
+    if (threadIdx.x >= 32 && threadIdx.x < 32 + NP) {
+      const int k = threadIdx.x - 32;
+      const double tau = s_rs[NP + k], u = s_rs[k], tr = s_rs[0] + s_rs[1];
+      s_mine[k] = EM ? 0.5 * (tau + (double)N * u)
+                     : tau + (double)N * (2.0 * c.mu0 * u + (k < 2 ? c.lam0 * tr : 0.0));
+    }
+    for (int st = 0; st < sp.m; ++st) stage_any<NP, false, true, NP, kTR, true>(cols, tws, sp, st, ncl, tile);
+    if (threadIdx.x < kSums) cluster.map_shared_rank(s_part, 0)[rank * kSums + threadIdx.x] = s_mine[threadIdx.x];
+    cluster.sync();
+  }
+
+  // iterate it - 1 is the one returned: its spectrum from the state it was made with, inverse y-DFT, and its
+  // rows to the eps buffer the output pass reads
+  const int ret = it - 1;
+  for (int pp = 0; pp < np; ++pp) {
+    const int p = p0 + pp;
+    const float4* g = priv(pp, ret & 1);
+    if constexpr (EM) {
+      const bool hasB = 2 * p + 1 < H;
+      for (int i = threadIdx.x; i < 2 * N; i += kTR) {
+        const int pos = i >> 1, h = i & 1;
+        float* T = reinterpret_cast<float*>(cols + (size_t)pp * tile + pl.at(pos));
+        const float2* u = reinterpret_cast<const float2*>(g) + 6 * pos + 3 * h;
+#pragma unroll
+        for (int k = 0; k < NP; ++k) {
+          const float2 x = h && !hasB ? make_float2(0.f, 0.f) : u[k];
+          T[4 * k + h] = x.x;
+          T[4 * k + 2 + h] = x.y;
+        }
+      }
+    } else {
+      const GreenPair gp(A, c, fp, 2 * p, pair);
+      for (int pos = threadIdx.x; pos < N; pos += kTR)
+        gp.spectrum(cols + (size_t)pp * tile + pl.at(pos), sx[pos], pos == 0, g[2 * pos], g[2 * pos + 1]);
+    }
+  }
+  __syncthreads();
+  for (int st = 0; st < sp.m; ++st) stage_any<NP, false, true, NP, kTR, true>(cols, tws, sp, st, ncl, tile);
+  float4* out = static_cast<float4*>(A.eps[ret & 1]);
+  for (int i = threadIdx.x; i < np * N * NP; i += kTR) {
+    const int pp = i / (N * NP), r = i - pp * (N * NP), y = r / NP, k = r - y * NP;
+    out[tile_index(c, N, l, p0 + pp, y) + k] = cols[(size_t)pp * tile + pl.at(y) + k];
+  }
+  cluster.sync();  // no CTA leaves while another may still write to its shared memory
+}
+
+}  // namespace
+
+// Taken when the whole batch fits: every grid's state within kMaxCluster CTAs (n up to about 250) and every
+// cluster on the chip at once.  A cluster's iteration is a chain of short stages whatever else runs, so
+// further waves of clusters lose to the passes, which fill the chip (64 random-disk cells, 39 of their 64
+// grids eligible: 8.4 ms in passes, 11.2 ms with the small grids on chip first), and small grids beside
+// large ones ride along in the passes' launches (the 2D sweep: 28.9 ms, 30.1 ms).  Within that, a grid is
+// spread until a CTA holds about four row groups or the chip is full.
+int resident2d_solve(const SolveArgs& A, const std::vector<CellDev>& cells, int L, int* list, int nphase_cell,
+                     cudaStream_t st, int* count) {
+  *count = 0;
+  constexpr int kSms = 152;
+  const bool em = A.scheme == HOM_SCHEME_EYRE_MILTON;
+  std::vector<int> least(cells.size(), 0);
+  int ctas = 0;
+  const int pairs = (int)cells.size() * L;
+  if (pairs > kSms) return HOM_OK;
+  for (size_t i = 0; i < cells.size(); ++i) {
+    const int n = cells[i].n;
+    const int tile = res_tile(n, !(n & 1), 2);  // an upper bound for any first radix
+    for (int C = 1; C <= kMaxCluster && !least[i]; C *= 2)
+      if (res_shape(n, C, nphase_cell, tile, em).bytes <= kResSmem) least[i] = C;
+    ctas += least[i] * L;
+    if (!least[i] || ctas > kSms) return HOM_OK;
+  }
+  struct Group {
+    std::vector<int> pairs;
+    size_t bytes = 0, full = 0;  // without and with the private state on chip
+  } by_size[4];
+  for (size_t i = 0; i < cells.size(); ++i) {
+    const int n = cells[i].n, G = (n + kFastRows - 1) / kFastRows;
+    int C = least[i];
+    while (C < kMaxCluster && (ctas + C * L) <= kSms && pairs * C * 2 <= kSms && (G + C - 1) / C > 4) {
+      ctas += C * L;
+      C *= 2;
+    }
+    Group& g = by_size[C == 1 ? 0 : C == 2 ? 1 : C == 4 ? 2 : 3];
+    for (int l = 0; l < L; ++l) g.pairs.push_back((int)i * L + l);
+    const ResShape sh = res_shape(n, C, nphase_cell, res_tile(n, !(n & 1), 2), em);
+    g.bytes = std::max(g.bytes, sh.bytes);
+    g.full = std::max(g.full, sh.bytes + sh.priv);
+  }
+  std::vector<int> all;
+  for (int q = 3; q >= 0; --q) all.insert(all.end(), by_size[q].pairs.begin(), by_size[q].pairs.end());
+  HOM_CUDA_TRY(cudaMemcpyAsync(list, all.data(), all.size() * sizeof(int), cudaMemcpyHostToDevice, st));
+  const int* at = list;
+  for (int q = 3; q >= 0; --q) {
+    const Group& g = by_size[q];
+    if (g.pairs.empty()) continue;
+    auto kernel = em ? k_resident2d<true> : k_resident2d<false>;
+    HOM_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmem));
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = 1u << q;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)g.pairs.size() << q);
+    cfg.blockDim = dim3(kTR);
+    const int priv_on_chip = g.full <= kResSmem;
+    cfg.dynamicSmemBytes = priv_on_chip ? g.full : g.bytes;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    HOM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, A, at, priv_on_chip));
+    at += g.pairs.size();
+  }
+  HOM_CUDA_TRY(cudaStreamSynchronize(st));  // the list's host copy goes out of scope
+  *count = (int)all.size();
+  return HOM_OK;
+}
+
+}  // namespace hom

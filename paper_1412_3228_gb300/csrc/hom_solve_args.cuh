@@ -46,6 +46,8 @@ struct SolveArgs {
   int* it_dev;
   int* nactive;
   unsigned long long* done;  // control kernel: arrivals (low half), active pairs (high half)
+  double* ctl_part;  // control kernel, pairs split over CTAs: [npairs][slices][nc + 3], and their arrivals
+  int* ctl_cnt;
   unsigned long long* bytes;  // [HOM_NKERNEL]
   int L, criterion, max_iter, diverge_window, stall_window;
   int green;  // HOM_GREEN_CONTINUOUS or HOM_GREEN_ROTATED

@@ -31,6 +31,7 @@
 #include "hom_plan.h"
 #include "hom_solve_args.cuh"
 #include "hom_em.cuh"
+#include "hom_control.cuh"
 #include "hom_fast2d.h"
 #include "hom_cg.cuh"
 
@@ -661,35 +662,42 @@ __global__ void __launch_bounds__(kThreads) k_ypass(SolveArgs A) {
 // One CTA per (cell, load): FP64 sums of the pair's partials (per-task partials of the row pass
 // and of the Green pass, summed in a fixed order: deterministic), equilibrium errors, stopping
 // rule.  The last CTA to finish counts the active pairs and advances the iteration.
-// Bound by latency: a chain of a few dependent loads, FP64 sums and FP64 divisions.  Each thread keeps
-// several tasks' loads in flight, the CTA grows with the pair's task count (ctl_threads: 4590 + 4590
-// tasks of a 135^3 pair on 128 threads took 56 us, on 1024 32 us), and the scalar FP64 chain
-// (square roots and divisions, hundreds of cycles each) runs side by side in the lanes of one warp
-// instead of one after the other in one thread (45^2, 3 pairs: 13.0 us, now 8.6 us).
-constexpr int kCtlMaxThreads = 1024;
-inline unsigned ctl_threads(int most_tasks) {
-  unsigned t = 128;
-  while (t < (unsigned)kCtlMaxThreads && (int)t * 4 < most_tasks) t *= 2;
-  return t;
+// Bound by latency (a chain of a few dependent loads) and, for pairs of many tasks, by FP64 additions: an
+// SM does two per cycle.  Each thread keeps several tasks' loads in flight; the block sums go through shared
+// memory, one warp per total (a shuffle tree in every warp would spend 32 lanes on every addition); a pair of
+// more than kCtlSlice tasks is split over CTAs, the last of which adds the slices in order.  Launches of
+// 128 threads and one CTA per pair took 56 us at 135^3 (6 pairs of 4590 + 4590 tasks), 1024 threads 32 us;
+// now 16 us.
+constexpr int kCtlThreads = 256;
+constexpr int kCtlSlice = 1024;
+constexpr int kCtlMaxSlices = 16;
+inline unsigned ctl_slices(int most_tasks) {
+  return (unsigned)std::min(kCtlMaxSlices, std::max(1, (most_tasks + kCtlSlice / 2) / kCtlSlice));
 }
 template <int NC>
-__global__ void __launch_bounds__(kCtlMaxThreads) k_control(SolveArgs A) {
-  __shared__ double s_red[kCtlMaxThreads / 32][NC + 3];
-  const int pair = blockIdx.x;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nthr = blockDim.x, nw = nthr >> 5;
+__global__ void __launch_bounds__(kCtlThreads) k_control(SolveArgs A) {
+  constexpr int K = NC + 3;
+  __shared__ double s_val[K][kCtlThreads];
+  __shared__ double s_tot[K];
+  __shared__ int s_last;
+  const int pair = blockIdx.x, slice = blockIdx.y, slices = gridDim.y;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int it = *A.it_dev;
   int still = 0;  // thread 0: the pair stays active
   if (A.active[pair]) {
     const PairDev pr = A.pairs[pair];
     // v[0..NC): sigma sums, v[NC]: residual sum, v[NC + 1]: normalised residual sum, v[NC + 2]:
     // compatibility residual sum (Eyre-Milton scheme)
-    double v[NC + 3];
+    double v[K];
 #pragma unroll
-    for (int k = 0; k < NC + 3; ++k) v[k] = 0.0;
+    for (int k = 0; k < K; ++k) v[k] = 0.0;
     const double* pR = A.partR + (size_t)pr.load * NC;
     const size_t rs = (size_t)A.L * NC;
+    const int nr = pr.rtask1 - pr.rtask0, nc = pr.ctask1 - pr.ctask0;
+    const int r1 = pr.rtask0 + (int)((long long)nr * (slice + 1) / slices);
+    const int c1 = pr.ctask0 + (int)((long long)nc * (slice + 1) / slices);
 #pragma unroll 4
-    for (int tk = pr.rtask0 + (int)threadIdx.x; tk < pr.rtask1; tk += nthr) {
+    for (int tk = pr.rtask0 + (int)((long long)nr * slice / slices) + (int)threadIdx.x; tk < r1; tk += kCtlThreads) {
       const double* p = pR + (size_t)tk * rs;
 #pragma unroll
       for (int k = 0; k < NC; ++k) v[k] += p[k];
@@ -697,102 +705,48 @@ __global__ void __launch_bounds__(kCtlMaxThreads) k_control(SolveArgs A) {
     const double2* pC = reinterpret_cast<const double2*>(A.partC);
     const bool em = A.partE != nullptr;
 #pragma unroll 4
-    for (int tk = pr.ctask0 + (int)threadIdx.x; tk < pr.ctask1; tk += nthr) {
+    for (int tk = pr.ctask0 + (int)((long long)nc * slice / slices) + (int)threadIdx.x; tk < c1; tk += kCtlThreads) {
       const double2 q = pC[tk];
       v[NC] += q.x;
       v[NC + 1] += q.y;
       if (em) v[NC + 2] += A.partE[tk];
     }
 #pragma unroll
-    for (int k = 0; k < NC + 3; ++k)
-      if (k < NC + 2 || em)
-        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-    if (lane == 0)
-#pragma unroll
-      for (int k = 0; k < NC + 3; ++k) s_red[wid][k] = v[k];
+    for (int k = 0; k < K; ++k) s_val[k][threadIdx.x] = v[k];
     __syncthreads();
-    if (wid == 0) {
-      const double nv = (double)A.cells[pr.cell].nv;
-      double sum = 0.0;  // lane k: total k
-      if (lane < NC + 3)
-        for (int w = 0; w < nw; ++w) sum += s_red[w][lane];
-      double den2 = 0.0, e2 = 0.0;
+    for (int k = wid; k < K; k += kCtlThreads / 32) {
+      double x = 0.0;
 #pragma unroll
-      for (int k = 0; k < NC; ++k) {
-        const double x = __shfl_sync(0xffffffffu, sum, k);
-        den2 += x * x;
-      }
-      if (em && lane == NC + 2) {
-        const double* Ep = A.E + (size_t)pair * NC;
-        for (int k = 0; k < NC; ++k) e2 += Ep[k] * Ep[k];
-      }
-      // lanes 0 .. NC - 1: the mean stress; NC and NC + 1: e and e_n; NC + 2: e_c
-      double num = sum, den = nv;
-      if (lane >= NC && lane < NC + 3) {
-        if (A.res0 && lane < NC + 2) {  // adjoint: relative to the first iterate's residual
-          double* r0 = A.res0 + 2 * pair + (lane - NC);
-          if (it == 0) *r0 = sum;
-          den = *r0;
-          num = den > 0.0 ? sum / den : 0.0;
-          den = 1.0;
-        } else if (lane < NC + 2) {
-          den = den2;
-        } else {
-          den = e2;
-        }
-        num = sqrt(num);
-        den = sqrt(den) * (lane == NC + 2 ? nv : 1.0);
-      }
-      const double q = num / den;
-      if (lane < NC) A.mean_sigma[(size_t)pair * NC + lane] = q;
-      const double e = __shfl_sync(0xffffffffu, q, NC), en = __shfl_sync(0xffffffffu, q, NC + 1),
-                   ec = __shfl_sync(0xffffffffu, q, NC + 2);
-      if (lane == 0) {
-        A.err[pair] = e;
-        A.errn[pair] = en;
-        double crit = A.criterion == HOM_CRIT_E ? e : en;
-        if (em) {  // Eyre-Milton: e_c = |eps_hat - P eps_hat| / (N_v |E|) must pass too
-          A.errc[pair] = ec;
-          crit = fmax(crit, ec);
-          if (!isfinite(ec)) crit = ec;
-        }
-        int st = -1;
-        const bool skip = A.warm && it == 0;  // warm start: g of the caller's field is unknown
-        if (A.hist && !A.inner && it <= A.max_iter)
-          A.hist[(size_t)pair * (A.max_iter + 1) + it] = skip ? (double)NAN : crit;
-        if (A.inner) {  // defect-correction inner solve: a fixed number of iterations, no error test
-          if (it >= A.kinner[pair]) st = HOM_STATUS_MAX_ITER;
-        } else if (skip) {
-          if (it >= A.max_iter) st = HOM_STATUS_MAX_ITER;
-        } else if (!isfinite(crit)) st = HOM_STATUS_DIVERGED;
-        else if (crit < A.tol) st = HOM_STATUS_CONVERGED;
-        else if (it >= A.max_iter) st = HOM_STATUS_MAX_ITER;
-        else {
-          if (A.diverge_window > 0) {
-            int gcount = crit > A.last_err[pair] ? A.grow[pair] + 1 : 0;
-            A.grow[pair] = gcount;
-            if (gcount >= A.diverge_window) st = HOM_STATUS_DIVERGED;
-          }
-          // stagnation: no new smallest error for stall_window iterations (the FP32 floor)
-          if (st < 0 && A.stall_window > 0) {
-            if (crit < A.best_err[pair]) {
-              A.best_err[pair] = crit;
-              A.best_it[pair] = it;
-            } else if (it - A.best_it[pair] >= A.stall_window) {
-              st = HOM_STATUS_STALLED;
-            }
-          }
-        }
-        if (!skip) A.last_err[pair] = crit;
-        if (st >= 0) {
-          A.status[pair] = st;
-          A.iters[pair] = it;
-          A.active[pair] = 0;
-        } else {
-          still = 1;
-        }
-      }
+      for (int i = 0; i < kCtlThreads / 32; ++i) x += s_val[k][i * 32 + lane];
+      for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+      if (lane == 0) s_tot[k] = x;
     }
+    __syncthreads();
+    bool last = true;
+    if (slices > 1) {
+      if (threadIdx.x < K) {
+        A.ctl_part[((size_t)pair * slices + slice) * K + threadIdx.x] = s_tot[threadIdx.x];
+        __threadfence();
+      }
+      __syncthreads();
+      if (threadIdx.x == 0) s_last = atomicAdd(A.ctl_cnt + pair, 1) == slices - 1;
+      __syncthreads();
+      last = s_last;
+    }
+    if (!last) return;
+    if (wid == 0) {
+      double sum = lane < K ? s_tot[lane] : 0.0;  // lane k: total k
+      if (slices > 1) {
+        __threadfence();
+        sum = 0.0;
+        if (lane < K)
+          for (int q = 0; q < slices; ++q) sum += __ldcg(A.ctl_part + ((size_t)pair * slices + q) * K + lane);
+        if (lane == 0) A.ctl_cnt[pair] = 0;
+      }
+      still = control_pair<NC>(A, pair, (double)A.cells[pr.cell].nv, sum, it);
+    }
+  } else if (slice > 0) {
+    return;
   }
   if (threadIdx.x == 0) {
     // arrivals in the low half, active pairs in the high half: the last CTA has both
@@ -1592,20 +1546,20 @@ int refine_solve(SolveArgs& A, unsigned char* ws, int npairs, int nc, const hom_
       if ((rc = allow_smem(k_ypass<double, false, 15>, smem_y64)) != HOM_OK) return rc;
     }
     const unsigned nR = (unsigned)lay.tR.size(), nC = (unsigned)lay.tC.size(), nY = (unsigned)lay.tY.size();
-    const unsigned nctl = ctl_threads(most_tasks(lay));
+    const unsigned nctl = ctl_slices(most_tasks(lay));
     auto iter64 = [&]() {
       k_row<double, DIM, false, 15><<<nR, kThreads, smem_row64, st>>>(A64);
       if (DIM == 3) k_ypass<double, true, 15><<<nY, kThreads, smem_y64, st>>>(A64);
       k_green<double, DIM, 15><<<nC, kThreads, smem_green64, st>>>(A64);
       if (DIM == 3) k_ypass<double, false, 15><<<nY, kThreads, smem_y64, st>>>(A64);
-      k_control<nc_of_dim<DIM>()><<<(unsigned)npairs, nctl, 0, st>>>(A64);
+      k_control<nc_of_dim<DIM>()><<<dim3((unsigned)npairs, nctl), kCtlThreads, 0, st>>>(A64);
     };
     auto iter32 = [&]() {
       k_row<float, DIM, false, MAXR><<<nR, kThreads, lay.smem_row, st>>>(Ain);
       if (DIM == 3) k_ypass<float, true, MAXR><<<nY, kThreads, lay.smem_y, st>>>(Ain);
       k_green<float, DIM, MAXR><<<nC, kThreads, lay.smem_green, st>>>(Ain);
       if (DIM == 3) k_ypass<float, false, MAXR><<<nY, kThreads, lay.smem_y, st>>>(Ain);
-      k_control<nc_of_dim<DIM>()><<<(unsigned)npairs, nctl, 0, st>>>(Ain);
+      k_control<nc_of_dim<DIM>()><<<dim3((unsigned)npairs, nctl), kCtlThreads, 0, st>>>(Ain);
     };
     const dim3 eg(64, (unsigned)npairs);
     float2* e32a = static_cast<float2*>(A.eps[0]);
@@ -1749,6 +1703,9 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
   const size_t o_int = take((size_t)npairs * 5 * sizeof(int) + 64);
   const size_t o_dbl = take((size_t)npairs * (4 + nc) * sizeof(double));
   const size_t o_bytes = take(HOM_NKERNEL * sizeof(unsigned long long));
+  const unsigned slices = ctl_slices(most_tasks(lay));  // only pairs of many tasks have partial sums to exchange
+  const size_t o_ctlp = slices > 1 ? take((size_t)npairs * slices * (nc + 3) * sizeof(double)) : 0;
+  const size_t o_ctlc = slices > 1 ? take((size_t)npairs * sizeof(int)) : 0;
   const size_t o_res0 = adj ? take((size_t)npairs * 2 * sizeof(double)) : 0;
   constexpr int NS = DIM == 2 ? 6 : 21;
   const size_t o_partE = em ? take(lay.tC.size() * sizeof(double)) : 0;
@@ -1802,6 +1759,7 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
     }
   }
   const size_t o_cphase = lay.fast ? take(cell_phases.size() * sizeof(int)) : 0;
+  const size_t o_reslist = lay.fast && DIM == 2 ? take((size_t)npairs * sizeof(int)) : 0;
   const size_t o_fplans = lay.fast ? take(lay.fplans.size() * sizeof(FastPlanDev)) : 0;
   const size_t o_stage_e = need_stage && out->eps && !eps_dev ? take(lay.fld_elems * sizeof(T)) : 0;
   const size_t o_stage_s = need_stage && out->sigma && !sig_dev ? take(lay.fld_elems * sizeof(T)) : 0;
@@ -1861,6 +1819,7 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
   HOM_CUDA_TRY(cudaMemsetAsync(ws + o_eps0, 0, lay.ws_elems * sizeof(V), st));
   HOM_CUDA_TRY(cudaMemsetAsync(ws + o_g, 0, lay.g_elems * sizeof(V), st));
   HOM_CUDA_TRY(cudaMemsetAsync(ws + o_bytes, 0, HOM_NKERNEL * sizeof(unsigned long long), st));
+  if (slices > 1) HOM_CUDA_TRY(cudaMemsetAsync(ws + o_ctlc, 0, (size_t)npairs * sizeof(int), st));
   HOM_CUDA_TRY(cudaMemsetAsync(ws + o_dbg, 0, 4 * sizeof(unsigned int), st));
   if (out->history && !hist_dev)  // staged: the entries the solve does not write keep the caller's values
     HOM_CUDA_TRY(cudaMemcpyAsync(ws + o_hist, out->history, hist_elems * sizeof(double), cudaMemcpyHostToDevice, st));
@@ -1914,6 +1873,8 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
   A.best_err = db + 3 * npairs;
   A.mean_sigma = db + 4 * npairs;
   A.bytes = reinterpret_cast<unsigned long long*>(ws + o_bytes);
+  A.ctl_part = slices > 1 ? reinterpret_cast<double*>(ws + o_ctlp) : nullptr;
+  A.ctl_cnt = slices > 1 ? reinterpret_cast<int*>(ws + o_ctlc) : nullptr;
   A.L = L;
   A.criterion = opts->criterion;
   A.max_iter = opts->max_iter;
@@ -1981,7 +1942,7 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
   Timer tm{out->stats, st, {}};
   const unsigned nR = (unsigned)lay.tR.size(), nC = (unsigned)lay.tC.size(), nY = (unsigned)lay.tY.size();
   NvtxRange nvtx_init_("hom_solve: initial state");
-  const unsigned nCtl = (unsigned)npairs, nctl = ctl_threads(most_tasks(lay));  // one control CTA per (cell, load)
+  const unsigned nCtl = (unsigned)npairs, nctl = ctl_slices(most_tasks(lay));  // control CTAs: (cell, load) pairs x slices
   tm.begin(HOM_K_INIT);
   k_init_pairs<<<(npairs + 255) / 256, 256, 0, st>>>(A);
   if (em) {
@@ -2008,6 +1969,12 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
 
   const int check = opts->check_every > 0 ? opts->check_every : 8;
   int host_nactive = npairs;
+  if (DIM == 2 && lay.fast && !adj && !out->stats && !ext) {
+    // pairs on small grids run to their own stopping point on chip; the passes below see them inactive
+    int nres = 0;
+    if ((rc = resident2d_solve(A, lay.cells, L, reinterpret_cast<int*>(ws + o_reslist), nph_max, st, &nres)) != HOM_OK) return rc;
+    host_nactive -= nres;
+  }
   int launched = 0;
   const dim3 cg_grid((unsigned)npairs, (unsigned)cg_nchunk);
   auto one_pass = [&]() {
@@ -2047,7 +2014,7 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
       k_cg_control<kCgUpdate><<<nCtl, kCgCtlThreads, 0, st>>>(A, G, nc);
       k_cg_elems<T, DIM, kCgDir><<<cg_grid, kCgThreads, 0, st>>>(A, G);
     } else {
-      k_control<nc_of_dim<DIM>()><<<nCtl, nctl, 0, st>>>(A);
+      k_control<nc_of_dim<DIM>()><<<dim3(nCtl, nctl), kCtlThreads, 0, st>>>(A);
     }
     tm.end();
   };
@@ -2064,7 +2031,7 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
     HOM_CUDA_TRY(cudaStreamSynchronize(st));
   }
   NvtxRange nvtx_iter_("hom_solve: iterations");
-  if (opts->use_graph && !out->stats && !cg) {
+  if (opts->use_graph && !out->stats && !cg && host_nactive > 0) {
     // The whole solve as one graph launch: a conditional WHILE node whose body is one iteration
     // (the passes and the control kernel); the control kernel clears the condition once no pair is
     // active or max_iter + 1 iterations ran, so the host waits once instead of polling.  The body
@@ -2332,34 +2299,51 @@ int solve_entry(const hom_cell* cells, int ncells, const hom_material* mat, cons
       std::vector<double> ms_sigma((size_t)ncells * L * nc_of(dim));
       std::string report;
       double best = 1e300;
-      for (const Cand& cd : cands) {
+      // The time per iteration of a candidate is that of the call as it would run (whatever mix of passes
+      // and on-chip solver it takes), from the difference of two fixed budgets: set-up drops out.
+      cudaEvent_t ev[2] = {};
+      HOM_CUDA_TRY(cudaEventCreate(&ev[0]));
+      if (cudaEventCreate(&ev[1]) != cudaSuccess) {
+        cudaEventDestroy(ev[0]);
+        return set_error(HOM_ERR_CUDA, "autotuner: event creation failed");
+      }
+      int tune_rc = HOM_OK;
+      auto timed = [&](const Cand& cd, int iters) {
         hom_solve_opts t = *opts;
         t.passes = cd.passes;
         t.max_radix = cd.radix;
         t.tol = -1.0;  // a fixed number of iterations, no early stop
-        t.max_iter = 4;
+        t.max_iter = iters;
         t.use_graph = 0;
         t.tune = 0;
-        double ms = 0.0;
-        for (int rep = 0; rep < 2; ++rep) {  // the first call builds plans and workspace
-          hom_kernel_stats ks{};
-          hom_result tr{};
-          tr.mean_sigma = ms_sigma.data();
-          tr.stats = &ks;
-          const int rc = dispatch(&t, &tr);
-          if (rc != HOM_OK && rc != HOM_ERR_NOT_CONVERGED && rc != HOM_ERR_DIVERGED) return rc;
-          ms = 0.0;
-          for (int k = HOM_K_ROW; k <= HOM_K_CONTROL; ++k) ms += ks.ms[k];
-        }
+        hom_result tr{};
+        tr.mean_sigma = ms_sigma.data();
+        cudaEventRecord(ev[0], st);
+        const int rc = dispatch(&t, &tr);
+        cudaEventRecord(ev[1], st);
+        if (rc != HOM_OK && rc != HOM_ERR_NOT_CONVERGED && rc != HOM_ERR_DIVERGED) tune_rc = rc;
+        float ms = 0.f;
+        cudaEventSynchronize(ev[1]);
+        cudaEventElapsedTime(&ms, ev[0], ev[1]);
+        return (double)ms;
+      };
+      for (const Cand& cd : cands) {
+        timed(cd, 4);  // the first call builds plans and workspace
+        const double few = std::min(timed(cd, 4), timed(cd, 4)), more = std::min(timed(cd, 16), timed(cd, 16));
+        if (tune_rc != HOM_OK) break;
+        const double ms = std::max(0.0, more - few) / 12.0;
         char line[160];
         std::snprintf(line, sizeof(line), "%s%s r%d %.3f ms", report.empty() ? "" : " | ",
-                      cd.passes == HOM_PASSES_AUTO ? "specialised" : "generic", cd.radix, ms / 5.0);
+                      cd.passes == HOM_PASSES_AUTO ? "specialised" : "generic", cd.radix, ms);
         report += line;
         if (ms < best) {
           best = ms;
           choice = TuneChoice{cd.passes, cd.radix};
         }
       }
+      cudaEventDestroy(ev[0]);
+      cudaEventDestroy(ev[1]);
+      if (tune_rc != HOM_OK) return tune_rc;
       keep_tuned(key, choice, report);
     }
     o.passes = choice.passes;
