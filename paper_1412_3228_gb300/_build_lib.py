@@ -22,7 +22,7 @@ LIB = os.path.join(BUILD, "libhom.so")
 BUILD_DEBUG = os.path.join(HERE, "_build_debug")
 LIB_DEBUG = os.path.join(BUILD_DEBUG, "libhom.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
-SOURCES = ["hom_capi.cu", "hom_filter.cu", "hom_solver.cu", "hom_fast2d.cu", "hom_fast3d.cu", "hom_noalloc.cu", "hom_backward.cu", "hom_extrap.cu"]
+SOURCES = ["hom_capi.cu", "hom_filter.cu", "hom_solver.cu", "hom_fast2d.cu", "hom_resident2d.cu", "hom_fast3d.cu", "hom_noalloc.cu", "hom_backward.cu", "hom_extrap.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -56,10 +56,6 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False) -> st
         common += ["-Xptxas", "-v"]
     if os.environ.get("HOM_THREADS"):  # threads per CTA of the solver passes (tuning)
         common += ["-DHOM_THREADS=%d" % int(os.environ["HOM_THREADS"])]
-    if os.environ.get("HOM_GREEN_TW2"):  # Green pass with a scalar twiddle table (tuning)
-        common += ["-DHOM_GREEN_TW2=%d" % int(os.environ["HOM_GREEN_TW2"])]
-    if os.environ.get("HOM_ROW_TW2"):  # row pass with a scalar twiddle table (tuning)
-        common += ["-DHOM_ROW_TW2=%d" % int(os.environ["HOM_ROW_TW2"])]
     if os.environ.get("HOM_FAST3D_THREADS"):  # threads per CTA of the specialised 3D passes (tuning)
         common += ["-DHOM_FAST3D_THREADS=%d" % int(os.environ["HOM_FAST3D_THREADS"])]
     if os.environ.get("HOM_FAST_THREADS"):  # threads per CTA of the specialised 2D passes (tuning)
