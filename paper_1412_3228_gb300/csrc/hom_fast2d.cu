@@ -286,8 +286,8 @@ __device__ __forceinline__ void prefetch_row_task(const SolveArgs& A, int task) 
 
 // One CTA per task.  `ahead` is the number of CTAs resident on the device at once: task b + ahead
 // is about the one that starts when this CTA ends, so CTA b prefetches its first load into L2.
-// RUN: radices up to RUN read from the plan (any size; see k_row_r2d); 0: compiled ones.
-template <bool OUT, bool SRC, bool EM, int RUN>
+// RUN: radices read from the plan (any size; see k_row_r2d).
+template <bool OUT, bool SRC, bool EM, bool RUN>
 __device__ __forceinline__ void row_task(const SolveArgs& A, int ntasks, int ahead) {
   HOM_DBG_POISON();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -302,9 +302,8 @@ __device__ __forceinline__ void row_task(const SolveArgs& A, int ntasks, int ahe
                         t.load < A.L, (size_t)task))
     return;
   const FastPlanDev& fp = A.fplans[c.fplan];
-  if constexpr (RUN > 0) {
-    __shared__ RunPlan sp;
-    row_body<OUT, SRC, EM>(RunN<NP, RUN>(stage_plan(fp.run, sp, kT)), A, task, t, c, fp, s, sh);
+  if constexpr (RUN) {
+    row_body<OUT, SRC, EM>(RunN<NP>(fp.run), A, task, t, c, fp, s, sh);
   } else {
     switch (c.n) {
       case 45: row_body<OUT, SRC, EM>(FixedN<45, NP>(), A, task, t, c, fp, s, sh); break;
@@ -319,16 +318,15 @@ __device__ __forceinline__ void row_task(const SolveArgs& A, int ntasks, int ahe
 }
 template <bool OUT, bool SRC, bool EM = false>
 __global__ void __launch_bounds__(kT, 3) k_row_f2d(SolveArgs A, int ntasks, int ahead) {
-  row_task<OUT, SRC, EM, 0>(A, ntasks, ahead);
+  row_task<OUT, SRC, EM, false>(A, ntasks, ahead);
 }
-// The same pass with radices read from a plan, for batches that hold a size without compiled ones.  Radices
-// up to 16 (lane pairs) take 128 registers, two CTAs per SM; batches whose plans stay at 9 and below run the
-// 80-register variant, three CTAs per SM.  Measured against the generic row pass, which keeps two real rows
-// per complex line and scalar arithmetic: 2 cells of 512^2, 3 loads: 72 us generic, 55 us with 128
-// registers, 39 us with 80; 143^2: 43 us generic, 20 us.
-template <bool OUT, bool SRC, bool EM, int MAXR>
-__global__ void __launch_bounds__(kT, MAXR > 9 ? 2 : 3) k_row_r2d(SolveArgs A, int ntasks, int ahead) {
-  row_task<OUT, SRC, EM, MAXR>(A, ntasks, ahead);
+// The same pass with radices read from a plan, for batches that hold a size without compiled ones: the
+// largest radix (16 lane pairs) takes 128 registers, two CTAs per SM.  Measured against the generic
+// row pass, which keeps two real rows per complex line and scalar arithmetic: 2 cells of 512^2, 3 loads:
+// 55 us (72 us generic); 143^2: 20 us (43 us).
+template <bool OUT, bool SRC, bool EM = false>
+__global__ void __launch_bounds__(kT, 2) k_row_r2d(SolveArgs A, int ntasks, int ahead) {
+  row_task<OUT, SRC, EM, true>(A, ntasks, ahead);
 }
 
 // eps = E: the stored x-spectrum holds E at kx = 0 of every row (lane A of pair 0), zero elsewhere.
@@ -556,7 +554,7 @@ __device__ __forceinline__ void prefetch_green_task(const SolveArgs& A, int task
 }
 
 // One CTA per task; CTA b prefetches task b + ahead into L2 (see k_row_f2d).
-template <bool EM, int RUN>
+template <bool EM, bool RUN>
 __device__ __forceinline__ void green_task(const SolveArgs& A, int ntasks, int ahead) {
   HOM_DBG_POISON();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -569,9 +567,8 @@ __device__ __forceinline__ void green_task(const SolveArgs& A, int ntasks, int a
   if (!HOM_CHECK(A, t.kx0 >= 0 && (t.kx0 & 1) == 0 && t.kx0 < c.H && t.load >= 0 && t.load < A.L, (size_t)task))
     return;
   const FastPlanDev& fp = A.fplans[c.fplan];
-  if constexpr (RUN > 0) {
-    __shared__ RunPlan sp;
-    green_body<EM>(RunN<NP, RUN>(stage_plan(fp.run, sp, kT)), A, task, t, c, fp, s);
+  if constexpr (RUN) {
+    green_body<EM>(RunN<NP>(fp.run), A, task, t, c, fp, s);
   } else {
     switch (c.n) {
       case 45: green_body<EM>(FixedN<45, NP>(), A, task, t, c, fp, s); break;
@@ -586,13 +583,13 @@ __device__ __forceinline__ void green_task(const SolveArgs& A, int ntasks, int a
 }
 template <bool EM = false>
 __global__ void __launch_bounds__(kT, 3) k_green_f2d(SolveArgs A, int ntasks, int ahead) {
-  green_task<EM, 0>(A, ntasks, ahead);
+  green_task<EM, false>(A, ntasks, ahead);
 }
-// Radices read from a plan (see k_row_r2d): 2 cells of 512^2, 3 loads: 103 us generic, 45 us with 128
-// registers, 33 us with 80; 143^2: 42 us generic, 19 us.
-template <bool EM, int MAXR>
-__global__ void __launch_bounds__(kT, MAXR > 9 ? 2 : 3) k_green_r2d(SolveArgs A, int ntasks, int ahead) {
-  green_task<EM, MAXR>(A, ntasks, ahead);
+// Radices read from a plan (see k_row_r2d): 2 cells of 512^2, 3 loads: 45 us (103 us generic); 143^2:
+// 19 us (42 us).
+template <bool EM = false>
+__global__ void __launch_bounds__(kT, 2) k_green_r2d(SolveArgs A, int ntasks, int ahead) {
+  green_task<EM, true>(A, ntasks, ahead);
 }
 
 // ------------------------------------------------------------------ labels in transform order
@@ -820,22 +817,24 @@ int launch_tasks(K kernel, const SolveArgs& A, unsigned ntasks, size_t smem, cud
 }
 }  // namespace
 
-// `run`: 0 for compiled radices, else the largest radix of the batch's plans.
-#define HOM_LAUNCH_ROW(OUT, SRC, EM)                                                                             \
-  (run == 0 ? launch_tasks(k_row_f2d<OUT, SRC, EM>, A, ntasks, smem, st)                                         \
-            : run <= 9 ? launch_tasks(k_row_r2d<OUT, SRC, EM, 9>, A, ntasks, smem, st)                           \
-                       : launch_tasks(k_row_r2d<OUT, SRC, EM, 16>, A, ntasks, smem, st))
-int fast2d_row(const SolveArgs& A, unsigned ntasks, size_t smem, int run, cudaStream_t st) {
-  if (A.scheme == HOM_SCHEME_EYRE_MILTON) return HOM_LAUNCH_ROW(false, false, true);
-  if (A.src) return HOM_LAUNCH_ROW(false, true, false);  // adjoint solve: the constitutive step takes the source term
-  return HOM_LAUNCH_ROW(false, false, false);
+int fast2d_row(const SolveArgs& A, unsigned ntasks, size_t smem, bool run, cudaStream_t st) {
+  if (A.scheme == HOM_SCHEME_EYRE_MILTON)
+    return run ? launch_tasks(k_row_r2d<false, false, true>, A, ntasks, smem, st)
+               : launch_tasks(k_row_f2d<false, false, true>, A, ntasks, smem, st);
+  if (A.src)  // adjoint solve: the constitutive step takes the source term
+    return run ? launch_tasks(k_row_r2d<false, true>, A, ntasks, smem, st)
+               : launch_tasks(k_row_f2d<false, true>, A, ntasks, smem, st);
+  return run ? launch_tasks(k_row_r2d<false, false>, A, ntasks, smem, st)
+             : launch_tasks(k_row_f2d<false, false>, A, ntasks, smem, st);
 }
 
-int fast2d_out(const SolveArgs& A, unsigned ntasks, size_t smem, int run, cudaStream_t st) {
-  if (A.scheme == HOM_SCHEME_EYRE_MILTON) return HOM_LAUNCH_ROW(true, false, true);
-  return HOM_LAUNCH_ROW(true, false, false);
+int fast2d_out(const SolveArgs& A, unsigned ntasks, size_t smem, bool run, cudaStream_t st) {
+  if (A.scheme == HOM_SCHEME_EYRE_MILTON)
+    return run ? launch_tasks(k_row_r2d<true, false, true>, A, ntasks, smem, st)
+               : launch_tasks(k_row_f2d<true, false, true>, A, ntasks, smem, st);
+  return run ? launch_tasks(k_row_r2d<true, false>, A, ntasks, smem, st)
+             : launch_tasks(k_row_f2d<true, false>, A, ntasks, smem, st);
 }
-#undef HOM_LAUNCH_ROW
 
 int fast2d_init(const SolveArgs& A, int ncells, cudaStream_t st) {
   dim3 grid(64, (unsigned)std::min(ncells, 65535));
@@ -844,16 +843,10 @@ int fast2d_init(const SolveArgs& A, int ncells, cudaStream_t st) {
   return HOM_OK;
 }
 
-namespace {
-template <bool EM>
-int launch_green(const SolveArgs& A, unsigned ntasks, size_t smem, int run, cudaStream_t st) {
-  if (run == 0) return launch_tasks(k_green_f2d<EM>, A, ntasks, smem, st);
-  return run <= 9 ? launch_tasks(k_green_r2d<EM, 9>, A, ntasks, smem, st) : launch_tasks(k_green_r2d<EM, 16>, A, ntasks, smem, st);
-}
-}  // namespace
-int fast2d_green(const SolveArgs& A, unsigned ntasks, size_t smem, int run, cudaStream_t st) {
-  return A.scheme == HOM_SCHEME_EYRE_MILTON ? launch_green<true>(A, ntasks, smem, run, st)
-                                            : launch_green<false>(A, ntasks, smem, run, st);
+int fast2d_green(const SolveArgs& A, unsigned ntasks, size_t smem, bool run, cudaStream_t st) {
+  if (A.scheme == HOM_SCHEME_EYRE_MILTON)
+    return run ? launch_tasks(k_green_r2d<true>, A, ntasks, smem, st) : launch_tasks(k_green_f2d<true>, A, ntasks, smem, st);
+  return run ? launch_tasks(k_green_r2d<false>, A, ntasks, smem, st) : launch_tasks(k_green_f2d<false>, A, ntasks, smem, st);
 }
 
 int fast2d_permute_labels(const SolveArgs& A, int ncells, long long max_nv, cudaStream_t st) {

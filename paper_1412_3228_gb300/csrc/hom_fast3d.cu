@@ -392,8 +392,8 @@ __device__ __forceinline__ void prefetch_row3_task(const SolveArgs& A, int task)
 }
 
 // One CTA per task; CTA b prefetches the first load of task b + ahead (about the task that starts
-// when this CTA ends: `ahead` CTAs are resident at once) into L2.  RUN: radices up to RUN read from the plan.
-template <bool OUT, bool SRC, bool EM, int RUN>
+// when this CTA ends: `ahead` CTAs are resident at once) into L2.  RUN: radices read from the plan.
+template <bool OUT, bool SRC, bool EM, bool RUN>
 __device__ __forceinline__ void row3_task(const SolveArgs& A, int ntasks, int ahead) {
   HOM_DBG_POISON();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -408,9 +408,8 @@ __device__ __forceinline__ void row3_task(const SolveArgs& A, int ntasks, int ah
                         t.row0 / c.n == (t.row0 + t.nrows - 1) / c.n && t.load < A.L, (size_t)task))
     return;
   const FastPlanDev& fp = A.fplans[c.fplan];
-  if constexpr (RUN > 0) {
-    __shared__ RunPlan sp;
-    row3_body<OUT, SRC, EM>(RunN<SP, RUN>(stage_plan(fp.run, sp, kT3)), A, task, t, c, fp, s, sh);
+  if constexpr (RUN) {
+    row3_body<OUT, SRC, EM>(RunN<SP>(fp.run), A, task, t, c, fp, s, sh);
   } else {
     switch (c.n) {
       case 27: row3_body<OUT, SRC, EM>(FixedN<27, SP>(), A, task, t, c, fp, s, sh); break;
@@ -424,14 +423,13 @@ __device__ __forceinline__ void row3_task(const SolveArgs& A, int ntasks, int ah
 }
 template <bool OUT, bool SRC, bool EM = false>
 __global__ void __launch_bounds__(kT3, kMinB3) k_row_f3d(SolveArgs A, int ntasks, int ahead) {
-  row3_task<OUT, SRC, EM, 0>(A, ntasks, ahead);
+  row3_task<OUT, SRC, EM, false>(A, ntasks, ahead);
 }
 // The same pass with radices read from a plan, for batches that hold a size without compiled ones (128
-// registers for radices up to 16, 80 up to 9).  Measured at 64^3, 6 loads: 112 us for the generic row pass,
-// 111 us with 128 registers, 101 us with 80.
-template <bool OUT, bool SRC, bool EM, int MAXR>
-__global__ void __launch_bounds__(kT3, MAXR > 9 ? kRunB3 : kMinB3) k_row_r3d(SolveArgs A, int ntasks, int ahead) {
-  row3_task<OUT, SRC, EM, MAXR>(A, ntasks, ahead);
+// registers for radix 16).  Measured against the generic row pass at 64^3, 6 loads: 111 us (112 us).
+template <bool OUT, bool SRC, bool EM = false>
+__global__ void __launch_bounds__(kT3, kRunB3) k_row_r3d(SolveArgs A, int ntasks, int ahead) {
+  row3_task<OUT, SRC, EM, true>(A, ntasks, ahead);
 }
 
 #ifndef HOM_3D_GREEN_GPF
@@ -510,7 +508,7 @@ __device__ __forceinline__ void ypass3_body(const PL& pl, const SolveArgs& A, co
   }
 }
 
-template <bool FWD, int RUN>
+template <bool FWD, bool RUN>
 __device__ __forceinline__ void ypass3_task(const SolveArgs& A) {
   HOM_DBG_POISON();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -521,9 +519,8 @@ __device__ __forceinline__ void ypass3_task(const SolveArgs& A) {
                         t.load >= 0 && t.load < A.L, (size_t)blockIdx.x))
     return;
   const FastPlanDev& fp = A.fplans[c.fplan];
-  if constexpr (RUN > 0) {
-    __shared__ RunPlan sp;
-    ypass3_body<FWD>(RunN<SP, RUN>(stage_plan(fp.run, sp, kT3)), A, t, c, fp, s);
+  if constexpr (RUN) {
+    ypass3_body<FWD>(RunN<SP>(fp.run), A, t, c, fp, s);
   } else {
     switch (c.n) {
       case 27: ypass3_body<FWD>(FixedN<27, SP>(), A, t, c, fp, s); break;
@@ -537,13 +534,12 @@ __device__ __forceinline__ void ypass3_task(const SolveArgs& A) {
 }
 template <bool FWD>
 __global__ void __launch_bounds__(kT3, 1024 / kT3) k_ypass_f3d(SolveArgs A) {
-  ypass3_task<FWD, 0>(A);
+  ypass3_task<FWD, false>(A);
 }
-// radices read from a plan: 64^3, 6 loads: 115-120 us for the generic passes, 58 us with 128 registers, 44 us
-// with 80
-template <bool FWD, int MAXR>
-__global__ void __launch_bounds__(kT3, MAXR > 9 ? kRunB3 : kMinB3) k_ypass_r3d(SolveArgs A) {
-  ypass3_task<FWD, MAXR>(A);
+// radices read from a plan: 64^3, 6 loads: 58 us (115-120 us for the generic passes)
+template <bool FWD>
+__global__ void __launch_bounds__(kT3, kRunB3) k_ypass_r3d(SolveArgs A) {
+  ypass3_task<FWD, true>(A);
 }
 
 // ------------------------------------------------------------------ Green pass (z lines)
@@ -793,7 +789,7 @@ __device__ __forceinline__ void green3_body(const PL& pl, const SolveArgs& A, co
   }
 }
 
-template <bool EM, int RUN>
+template <bool EM, bool RUN>
 __device__ __forceinline__ void green3_task(const SolveArgs& A) {
   HOM_DBG_POISON();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -804,9 +800,8 @@ __device__ __forceinline__ void green3_task(const SolveArgs& A) {
                         t.load >= 0 && t.load < A.L, (size_t)blockIdx.x))
     return;
   const FastPlanDev& fp = A.fplans[c.fplan];
-  if constexpr (RUN > 0) {
-    __shared__ RunPlan sp;
-    green3_body<EM>(RunN<SP, RUN>(stage_plan(fp.run, sp, kT3)), A, t, c, fp, s);
+  if constexpr (RUN) {
+    green3_body<EM>(RunN<SP>(fp.run), A, t, c, fp, s);
   } else {
     switch (c.n) {
       case 27: green3_body<EM>(FixedN<27, SP>(), A, t, c, fp, s); break;
@@ -820,12 +815,12 @@ __device__ __forceinline__ void green3_task(const SolveArgs& A) {
 }
 template <bool EM = false>
 __global__ void __launch_bounds__(kT3, kMinB3) k_green_f3d(SolveArgs A) {
-  green3_task<EM, 0>(A);
+  green3_task<EM, false>(A);
 }
-// radices read from a plan: 64^3, 6 loads: 179 us generic, 81 us with 128 registers, 62 us with 80
-template <bool EM, int MAXR>
-__global__ void __launch_bounds__(kT3, MAXR > 9 ? kRunB3 : kMinB3) k_green_r3d(SolveArgs A) {
-  green3_task<EM, MAXR>(A);
+// radices read from a plan: 64^3, 6 loads: 81 us (179 us generic)
+template <bool EM = false>
+__global__ void __launch_bounds__(kT3, kRunB3) k_green_r3d(SolveArgs A) {
+  green3_task<EM, true>(A);
 }
 
 // eps = E: the stored x-spectrum holds E at kx = 0 (lane A of pair 0) of every row, zero elsewhere.
@@ -906,27 +901,34 @@ int launch_lines3(K kernel, const SolveArgs& A, unsigned ntasks, size_t smem, cu
 }
 }  // namespace
 
-// `run`: 0 for compiled radices, else the largest radix of the batch's plans.
-#define HOM_LAUNCH3(LAUNCH, NAME, ...)                                                                           \
-  (run == 0 ? LAUNCH(k_##NAME##_f3d<__VA_ARGS__>, A, ntasks, smem, st)                                           \
-            : run <= 9 ? LAUNCH(k_##NAME##_r3d<__VA_ARGS__, 9>, A, ntasks, smem, st)                             \
-                       : LAUNCH(k_##NAME##_r3d<__VA_ARGS__, 16>, A, ntasks, smem, st))
-int fast3d_row(const SolveArgs& A, unsigned ntasks, size_t smem, bool out, int run, cudaStream_t st) {
+int fast3d_row(const SolveArgs& A, unsigned ntasks, size_t smem, bool out, bool run, cudaStream_t st) {
+  if (A.scheme == HOM_SCHEME_EYRE_MILTON) {
+    if (out)
+      return run ? launch_row3(k_row_r3d<true, false, true>, A, ntasks, smem, st)
+                 : launch_row3(k_row_f3d<true, false, true>, A, ntasks, smem, st);
+    return run ? launch_row3(k_row_r3d<false, false, true>, A, ntasks, smem, st)
+               : launch_row3(k_row_f3d<false, false, true>, A, ntasks, smem, st);
+  }
+  if (out)
+    return run ? launch_row3(k_row_r3d<true, false>, A, ntasks, smem, st)
+               : launch_row3(k_row_f3d<true, false>, A, ntasks, smem, st);
+  if (A.src)  // adjoint solve: the constitutive step takes the source term
+    return run ? launch_row3(k_row_r3d<false, true>, A, ntasks, smem, st)
+               : launch_row3(k_row_f3d<false, true>, A, ntasks, smem, st);
+  return run ? launch_row3(k_row_r3d<false, false>, A, ntasks, smem, st)
+             : launch_row3(k_row_f3d<false, false>, A, ntasks, smem, st);
+}
+
+int fast3d_ypass(const SolveArgs& A, unsigned ntasks, size_t smem, bool fwd, bool run, cudaStream_t st) {
+  if (fwd) return run ? launch_lines3(k_ypass_r3d<true>, A, ntasks, smem, st) : launch_lines3(k_ypass_f3d<true>, A, ntasks, smem, st);
+  return run ? launch_lines3(k_ypass_r3d<false>, A, ntasks, smem, st) : launch_lines3(k_ypass_f3d<false>, A, ntasks, smem, st);
+}
+
+int fast3d_green(const SolveArgs& A, unsigned ntasks, size_t smem, bool run, cudaStream_t st) {
   if (A.scheme == HOM_SCHEME_EYRE_MILTON)
-    return out ? HOM_LAUNCH3(launch_row3, row, true, false, true) : HOM_LAUNCH3(launch_row3, row, false, false, true);
-  if (out) return HOM_LAUNCH3(launch_row3, row, true, false, false);
-  if (A.src) return HOM_LAUNCH3(launch_row3, row, false, true, false);  // adjoint solve: the source term
-  return HOM_LAUNCH3(launch_row3, row, false, false, false);
+    return run ? launch_lines3(k_green_r3d<true>, A, ntasks, smem, st) : launch_lines3(k_green_f3d<true>, A, ntasks, smem, st);
+  return run ? launch_lines3(k_green_r3d<false>, A, ntasks, smem, st) : launch_lines3(k_green_f3d<false>, A, ntasks, smem, st);
 }
-
-int fast3d_ypass(const SolveArgs& A, unsigned ntasks, size_t smem, bool fwd, int run, cudaStream_t st) {
-  return fwd ? HOM_LAUNCH3(launch_lines3, ypass, true) : HOM_LAUNCH3(launch_lines3, ypass, false);
-}
-
-int fast3d_green(const SolveArgs& A, unsigned ntasks, size_t smem, int run, cudaStream_t st) {
-  return A.scheme == HOM_SCHEME_EYRE_MILTON ? HOM_LAUNCH3(launch_lines3, green, true) : HOM_LAUNCH3(launch_lines3, green, false);
-}
-#undef HOM_LAUNCH3
 
 int fast3d_init(const SolveArgs& A, int ncells, cudaStream_t st) {
   dim3 grid(64, (unsigned)std::min(ncells, 65535));
