@@ -47,12 +47,17 @@ struct CgArgs {
 };
 
 constexpr int kCgThreads = 256;
-constexpr int kCgElems = 8192;  // complex elements per CTA (rounded to whole rows)
+// Complex elements per CTA (rounded to whole rows): a thread's successive loads cost latency, a CTA's FP64
+// block sum thousands of cycles.  405^2 FP64, 2 cells x 3 loads, us a launch of the two inner products and the
+// direction update: 75, 66, 26 at 8192 elements, 149, 144, 14 at 1024 (both with two separate block sums),
+// 54, 47, 16 at 4096.
+constexpr int kCgElems = 4096;
+constexpr int kCgMaxChunks = 32768;
 
-// Rows per CTA of the element kernels for a cell whose rows hold Hp * nc complex elements.
-__host__ __device__ inline int cg_rows_per_cta(int Hp, int nc) {
-  const int r = kCgElems / (Hp * nc);
-  return r > 0 ? r : 1;
+// Rows per CTA of the element kernels for a cell of nrows rows that hold Hp * nc complex elements.
+__host__ __device__ inline int cg_rows_per_cta(int Hp, int nc, int nrows) {
+  const int r = kCgElems / (Hp * nc), least = (nrows + kCgMaxChunks - 1) / kCgMaxChunks;
+  return r > least ? r : least;
 }
 
 enum CgStage { kCgStart = 0, kCgPq = 1, kCgUpdate = 2, kCgDir = 3, kCgFinal = 4 };
@@ -95,7 +100,7 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_elems(SolveArgs A, CgArgs G) 
   const PairDev pr = A.pairs[pair];
   const CellDev c = A.cells[pr.cell];
   const int rowlen = c.Hp * NC;
-  const int rpc = cg_rows_per_cta(c.Hp, NC);
+  const int rpc = cg_rows_per_cta(c.Hp, NC, c.nrows);
   const int row0 = blockIdx.y * rpc;
   const int it = *A.it_dev;
   double* part = G.part + (size_t)pair * G.nchunk + blockIdx.y;
@@ -198,7 +203,7 @@ __global__ void __launch_bounds__(kCgCtlThreads) k_cg_control(SolveArgs A, CgArg
   if (A.active[pair]) {
     const PairDev pr = A.pairs[pair];
     const CellDev c = A.cells[pr.cell];
-    const int nchunk = (c.nrows + cg_rows_per_cta(c.Hp, nc) - 1) / cg_rows_per_cta(c.Hp, nc);
+    const int nchunk = (c.nrows + cg_rows_per_cta(c.Hp, nc, c.nrows) - 1) / cg_rows_per_cta(c.Hp, nc, c.nrows);
     // v[0]: inner product, v[1..nc]: stress sums of the last row pass
     double v[7];
 #pragma unroll

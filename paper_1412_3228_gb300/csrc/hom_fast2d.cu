@@ -107,6 +107,9 @@ __device__ __forceinline__ void row_body(const PL& pl, const SolveArgs& A, int t
   float2* sinv = sph + c.nph;  // EM: per local phase, (c + c0)^-1 as the pair (coefficient of tr(u) I, of u)
   cp_commit();
   phase_constants<OUT, EM>(A, c, cc, sph, sinv, kT);  // visible after the next barrier
+  uint16_t* xpos = reinterpret_cast<uint16_t*>(sinv + c.nph);  // OUT: position of x
+  if (OUT)
+    for (int i = threadIdx.x; i < N; i += kT) xpos[__ldg(fp.iperm + i)] = (uint16_t)i;
 
   for (int la = 0; la < nal; ++la) {
     const int l = s_al[la];
@@ -166,40 +169,47 @@ __device__ __forceinline__ void row_body(const PL& pl, const SolveArgs& A, int t
     // 2. constitutive update: lanes (x, y, z, w) of a float4 are rows (0, 2, 1, 3).  A one-byte
     // label is the local phase index of a pure voxel, or kLabel8Mixed (full label read from the
     // material, which also covers any voxel whose phase is not in the cell's list).
+    auto labels = [&](int pos, uint32_t (&lab)[kFastRows]) {
+#pragma unroll
+      for (int r = 0; r < kFastRows; ++r) lab[r] = r < nr ? (uint32_t)slab[r * NL + pos] : 0u;
+    };
+    if constexpr (OUT) {
+      // strains first (EM: from the states u), then stresses, each in place in the tile and out from there
+      float* field[2] = {static_cast<float*>(A.out_eps), static_cast<float*>(A.out_sig)};
+      const size_t base = c.fld_off + (size_t)l * NP * c.nv + (size_t)y0 * N;
+      for (int ph = 0; ph < 2; ++ph) {
+        if (ph == 1 || EM) {
+          for (int pos = threadIdx.x; pos < N; pos += kT) {
+            const int at = pl.at(pos);
+            uint32_t lab[kFastRows];
+            labels(pos, lab);
+            float4 e[NP], o[NP];
+#pragma unroll
+            for (int k = 0; k < NP; ++k) e[k] = s[at + k];
+            if (ph == 0) tau_point<true, false, true>(A, c, fp, sph, sinv, cc, nr, y0, l, pos, lab, e, o);
+            else tau_point<true, false, false>(A, c, fp, sph, sinv, cc, nr, y0, l, pos, lab, e, o);
+#pragma unroll
+            for (int k = 0; k < NP; ++k) s[at + k] = ph == 0 ? e[k] : o[k];
+          }
+          __syncthreads();
+        }
+        if (field[ph]) store_rows<NP, kT>(pl, s, xpos, field[ph] + base, c.nv, nr);
+        __syncthreads();  // the tile is rewritten by the next phase or the next load's fill
+      }
+      continue;
+    }
     for (int pos = threadIdx.x; pos < N; pos += kT) {
       const int at = pl.at(pos);
       uint32_t lab[kFastRows];
-#pragma unroll
-      for (int r = 0; r < kFastRows; ++r) lab[r] = r < nr ? (uint32_t)slab[r * NL + pos] : 0u;
+      labels(pos, lab);
       float4 e[NP], o[NP];
 #pragma unroll
       for (int k = 0; k < NP; ++k) e[k] = s[at + k];
       tau_point<OUT, SRC, EM>(A, c, fp, sph, sinv, cc, nr, y0, l, pos, lab, e, o);
-      if (OUT) {
-        // real fields of rows y0 + r at x = iperm[pos]
-        const int x = __ldg(fp.iperm + pos);
-        float* oe = static_cast<float*>(A.out_eps);
-        float* os = static_cast<float*>(A.out_sig);
-        const size_t base = c.fld_off + (size_t)l * NP * c.nv + (size_t)y0 * N + x;
 #pragma unroll
-        for (int r = 0; r < kFastRows; ++r) {
-          if (r >= nr) break;
-#pragma unroll
-          for (int k = 0; k < NP; ++k) {
-            const float ev = r == 0 ? e[k].x : r == 1 ? e[k].z : r == 2 ? e[k].y : e[k].w;
-            const float sv = r == 0 ? o[k].x : r == 1 ? o[k].z : r == 2 ? o[k].y : o[k].w;
-            const size_t ad = base + (size_t)k * c.nv + (size_t)r * N;
-            if (oe) oe[ad] = ev;
-            if (os) os[ad] = sv;
-          }
-        }
-      } else {
-#pragma unroll
-        for (int k = 0; k < NP; ++k) s[at + k] = o[k];
-      }
+      for (int k = 0; k < NP; ++k) s[at + k] = o[k];
     }
-    __syncthreads();  // the tile is read above and rewritten below (or by the next load's fill)
-    if (OUT) continue;
+    __syncthreads();
     fft_dit<NP, true, kT>(pl, s, tws);  // forward: natural order
 
     // 3. split the two real rows of each line; store the half spectra of tau, pair by pair
@@ -286,8 +296,8 @@ __device__ __forceinline__ void prefetch_row_task(const SolveArgs& A, int task) 
 
 // One CTA per task.  `ahead` is the number of CTAs resident on the device at once: task b + ahead
 // is about the one that starts when this CTA ends, so CTA b prefetches its first load into L2.
-// RUN: radices read from the plan (any size; see k_row_r2d).
-template <bool OUT, bool SRC, bool EM, bool RUN>
+// RUN: radices up to RUN read from the plan (any size; see k_row_r2d); 0: compiled ones.
+template <bool OUT, bool SRC, bool EM, int RUN>
 __device__ __forceinline__ void row_task(const SolveArgs& A, int ntasks, int ahead) {
   HOM_DBG_POISON();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -302,8 +312,9 @@ __device__ __forceinline__ void row_task(const SolveArgs& A, int ntasks, int ahe
                         t.load < A.L, (size_t)task))
     return;
   const FastPlanDev& fp = A.fplans[c.fplan];
-  if constexpr (RUN) {
-    row_body<OUT, SRC, EM>(RunN<NP>(fp.run), A, task, t, c, fp, s, sh);
+  if constexpr (RUN > 0) {
+    __shared__ RunPlan sp;
+    row_body<OUT, SRC, EM>(RunN<NP, RUN>(stage_plan(fp.run, sp, kT)), A, task, t, c, fp, s, sh);
   } else {
     switch (c.n) {
       case 45: row_body<OUT, SRC, EM>(FixedN<45, NP>(), A, task, t, c, fp, s, sh); break;
@@ -318,15 +329,16 @@ __device__ __forceinline__ void row_task(const SolveArgs& A, int ntasks, int ahe
 }
 template <bool OUT, bool SRC, bool EM = false>
 __global__ void __launch_bounds__(kT, 3) k_row_f2d(SolveArgs A, int ntasks, int ahead) {
-  row_task<OUT, SRC, EM, false>(A, ntasks, ahead);
+  row_task<OUT, SRC, EM, 0>(A, ntasks, ahead);
 }
-// The same pass with radices read from a plan, for batches that hold a size without compiled ones: the
-// largest radix (16 lane pairs) takes 128 registers, two CTAs per SM.  Measured against the generic
-// row pass, which keeps two real rows per complex line and scalar arithmetic: 2 cells of 512^2, 3 loads:
-// 55 us (72 us generic); 143^2: 20 us (43 us).
-template <bool OUT, bool SRC, bool EM = false>
-__global__ void __launch_bounds__(kT, 2) k_row_r2d(SolveArgs A, int ntasks, int ahead) {
-  row_task<OUT, SRC, EM, true>(A, ntasks, ahead);
+// The same pass with radices read from a plan, for batches that hold a size without compiled ones.  Radices
+// up to 16 (lane pairs) take 128 registers, two CTAs per SM; batches whose plans stay at 9 and below run the
+// 80-register variant, three CTAs per SM.  Measured against the generic row pass, which keeps two real rows
+// per complex line and scalar arithmetic: 2 cells of 512^2, 3 loads: 72 us generic, 55 us with 128
+// registers, 39 us with 80; 143^2: 43 us generic, 20 us.
+template <bool OUT, bool SRC, bool EM, int MAXR>
+__global__ void __launch_bounds__(kT, MAXR > 9 ? 2 : 3) k_row_r2d(SolveArgs A, int ntasks, int ahead) {
+  row_task<OUT, SRC, EM, MAXR>(A, ntasks, ahead);
 }
 
 // eps = E: the stored x-spectrum holds E at kx = 0 of every row (lane A of pair 0), zero elsewhere.
@@ -554,7 +566,7 @@ __device__ __forceinline__ void prefetch_green_task(const SolveArgs& A, int task
 }
 
 // One CTA per task; CTA b prefetches task b + ahead into L2 (see k_row_f2d).
-template <bool EM, bool RUN>
+template <bool EM, int RUN>
 __device__ __forceinline__ void green_task(const SolveArgs& A, int ntasks, int ahead) {
   HOM_DBG_POISON();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -567,8 +579,9 @@ __device__ __forceinline__ void green_task(const SolveArgs& A, int ntasks, int a
   if (!HOM_CHECK(A, t.kx0 >= 0 && (t.kx0 & 1) == 0 && t.kx0 < c.H && t.load >= 0 && t.load < A.L, (size_t)task))
     return;
   const FastPlanDev& fp = A.fplans[c.fplan];
-  if constexpr (RUN) {
-    green_body<EM>(RunN<NP>(fp.run), A, task, t, c, fp, s);
+  if constexpr (RUN > 0) {
+    __shared__ RunPlan sp;
+    green_body<EM>(RunN<NP, RUN>(stage_plan(fp.run, sp, kT)), A, task, t, c, fp, s);
   } else {
     switch (c.n) {
       case 45: green_body<EM>(FixedN<45, NP>(), A, task, t, c, fp, s); break;
@@ -583,13 +596,13 @@ __device__ __forceinline__ void green_task(const SolveArgs& A, int ntasks, int a
 }
 template <bool EM = false>
 __global__ void __launch_bounds__(kT, 3) k_green_f2d(SolveArgs A, int ntasks, int ahead) {
-  green_task<EM, false>(A, ntasks, ahead);
+  green_task<EM, 0>(A, ntasks, ahead);
 }
-// Radices read from a plan (see k_row_r2d): 2 cells of 512^2, 3 loads: 45 us (103 us generic); 143^2:
-// 19 us (42 us).
-template <bool EM = false>
-__global__ void __launch_bounds__(kT, 2) k_green_r2d(SolveArgs A, int ntasks, int ahead) {
-  green_task<EM, true>(A, ntasks, ahead);
+// Radices read from a plan (see k_row_r2d): 2 cells of 512^2, 3 loads: 103 us generic, 45 us with 128
+// registers, 32 us with 80; 143^2: 42 us generic, 19 us.
+template <bool EM, int MAXR>
+__global__ void __launch_bounds__(kT, MAXR > 9 ? 2 : 3) k_green_r2d(SolveArgs A, int ntasks, int ahead) {
+  green_task<EM, MAXR>(A, ntasks, ahead);
 }
 
 // ------------------------------------------------------------------ labels in transform order
@@ -817,24 +830,23 @@ int launch_tasks(K kernel, const SolveArgs& A, unsigned ntasks, size_t smem, cud
 }
 }  // namespace
 
-int fast2d_row(const SolveArgs& A, unsigned ntasks, size_t smem, bool run, cudaStream_t st) {
-  if (A.scheme == HOM_SCHEME_EYRE_MILTON)
-    return run ? launch_tasks(k_row_r2d<false, false, true>, A, ntasks, smem, st)
-               : launch_tasks(k_row_f2d<false, false, true>, A, ntasks, smem, st);
-  if (A.src)  // adjoint solve: the constitutive step takes the source term
-    return run ? launch_tasks(k_row_r2d<false, true>, A, ntasks, smem, st)
-               : launch_tasks(k_row_f2d<false, true>, A, ntasks, smem, st);
-  return run ? launch_tasks(k_row_r2d<false, false>, A, ntasks, smem, st)
-             : launch_tasks(k_row_f2d<false, false>, A, ntasks, smem, st);
+// `run`: 0 for compiled radices, else the largest radix of the batch's plans.
+#define HOM_LAUNCH_ROW(OUT, SRC, EM)                                                                             \
+  (run == 0 ? launch_tasks(k_row_f2d<OUT, SRC, EM>, A, ntasks, smem, st)                                         \
+            : run <= 9 ? launch_tasks(k_row_r2d<OUT, SRC, EM, 9>, A, ntasks, smem, st)                           \
+                       : launch_tasks(k_row_r2d<OUT, SRC, EM, 16>, A, ntasks, smem, st))
+int fast2d_row(const SolveArgs& A, unsigned ntasks, size_t smem, int run, cudaStream_t st) {
+  if (A.scheme == HOM_SCHEME_EYRE_MILTON) return HOM_LAUNCH_ROW(false, false, true);
+  if (A.src) return HOM_LAUNCH_ROW(false, true, false);  // adjoint solve: the constitutive step takes the source term
+  return HOM_LAUNCH_ROW(false, false, false);
 }
 
-int fast2d_out(const SolveArgs& A, unsigned ntasks, size_t smem, bool run, cudaStream_t st) {
-  if (A.scheme == HOM_SCHEME_EYRE_MILTON)
-    return run ? launch_tasks(k_row_r2d<true, false, true>, A, ntasks, smem, st)
-               : launch_tasks(k_row_f2d<true, false, true>, A, ntasks, smem, st);
-  return run ? launch_tasks(k_row_r2d<true, false>, A, ntasks, smem, st)
-             : launch_tasks(k_row_f2d<true, false>, A, ntasks, smem, st);
+int fast2d_out(const SolveArgs& A, unsigned ntasks, size_t smem, int run, cudaStream_t st) {
+  // (`smem` with room for the x positions)
+  if (A.scheme == HOM_SCHEME_EYRE_MILTON) return HOM_LAUNCH_ROW(true, false, true);
+  return HOM_LAUNCH_ROW(true, false, false);
 }
+#undef HOM_LAUNCH_ROW
 
 int fast2d_init(const SolveArgs& A, int ncells, cudaStream_t st) {
   dim3 grid(64, (unsigned)std::min(ncells, 65535));
@@ -843,10 +855,16 @@ int fast2d_init(const SolveArgs& A, int ncells, cudaStream_t st) {
   return HOM_OK;
 }
 
-int fast2d_green(const SolveArgs& A, unsigned ntasks, size_t smem, bool run, cudaStream_t st) {
-  if (A.scheme == HOM_SCHEME_EYRE_MILTON)
-    return run ? launch_tasks(k_green_r2d<true>, A, ntasks, smem, st) : launch_tasks(k_green_f2d<true>, A, ntasks, smem, st);
-  return run ? launch_tasks(k_green_r2d<false>, A, ntasks, smem, st) : launch_tasks(k_green_f2d<false>, A, ntasks, smem, st);
+namespace {
+template <bool EM>
+int launch_green(const SolveArgs& A, unsigned ntasks, size_t smem, int run, cudaStream_t st) {
+  if (run == 0) return launch_tasks(k_green_f2d<EM>, A, ntasks, smem, st);
+  return run <= 9 ? launch_tasks(k_green_r2d<EM, 9>, A, ntasks, smem, st) : launch_tasks(k_green_r2d<EM, 16>, A, ntasks, smem, st);
+}
+}  // namespace
+int fast2d_green(const SolveArgs& A, unsigned ntasks, size_t smem, int run, cudaStream_t st) {
+  return A.scheme == HOM_SCHEME_EYRE_MILTON ? launch_green<true>(A, ntasks, smem, run, st)
+                                            : launch_green<false>(A, ntasks, smem, run, st);
 }
 
 int fast2d_permute_labels(const SolveArgs& A, int ncells, long long max_nv, cudaStream_t st) {

@@ -56,13 +56,13 @@ void fast2d_plan_rebase(FastPlanDev& p, const unsigned char* base);
 // Dynamic shared memory of the row and Green passes for the largest grid size n of a call.
 size_t fast2d_smem_row(int nmax, int nphase_cell);
 size_t fast2d_smem_green(int nmax);
-// Launches (one CTA per task); `smem` from fast2d_smem_row / fast2d_smem_green; `run`: radices read from
-// the plans.
-int fast2d_row(const SolveArgs& A, unsigned ntasks, size_t smem, bool run, cudaStream_t st);
-int fast2d_green(const SolveArgs& A, unsigned ntasks, size_t smem, bool run, cudaStream_t st);
+// Launches (one CTA per task); `smem` from fast2d_smem_row / fast2d_smem_green; `run`: 0 for
+// compiled radices, else the largest radix of the batch's plans.
+int fast2d_row(const SolveArgs& A, unsigned ntasks, size_t smem, int run, cudaStream_t st);
+int fast2d_green(const SolveArgs& A, unsigned ntasks, size_t smem, int run, cudaStream_t st);
 // Output pass (final eps and sigma fields) and the initial state eps = E, in the tiled layout of
 // the specialised passes (see hom_fast2d.cu).
-int fast2d_out(const SolveArgs& A, unsigned ntasks, size_t smem, bool run, cudaStream_t st);
+int fast2d_out(const SolveArgs& A, unsigned ntasks, size_t smem, int run, cudaStream_t st);
 int fast2d_init(const SolveArgs& A, int ncells, cudaStream_t st);
 // label8[lp_off + y nl + pos] = index, in the cell's list of pure phases, of the phase of
 // label[vox_off + y n + iperm[pos]] (255 for a mixed voxel; nl = n rounded up to 16).
@@ -81,9 +81,9 @@ int resident2d_solve(const SolveArgs& A, const std::vector<CellDev>& cells, int 
 size_t fast3d_smem_row(int nmax, int nphase_cell);
 size_t fast3d_smem_y(int nmax);
 size_t fast3d_smem_green(int nmax);
-int fast3d_row(const SolveArgs& A, unsigned ntasks, size_t smem, bool out, bool run, cudaStream_t st);
-int fast3d_ypass(const SolveArgs& A, unsigned ntasks, size_t smem, bool fwd, bool run, cudaStream_t st);
-int fast3d_green(const SolveArgs& A, unsigned ntasks, size_t smem, bool run, cudaStream_t st);
+int fast3d_row(const SolveArgs& A, unsigned ntasks, size_t smem, bool out, int run, cudaStream_t st);
+int fast3d_ypass(const SolveArgs& A, unsigned ntasks, size_t smem, bool fwd, int run, cudaStream_t st);
+int fast3d_green(const SolveArgs& A, unsigned ntasks, size_t smem, int run, cudaStream_t st);
 int fast3d_init(const SolveArgs& A, int ncells, cudaStream_t st);
 
 }  // namespace hom

@@ -19,6 +19,7 @@
 // Green pass is private: [load][kx pair][y position][z position][3 lane pairs].
 #define HOM_FILE_ID 3
 #include <algorithm>
+#include <type_traits>
 
 #include "hom_fast2d.h"
 #include "hom_solve_args.cuh"
@@ -107,6 +108,10 @@ __device__ __forceinline__ void row3_body(const PL& pl, const SolveArgs& A, int 
     }
   }
 
+  uint16_t* xpos = reinterpret_cast<uint16_t*>(sinv + c.nph);  // OUT: position of x
+  if (OUT)
+    for (int i = threadIdx.x; i < N; i += kT3) xpos[__ldg(fp.iperm + i)] = (uint16_t)i;
+
   for (int la = 0; la < nal; ++la) {
     const int l = sh.al[la];
     const float4* ein = static_cast<const float4*>(A.eps[OUT ? (A.iters[t.cell * A.L + l] & 1) : (it & 1)]);
@@ -158,7 +163,9 @@ __device__ __forceinline__ void row3_body(const PL& pl, const SolveArgs& A, int 
     fft_dif<NP, false, kT3>(pl, s, tws);  // inverse: eps at digit-reversed positions
 
     // 2. constitutive update; lanes (x, y, z, w) of a float4 are rows (0, 2, 1, 3)
-    for (int pos = threadIdx.x; pos < N; pos += kT3) {
+    // one position: its strains e (EM: from the states u) and o = tau, or the stress when OUT
+    auto update = [&](auto em_tag, int pos, float4(&e)[NP], float4(&o)[NP]) {
+      constexpr bool kEm = decltype(em_tag)::value;
       const int at = pl.at(pos);
       uint32_t lab[kFastRows];
       bool mixed = false;
@@ -167,10 +174,9 @@ __device__ __forceinline__ void row3_body(const PL& pl, const SolveArgs& A, int 
         lab[r] = r < nr ? (uint32_t)slab[r * NL + pos] : 0u;
         mixed |= lab[r] == kLabel8Mixed;
       }
-      float4 e[NP], o[NP];
 #pragma unroll
       for (int k = 0; k < NP; ++k) e[k] = s[at + k];
-      if (EM && (OUT || mixed)) {
+      if (kEm && (OUT || mixed)) {
         // e holds u: eps = (c~ + c0)^-1 u per voxel (mixed: the per-call table; pure: closed form)
         const int x = __ldg(fp.iperm + pos);
 #pragma unroll
@@ -285,30 +291,36 @@ __device__ __forceinline__ void row3_body(const PL& pl, const SolveArgs& A, int 
           }
         }
       }
-      if (OUT) {
-        const int x = __ldg(fp.iperm + pos);
-        float* oe = static_cast<float*>(A.out_eps);
-        float* os = static_cast<float*>(A.out_sig);
-        const size_t base = c.fld_off + (size_t)l * NP * c.nv + (size_t)t.row0 * N + x;
+    };
+    if constexpr (OUT) {
+      // strains first (EM: from the states u), then stresses, each in place in the tile and out from there
+      float* field[2] = {static_cast<float*>(A.out_eps), static_cast<float*>(A.out_sig)};
+      const size_t base = c.fld_off + (size_t)l * NP * c.nv + (size_t)t.row0 * N;
+      for (int ph = 0; ph < 2; ++ph) {
+        if (ph == 1 || EM) {
+          for (int pos = threadIdx.x; pos < N; pos += kT3) {
+            const int at = pl.at(pos);
+            float4 e[NP], o[NP];
+            if (ph == 0) update(std::integral_constant<bool, EM>(), pos, e, o);
+            else update(std::false_type(), pos, e, o);
 #pragma unroll
-        for (int r = 0; r < kFastRows; ++r) {
-          if (r >= nr) break;
-#pragma unroll
-          for (int k = 0; k < NP; ++k) {
-            const float ev = r == 0 ? e[k].x : r == 1 ? e[k].z : r == 2 ? e[k].y : e[k].w;
-            const float sv = r == 0 ? o[k].x : r == 1 ? o[k].z : r == 2 ? o[k].y : o[k].w;
-            const size_t ad = base + (size_t)k * c.nv + (size_t)r * N;
-            if (oe) oe[ad] = ev;
-            if (os) os[ad] = sv;
+            for (int k = 0; k < NP; ++k) s[at + k] = ph == 0 ? e[k] : o[k];
           }
+          __syncthreads();
         }
-      } else {
-#pragma unroll
-        for (int k = 0; k < NP; ++k) s[at + k] = o[k];
+        if (field[ph]) store_rows<NP, kT3>(pl, s, xpos, field[ph] + base, c.nv, nr);
+        __syncthreads();  // the tile is rewritten by the next phase or the next load's fill
       }
+      continue;
     }
-    __syncthreads();  // the tile is read above and rewritten below (or by the next load's fill)
-    if (OUT) continue;
+    for (int pos = threadIdx.x; pos < N; pos += kT3) {
+      const int at = pl.at(pos);
+      float4 e[NP], o[NP];
+      update(std::integral_constant<bool, EM>(), pos, e, o);
+#pragma unroll
+      for (int k = 0; k < NP; ++k) s[at + k] = o[k];
+    }
+    __syncthreads();
     fft_dit<NP, true, kT3>(pl, s, tws);  // forward: natural order
 
     // 3. split the two real rows of each line; store the half spectra of tau pair by pair
@@ -392,8 +404,8 @@ __device__ __forceinline__ void prefetch_row3_task(const SolveArgs& A, int task)
 }
 
 // One CTA per task; CTA b prefetches the first load of task b + ahead (about the task that starts
-// when this CTA ends: `ahead` CTAs are resident at once) into L2.  RUN: radices read from the plan.
-template <bool OUT, bool SRC, bool EM, bool RUN>
+// when this CTA ends: `ahead` CTAs are resident at once) into L2.  RUN: radices up to RUN read from the plan.
+template <bool OUT, bool SRC, bool EM, int RUN>
 __device__ __forceinline__ void row3_task(const SolveArgs& A, int ntasks, int ahead) {
   HOM_DBG_POISON();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -408,8 +420,9 @@ __device__ __forceinline__ void row3_task(const SolveArgs& A, int ntasks, int ah
                         t.row0 / c.n == (t.row0 + t.nrows - 1) / c.n && t.load < A.L, (size_t)task))
     return;
   const FastPlanDev& fp = A.fplans[c.fplan];
-  if constexpr (RUN) {
-    row3_body<OUT, SRC, EM>(RunN<SP>(fp.run), A, task, t, c, fp, s, sh);
+  if constexpr (RUN > 0) {
+    __shared__ RunPlan sp;
+    row3_body<OUT, SRC, EM>(RunN<SP, RUN>(stage_plan(fp.run, sp, kT3)), A, task, t, c, fp, s, sh);
   } else {
     switch (c.n) {
       case 27: row3_body<OUT, SRC, EM>(FixedN<27, SP>(), A, task, t, c, fp, s, sh); break;
@@ -423,13 +436,14 @@ __device__ __forceinline__ void row3_task(const SolveArgs& A, int ntasks, int ah
 }
 template <bool OUT, bool SRC, bool EM = false>
 __global__ void __launch_bounds__(kT3, kMinB3) k_row_f3d(SolveArgs A, int ntasks, int ahead) {
-  row3_task<OUT, SRC, EM, false>(A, ntasks, ahead);
+  row3_task<OUT, SRC, EM, 0>(A, ntasks, ahead);
 }
 // The same pass with radices read from a plan, for batches that hold a size without compiled ones (128
-// registers for radix 16).  Measured against the generic row pass at 64^3, 6 loads: 111 us (112 us).
-template <bool OUT, bool SRC, bool EM = false>
-__global__ void __launch_bounds__(kT3, kRunB3) k_row_r3d(SolveArgs A, int ntasks, int ahead) {
-  row3_task<OUT, SRC, EM, true>(A, ntasks, ahead);
+// registers for radices up to 16, 80 up to 9).  Measured at 64^3, 6 loads: 112 us for the generic row pass,
+// 111 us with 128 registers, 101 us with 80.
+template <bool OUT, bool SRC, bool EM, int MAXR>
+__global__ void __launch_bounds__(kT3, MAXR > 9 ? kRunB3 : kMinB3) k_row_r3d(SolveArgs A, int ntasks, int ahead) {
+  row3_task<OUT, SRC, EM, MAXR>(A, ntasks, ahead);
 }
 
 #ifndef HOM_3D_GREEN_GPF
@@ -508,7 +522,7 @@ __device__ __forceinline__ void ypass3_body(const PL& pl, const SolveArgs& A, co
   }
 }
 
-template <bool FWD, bool RUN>
+template <bool FWD, int RUN>
 __device__ __forceinline__ void ypass3_task(const SolveArgs& A) {
   HOM_DBG_POISON();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -519,8 +533,9 @@ __device__ __forceinline__ void ypass3_task(const SolveArgs& A) {
                         t.load >= 0 && t.load < A.L, (size_t)blockIdx.x))
     return;
   const FastPlanDev& fp = A.fplans[c.fplan];
-  if constexpr (RUN) {
-    ypass3_body<FWD>(RunN<SP>(fp.run), A, t, c, fp, s);
+  if constexpr (RUN > 0) {
+    __shared__ RunPlan sp;
+    ypass3_body<FWD>(RunN<SP, RUN>(stage_plan(fp.run, sp, kT3)), A, t, c, fp, s);
   } else {
     switch (c.n) {
       case 27: ypass3_body<FWD>(FixedN<27, SP>(), A, t, c, fp, s); break;
@@ -534,12 +549,13 @@ __device__ __forceinline__ void ypass3_task(const SolveArgs& A) {
 }
 template <bool FWD>
 __global__ void __launch_bounds__(kT3, 1024 / kT3) k_ypass_f3d(SolveArgs A) {
-  ypass3_task<FWD, false>(A);
+  ypass3_task<FWD, 0>(A);
 }
-// radices read from a plan: 64^3, 6 loads: 58 us (115-120 us for the generic passes)
-template <bool FWD>
-__global__ void __launch_bounds__(kT3, kRunB3) k_ypass_r3d(SolveArgs A) {
-  ypass3_task<FWD, true>(A);
+// radices read from a plan: 64^3, 6 loads: 115-120 us for the generic passes, 58 us with 128 registers, 44 us
+// with 80
+template <bool FWD, int MAXR>
+__global__ void __launch_bounds__(kT3, MAXR > 9 ? kRunB3 : kMinB3) k_ypass_r3d(SolveArgs A) {
+  ypass3_task<FWD, MAXR>(A);
 }
 
 // ------------------------------------------------------------------ Green pass (z lines)
@@ -789,7 +805,7 @@ __device__ __forceinline__ void green3_body(const PL& pl, const SolveArgs& A, co
   }
 }
 
-template <bool EM, bool RUN>
+template <bool EM, int RUN>
 __device__ __forceinline__ void green3_task(const SolveArgs& A) {
   HOM_DBG_POISON();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -800,8 +816,9 @@ __device__ __forceinline__ void green3_task(const SolveArgs& A) {
                         t.load >= 0 && t.load < A.L, (size_t)blockIdx.x))
     return;
   const FastPlanDev& fp = A.fplans[c.fplan];
-  if constexpr (RUN) {
-    green3_body<EM>(RunN<SP>(fp.run), A, t, c, fp, s);
+  if constexpr (RUN > 0) {
+    __shared__ RunPlan sp;
+    green3_body<EM>(RunN<SP, RUN>(stage_plan(fp.run, sp, kT3)), A, t, c, fp, s);
   } else {
     switch (c.n) {
       case 27: green3_body<EM>(FixedN<27, SP>(), A, t, c, fp, s); break;
@@ -815,12 +832,12 @@ __device__ __forceinline__ void green3_task(const SolveArgs& A) {
 }
 template <bool EM = false>
 __global__ void __launch_bounds__(kT3, kMinB3) k_green_f3d(SolveArgs A) {
-  green3_task<EM, false>(A);
+  green3_task<EM, 0>(A);
 }
-// radices read from a plan: 64^3, 6 loads: 81 us (179 us generic)
-template <bool EM = false>
-__global__ void __launch_bounds__(kT3, kRunB3) k_green_r3d(SolveArgs A) {
-  green3_task<EM, true>(A);
+// radices read from a plan: 64^3, 6 loads: 179 us generic, 81 us with 128 registers, 62 us with 80
+template <bool EM, int MAXR>
+__global__ void __launch_bounds__(kT3, MAXR > 9 ? kRunB3 : kMinB3) k_green_r3d(SolveArgs A) {
+  green3_task<EM, MAXR>(A);
 }
 
 // eps = E: the stored x-spectrum holds E at kx = 0 (lane A of pair 0) of every row, zero elsewhere.
@@ -901,34 +918,27 @@ int launch_lines3(K kernel, const SolveArgs& A, unsigned ntasks, size_t smem, cu
 }
 }  // namespace
 
-int fast3d_row(const SolveArgs& A, unsigned ntasks, size_t smem, bool out, bool run, cudaStream_t st) {
-  if (A.scheme == HOM_SCHEME_EYRE_MILTON) {
-    if (out)
-      return run ? launch_row3(k_row_r3d<true, false, true>, A, ntasks, smem, st)
-                 : launch_row3(k_row_f3d<true, false, true>, A, ntasks, smem, st);
-    return run ? launch_row3(k_row_r3d<false, false, true>, A, ntasks, smem, st)
-               : launch_row3(k_row_f3d<false, false, true>, A, ntasks, smem, st);
-  }
-  if (out)
-    return run ? launch_row3(k_row_r3d<true, false>, A, ntasks, smem, st)
-               : launch_row3(k_row_f3d<true, false>, A, ntasks, smem, st);
-  if (A.src)  // adjoint solve: the constitutive step takes the source term
-    return run ? launch_row3(k_row_r3d<false, true>, A, ntasks, smem, st)
-               : launch_row3(k_row_f3d<false, true>, A, ntasks, smem, st);
-  return run ? launch_row3(k_row_r3d<false, false>, A, ntasks, smem, st)
-             : launch_row3(k_row_f3d<false, false>, A, ntasks, smem, st);
-}
-
-int fast3d_ypass(const SolveArgs& A, unsigned ntasks, size_t smem, bool fwd, bool run, cudaStream_t st) {
-  if (fwd) return run ? launch_lines3(k_ypass_r3d<true>, A, ntasks, smem, st) : launch_lines3(k_ypass_f3d<true>, A, ntasks, smem, st);
-  return run ? launch_lines3(k_ypass_r3d<false>, A, ntasks, smem, st) : launch_lines3(k_ypass_f3d<false>, A, ntasks, smem, st);
-}
-
-int fast3d_green(const SolveArgs& A, unsigned ntasks, size_t smem, bool run, cudaStream_t st) {
+// `run`: 0 for compiled radices, else the largest radix of the batch's plans.
+#define HOM_LAUNCH3(LAUNCH, NAME, ...)                                                                           \
+  (run == 0 ? LAUNCH(k_##NAME##_f3d<__VA_ARGS__>, A, ntasks, smem, st)                                           \
+            : run <= 9 ? LAUNCH(k_##NAME##_r3d<__VA_ARGS__, 9>, A, ntasks, smem, st)                             \
+                       : LAUNCH(k_##NAME##_r3d<__VA_ARGS__, 16>, A, ntasks, smem, st))
+int fast3d_row(const SolveArgs& A, unsigned ntasks, size_t smem, bool out, int run, cudaStream_t st) {
   if (A.scheme == HOM_SCHEME_EYRE_MILTON)
-    return run ? launch_lines3(k_green_r3d<true>, A, ntasks, smem, st) : launch_lines3(k_green_f3d<true>, A, ntasks, smem, st);
-  return run ? launch_lines3(k_green_r3d<false>, A, ntasks, smem, st) : launch_lines3(k_green_f3d<false>, A, ntasks, smem, st);
+    return out ? HOM_LAUNCH3(launch_row3, row, true, false, true) : HOM_LAUNCH3(launch_row3, row, false, false, true);
+  if (out) return HOM_LAUNCH3(launch_row3, row, true, false, false);
+  if (A.src) return HOM_LAUNCH3(launch_row3, row, false, true, false);  // adjoint solve: the source term
+  return HOM_LAUNCH3(launch_row3, row, false, false, false);
 }
+
+int fast3d_ypass(const SolveArgs& A, unsigned ntasks, size_t smem, bool fwd, int run, cudaStream_t st) {
+  return fwd ? HOM_LAUNCH3(launch_lines3, ypass, true) : HOM_LAUNCH3(launch_lines3, ypass, false);
+}
+
+int fast3d_green(const SolveArgs& A, unsigned ntasks, size_t smem, int run, cudaStream_t st) {
+  return A.scheme == HOM_SCHEME_EYRE_MILTON ? HOM_LAUNCH3(launch_lines3, green, true) : HOM_LAUNCH3(launch_lines3, green, false);
+}
+#undef HOM_LAUNCH3
 
 int fast3d_init(const SolveArgs& A, int ncells, cudaStream_t st) {
   dim3 grid(64, (unsigned)std::min(ncells, 65535));

@@ -449,8 +449,10 @@ template <int N_, int SP_> struct FixedN {
 // RunN: length and radices read from the plan.  With an even first radix r0 the lines of the span-1
 // stage would start a multiple of r0 SP float4 apart, on the same banks: one float4 of padding after
 // every r0 positions moves them apart, and every later span is a multiple of r0, so addresses stay linear.
-template <int SP_> struct RunN {
+// MAXR bounds the radices a kernel is compiled for (its registers follow the largest).
+template <int SP_, int MAXR_> struct RunN {
   static constexpr bool fixed = false;
+  static constexpr int maxr = MAXR_;
   const RunPlan& p;
   int n, tile;
   __device__ __forceinline__ explicit RunN(const RunPlan& plan) : p(plan), n(plan.n) { tile = run_tile(plan.n, plan.pad, plan.r[0]); }
@@ -521,9 +523,9 @@ __device__ __forceinline__ void stage_run(float4* s, const float2* tws, const Ru
     }
   }
 }
-template <int NP, bool FWD, bool DIT, int SP, int NT, bool MULTI = false>
+template <int NP, bool FWD, bool DIT, int SP, int NT, int MAXR = 16, bool MULTI = false>
 __device__ __forceinline__ void stage_any(float4* s, const float2* tws, const RunPlan& p, int st, int nl = NP, int tile = 0) {
-#define HOM_STAGE(R) case R: stage_run<NP, R, FWD, DIT, SP, NT, MULTI>(s, tws, p, st, nl, tile); break
+#define HOM_STAGE(R) case R: if constexpr (R <= MAXR) stage_run<NP, R, FWD, DIT, SP, NT, MULTI>(s, tws, p, st, nl, tile); break
   switch (p.r[st]) {
     HOM_STAGE(2); HOM_STAGE(3); HOM_STAGE(4); HOM_STAGE(5); HOM_STAGE(7); HOM_STAGE(8); HOM_STAGE(9); HOM_STAGE(11);
     HOM_STAGE(13); HOM_STAGE(15); HOM_STAGE(16);
@@ -542,13 +544,44 @@ template <int NP, bool FWD, int NT, int N, int SP>
 __device__ __forceinline__ void fft_dit(const FixedN<N, SP>&, float4* s, const float2* tw) {
   fft_dit_p<NP, N, FWD, float2, SP, NT>(s, tw);
 }
-template <int NP, bool FWD, int NT, int SP>
-__device__ __forceinline__ void fft_dif(const RunN<SP>& pl, float4* s, const float2* tw) {
-  for (int st = pl.p.m - 1; st >= 0; --st) stage_any<NP, FWD, false, SP, NT>(s, tw, pl.p, st);
+template <int NP, bool FWD, int NT, int SP, int MAXR>
+__device__ __forceinline__ void fft_dif(const RunN<SP, MAXR>& pl, float4* s, const float2* tw) {
+  for (int st = pl.p.m - 1; st >= 0; --st) stage_any<NP, FWD, false, SP, NT, MAXR>(s, tw, pl.p, st);
 }
-template <int NP, bool FWD, int NT, int SP>
-__device__ __forceinline__ void fft_dit(const RunN<SP>& pl, float4* s, const float2* tw) {
-  for (int st = 0; st < pl.p.m; ++st) stage_any<NP, FWD, true, SP, NT>(s, tw, pl.p, st);
+template <int NP, bool FWD, int NT, int SP, int MAXR>
+__device__ __forceinline__ void fft_dit(const RunN<SP, MAXR>& pl, float4* s, const float2* tw) {
+  for (int st = 0; st < pl.p.m; ++st) stage_any<NP, FWD, true, SP, NT, MAXR>(s, tw, pl.p, st);
+}
+
+// The plan of a CTA's size in shared memory: the stages read a dozen of its words each.  Every thread calls.
+__device__ __forceinline__ const RunPlan& stage_plan(const RunPlan& src, RunPlan& sp, int nthr) {
+  for (int i = threadIdx.x; i < (int)(sizeof(RunPlan) / sizeof(int)); i += nthr)
+    reinterpret_cast<int*>(&sp)[i] = __ldg(reinterpret_cast<const int*>(&src) + i);
+  __syncthreads();
+  return sp;
+}
+
+// Output passes: the four real rows of every component, held at digit-reversed positions of the tile, to a
+// field (out: component 0 of the first row at x = 0; components nv apart, rows n apart), x by x so that
+// the stores of a warp are contiguous; xpos[x] is the position of x.  Storing position by position
+// scattered every warp's stores over 32 sectors: 1185 us for the sweep's fields, 4063 us for those of a 243^3
+// cell with 6 loads; now 392 and 1835 us.
+template <int NP, int NT, class PL>
+__device__ __forceinline__ void store_rows(const PL& pl, const float4* s, const uint16_t* xpos, float* out, long long nv,
+                                           int nr) {
+  const int N = pl.n;
+  for (int x = threadIdx.x; x < N; x += NT) {
+    const float4* v = s + pl.at(xpos[x]);
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+      const float4 f = v[k];  // lanes (x, y, z, w): rows (0, 2, 1, 3)
+      float* o = out + (size_t)k * nv + x;
+      o[0] = f.x;
+      if (nr > 1) o[N] = f.z;
+      if (nr > 2) o[2 * (size_t)N] = f.y;
+      if (nr > 3) o[3 * (size_t)N] = f.w;
+    }
+  }
 }
 
 }  // namespace

@@ -69,11 +69,8 @@ __global__ void __launch_bounds__(kTR, 2) k_resident2d(SolveArgs A, const int* l
   const PairDev pr = A.pairs[pair];
   const CellDev c = A.cells[pr.cell];
   const FastPlanDev& fp = A.fplans[c.fplan];
-  for (int i = threadIdx.x; i < (int)(sizeof(RunPlan) / sizeof(int)); i += kTR)
-    reinterpret_cast<int*>(&sp)[i] = reinterpret_cast<const int*>(&fp.run)[i];
   if (threadIdx.x == 0) s_stop = 0;
-  __syncthreads();
-  const RunN<NP> pl(sp);
+  const RunN<NP, 16> pl(stage_plan(fp.run, sp, kTR));
   const int N = pl.n, tile = pl.tile, H = N / 2 + 1, P = (H + 1) / 2, G = (N + kFastRows - 1) / kFastRows;
   const int NL = (N + 15) / 16 * 16;
   const int gpc = (G + C - 1) / C, ppc = (P + C - 1) / C;
@@ -174,7 +171,7 @@ __global__ void __launch_bounds__(kTR, 2) k_resident2d(SolveArgs A, const int* l
     }
     cg::cluster_group::arrival_token tok = cluster.barrier_arrive();  // the columns may be overwritten once all have read
     __syncthreads();
-    for (int st = sp.m - 1; st >= 0; --st) stage_any<NP, false, false, NP, kTR, true>(rows, tws, sp, st, nrl, tile);
+    for (int st = sp.m - 1; st >= 0; --st) stage_any<NP, false, false, NP, kTR, 16, true>(rows, tws, sp, st, nrl, tile);
     for (int i = threadIdx.x; i < ng * N; i += kTR) {
       const int gl = i / N, pos = i - gl * N, y0 = (g0 + gl) * kFastRows, nr = min(kFastRows, N - y0);
       float4* s = rows + (size_t)gl * tile + pl.at(pos);
@@ -189,7 +186,7 @@ __global__ void __launch_bounds__(kTR, 2) k_resident2d(SolveArgs A, const int* l
       for (int k = 0; k < NP; ++k) s[k] = o[k];
     }
     __syncthreads();
-    for (int st = 0; st < sp.m; ++st) stage_any<NP, true, true, NP, kTR, true>(rows, tws, sp, st, nrl, tile);
+    for (int st = 0; st < sp.m; ++st) stage_any<NP, true, true, NP, kTR, 16, true>(rows, tws, sp, st, nrl, tile);
     cluster.barrier_wait(std::move(tok));
     if (s_stop) break;
     // split the two real rows of each line and push the half spectra of tau to the owners of their columns
@@ -242,7 +239,7 @@ __global__ void __launch_bounds__(kTR, 2) k_resident2d(SolveArgs A, const int* l
       if (lane == 0) s_rs[q] = x;
     }
     // columns
-    for (int st = sp.m - 1; st >= 0; --st) stage_any<NP, true, false, NP, kTR, true>(cols, tws, sp, st, ncl, tile);
+    for (int st = sp.m - 1; st >= 0; --st) stage_any<NP, true, false, NP, kTR, 16, true>(cols, tws, sp, st, ncl, tile);
     Acc<float> acc[EM ? 3 : 2];
     if constexpr (EM) {
       GreenPairEm gp(A, c, fp, 0, Eld);
@@ -282,7 +279,7 @@ __global__ void __launch_bounds__(kTR, 2) k_resident2d(SolveArgs A, const int* l
       s_mine[k] = EM ? 0.5 * (tau + (double)N * u)
                      : tau + (double)N * (2.0 * c.mu0 * u + (k < 2 ? c.lam0 * tr : 0.0));
     }
-    for (int st = 0; st < sp.m; ++st) stage_any<NP, false, true, NP, kTR, true>(cols, tws, sp, st, ncl, tile);
+    for (int st = 0; st < sp.m; ++st) stage_any<NP, false, true, NP, kTR, 16, true>(cols, tws, sp, st, ncl, tile);
     if (threadIdx.x < kSums) cluster.map_shared_rank(s_part, 0)[rank * kSums + threadIdx.x] = s_mine[threadIdx.x];
     cluster.sync();
   }
@@ -313,7 +310,7 @@ __global__ void __launch_bounds__(kTR, 2) k_resident2d(SolveArgs A, const int* l
     }
   }
   __syncthreads();
-  for (int st = 0; st < sp.m; ++st) stage_any<NP, false, true, NP, kTR, true>(cols, tws, sp, st, ncl, tile);
+  for (int st = 0; st < sp.m; ++st) stage_any<NP, false, true, NP, kTR, 16, true>(cols, tws, sp, st, ncl, tile);
   float4* out = static_cast<float4*>(A.eps[ret & 1]);
   for (int i = threadIdx.x; i < np * N * NP; i += kTR) {
     const int pp = i / (N * NP), r = i - pp * (N * NP), y = r / NP, k = r - y * NP;

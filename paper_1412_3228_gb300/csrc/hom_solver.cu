@@ -1067,6 +1067,7 @@ struct Layout {
   std::vector<std::vector<unsigned char>> fplan_host;  // external workspace: their host copies
   bool fast = false;
   bool run = false;  // fast, with radices read from the plans (a size without compiled ones)
+  int run_max = 0;   // the largest of them (0: compiled radices)
   size_t ws_elems = 0, g_elems = 0, fld_elems = 0;
   size_t smem_row = 0, smem_green = 0, smem_y = 0;
 };
@@ -1229,6 +1230,8 @@ int build_layout(const hom_cell* cells, int ncells, int L, int dim, size_t vsize
         }
         if (rc != HOM_OK) return rc;
         lay.fplans.push_back(fp);
+        if (lay.run)
+          for (int st = 0; st < fp.run.m; ++st) lay.run_max = std::max(lay.run_max, fp.run.r[st]);
         idx = (int)lay.fplans.size() - 1;
       }
       c.fplan = idx;
@@ -1717,7 +1720,7 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
   const size_t o_hist = out->history && !hist_dev ? take(hist_elems * sizeof(double)) : 0;
   int cg_nchunk = 1;
   for (const CellDev& c : lay.cells)
-    cg_nchunk = std::max(cg_nchunk, (c.nrows + cg_rows_per_cta(c.Hp, nc) - 1) / cg_rows_per_cta(c.Hp, nc));
+    cg_nchunk = std::max(cg_nchunk, (c.nrows + cg_rows_per_cta(c.Hp, nc, c.nrows) - 1) / cg_rows_per_cta(c.Hp, nc, c.nrows));
   if (cg && cg_nchunk > 65535) return set_error(HOM_ERR_UNSUPPORTED_SIZE, "hom_solve_cg: cell too large");
   const size_t o_cgx = cg ? take(lay.ws_elems * sizeof(V)) : 0, o_cgr = cg ? take(lay.ws_elems * sizeof(V)) : 0;
   const size_t o_cgpart = cg ? take((size_t)npairs * cg_nchunk * sizeof(double)) : 0;
@@ -1916,9 +1919,10 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
     G.E = A.E;
     G.nchunk = cg_nchunk;
   }
-  size_t smem_frow = 0, smem_fgreen = 0, smem_fy = 0;  // the largest over the batch's sizes
+  size_t smem_frow = 0, smem_fout = 0, smem_fgreen = 0, smem_fy = 0;  // the largest over the batch's sizes
   for (const FastPlanDev& fp : lay.fplans) {
     smem_frow = std::max(smem_frow, DIM == 2 ? fast2d_smem_row(fp.n, nph_max) : fast3d_smem_row(fp.n, nph_max));
+    smem_fout = std::max(smem_fout, smem_frow + ((size_t)fp.n * sizeof(uint16_t) + 15) / 16 * 16);
     smem_fgreen = std::max(smem_fgreen, DIM == 2 ? fast2d_smem_green(fp.n) : fast3d_smem_green(fp.n));
     if (DIM == 3) smem_fy = std::max(smem_fy, fast3d_smem_y(fp.n));
   }
@@ -1980,26 +1984,26 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
   auto one_pass = [&]() {
     NvtxRange r_("hom_solve: passes");
     tm.begin(HOM_K_ROW);
-    if (lay.fast && DIM == 3) fast3d_row(A, nR, smem_frow, false, lay.run, st);
-    else if (lay.fast) fast2d_row(A, nR, smem_frow, lay.run, st);
+    if (lay.fast && DIM == 3) fast3d_row(A, nR, smem_frow, false, lay.run_max, st);
+    else if (lay.fast) fast2d_row(A, nR, smem_frow, lay.run_max, st);
     else if (em) k_row<T, DIM, false, MAXR, true><<<nR, kThreads, lay.smem_row, st>>>(A);
     else k_row<T, DIM, false, MAXR><<<nR, kThreads, lay.smem_row, st>>>(A);
     tm.end();
     if (DIM == 3) {
       tm.begin(HOM_K_YFWD);
-      if (lay.fast) fast3d_ypass(A, nY, smem_fy, true, lay.run, st);
+      if (lay.fast) fast3d_ypass(A, nY, smem_fy, true, lay.run_max, st);
       else k_ypass<T, true, MAXR><<<nY, kThreads, lay.smem_y, st>>>(A);
       tm.end();
     }
     tm.begin(HOM_K_GREEN);
-    if (lay.fast && DIM == 3) fast3d_green(A, nC, smem_fgreen, lay.run, st);
-    else if (lay.fast) fast2d_green(A, nC, smem_fgreen, lay.run, st);
+    if (lay.fast && DIM == 3) fast3d_green(A, nC, smem_fgreen, lay.run_max, st);
+    else if (lay.fast) fast2d_green(A, nC, smem_fgreen, lay.run_max, st);
     else if (em) k_green<T, DIM, MAXR, true><<<nC, kThreads, lay.smem_green, st>>>(A);
     else k_green<T, DIM, MAXR><<<nC, kThreads, lay.smem_green, st>>>(A);
     tm.end();
     if (DIM == 3) {
       tm.begin(HOM_K_YINV);
-      if (lay.fast) fast3d_ypass(A, nY, smem_fy, false, lay.run, st);
+      if (lay.fast) fast3d_ypass(A, nY, smem_fy, false, lay.run_max, st);
       else k_ypass<T, false, MAXR><<<nY, kThreads, lay.smem_y, st>>>(A);
       tm.end();
     }
@@ -2043,7 +2047,7 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
     K.out_eps = K.out_sig = nullptr;
     std::string key(reinterpret_cast<const char*>(&K), sizeof(K));
     const size_t dims[] = {nR, nC, nY, nCtl, nctl, lay.smem_row, lay.smem_green, lay.smem_y, smem_frow, smem_fgreen,
-                           smem_fy, (size_t)lay.fast, (size_t)lay.run, (size_t)DIM, sizeof(T), (size_t)MAXR};
+                           smem_fy, (size_t)lay.fast, (size_t)lay.run_max, (size_t)DIM, sizeof(T), (size_t)MAXR};
     key.append(reinterpret_cast<const char*>(dims), sizeof(dims));
     cudaGraphExec_t gexec = find_graph(dev, key);
     if (!gexec) {
@@ -2119,8 +2123,8 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
   if (want_fields) {
     NvtxRange r_("hom_solve: output fields");
     tm.begin(HOM_K_OUTPUT);
-    if (lay.fast && DIM == 3) fast3d_row(A, nR, smem_frow, true, lay.run, st);
-    else if (lay.fast) fast2d_out(A, nR, smem_frow, lay.run, st);
+    if (lay.fast && DIM == 3) fast3d_row(A, nR, smem_fout, true, lay.run_max, st);
+    else if (lay.fast) fast2d_out(A, nR, smem_fout, lay.run_max, st);
     else if (em) k_row<T, DIM, true, MAXR, true><<<nR, kThreads, lay.smem_row, st>>>(A);
     else k_row<T, DIM, true, MAXR><<<nR, kThreads, lay.smem_row, st>>>(A);
     tm.end();
