@@ -1131,13 +1131,11 @@ int build_layout(const hom_cell* cells, int ncells, int L, int dim, size_t vsize
   const size_t kMaxSmem = 227 * 1024;
   // The specialised passes take 4-row and 2-column tasks; the output pass (generic row kernel)
   // then needs 4 rows of every load on chip.
-  // The row radices are compiled in where every size of the batch has them, else read from plans (not
-  // for the no-allocation entry point, whose scratch rules are fixed by the sizes it documents).
+  // The radices are compiled in where every size of the batch has them, else read from plans.
   if (lay.fast) {
     for (int ci = 0; ci < ncells; ++ci) {
       const int n = cells[ci].n;
       if (!(dim == 2 ? fast2d_size(n) : fast3d_size(n))) lay.run = true;
-      if (external && lay.run) lay.fast = false;
       if (!(dim == 2 ? run2d_size(n) : run3d_size(n))) lay.fast = false;
     }
     if (lay.run) {  // what the one-byte labels and their kernel cannot hold stays on the generic passes
@@ -1773,6 +1771,11 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
   for (size_t i = 0; i < lay.fplan_host.size(); ++i) o_fplan_tab[i] = take(lay.fplan_host[i].size());
   void* wsv = nullptr;
   if (ext) {
+    if (off > ext->capacity && lay.run) {  // the generic passes take less scratch (no one-byte labels)
+      hom_solve_opts g = *opts;
+      g.passes = HOM_PASSES_GENERIC;
+      return run_solve<T, DIM, MAXR>(cells, ncells, mat, E, L, c0, &g, out, st, ext, adj, cg);
+    }
     if (off > ext->capacity)
       return set_error(HOM_ERR_UNSUPPORTED_SIZE,
                        "this batch needs %zu bytes of solver scratch; the fixed scratch array holds %zu bytes", off,
@@ -1973,7 +1976,7 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
 
   const int check = opts->check_every > 0 ? opts->check_every : 8;
   int host_nactive = npairs;
-  if (DIM == 2 && lay.fast && !adj && !out->stats && !ext) {
+  if (DIM == 2 && lay.fast && !adj && !out->stats) {
     // pairs on small grids run to their own stopping point on chip; the passes below see them inactive
     int nres = 0;
     if ((rc = resident2d_solve(A, lay.cells, L, reinterpret_cast<int*>(ws + o_reslist), nph_max, st, &nres)) != HOM_OK) return rc;
