@@ -29,10 +29,9 @@ __device__ __forceinline__ int control_pair(const SolveArgs& A, int pair, double
     const double* Ep = A.E + (size_t)pair * NC;
     for (int k = 0; k < NC; ++k) e2 += Ep[k] * Ep[k];
   }
-  // An iterate clearly above the tolerance goes on without a square root or a division (the FP64 chain took
-  // 2-3 us of every iteration): its errors are asked for only by the history and by the stagnation and
-  // divergence windows.
-  if (!A.res0 && !A.hist && !A.inner && !A.warm && A.diverge_window == 0 && A.stall_window == 0 && it < A.max_iter) {
+  // An iterate clearly above the tolerance whose errors nobody reads goes on without a square root or a
+  // division (the FP64 chain took 2-3 us of every iteration).
+  if (A.quiet && it < A.max_iter) {
     const double q = __shfl_sync(0xffffffffu, sum, A.criterion == HOM_CRIT_E ? NC : NC + 1);
     const double c2 = em ? __shfl_sync(0xffffffffu, sum, NC + 2) : 0.0;
     const double t2 = (A.tol > 0.0 ? A.tol * A.tol : 0.0) * (1.0 + 1e-9);

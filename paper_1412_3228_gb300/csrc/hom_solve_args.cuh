@@ -52,6 +52,10 @@ struct SolveArgs {
   int L, criterion, max_iter, diverge_window, stall_window;
   int green;  // HOM_GREEN_CONTINUOUS or HOM_GREEN_ROTATED
   int inner;  // defect-correction inner solve: the control kernel only counts iterations
+  // 1: nobody reads the mean stress and the errors of an iterate that goes on (no history, no stagnation or
+  // divergence window, no adjoint or warm start, and not a check of the defect correction, whose results
+  // are those of the last iterate checked whether it passes or not)
+  int quiet;
   const int* kinner;  // inner solve: per-pair iteration count (the pair stops at kinner[p])
   double tol;
   void* out_eps;

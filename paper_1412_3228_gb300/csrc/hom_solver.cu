@@ -1515,6 +1515,7 @@ int refine_solve(SolveArgs& A, unsigned char* ws, int npairs, int nc, const hom_
       X.mean_sigma = db + 4 * (size_t)npairs;
       X.diverge_window = 0;
       X.stall_window = 0;
+      X.quiet = 0;  // the last check's mean stress and errors are the results, above tol too
       X.cond = 0;
       X.use_cond = 0;
     };
@@ -1904,6 +1905,7 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
   A.partE = em ? reinterpret_cast<double*>(ws + o_partE) : nullptr;
   A.errc = em ? reinterpret_cast<double*>(ws + o_errc) : nullptr;
   A.em_minv = em ? ws + o_minv : nullptr;
+  A.quiet = !adj && !warm && !A.hist && A.diverge_window == 0 && A.stall_window == 0;
   A.fplans = lay.fast ? reinterpret_cast<const FastPlanDev*>(ws + o_fplans) : nullptr;
   A.label8 = lay.fast ? reinterpret_cast<const uint8_t*>(ws + o_lperm) : nullptr;
   A.cell_phases = lay.fast ? reinterpret_cast<const int*>(ws + o_cphase) : nullptr;
