@@ -814,14 +814,6 @@ size_t fast2d_smem_green(int nmax) {
 
 namespace {
 template <typename K>
-int opt_in(K kernel, size_t bytes) {
-  if (bytes > 48 * 1024) HOM_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-  return HOM_OK;
-}
-}  // namespace
-
-namespace {
-template <typename K>
 int launch_tasks(K kernel, const SolveArgs& A, unsigned ntasks, size_t smem, cudaStream_t st) {
   int rc = opt_in(kernel, smem);
   if (rc != HOM_OK) return rc;

@@ -867,12 +867,6 @@ __global__ void k_init_f3d(SolveArgs A, int ncells) {
   }
 }
 
-template <typename K>
-int opt_in3(K kernel, size_t bytes) {
-  if (bytes > 48 * 1024) HOM_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-  return HOM_OK;
-}
-
 }  // namespace
 
 bool fast3d_size(int n) {
@@ -904,14 +898,14 @@ size_t fast3d_smem_green(int nmax) {
 namespace {
 template <typename K>
 int launch_row3(K kernel, const SolveArgs& A, unsigned ntasks, size_t smem, cudaStream_t st) {
-  int rc = opt_in3(kernel, smem);
+  int rc = opt_in(kernel, smem);
   if (rc != HOM_OK) return rc;
   kernel<<<ntasks, kT3, smem, st>>>(A, (int)ntasks, resident_ctas(kernel, kT3, smem));
   return HOM_OK;
 }
 template <typename K>
 int launch_lines3(K kernel, const SolveArgs& A, unsigned ntasks, size_t smem, cudaStream_t st) {
-  int rc = opt_in3(kernel, smem);
+  int rc = opt_in(kernel, smem);
   if (rc != HOM_OK) return rc;
   kernel<<<ntasks, kT3, smem, st>>>(A);
   return HOM_OK;

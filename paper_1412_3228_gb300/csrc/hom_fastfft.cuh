@@ -11,6 +11,7 @@
 
 #include "hom_common.cuh"
 #include "hom_fast2d.h"
+#include "hom_internal.h"
 
 namespace hom {
 namespace {
@@ -19,6 +20,19 @@ namespace {
 #define HOM_FAST_THREADS 256
 #endif
 constexpr int kT = HOM_FAST_THREADS;  // threads per CTA (a build-time tunable)
+
+// Lets `kernel` be launched with `bytes` of dynamic shared memory.  The limit a kernel starts with, 48 KB,
+// holds its static arrays too (loads' bookkeeping, plan, block sums: below 4 KB in every pass), so launches
+// from 44 KB on raise it, always to the same value: neither the order of calls nor other threads matter.
+constexpr size_t kPassSmem = (size_t)(227 - 4) * 1024;
+template <typename K>
+int opt_in(K kernel, size_t bytes) {
+  if (bytes > kPassSmem)
+    return set_error(HOM_ERR_UNSUPPORTED_SIZE, "a pass needs %zu bytes of shared memory, it can have %zu", bytes, kPassSmem);
+  if (bytes > 44 * 1024)
+    HOM_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPassSmem));
+  return HOM_OK;
+}
 
 // CTAs of `kernel` resident on the device at once (the prefetch distance of the passes), cached
 // per kernel for the last (device, shared-memory size) asked.

@@ -1986,29 +1986,33 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
   }
   int launched = 0;
   const dim3 cg_grid((unsigned)npairs, (unsigned)cg_nchunk);
+  int pass_rc = HOM_OK;  // the first pass that could not be launched
+  auto launched_ok = [&](int r) {
+    if (pass_rc == HOM_OK) pass_rc = r;
+  };
   auto one_pass = [&]() {
     NvtxRange r_("hom_solve: passes");
     tm.begin(HOM_K_ROW);
-    if (lay.fast && DIM == 3) fast3d_row(A, nR, smem_frow, false, lay.run_max, st);
-    else if (lay.fast) fast2d_row(A, nR, smem_frow, lay.run_max, st);
+    if (lay.fast && DIM == 3) launched_ok(fast3d_row(A, nR, smem_frow, false, lay.run_max, st));
+    else if (lay.fast) launched_ok(fast2d_row(A, nR, smem_frow, lay.run_max, st));
     else if (em) k_row<T, DIM, false, MAXR, true><<<nR, kThreads, lay.smem_row, st>>>(A);
     else k_row<T, DIM, false, MAXR><<<nR, kThreads, lay.smem_row, st>>>(A);
     tm.end();
     if (DIM == 3) {
       tm.begin(HOM_K_YFWD);
-      if (lay.fast) fast3d_ypass(A, nY, smem_fy, true, lay.run_max, st);
+      if (lay.fast) launched_ok(fast3d_ypass(A, nY, smem_fy, true, lay.run_max, st));
       else k_ypass<T, true, MAXR><<<nY, kThreads, lay.smem_y, st>>>(A);
       tm.end();
     }
     tm.begin(HOM_K_GREEN);
-    if (lay.fast && DIM == 3) fast3d_green(A, nC, smem_fgreen, lay.run_max, st);
-    else if (lay.fast) fast2d_green(A, nC, smem_fgreen, lay.run_max, st);
+    if (lay.fast && DIM == 3) launched_ok(fast3d_green(A, nC, smem_fgreen, lay.run_max, st));
+    else if (lay.fast) launched_ok(fast2d_green(A, nC, smem_fgreen, lay.run_max, st));
     else if (em) k_green<T, DIM, MAXR, true><<<nC, kThreads, lay.smem_green, st>>>(A);
     else k_green<T, DIM, MAXR><<<nC, kThreads, lay.smem_green, st>>>(A);
     tm.end();
     if (DIM == 3) {
       tm.begin(HOM_K_YINV);
-      if (lay.fast) fast3d_ypass(A, nY, smem_fy, false, lay.run_max, st);
+      if (lay.fast) launched_ok(fast3d_ypass(A, nY, smem_fy, false, lay.run_max, st));
       else k_ypass<T, false, MAXR><<<nY, kThreads, lay.smem_y, st>>>(A);
       tm.end();
     }
@@ -2086,9 +2090,13 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
         cudaGraph_t body = nullptr;
         ce = cudaStreamEndCapture(cap, &body);
       }
-      if (ce == cudaSuccess) ce = cudaGraphInstantiate(&gexec, graph, 0);
+      if (ce == cudaSuccess && pass_rc == HOM_OK) ce = cudaGraphInstantiate(&gexec, graph, 0);
       if (cap) cudaStreamDestroy(cap);
       cudaGraphDestroy(graph);
+      if (pass_rc != HOM_OK) {
+        cudaGetLastError();
+        return pass_rc;
+      }
       if (ce != cudaSuccess) {
         cudaGetLastError();
         return set_error(HOM_ERR_CUDA, "whole-solve graph: %s", cudaGetErrorString(ce));
@@ -2106,6 +2114,7 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
     const int k = std::min(check, remaining);
     for (int i = 0; i < k; ++i) one_iteration();
     launched += k;
+    if (pass_rc != HOM_OK) return pass_rc;
     HOM_CUDA_TRY(cudaGetLastError());
     HOM_CUDA_TRY(cudaMemcpyAsync(&host_nactive, A.nactive, sizeof(int), cudaMemcpyDeviceToHost, st));
     HOM_CUDA_TRY(cudaStreamSynchronize(st));
@@ -2128,12 +2137,13 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
   if (want_fields) {
     NvtxRange r_("hom_solve: output fields");
     tm.begin(HOM_K_OUTPUT);
-    if (lay.fast && DIM == 3) fast3d_row(A, nR, smem_fout, true, lay.run_max, st);
-    else if (lay.fast) fast2d_out(A, nR, smem_fout, lay.run_max, st);
+    if (lay.fast && DIM == 3) launched_ok(fast3d_row(A, nR, smem_fout, true, lay.run_max, st));
+    else if (lay.fast) launched_ok(fast2d_out(A, nR, smem_fout, lay.run_max, st));
     else if (em) k_row<T, DIM, true, MAXR, true><<<nR, kThreads, lay.smem_row, st>>>(A);
     else k_row<T, DIM, true, MAXR><<<nR, kThreads, lay.smem_row, st>>>(A);
     tm.end();
     HOM_CUDA_TRY(cudaGetLastError());
+    if (pass_rc != HOM_OK) return pass_rc;
     if (out->eps && !eps_dev)
       HOM_CUDA_TRY(cudaMemcpyAsync(out->eps, ws + o_stage_e, lay.fld_elems * sizeof(T), cudaMemcpyDeviceToHost, st));
     if (out->sigma && !sig_dev)
