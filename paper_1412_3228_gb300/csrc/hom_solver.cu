@@ -1677,6 +1677,7 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
   const bool em = opts->scheme == HOM_SCHEME_EYRE_MILTON && !cg && !adj && !ext;
   // a warm start converts the caller's real field on the generic passes' layout
   const bool warm = opts->warm_start != 0 && !cg && !adj && !ext;
+  if (warm && !out->eps) return set_error(HOM_ERR_INVALID_ARG, "hom_solve: a warm start without an initial field");
   lay.fast = std::is_same<T, float>::value && !cg && opts->passes != HOM_PASSES_GENERIC &&
              opts->green == HOM_GREEN_CONTINUOUS && !refine && !warm;
   int rc = build_layout(cells, ncells, L, DIM, sizeof(V), MAXR, c0, ext != nullptr, lay, em);
@@ -2302,8 +2303,11 @@ int solve_entry(const hom_cell* cells, int ncells, const hom_material* mat, cons
     std::vector<int> ns;
     for (int c = 0; c < ncells; ++c) ns.push_back(cells[c].n);
     std::sort(ns.begin(), ns.end());
+    // defect correction and warm starts run on the generic passes: a choice of their own, over their radices
+    const bool generic = opts->refine > 0 || opts->warm_start != 0;
     std::string key = "dev" + std::to_string(dev) + " dim" + std::to_string(dim) + " L" + std::to_string(L) +
-                      " green" + std::to_string(opts->green) + " scheme" + std::to_string(opts->scheme) + " n";
+                      " green" + std::to_string(opts->green) + " scheme" + std::to_string(opts->scheme) +
+                      (generic ? " generic n" : " n");
     for (size_t i = 0; i < ns.size(); ++i) {
       size_t j = i;
       while (j + 1 < ns.size() && ns[j + 1] == ns[i]) ++j;
@@ -2313,8 +2317,9 @@ int solve_entry(const hom_cell* cells, int ncells, const hom_material* mat, cons
     TuneChoice choice{};
     if (!find_tuned(key, &choice)) {
       struct Cand { int passes, radix; };
-      const Cand cands[] = {{HOM_PASSES_AUTO, 27}, {HOM_PASSES_GENERIC, 15}, {HOM_PASSES_GENERIC, 27},
-                            {HOM_PASSES_GENERIC, 45}};
+      Cand cands[] = {{HOM_PASSES_AUTO, 27}, {HOM_PASSES_GENERIC, 15}, {HOM_PASSES_GENERIC, 27},
+                      {HOM_PASSES_GENERIC, 45}};
+      if (generic) cands[0].passes = HOM_PASSES_GENERIC;
       std::vector<double> ms_sigma((size_t)ncells * L * nc_of(dim));
       std::string report;
       double best = 1e300;
@@ -2331,6 +2336,9 @@ int solve_entry(const hom_cell* cells, int ncells, const hom_material* mat, cons
         hom_solve_opts t = *opts;
         t.passes = cd.passes;
         t.max_radix = cd.radix;
+        // a trial has no field to start from, and its iterations are those of the plain scheme
+        t.warm_start = 0;
+        t.refine = 0;
         t.tol = -1.0;  // a fixed number of iterations, no early stop
         t.max_iter = iters;
         t.use_graph = 0;
