@@ -235,12 +235,12 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
 
 
 def _mixed_estimate(cells) -> int:
-    """Room for the mixed voxels of a batch: the voxels whose filter ball meets a surface lie in a band
-    of twice the filter radius about it (3D packs hold more of them than a sixteenth of their voxels,
-    and a table that is too small costs a second build).  Overlapping primitives only overestimate."""
+    """Mixed voxels of a batch: those whose filter ball meets a surface lie in a band of twice the filter
+    radius about it.  Overlapping primitives only overestimate; what the library will refuse (sizes,
+    dimensions, radii out of range) counts for nothing."""
     total = 0.0
     for c in cells:
-        if c.rule == 0:
+        if c.rule == 0 or c.dim not in (2, 3) or c.n < 1:
             continue
         band = 2.0 * float(c.radius_px) + 0.5
         part = 0.0
@@ -252,8 +252,16 @@ def _mixed_estimate(cells) -> int:
                 part += 2.0 * math.pi * r * band
             else:
                 part += 4.0 * math.pi * (r * r + band * band / 12.0) * band
-        total += min(part, float(c.n) ** c.dim)
+        if part > 0.0:  # (not NaN)
+            total += min(part, float(c.n) ** c.dim)
     return int(total) + 1
+
+
+def _mixed_capacity(cells, nvox: int) -> int:
+    """Entries of the first mixed table (about 300 bytes each in 3D): the estimate where it asks for more than a
+    sixteenth of the voxels (3D packs do: 14 % at 135^3, and a table that is too small costs a second build), up
+    to a quarter of them, or 2^18 entries.  Beyond that the second build has the exact count."""
+    return max(1024, nvox // 16, min(_mixed_estimate(cells), max(nvox // 4, 1 << 18)))
 
 
 def hom_filter_build(cells: Sequence, phases: Sequence[Tuple[float, float]], device=None, stream=None,
@@ -274,7 +282,7 @@ def hom_filter_build(cells: Sequence, phases: Sequence[Tuple[float, float]], dev
     label = torch.empty(nvox, dtype=torch.int32, device=device)
     phase_c64 = torch.empty(nphase * ns, dtype=torch.float64, device=device)
     phase_c32 = torch.empty(nphase * ns, dtype=torch.float32, device=device)
-    cap = capacity if capacity is not None else max(1024, nvox // 16, _mixed_estimate(cells))
+    cap = capacity if capacity is not None else _mixed_capacity(cells, nvox)
     for _attempt in range(2):
         mixed = dict(
             mixed_c64=torch.empty(cap * ns, dtype=torch.float64, device=device),
