@@ -474,27 +474,6 @@ template <int SP_, int MAXR_> struct RunN {
   __device__ __forceinline__ int at(int pos) const { return pos * SP_ + (p.pad ? fdiv(pos, p.d_r0) : 0); }
 };
 
-// Twiddles w^q (q < R) of one butterfly: w and every fourth power come from the table, the others are
-// products of at most three factors, formed where they are used (few registers stay live).
-template <int R> struct TwPow {
-  float2 w1, w2, w3, w4, w8, w12;
-  __device__ __forceinline__ TwPow(const float2* tw, int L, int j) {
-    w1 = tw[j];
-    w2 = cmul1(w1, w1);
-    w3 = cmul1(w2, w1);
-    w4 = w8 = w12 = w1;
-    if constexpr (R > 4) w4 = tw[3 * L + j];
-    if constexpr (R > 8) w8 = R > 9 ? tw[7 * L + j] : cmul1(w4, w4);
-    if constexpr (R > 12) w12 = tw[11 * L + j];
-  }
-  __device__ __forceinline__ float2 operator()(int q) const {
-    const float2 hi = q < 8 ? w4 : q < 12 ? w8 : w12;
-    const int r = q & 3;
-    if (q < 4) return r == 1 ? w1 : r == 2 ? w2 : w3;
-    return r == 0 ? hi : cmul1(hi, r == 1 ? w1 : r == 2 ? w2 : w3);
-  }
-};
-
 // One stage with its span read from the plan (see stage_p).
 // MULTI: over nl lines, NP of each tile of `tile` float4, instead of the NP lines of one.
 template <int NP, int R, bool FWD, bool DIT, int SP, int NT, bool MULTI = false>
@@ -514,9 +493,8 @@ __device__ __forceinline__ void stage_run(float4* s, const float2* tws, const Ru
 #pragma unroll
       for (int q = 1; q < R; ++q) v[q] = ldp(base[q * qs]);
       if (L > 1) {
-        const TwPow<R> w(tw, L, j);
 #pragma unroll
-        for (int q = 1; q < R; ++q) v[q] = twmul<FWD>(v[q], w(q));
+        for (int q = 1; q < R; ++q) v[q] = twmul<FWD>(v[q], tw[(q - 1) * L + j]);
       }
       dftp<R, FWD>(v);
 #pragma unroll
@@ -527,9 +505,8 @@ __device__ __forceinline__ void stage_run(float4* s, const float2* tws, const Ru
       dftp<R, FWD>(v);
       base[0] = stp(v[0]);
       if (L > 1) {
-        const TwPow<R> w(tw, L, j);
 #pragma unroll
-        for (int q = 1; q < R; ++q) base[q * qs] = stp(twmul<FWD>(v[out_pos<R>(q)], w(q)));
+        for (int q = 1; q < R; ++q) base[q * qs] = stp(twmul<FWD>(v[out_pos<R>(q)], tw[(q - 1) * L + j]));
       } else {
 #pragma unroll
         for (int q = 1; q < R; ++q) base[q * qs] = stp(v[out_pos<R>(q)]);
