@@ -61,7 +61,11 @@ __device__ __forceinline__ void tau_point(const SolveArgs& A, const CellDev& c, 
   const float lam_em = cc.lam0, mu2_em = cc.mu2;  // EM: the reference medium of (c + c0)^-1, also when OUT
   bool mixed = false;
 #pragma unroll
-  for (int r = 0; r < kFastRows; ++r) mixed |= lab[r] == kLabel8Mixed;
+  for (int r = 0; r < kFastRows; ++r) {
+    // debug builds: a phase of the cell's list
+    if (!HOM_CHECK(A, lab[r] == kLabel8Mixed || lab[r] < (uint32_t)c.nph, lab[r])) lab[r] = 0;
+    mixed |= lab[r] == kLabel8Mixed;
+  }
   uint32_t loc[kFastRows];  // the one-byte labels (EM: per-phase constants of pure voxels)
 #pragma unroll
   for (int r = 0; r < kFastRows; ++r) loc[r] = lab[r];

@@ -65,7 +65,11 @@ __global__ void __launch_bounds__(kTR, 2) k_resident2d(SolveArgs A, const int* l
   __shared__ int s_stop;
   cg::cluster_group cluster = cg::this_cluster();
   const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  HOM_DBG_POISON();
   const int pair = list[blockIdx.x / C];
+  // debug builds: a pair of the batch (every CTA of the cluster finds the same and leaves before the first
+  // cluster barrier, here and below)
+  if (!HOM_CHECK(A, pair >= 0 && pair < A.npairs, (size_t)pair)) return;
   const PairDev pr = A.pairs[pair];
   const CellDev c = A.cells[pr.cell];
   const FastPlanDev& fp = A.fplans[c.fplan];
@@ -90,6 +94,17 @@ __global__ void __launch_bounds__(kTR, 2) k_resident2d(SolveArgs A, const int* l
   float2* sinv = sph + c.nph;
   constexpr int GP = EM ? 3 : 2;  // float4 per position of the Green step's private state
   float4* s_priv = reinterpret_cast<float4*>(sph + 2 * c.nph);  // [buffer][pair][position][GP]
+
+  // debug builds: the arrays above end within the launch's dynamic shared memory, every pair's tile and
+  // private state within the workspace (2 complex elements a float4), the grid within the labels, every
+  // position within its tile, every kx pair with an owner
+  if (!HOM_CHECK(A, reinterpret_cast<unsigned char*>(s_priv + (priv_on_chip ? 2 * (size_t)ppc * N * GP : 0)) <=
+                        smem_raw + dynamic_smem(), pair) ||
+      !HOM_CHECK(A, 2 * tile_index(c, N, l, P - 1, N) <= A.n_ws, pair) ||
+      !HOM_CHECK(A, c.g_off + ((size_t)l * (c.Hp / 2) + P) * N * 2 * GP <= A.n_g, pair) ||
+      !HOM_CHECK(A, (size_t)(c.vox_off + c.nv) <= A.n_lab, pair) || !HOM_CHECK(A, pl.at(N - 1) + NP <= tile, pair) ||
+      !HOM_CHECK(A, P <= ppc * C && G <= gpc * C, pair))
+    return;
 
   CellConst<float> cc;
   cell_const(c, cc);

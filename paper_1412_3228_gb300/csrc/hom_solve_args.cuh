@@ -103,12 +103,18 @@ __device__ __forceinline__ bool dbg_ok(unsigned int* w, bool ok, unsigned file, 
   return false;
 }
 
+// Bytes of dynamic shared memory this launch has.
+__device__ __forceinline__ size_t dynamic_smem() {
+  unsigned int bytes;
+  asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(bytes));
+  return bytes;
+}
+
 // Debug builds fill a pass kernel's dynamic shared memory with all-ones bytes (NaN in FP32 and
 // FP64) before use, so a read of an element nobody wrote shows up as a NaN result.
 __device__ __forceinline__ void dbg_poison_smem() {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  unsigned int bytes;
-  asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(bytes));
+  const unsigned int bytes = (unsigned)dynamic_smem();
   uint32_t* p = reinterpret_cast<uint32_t*>(smem_raw);
   for (unsigned i = threadIdx.x; i < bytes / 4; i += blockDim.x) p[i] = 0xFFFFFFFFu;
   __syncthreads();
