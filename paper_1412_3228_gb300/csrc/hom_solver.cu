@@ -2324,14 +2324,15 @@ int solve_entry(const hom_cell* cells, int ncells, const hom_material* mat, cons
       std::string report;
       double best = 1e300;
       // The time per iteration of a candidate is that of the call as it would run (whatever mix of passes
-      // and on-chip solver it takes), from the difference of two fixed budgets: set-up drops out.
+      // and on-chip solver it takes), from the difference of two fixed budgets: set-up drops out.  A caller
+      // waits for the trials, so they are few: 1, 1 and 8 iterations a candidate.
       cudaEvent_t ev[2] = {};
       HOM_CUDA_TRY(cudaEventCreate(&ev[0]));
       if (cudaEventCreate(&ev[1]) != cudaSuccess) {
         cudaEventDestroy(ev[0]);
         return set_error(HOM_ERR_CUDA, "autotuner: event creation failed");
       }
-      int tune_rc = HOM_OK;
+      int tune_rc = HOM_OK, trial_iters = 0;
       auto timed = [&](const Cand& cd, int iters) {
         hom_solve_opts t = *opts;
         t.passes = cd.passes;
@@ -2340,7 +2341,8 @@ int solve_entry(const hom_cell* cells, int ncells, const hom_material* mat, cons
         t.warm_start = 0;
         t.refine = 0;
         t.tol = -1.0;  // a fixed number of iterations, no early stop
-        t.max_iter = iters;
+        t.max_iter = iters - 1;  // max_iter Green-operator applications make one iterate more
+        trial_iters += iters;
         t.use_graph = 0;
         t.tune = 0;
         hom_result tr{};
@@ -2355,10 +2357,10 @@ int solve_entry(const hom_cell* cells, int ncells, const hom_material* mat, cons
         return (double)ms;
       };
       for (const Cand& cd : cands) {
-        timed(cd, 4);  // the first call builds plans and workspace
-        const double few = std::min(timed(cd, 4), timed(cd, 4)), more = std::min(timed(cd, 16), timed(cd, 16));
+        timed(cd, 1);  // the first call builds plans and workspace
+        const double few = timed(cd, 1), more = timed(cd, 8);
         if (tune_rc != HOM_OK) break;
-        const double ms = std::max(0.0, more - few) / 12.0;
+        const double ms = std::max(0.0, more - few) / 7.0;
         char line[160];
         std::snprintf(line, sizeof(line), "%s%s r%d %.3f ms", report.empty() ? "" : " | ",
                       cd.passes == HOM_PASSES_AUTO ? "specialised" : "generic", cd.radix, ms);
@@ -2371,7 +2373,7 @@ int solve_entry(const hom_cell* cells, int ncells, const hom_material* mat, cons
       cudaEventDestroy(ev[0]);
       cudaEventDestroy(ev[1]);
       if (tune_rc != HOM_OK) return tune_rc;
-      keep_tuned(key, choice, report);
+      keep_tuned(key, choice, report + " (" + std::to_string(trial_iters) + " trial iterations)");
     }
     o.passes = choice.passes;
     o.max_radix = choice.radix;
