@@ -715,11 +715,10 @@ int fast2d_plan_host(int n, bool run, std::vector<unsigned char>& h, FastPlanDev
   if (radix.empty() || !build_host_plan_radices(n, radix, hp))
     return set_error(HOM_ERR_UNSUPPORTED_SIZE, "no specialised plan for n = %d", n);
   auto up = [](size_t b) { return (b + 255) / 256 * 256; };
-  const size_t b_tw = up((size_t)n * 16), b_ip = up((size_t)n * 2), b_xp = up((size_t)n * 4), b_xn = up((size_t)n * 4),
-               b_t2 = up((size_t)n * 8 + 8);
-  h.assign(b_tw + b_ip + b_xp + b_xn + b_t2, 0);
+  const size_t b_ip = up((size_t)n * 2), b_xp = up((size_t)n * 4), b_xn = up((size_t)n * 4), b_tw = up((size_t)n * 8 + 8);
+  h.assign(b_ip + b_xp + b_xn + b_tw, 0);
   // per-stage twiddle tables (stages with span L > 1): entry (q - 1) L + j = w^(j q n / (L R))
-  float* tw = reinterpret_cast<float*>(h.data());
+  float* tw = reinterpret_cast<float*>(h.data() + b_ip + b_xp + b_xn);
   {
     size_t e = 0;
     for (size_t st = 1; st < hp.radix.size(); ++st) {
@@ -727,27 +726,23 @@ int fast2d_plan_host(int n, bool run, std::vector<unsigned char>& h, FastPlanDev
       for (int q = 1; q < R; ++q)
         for (int j = 0; j < L; ++j, ++e) {
           const int t = (j * q * TS) % n;
-          tw[4 * e] = tw[4 * e + 1] = (float)hp.tw[2 * t];
-          tw[4 * e + 2] = tw[4 * e + 3] = (float)hp.tw[2 * t + 1];
-          float* t2 = reinterpret_cast<float*>(h.data() + b_tw + b_ip + b_xp + b_xn);
-          t2[2 * e] = (float)hp.tw[2 * t];
-          t2[2 * e + 1] = (float)hp.tw[2 * t + 1];
+          tw[2 * e] = (float)hp.tw[2 * t];
+          tw[2 * e + 1] = (float)hp.tw[2 * t + 1];
         }
     }
   }
-  uint16_t* ip = reinterpret_cast<uint16_t*>(h.data() + b_tw);
+  uint16_t* ip = reinterpret_cast<uint16_t*>(h.data());
   for (int k = 0; k < n; ++k) ip[hp.perm[k]] = (uint16_t)k;
-  float* xp = reinterpret_cast<float*>(h.data() + b_tw + b_ip);
-  float* xn = reinterpret_cast<float*>(h.data() + b_tw + b_ip + b_xp);
+  float* xp = reinterpret_cast<float*>(h.data() + b_ip);
+  float* xn = reinterpret_cast<float*>(h.data() + b_ip + b_xp);
   for (int p = 0; p < n; ++p) xp[p] = (float)hp.xi[ip[p]];
   for (int k = 0; k < n; ++k) xn[k] = (float)hp.xi[k];
   // table pointers as byte offsets from the start of the tables (fast2d_plan_rebase adds the base)
   FastPlanDev p{};
-  p.tw4 = reinterpret_cast<const float4*>(size_t(0));
-  p.iperm = reinterpret_cast<const uint16_t*>(b_tw);
-  p.xipos = reinterpret_cast<const float*>(b_tw + b_ip);
-  p.xinat = reinterpret_cast<const float*>(b_tw + b_ip + b_xp);
-  p.tw2 = reinterpret_cast<const float2*>(b_tw + b_ip + b_xp + b_xn);
+  p.iperm = reinterpret_cast<const uint16_t*>(size_t(0));
+  p.xipos = reinterpret_cast<const float*>(b_ip);
+  p.xinat = reinterpret_cast<const float*>(b_ip + b_xp);
+  p.tw2 = reinterpret_cast<const float2*>(b_ip + b_xp + b_xn);
   p.n = n;
   fill_run_plan(hp, p.run);
   *out = p;
@@ -756,7 +751,6 @@ int fast2d_plan_host(int n, bool run, std::vector<unsigned char>& h, FastPlanDev
 
 void fast2d_plan_rebase(FastPlanDev& p, const unsigned char* base) {
   auto at = [&](const void* off) { return base + reinterpret_cast<size_t>(off); };
-  p.tw4 = reinterpret_cast<const float4*>(at(p.tw4));
   p.iperm = reinterpret_cast<const uint16_t*>(at(p.iperm));
   p.xipos = reinterpret_cast<const float*>(at(p.xipos));
   p.xinat = reinterpret_cast<const float*>(at(p.xinat));

@@ -1,7 +1,7 @@
-// Specialised FP32 passes of the 2D fixed-point scheme (section 2, eqs. 1-a, 1-b, 2) for grid
-// sizes with a compile-time radix plan.  They compute what the generic row and Green passes of
-// hom_solver.cu compute, on the same mixed-domain state, task lists and partial sums; see
-// hom_fast2d.cu for the data layout in shared memory.
+// FP32 lane-pair passes of the fixed-point and Eyre-Milton schemes (section 2, eqs. 1-a, 1-b, 2), 2D and 3D,
+// with radices compiled in for a few sizes and read from a plan for every other, and the on-chip solver of
+// small 2D grids.  They compute what the generic passes of hom_solver.cu compute, on the same task lists and
+// partial sums; see hom_fast2d.cu for the data layouts.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -25,14 +25,13 @@ struct RunPlan {
   FastDiv d_nb[kMaxRunStages], d_L[kMaxRunStages], d_r0;
 };
 
-// Device tables of one grid size n (plan with the radices compiled into the specialised passes).
+// Device tables of one grid size n, in the digit order of its radices (compiled in or of `run`).
 struct FastPlanDev {
-  const float4* tw4;      // (cos, cos, -sin, -sin)(2 pi t / n), t < n: twiddles duplicated per lane
   const uint16_t* iperm;  // iperm[pos]: index held at position pos after a DIF transform
   const float* xipos;     // 2 pi a(iperm[pos]): wave number of the bin at position pos
   const float* xinat;     // 2 pi a(k) in natural order
-  const float2* tw2;      // the twiddle tables as (cos, -sin) pairs
-  int n, pad;
+  const float2* tw2;      // the stages' twiddle tables, (cos, -sin) pairs
+  int n;
   RunPlan run;            // the same transform for the run-time-size passes
 };
 
@@ -69,9 +68,9 @@ int fast2d_init(const SolveArgs& A, int ncells, cudaStream_t st);
 int fast2d_permute_labels(const SolveArgs& A, int ncells, long long max_nv, cudaStream_t st);
 void fast2d_release();
 
-// On-chip solver of the small grids of a batch (hom_resident2d.cu): runs every pair whose grid fits a
-// thread-block cluster to its stopping point and leaves it inactive, its iterate where the output pass
-// reads it.  `list` holds room for every pair; *count receives the number of pairs taken.
+// On-chip solver of batches of small grids (hom_resident2d.cu): where every pair of the batch fits, runs all of
+// them to their stopping points and leaves them inactive, their iterates where the output pass reads them.
+// `list` holds room for every pair; *count receives the number of pairs taken, all or none.
 struct CellDev;
 int resident2d_solve(const SolveArgs& A, const std::vector<CellDev>& cells, int L, int* list, int nphase_cell,
                      cudaStream_t st, int* count);
