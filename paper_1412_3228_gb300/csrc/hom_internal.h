@@ -82,6 +82,7 @@ bool grid_supported(int n);
 struct ExternalWorkspace {
   unsigned char* base;
   size_t capacity;
+  bool compact = false;  // a call that did not fit tries again with the least scratch
 };
 
 // Adjoint Lippmann-Schwinger solve (used by hom_solve_backward): the same fixed point driven by a

@@ -1066,6 +1066,7 @@ struct Layout {
   std::vector<FastPlanDev> fplans;  // specialised FP32 passes: per-size tables
   std::vector<std::vector<unsigned char>> fplan_host;  // external workspace: their host copies
   bool fast = false;
+  bool compact = false;  // the least scratch: no smaller tasks than fit on chip, one control CTA per pair
   bool run = false;  // fast, with radices read from the plans (a size without compiled ones)
   int run_max = 0;   // the largest of them (0: compiled radices)
   size_t ws_elems = 0, g_elems = 0, fld_elems = 0;
@@ -1084,6 +1085,9 @@ int most_tasks(const Layout& lay) {
   for (const PairDev& p : lay.pairs) m = std::max(m, std::max(p.rtask1 - p.rtask0, p.ctask1 - p.ctask0));
   return m;
 }
+
+// Control CTAs per pair.
+unsigned control_slices(const Layout& lay) { return lay.compact ? 1u : ctl_slices(most_tasks(lay)); }
 
 template <int DIM> constexpr int nc_of_dim() { return DIM == 2 ? 3 : 6; }
 
@@ -1176,7 +1180,7 @@ int build_layout(const hom_cell* cells, int ncells, int L, int dim, size_t vsize
     row_total += ((size_t)(dim == 2 ? n : n * n) + r - 1) / r;
     col_total += (size_t)(n / 2 + q) / q * L * (dim == 2 ? 1 : n);
   }
-  const bool split_loads = lay.fast && L > 1 && row_total < kFewTasks;
+  const bool split_loads = !lay.compact && lay.fast && L > 1 && row_total < kFewTasks;
   for (int ci = 0; ci < ncells; ++ci) {
     const hom_cell& k = cells[ci];
     CellDev c{};
@@ -1259,7 +1263,7 @@ int build_layout(const hom_cell* cells, int ncells, int L, int dim, size_t vsize
     // row-pass tasks: as many rows as fit in the shared-memory budget with every load active
     const size_t line_bytes = (size_t)k.n * vsize;
     int r = rows_fit(k.n);
-    if (!lay.fast) {
+    if (!lay.fast && !lay.compact) {
       const int fit = r;
       r = spread(fit, row_total);
       // an odd number of real rows leaves half of a complex line empty (405^2 FP64, 3 loads: tasks of one
@@ -1271,7 +1275,7 @@ int build_layout(const hom_cell* cells, int ncells, int L, int dim, size_t vsize
     if (need_r > kMaxSmem) return set_error(HOM_ERR_UNSUPPORTED_SIZE, "row of n = %d with %d loads does not fit on chip", k.n, L);
     lay.smem_row = std::max(lay.smem_row, need_r);
     if (lay.fast) r = std::min(kFastRows, c.nrows);
-    const int ntk = lay.fast ? cols_fit(k.n) : spread(cols_fit(k.n), col_total);
+    const int ntk = lay.fast || lay.compact ? cols_fit(k.n) : spread(cols_fit(k.n), col_total);
     const size_t need_l = ((size_t)ntk * nc + 2) * line_bytes;
     lay.smem_green = std::max(lay.smem_green, need_l);
     lay.smem_y = std::max(lay.smem_y, need_l);
@@ -1548,7 +1552,7 @@ int refine_solve(SolveArgs& A, unsigned char* ws, int npairs, int nc, const hom_
       if ((rc = allow_smem(k_ypass<double, false, 15>, smem_y64)) != HOM_OK) return rc;
     }
     const unsigned nR = (unsigned)lay.tR.size(), nC = (unsigned)lay.tC.size(), nY = (unsigned)lay.tY.size();
-    const unsigned nctl = ctl_slices(most_tasks(lay));
+    const unsigned nctl = control_slices(lay);
     auto iter64 = [&]() {
       k_row<double, DIM, false, 15><<<nR, kThreads, smem_row64, st>>>(A64);
       if (DIM == 3) k_ypass<double, true, 15><<<nY, kThreads, smem_y64, st>>>(A64);
@@ -1680,6 +1684,7 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
   if (warm && !out->eps) return set_error(HOM_ERR_INVALID_ARG, "hom_solve: a warm start without an initial field");
   lay.fast = std::is_same<T, float>::value && !cg && opts->passes != HOM_PASSES_GENERIC &&
              opts->green == HOM_GREEN_CONTINUOUS && !refine && !warm;
+  lay.compact = ext && ext->compact;
   int rc = build_layout(cells, ncells, L, DIM, sizeof(V), MAXR, c0, ext != nullptr, lay, em);
   if (rc != HOM_OK) return rc;
   const int npairs = ncells * L;
@@ -1706,7 +1711,7 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
   const size_t o_int = take((size_t)npairs * 5 * sizeof(int) + 64);
   const size_t o_dbl = take((size_t)npairs * (4 + nc) * sizeof(double));
   const size_t o_bytes = take(HOM_NKERNEL * sizeof(unsigned long long));
-  const unsigned slices = ctl_slices(most_tasks(lay));  // only pairs of many tasks have partial sums to exchange
+  const unsigned slices = control_slices(lay);  // only pairs of many tasks have partial sums to exchange
   const size_t o_ctlp = slices > 1 ? take((size_t)npairs * slices * (nc + 3) * sizeof(double)) : 0;
   const size_t o_ctlc = slices > 1 ? take((size_t)npairs * sizeof(int)) : 0;
   const size_t o_res0 = adj ? take((size_t)npairs * 2 * sizeof(double)) : 0;
@@ -1762,7 +1767,8 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
     }
   }
   const size_t o_cphase = lay.fast ? take(cell_phases.size() * sizeof(int)) : 0;
-  const size_t o_reslist = lay.fast && DIM == 2 ? take((size_t)npairs * sizeof(int)) : 0;
+  const bool on_chip = lay.fast && DIM == 2 && !adj && !out->stats && !lay.compact;
+  const size_t o_reslist = on_chip ? take((size_t)npairs * sizeof(int)) : 0;
   const size_t o_fplans = lay.fast ? take(lay.fplans.size() * sizeof(FastPlanDev)) : 0;
   const size_t o_stage_e = need_stage && out->eps && !eps_dev ? take(lay.fld_elems * sizeof(T)) : 0;
   const size_t o_stage_s = need_stage && out->sigma && !sig_dev ? take(lay.fld_elems * sizeof(T)) : 0;
@@ -1773,10 +1779,14 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
   for (size_t i = 0; i < lay.fplan_host.size(); ++i) o_fplan_tab[i] = take(lay.fplan_host[i].size());
   void* wsv = nullptr;
   if (ext) {
-    if (off > ext->capacity && lay.run) {  // the generic passes take less scratch (no one-byte labels)
+    // What speed costs in scratch goes first (partial sums of more tasks and control CTAs), then the passes
+    // with plan-read radices: the generic ones take less (no one-byte labels).
+    if (off > ext->capacity && (!ext->compact || lay.run)) {
+      ExternalWorkspace least = *ext;
       hom_solve_opts g = *opts;
-      g.passes = HOM_PASSES_GENERIC;
-      return run_solve<T, DIM, MAXR>(cells, ncells, mat, E, L, c0, &g, out, st, ext, adj, cg);
+      if (ext->compact) g.passes = HOM_PASSES_GENERIC;
+      least.compact = true;
+      return run_solve<T, DIM, MAXR>(cells, ncells, mat, E, L, c0, &g, out, st, &least, adj, cg);
     }
     if (off > ext->capacity)
       return set_error(HOM_ERR_UNSUPPORTED_SIZE,
@@ -1952,7 +1962,7 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
   Timer tm{out->stats, st, {}};
   const unsigned nR = (unsigned)lay.tR.size(), nC = (unsigned)lay.tC.size(), nY = (unsigned)lay.tY.size();
   NvtxRange nvtx_init_("hom_solve: initial state");
-  const unsigned nCtl = (unsigned)npairs, nctl = ctl_slices(most_tasks(lay));  // control CTAs: (cell, load) pairs x slices
+  const unsigned nCtl = (unsigned)npairs, nctl = control_slices(lay);  // control CTAs: (cell, load) pairs x slices
   tm.begin(HOM_K_INIT);
   k_init_pairs<<<(npairs + 255) / 256, 256, 0, st>>>(A);
   if (em) {
@@ -1979,7 +1989,7 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
 
   const int check = opts->check_every > 0 ? opts->check_every : 8;
   int host_nactive = npairs;
-  if (DIM == 2 && lay.fast && !adj && !out->stats) {
+  if (on_chip) {
     // pairs on small grids run to their own stopping point on chip; the passes below see them inactive
     int nres = 0;
     if ((rc = resident2d_solve(A, lay.cells, L, reinterpret_cast<int*>(ws + o_reslist), nph_max, st, &nres)) != HOM_OK) return rc;
