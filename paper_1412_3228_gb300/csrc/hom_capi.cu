@@ -23,6 +23,16 @@ int set_error(int code, const char* fmt, ...) {
   return code;
 }
 
+int sm_count() {
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) {
+    cudaGetLastError();
+    return 1;
+  }
+  return n;
+}
+
 bool grid_supported(int n) {
   std::vector<int> r;
   return n >= 3 && n <= kMaxN && factorize(n, r) && (int)r.size() <= kMaxStages;

@@ -42,6 +42,9 @@ int set_error(int code, const char* fmt, ...);
                               cudaGetErrorString(e_), __FILE__, __LINE__);                 \
   } while (0)
 
+// SMs of the current device.
+int sm_count();
+
 // ------------------------------------------------------------------ plans
 // Returns the device-resident plan of length n whose radices do not exceed max_radix (built
 // and uploaded on first use), or an error.

@@ -1117,15 +1117,15 @@ constexpr size_t kGreenBudget = (size_t)110 * 1024;
 constexpr size_t kRowBudget = (size_t)96 * 1024;
 
 // A batch of few or small cells leaves most of the chip idle when every CTA takes as much as its
-// shared memory holds: below kFewTasks tasks in a pass (four per SM) the tasks are made smaller, down
+// shared memory holds: below four tasks per SM in a pass the tasks are made smaller, down
 // to one row (two where they pair up) or one kx column, or one load per row task on the specialised
 // passes.  Measured (us per launch): the 61 cells of an FP64 convergence study: row 142 -> 111, Green 170
 // -> 146; 45^2 FP32 on the specialised passes: row 18.7 -> 13.8.
-constexpr size_t kFewTasks = 4 * 152;
-// Rows (or columns) per task, at most `fit`, that bring the pass's tasks (total at `fit`) near kFewTasks.
-int spread(int fit, size_t total) {
-  if (total >= kFewTasks || fit <= 1) return fit;
-  return (int)std::max<size_t>(1, fit * total / kFewTasks);
+inline size_t few_tasks() { return 4 * (size_t)sm_count(); }
+// Rows (or columns) per task, at most `fit`, that bring the pass's tasks (total at `fit`) near `few`.
+int spread(int fit, size_t total, size_t few) {
+  if (total >= few || fit <= 1) return fit;
+  return (int)std::max<size_t>(1, fit * total / few);
 }
 
 int build_layout(const hom_cell* cells, int ncells, int L, int dim, size_t vsize, int max_radix, const double* c0,
@@ -1180,7 +1180,8 @@ int build_layout(const hom_cell* cells, int ncells, int L, int dim, size_t vsize
     row_total += ((size_t)(dim == 2 ? n : n * n) + r - 1) / r;
     col_total += (size_t)(n / 2 + q) / q * L * (dim == 2 ? 1 : n);
   }
-  const bool split_loads = !lay.compact && lay.fast && L > 1 && row_total < kFewTasks;
+  const size_t few = few_tasks();
+  const bool split_loads = !lay.compact && lay.fast && L > 1 && row_total < few;
   for (int ci = 0; ci < ncells; ++ci) {
     const hom_cell& k = cells[ci];
     CellDev c{};
@@ -1265,7 +1266,7 @@ int build_layout(const hom_cell* cells, int ncells, int L, int dim, size_t vsize
     int r = rows_fit(k.n);
     if (!lay.fast && !lay.compact) {
       const int fit = r;
-      r = spread(fit, row_total);
+      r = spread(fit, row_total, few);
       // an odd number of real rows leaves half of a complex line empty (405^2 FP64, 3 loads: tasks of one
       // row, 9 real rows, took 329 us, tasks of 3 rows 288)
       if (r < fit && (r & 1) && (L * nc & 1)) ++r;
@@ -1275,7 +1276,7 @@ int build_layout(const hom_cell* cells, int ncells, int L, int dim, size_t vsize
     if (need_r > kMaxSmem) return set_error(HOM_ERR_UNSUPPORTED_SIZE, "row of n = %d with %d loads does not fit on chip", k.n, L);
     lay.smem_row = std::max(lay.smem_row, need_r);
     if (lay.fast) r = std::min(kFastRows, c.nrows);
-    const int ntk = lay.fast || lay.compact ? cols_fit(k.n) : spread(cols_fit(k.n), col_total);
+    const int ntk = lay.fast || lay.compact ? cols_fit(k.n) : spread(cols_fit(k.n), col_total, few);
     const size_t need_l = ((size_t)ntk * nc + 2) * line_bytes;
     lay.smem_green = std::max(lay.smem_green, need_l);
     lay.smem_y = std::max(lay.smem_y, need_l);
