@@ -68,12 +68,12 @@ int fast2d_init(const SolveArgs& A, int ncells, cudaStream_t st);
 int fast2d_permute_labels(const SolveArgs& A, int ncells, long long max_nv, cudaStream_t st);
 void fast2d_release();
 
-// On-chip solver of batches of small grids (hom_resident2d.cu): where every pair of the batch fits, runs all of
-// them to their stopping points and leaves them inactive, their iterates where the output pass reads them.
-// `list` holds room for every pair; *count receives the number of pairs taken, all or none.
+// On-chip solver of batches of small grids (hom_resident2d.cu): where every pair of the batch fits and it is the
+// faster way, runs all of them to their stopping points and leaves them inactive, their iterates where the output pass reads them.
+// `run` as above; `list` holds room for every pair; *count receives the number of pairs taken, all or none.
 struct CellDev;
-int resident2d_solve(const SolveArgs& A, const std::vector<CellDev>& cells, int L, int* list, int nphase_cell,
-                     cudaStream_t st, int* count);
+int resident2d_solve(const SolveArgs& A, const std::vector<CellDev>& cells, const std::vector<FastPlanDev>& plans, int L,
+                     int run, int* list, int nphase_cell, cudaStream_t st, int* count);
 
 // Specialised 3D passes (hom_fast3d.cu): row, y forward / inverse, Green (z lines), the initial
 // state eps = E and the output pass, on the kx-pair tiled state of those passes.

@@ -13,8 +13,8 @@
 //             others start the next rows; the flag comes back with the barrier after the pull.
 // Three cluster barriers an iteration, no launch and no trip through HBM.  The Green step's private state
 // (g, or u_hat of the Eyre-Milton scheme) has two buffers used in turn, in shared memory where they fit (n up
-// to about 190) and in the workspace otherwise: when iterate `it` passes, its own spectrum is rebuilt from the state it was made with, and its rows are left where
-// the output pass reads them.  The steps are those of the passes, so the iterates are too.
+// to about 190, Eyre-Milton 170) and in the workspace otherwise: when iterate `it` passes, its own spectrum is
+// rebuilt from the state it was made with, and its rows are left where the output pass reads them.  The steps are those of the passes, so the iterates are too.
 //
 // Measured, 40 iterations, 3 loads (whole call): 45^2, one cell: 1.72 ms in passes, 0.69 ms here; 143^2, two
 // cells: 3.67 ms (generic passes), 1.10 ms.
@@ -336,69 +336,132 @@ __global__ void __launch_bounds__(kTR, 2) k_resident2d(SolveArgs A, const int* l
 
 }  // namespace
 
-// Taken when the whole batch fits: every grid's state within kMaxCluster CTAs (n up to about 250) and every
-// cluster on the chip at once.  A cluster's iteration is a chain of short stages whatever else runs, so
-// further waves of clusters lose to the passes, which fill the chip (64 random-disk cells, 39 of their 64
-// grids eligible: 8.4 ms in passes, 11.2 ms with the small grids on chip first), and small grids beside
-// large ones ride along in the passes' launches (the 2D sweep: 28.9 ms, 30.1 ms).  Within that, a grid is
-// spread until a CTA holds about four row groups or the chip is full.
-int resident2d_solve(const SolveArgs& A, const std::vector<CellDev>& cells, int L, int* list, int nphase_cell,
-                     cudaStream_t st, int* count) {
+// Which batches run on chip: those whose every grid fits a cluster (n up to about 235), and whose clusters are
+// estimated faster than the passes.  A cluster's iteration is a chain of short stages whatever else runs, so
+// further waves of clusters soon lose to the passes, which fill the chip (64 random-disk cells, 39 of their 64
+// grids eligible: 8.4 ms in passes, 11.2 ms with the small grids on chip first), and small grids beside large
+// ones ride along in the passes' launches (the 2D sweep: 28.9 ms, 30.1 ms): a batch goes on chip as a whole or
+// not at all.
+//
+// The estimates, in us an iteration, follow measurements at n = 15 to 243, 1 to 48 pairs, both schemes:
+//   on chip: 8 + (0.007 + 0.0045 m) g n per wave of clusters, g row groups a CTA, m stages of the transform; 1.28
+//            times that for the Eyre-Milton scheme; cluster sizes run one after another.  105: 15.2, 150: 25 (three
+//            stages), 165: 24, 195: 32, 208: 34, 225: 37, 243: 43; Eyre-Milton 165: 31, 195: 41, 225: 49.
+//   passes : 16 + 16 per wave of their CTAs with radices from a plan (three an SM up to radix 9, else two):
+//            105 to 243: 30, 46 and 62 for one to three waves; 16 + 0.06 n per wave with compiled ones (135: 22 and
+//            33, 225: 28 and 45); 1.08 times that for the Eyre-Milton scheme.  These are a graph's; the
+//            host loop takes 5 more, and half of that is added for either, since a graph gives the loop's results bit
+//            for bit.
+// They cross near n = 210 (Eyre-Milton 180) for batches of one wave of passes, and below 225, which has compiled
+// radices; with two or three waves of passes most sizes that fit gain on chip (208, 12 pairs: 34 against 64),
+// unless their clusters take two waves too (152 SMs place about 15 clusters of 8 CTAs that fill an SM each:
+// 225, 16 pairs: 75 against 49; 165: 48 against 61).
+struct ResGroup {  // pairs of one cluster size
+  std::vector<int> pairs;
+  size_t bytes = 0, full = 0;  // dynamic shared memory without and with the private state on chip
+  double us = 0.0;             // an iteration of the slowest
+};
+double on_chip_us(const ResShape& sh, int n, int stages, bool em) {
+  return (em ? 1.28 : 1.0) * (8.0 + (0.007 + 0.0045 * stages) * sh.gpc * n);
+}
+double passes_us(const std::vector<CellDev>& cells, int L, int run, bool em, int sms) {
+  long long tasks = 0;
+  int nmax = 0;
+  for (const CellDev& c : cells) {
+    tasks += (long long)L * ((c.n / 2 + 2) / 2);
+    nmax = std::max(nmax, c.n);
+  }
+  const long long slots = (long long)sms * (run > 9 ? 2 : 3), waves = (tasks + slots - 1) / slots;
+  return (em ? 1.08 : 1.0) * (16.0 + (run ? 16.0 : 0.06 * nmax) * (double)waves) + 2.5;
+}
+// Clusters of `kernel` on the device at once, cached for the last few (device, kernel, size, shared memory) asked;
+// 0 where it can place none.
+template <typename K>
+int active_clusters(K kernel, const cudaLaunchConfig_t& cfg) {
+  struct Last { const void* k = nullptr; int dev = -1; unsigned size = 0; size_t smem = 0; int val = 0; };
+  static thread_local Last last[8];
+  static thread_local int next = 0;
+  const void* kp = reinterpret_cast<const void*>(kernel);
+  const unsigned size = cfg.attrs[0].val.clusterDim.x;
+  int dev = 0, n = 0;
+  cudaGetDevice(&dev);
+  for (const Last& e : last)
+    if (e.k == kp && e.dev == dev && e.size == size && e.smem == cfg.dynamicSmemBytes) return e.val;
+  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    n = 0;
+  }
+  last[next] = Last{kp, dev, size, cfg.dynamicSmemBytes, n};
+  next = (next + 1) & 7;
+  return n;
+}
+
+// Within that, a grid is spread until a CTA holds about four row groups or the chip is full.
+int resident2d_solve(const SolveArgs& A, const std::vector<CellDev>& cells, const std::vector<FastPlanDev>& plans, int L,
+                     int run, int* list, int nphase_cell, cudaStream_t st, int* count) {
   *count = 0;
-  constexpr int kSms = 152;
+  const int sms = sm_count();
   const bool em = A.scheme == HOM_SCHEME_EYRE_MILTON;
   std::vector<int> least(cells.size(), 0);
   int ctas = 0;
   const int pairs = (int)cells.size() * L;
-  if (pairs > kSms) return HOM_OK;
+  if (pairs > sms) return HOM_OK;
   for (size_t i = 0; i < cells.size(); ++i) {
     const int n = cells[i].n;
     const int tile = res_tile(n, !(n & 1), 2);  // an upper bound for any first radix
     for (int C = 1; C <= kMaxCluster && !least[i]; C *= 2)
       if (res_shape(n, C, nphase_cell, tile, em).bytes <= kResSmem) least[i] = C;
     ctas += least[i] * L;
-    if (!least[i] || ctas > kSms) return HOM_OK;
+    if (!least[i] || ctas > sms) return HOM_OK;
   }
-  struct Group {
-    std::vector<int> pairs;
-    size_t bytes = 0, full = 0;  // without and with the private state on chip
-  } by_size[4];
+  ResGroup by_size[4];
   for (size_t i = 0; i < cells.size(); ++i) {
     const int n = cells[i].n, G = (n + kFastRows - 1) / kFastRows;
     int C = least[i];
-    while (C < kMaxCluster && (ctas + C * L) <= kSms && pairs * C * 2 <= kSms && (G + C - 1) / C > 4) {
+    while (C < kMaxCluster && (ctas + C * L) <= sms && pairs * C * 2 <= sms && (G + C - 1) / C > 4) {
       ctas += C * L;
       C *= 2;
     }
-    Group& g = by_size[C == 1 ? 0 : C == 2 ? 1 : C == 4 ? 2 : 3];
+    ResGroup& g = by_size[C == 1 ? 0 : C == 2 ? 1 : C == 4 ? 2 : 3];
     for (int l = 0; l < L; ++l) g.pairs.push_back((int)i * L + l);
     const ResShape sh = res_shape(n, C, nphase_cell, res_tile(n, !(n & 1), 2), em);
     g.bytes = std::max(g.bytes, sh.bytes);
     g.full = std::max(g.full, sh.bytes + sh.priv);
+    g.us = std::max(g.us, on_chip_us(sh, n, plans[cells[i].fplan].run.m, em));
   }
+  auto kernel = em ? k_resident2d<true> : k_resident2d<false>;
+  HOM_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmem));
   std::vector<int> all;
-  for (int q = 3; q >= 0; --q) all.insert(all.end(), by_size[q].pairs.begin(), by_size[q].pairs.end());
+  cudaLaunchAttribute attr[4] = {};
+  cudaLaunchConfig_t cfg[4] = {};
+  int priv_on_chip[4] = {};
+  double chip_us = 0.0;
+  for (int q = 3; q >= 0; --q) {
+    const ResGroup& g = by_size[q];
+    if (g.pairs.empty()) continue;
+    all.insert(all.end(), g.pairs.begin(), g.pairs.end());
+    priv_on_chip[q] = g.full <= kResSmem;
+    attr[q].id = cudaLaunchAttributeClusterDimension;
+    attr[q].val.clusterDim.x = 1u << q;
+    attr[q].val.clusterDim.y = attr[q].val.clusterDim.z = 1;
+    cfg[q].gridDim = dim3((unsigned)g.pairs.size() << q);
+    cfg[q].blockDim = dim3(kTR);
+    cfg[q].dynamicSmemBytes = priv_on_chip[q] ? g.full : g.bytes;
+    cfg[q].stream = st;
+    cfg[q].attrs = &attr[q];
+    cfg[q].numAttrs = 1;
+    // a device (or a slice of one) that cannot place such a cluster leaves the batch to the passes
+    const int clusters = active_clusters(kernel, cfg[q]);
+    if (clusters < 1) return HOM_OK;
+    chip_us += g.us * (double)(((int)g.pairs.size() + clusters - 1) / clusters);
+  }
+  if (chip_us > passes_us(cells, L, run, em, sms)) return HOM_OK;
   HOM_CUDA_TRY(cudaMemcpyAsync(list, all.data(), all.size() * sizeof(int), cudaMemcpyHostToDevice, st));
   const int* at = list;
   for (int q = 3; q >= 0; --q) {
-    const Group& g = by_size[q];
-    if (g.pairs.empty()) continue;
-    auto kernel = em ? k_resident2d<true> : k_resident2d<false>;
-    HOM_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmem));
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = 1u << q;
-    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)g.pairs.size() << q);
-    cfg.blockDim = dim3(kTR);
-    const int priv_on_chip = g.full <= kResSmem;
-    cfg.dynamicSmemBytes = priv_on_chip ? g.full : g.bytes;
-    cfg.stream = st;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    HOM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, A, at, priv_on_chip));
-    at += g.pairs.size();
+    if (by_size[q].pairs.empty()) continue;
+    HOM_CUDA_TRY(cudaLaunchKernelEx(&cfg[q], kernel, A, at, priv_on_chip[q]));
+    at += by_size[q].pairs.size();
   }
   HOM_CUDA_TRY(cudaStreamSynchronize(st));  // the list's host copy goes out of scope
   *count = (int)all.size();

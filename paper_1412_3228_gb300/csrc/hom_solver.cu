@@ -1993,7 +1993,9 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
   if (on_chip) {
     // pairs on small grids run to their own stopping point on chip; the passes below see them inactive
     int nres = 0;
-    if ((rc = resident2d_solve(A, lay.cells, L, reinterpret_cast<int*>(ws + o_reslist), nph_max, st, &nres)) != HOM_OK) return rc;
+    if ((rc = resident2d_solve(A, lay.cells, lay.fplans, L, lay.run_max, reinterpret_cast<int*>(ws + o_reslist),
+                               nph_max, st, &nres)) != HOM_OK)
+      return rc;
     host_nactive -= nres;
   }
   int launched = 0;
