@@ -1116,16 +1116,107 @@ TaskL make_task(int cell, int load, int kx0, int ntk, int fixed, int nc, int dim
 constexpr size_t kGreenBudget = (size_t)110 * 1024;
 constexpr size_t kRowBudget = (size_t)96 * 1024;
 
-// A batch of few or small cells leaves most of the chip idle when every CTA takes as much as its
-// shared memory holds: below four tasks per SM in a pass the tasks are made smaller, down
-// to one row (two where they pair up) or one kx column, or one load per row task on the specialised
-// passes.  Measured (us per launch): the 61 cells of an FP64 convergence study: row 142 -> 111, Green 170
-// -> 146; 45^2 FP32 on the specialised passes: row 18.7 -> 13.8.
-inline size_t few_tasks() { return 4 * (size_t)sm_count(); }
-// Rows (or columns) per task, at most `fit`, that bring the pass's tasks (total at `fit`) near `few`.
-int spread(int fit, size_t total, size_t few) {
-  if (total >= few || fit <= 1) return fit;
-  return (int)std::max<size_t>(1, fit * total / few);
+// A batch of few or small cells leaves most of the chip idle when every CTA of the generic passes takes as much
+// as its shared memory holds; smaller tasks spread it, but each has a start of its own (task words, twiddles,
+// labels, a barrier per stage), and one task more than the SMs share out evenly costs a whole turn.  Below four
+// tasks per SM the sizes are therefore chosen by an estimate of the busiest SM's time.
+//   One grid size: a task of `lines` complex lines of length n costs n lines + fixed; of T tasks the SM gets
+//   ceil(T / SMs), two at a time in `pair` times the time of one (FP64 keeps an SM busy with one task, FP32 does
+//   not); over every size of task.
+//   Several: a task costs n (lines + start) + fixed; the larger of the largest task and of pair / 2 times the mean
+//   load plus `tail` mean tasks, over the sizes that bring two, three, four or six tasks to an SM.
+// Smaller tasks are taken where the estimate falls by more than `gain`.  The constants fit launches of 32 batches of
+// one size (2D 45 to 512, 3D 13 to 81, one to six loads, one to sixteen cells, up to 18 task sizes each) and of 19 of
+// several (2 to 61 cells): the sizes chosen take 0.2 to 4 % more than the best of those tried, and none more than
+// tasks as large as fit.  Us per launch, as large as fit -> chosen: FP64 45^3, 1 load: row 129 -> 50, Green 133 ->
+// 58; 26^3, 3 loads: 122 -> 39, 60 -> 51; 405^2, 3 loads: 153 and 184, both kept (a fixed target of four tasks
+// per SM gave 193 and 215); the 61 cells of a convergence study: 156 -> 137, 184 -> 148.
+struct TaskModel {
+  struct {
+    double fixed, pair, gain;
+  } one;
+  struct {
+    double fixed, start, pair, tail, gain;
+  } several;
+};
+constexpr TaskModel kRow64{{150.0, 1.8, 0.0}, {400.0, 1.0, 1.4, 1.0, 0.2}};
+constexpr TaskModel kCol64{{900.0, 1.9, 0.0}, {150.0, 0.5, 2.0, 0.5, 0.2}};
+constexpr TaskModel kRow32{{100.0, 1.0, 0.0}, {300.0, 0.0, 2.0, 0.5, 0.15}};
+constexpr TaskModel kCol32{{900.0, 1.4, 0.05}, {500.0, 3.0, 2.0, 0.5, 0.1}};
+struct PassCell {  // one cell's lines in a pass: `mult` times `units` rows or kx columns, at most `fit` a task
+  int n, fit;
+  long long units, mult;
+};
+// Rows (columns) per task of every cell.  `lines(k)`: complex lines of a task of k; `even`: tasks of an even number
+// where they are smaller (an odd number of real rows leaves half of a complex line empty).
+template <typename F>
+std::vector<int> task_sizes(const std::vector<PassCell>& cells, const TaskModel& m, int sms, bool even, F lines) {
+  auto tasks = [](const PassCell& c, int k) { return c.mult * ((c.units + k - 1) / k); };
+  std::vector<int> pick;
+  long long full = 0;
+  bool alike = true;
+  for (const PassCell& c : cells) {
+    pick.push_back(c.fit);
+    full += tasks(c, c.fit);
+    alike = alike && c.n == cells[0].n && c.fit == cells[0].fit;
+  }
+  if (full >= 4ll * sms) return pick;
+  double whole, best;
+  if (alike) {
+    const PassCell& c = cells[0];
+    auto estimate = [&](int k) {
+      const long long turns = (tasks(c, k) * (long long)cells.size() + sms - 1) / sms;
+      return ((double)(turns / 2) * m.one.pair + (double)(turns % 2)) * (c.n * lines(k) + m.one.fixed);
+    };
+    whole = best = estimate(c.fit);
+    for (int k = c.fit - 1; k >= 1; --k) {
+      const double t = estimate(k);
+      if (t < best && t < (1.0 - m.one.gain) * whole) {
+        best = t;
+        std::fill(pick.begin(), pick.end(), k);
+      }
+    }
+    return pick;
+  }
+  auto estimate = [&](const std::vector<int>& k) {
+    double sum = 0.0, most = 0.0;
+    long long T = 0;
+    for (size_t i = 0; i < cells.size(); ++i) {
+      const double c = cells[i].n * (lines(k[i]) + m.several.start) + m.several.fixed;
+      const long long t = tasks(cells[i], k[i]);
+      T += t;
+      sum += (double)t * c;
+      most = std::max(most, c);
+    }
+    return std::max(0.5 * m.several.pair * sum / sms + m.several.tail * sum / (double)T, most);
+  };
+  whole = best = estimate(pick);
+  std::vector<int> k(cells.size());
+  for (const int per : {2, 3, 4, 6}) {
+    const long long few = (long long)per * sms;
+    for (size_t i = 0; i < cells.size(); ++i) {
+      const int fit = cells[i].fit;
+      k[i] = full >= few ? fit : (int)std::max<long long>(1, fit * full / few);
+      if (even && k[i] < fit && (k[i] & 1)) ++k[i];
+    }
+    const double t = estimate(k);
+    if (t < best && t < (1.0 - m.several.gain) * whole) {
+      best = t;
+      pick = k;
+    }
+  }
+  return pick;
+}
+// One load per row task on the specialised passes, in place of every load (labels and twiddles are then read once):
+// `groups` tasks of L loads, or groups L of one.  In 2D in turns of what the SMs hold at once (three CTAs up to
+// radix 9 or with compiled radices, else two), a task's start costing about a load; 3D lines are short, and single
+// loads keep the SMs busier up to as many groups.  Us per launch, every load -> one load: 45^2, 3
+// loads: 16.5 -> 12.5; 405^2, 2 cells: 32 -> 28, 4 cells: 39.5, 44; 33^3, 6 loads: 38 -> 32; 45^3: 30, 32.
+bool one_load_tasks(long long groups, int L, int dim, int run, int sms) {
+  if (L < 2 || groups >= 4ll * sms) return false;
+  const long long slots = (long long)sms * (run > 9 ? 2 : 3);
+  auto turns = [&](long long tasks) { return (tasks + slots - 1) / slots; };
+  return dim == 3 ? groups <= slots : 2 * turns(groups * L) <= (L + 1) * turns(groups);
 }
 
 int build_layout(const hom_cell* cells, int ncells, int L, int dim, size_t vsize, int max_radix, const double* c0,
@@ -1174,14 +1265,26 @@ int build_layout(const hom_cell* cells, int ncells, int L, int dim, size_t vsize
     return std::min(lay.fast ? kFastCols : ntk, n / 2 + 1);
   };
   std::vector<int> task_rows, task_cols;
-  size_t row_total = 0, col_total = 0;
+  std::vector<PassCell> row_cells, col_cells;
+  long long groups = 0;  // of rows, on the specialised passes
   for (int ci = 0; ci < ncells; ++ci) {
-    const int n = cells[ci].n, r = lay.fast ? kFastRows : rows_fit(n), q = cols_fit(n);
-    row_total += ((size_t)(dim == 2 ? n : n * n) + r - 1) / r;
-    col_total += (size_t)(n / 2 + q) / q * L * (dim == 2 ? 1 : n);
+    const int n = cells[ci].n, nrows = dim == 2 ? n : n * n;
+    groups += (long long)((n + kFastRows - 1) / kFastRows) * (dim == 2 ? 1 : n);
+    row_cells.push_back(PassCell{n, rows_fit(n), nrows, 1});
+    col_cells.push_back(PassCell{n, cols_fit(n), n / 2 + 1, (long long)L * (dim == 2 ? 1 : n)});
   }
-  const size_t few = few_tasks();
-  const bool split_loads = !lay.compact && lay.fast && L > 1 && row_total < few;
+  if (!lay.fast && !lay.compact) {
+    const bool f64 = vsize == sizeof(double2);
+    const int sms = sm_count();
+    task_rows = task_sizes(row_cells, f64 ? kRow64 : kRow32, sms, (L * nc & 1) != 0,
+                           [&](int k) { return (double)((k * L * nc + 1) / 2); });
+    task_cols = task_sizes(col_cells, f64 ? kCol64 : kCol32, sms, false, [&](int k) { return (double)(k * nc); });
+  } else {
+    for (int ci = 0; ci < ncells; ++ci) {
+      task_rows.push_back(row_cells[ci].fit);
+      task_cols.push_back(col_cells[ci].fit);
+    }
+  }
   for (int ci = 0; ci < ncells; ++ci) {
     const hom_cell& k = cells[ci];
     CellDev c{};
@@ -1263,27 +1366,20 @@ int build_layout(const hom_cell* cells, int ncells, int L, int dim, size_t vsize
     lay.g_elems += (size_t)L * c.nrows * c.Hp * (em ? nc : dim);  // EM: u_hat (nc) instead of g (dim)
     // row-pass tasks: as many rows as fit in the shared-memory budget with every load active
     const size_t line_bytes = (size_t)k.n * vsize;
-    int r = rows_fit(k.n);
-    if (!lay.fast && !lay.compact) {
-      const int fit = r;
-      r = spread(fit, row_total, few);
-      // an odd number of real rows leaves half of a complex line empty (405^2 FP64, 3 loads: tasks of one
-      // row, 9 real rows, took 329 us, tasks of 3 rows 288)
-      if (r < fit && (r & 1) && (L * nc & 1)) ++r;
-    }
+    int r = task_rows[ci];
     // (passes with run-time radices refuse what the generic ones do, although they would hold it)
     const size_t need_r = row_lines(r) * line_bytes + (size_t)r * L * nc * (sizeof(long long) + 2 * vsize / 2);
     if (need_r > kMaxSmem) return set_error(HOM_ERR_UNSUPPORTED_SIZE, "row of n = %d with %d loads does not fit on chip", k.n, L);
     lay.smem_row = std::max(lay.smem_row, need_r);
     if (lay.fast) r = std::min(kFastRows, c.nrows);
-    const int ntk = lay.fast || lay.compact ? cols_fit(k.n) : spread(cols_fit(k.n), col_total, few);
+    const int ntk = task_cols[ci];
     const size_t need_l = ((size_t)ntk * nc + 2) * line_bytes;
     lay.smem_green = std::max(lay.smem_green, need_l);
     lay.smem_y = std::max(lay.smem_y, need_l);
-    task_rows.push_back(r);
-    task_cols.push_back(ntk);
+    task_rows[ci] = r;
     lay.cells.push_back(c);
   }
+  const bool split_loads = lay.fast && !lay.compact && one_load_tasks(groups, L, dim, lay.run_max, sm_count());
   // tasks, largest grids first: the small cells' tasks fill the end of each launch
   std::vector<int> order(ncells);
   for (int ci = 0; ci < ncells; ++ci) order[ci] = ci;
