@@ -74,7 +74,7 @@ extern "C" {
 #define HOM_FP32 0 /* FP32 fields, FFTs and Green operator; FP64 residual norm and averages   */
 #define HOM_FP64 1 /* FP64 everywhere                                                          */
 
-#define HOM_PASSES_AUTO 0    /* specialised FP32 passes where a compiled plan exists, else generic */
+#define HOM_PASSES_AUTO 0    /* FP32: on chip, specialised or generic passes, as is faster for the batch */
 #define HOM_PASSES_GENERIC 1 /* generic passes for every cell (any supported grid and precision)   */
 
 /* Discrete Green operator (section 2, eq. 2, and the modified operators its introduction cites). */

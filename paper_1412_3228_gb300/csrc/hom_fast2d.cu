@@ -705,6 +705,20 @@ void fill_run_plan(const HostPlan& hp, RunPlan& r) {
 }
 }  // namespace
 
+void run_plan_shape(int n, int* largest, int* stages) {
+  struct Shape { int n, largest, stages; };
+  static std::vector<Shape> known;  // every size asked for once
+  std::lock_guard<std::mutex> lk(g_fast_mu);
+  auto it = std::find_if(known.begin(), known.end(), [&](const Shape& s) { return s.n == n; });
+  if (it == known.end()) {
+    const std::vector<int> r = run_radices(n);
+    known.push_back({n, r.empty() ? 0 : *std::max_element(r.begin(), r.end()), (int)r.size()});
+    it = known.end() - 1;
+  }
+  *largest = it->largest;
+  *stages = it->stages;
+}
+
 bool run2d_size(int n) {  // the row pass's tile, twiddles and labels of 4 rows on chip, a few phases
   return grid_supported(n) && fast2d_smem_row(n, 64) <= 200 * 1024;
 }

@@ -44,6 +44,8 @@ bool fast2d_size(int n);
 bool fast3d_size(int n);
 bool run2d_size(int n);
 bool run3d_size(int n);
+// Largest radix and number of stages of the plan-read transform of size n.
+void run_plan_shape(int n, int* largest, int* stages);
 // Device tables of size n (built and uploaded on first use, kept until hom_release).  `run`: for the
 // passes with run-time radices, whose digit order differs from the compiled ones'.
 int fast2d_plan(int n, bool run, FastPlanDev* out);
@@ -74,6 +76,8 @@ void fast2d_release();
 struct CellDev;
 int resident2d_solve(const SolveArgs& A, const std::vector<CellDev>& cells, const std::vector<FastPlanDev>& plans, int L,
                      int run, int* list, int nphase_cell, cudaStream_t st, int* count);
+// Whether it will: the cells' sizes and the stages of their plans.
+bool resident2d_takes(const std::vector<int>& sizes, const std::vector<int>& stages, int L, int run, int nphase_cell, bool em);
 
 // Specialised 3D passes (hom_fast3d.cu): row, y forward / inverse, Green (z lines), the initial
 // state eps = E and the output pass, on the kx-pair tiled state of those passes.

@@ -334,7 +334,6 @@ __global__ void __launch_bounds__(kTR, 2) k_resident2d(SolveArgs A, const int* l
   cluster.sync();  // no CTA leaves while another may still write to its shared memory
 }
 
-}  // namespace
 
 // Which batches run on chip: those whose every grid fits a cluster (n up to about 235), and whose clusters are
 // estimated faster than the passes.  A cluster's iteration is a chain of short stages whatever else runs, so
@@ -364,12 +363,12 @@ struct ResGroup {  // pairs of one cluster size
 double on_chip_us(const ResShape& sh, int n, int stages, bool em) {
   return (em ? 1.28 : 1.0) * (8.0 + (0.007 + 0.0045 * stages) * sh.gpc * n);
 }
-double passes_us(const std::vector<CellDev>& cells, int L, int run, bool em, int sms) {
+double passes_us(const std::vector<int>& sizes, int L, int run, bool em, int sms) {
   long long tasks = 0;
   int nmax = 0;
-  for (const CellDev& c : cells) {
-    tasks += (long long)L * ((c.n / 2 + 2) / 2);
-    nmax = std::max(nmax, c.n);
+  for (int n : sizes) {
+    tasks += (long long)L * ((n / 2 + 2) / 2);
+    nmax = std::max(nmax, n);
   }
   const long long slots = (long long)sms * (run > 9 ? 2 : 3), waves = (tasks + slots - 1) / slots;
   return (em ? 1.08 : 1.0) * (16.0 + (run ? 16.0 : 0.06 * nmax) * (double)waves) + 2.5;
@@ -396,27 +395,31 @@ int active_clusters(K kernel, const cudaLaunchConfig_t& cfg) {
   return n;
 }
 
-// Within that, a grid is spread until a CTA holds about four row groups or the chip is full.
-int resident2d_solve(const SolveArgs& A, const std::vector<CellDev>& cells, const std::vector<FastPlanDev>& plans, int L,
-                     int run, int* list, int nphase_cell, cudaStream_t st, int* count) {
-  *count = 0;
-  const int sms = sm_count();
-  const bool em = A.scheme == HOM_SCHEME_EYRE_MILTON;
-  std::vector<int> least(cells.size(), 0);
+using ResKernel = void (*)(SolveArgs, const int*, int);
+ResKernel res_kernel(bool em) { return em ? k_resident2d<true> : k_resident2d<false>; }
+struct ResLaunch {  // one launch: the pairs of one cluster size
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr = {};
+  int priv_on_chip = 0;
+};
+// The launches of a batch that runs on chip (clusters of 2^q CTAs), or false: it runs in passes.  Within the rule
+// above, a grid is spread until a CTA holds about four row groups or the chip is full.
+bool res_launches(const std::vector<int>& sizes, const std::vector<int>& stages, int L, int run, int nphase_cell, bool em,
+                  ResGroup (&by_size)[4], ResLaunch (&launch)[4]) {
+  const int sms = sm_count(), pairs = (int)sizes.size() * L;
+  std::vector<int> least(sizes.size(), 0);
   int ctas = 0;
-  const int pairs = (int)cells.size() * L;
-  if (pairs > sms) return HOM_OK;
-  for (size_t i = 0; i < cells.size(); ++i) {
-    const int n = cells[i].n;
+  if (pairs > sms) return false;
+  for (size_t i = 0; i < sizes.size(); ++i) {
+    const int n = sizes[i];
     const int tile = res_tile(n, !(n & 1), 2);  // an upper bound for any first radix
     for (int C = 1; C <= kMaxCluster && !least[i]; C *= 2)
       if (res_shape(n, C, nphase_cell, tile, em).bytes <= kResSmem) least[i] = C;
     ctas += least[i] * L;
-    if (!least[i] || ctas > sms) return HOM_OK;
+    if (!least[i] || ctas > sms) return false;
   }
-  ResGroup by_size[4];
-  for (size_t i = 0; i < cells.size(); ++i) {
-    const int n = cells[i].n, G = (n + kFastRows - 1) / kFastRows;
+  for (size_t i = 0; i < sizes.size(); ++i) {
+    const int n = sizes[i], G = (n + kFastRows - 1) / kFastRows;
     int C = least[i];
     while (C < kMaxCluster && (ctas + C * L) <= sms && pairs * C * 2 <= sms && (G + C - 1) / C > 4) {
       ctas += C * L;
@@ -427,40 +430,62 @@ int resident2d_solve(const SolveArgs& A, const std::vector<CellDev>& cells, cons
     const ResShape sh = res_shape(n, C, nphase_cell, res_tile(n, !(n & 1), 2), em);
     g.bytes = std::max(g.bytes, sh.bytes);
     g.full = std::max(g.full, sh.bytes + sh.priv);
-    g.us = std::max(g.us, on_chip_us(sh, n, plans[cells[i].fplan].run.m, em));
+    g.us = std::max(g.us, on_chip_us(sh, n, stages[i], em));
   }
-  auto kernel = em ? k_resident2d<true> : k_resident2d<false>;
-  HOM_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmem));
-  std::vector<int> all;
-  cudaLaunchAttribute attr[4] = {};
-  cudaLaunchConfig_t cfg[4] = {};
-  int priv_on_chip[4] = {};
+  const ResKernel kernel = res_kernel(em);
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmem) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
   double chip_us = 0.0;
   for (int q = 3; q >= 0; --q) {
     const ResGroup& g = by_size[q];
     if (g.pairs.empty()) continue;
-    all.insert(all.end(), g.pairs.begin(), g.pairs.end());
-    priv_on_chip[q] = g.full <= kResSmem;
-    attr[q].id = cudaLaunchAttributeClusterDimension;
-    attr[q].val.clusterDim.x = 1u << q;
-    attr[q].val.clusterDim.y = attr[q].val.clusterDim.z = 1;
-    cfg[q].gridDim = dim3((unsigned)g.pairs.size() << q);
-    cfg[q].blockDim = dim3(kTR);
-    cfg[q].dynamicSmemBytes = priv_on_chip[q] ? g.full : g.bytes;
-    cfg[q].stream = st;
-    cfg[q].attrs = &attr[q];
-    cfg[q].numAttrs = 1;
+    ResLaunch& l = launch[q];
+    l.priv_on_chip = g.full <= kResSmem;
+    l.attr.id = cudaLaunchAttributeClusterDimension;
+    l.attr.val.clusterDim.x = 1u << q;
+    l.attr.val.clusterDim.y = l.attr.val.clusterDim.z = 1;
+    l.cfg.gridDim = dim3((unsigned)g.pairs.size() << q);
+    l.cfg.blockDim = dim3(kTR);
+    l.cfg.dynamicSmemBytes = l.priv_on_chip ? g.full : g.bytes;
+    l.cfg.attrs = &l.attr;
+    l.cfg.numAttrs = 1;
     // a device (or a slice of one) that cannot place such a cluster leaves the batch to the passes
-    const int clusters = active_clusters(kernel, cfg[q]);
-    if (clusters < 1) return HOM_OK;
+    const int clusters = active_clusters(kernel, l.cfg);
+    if (clusters < 1) return false;
     chip_us += g.us * (double)(((int)g.pairs.size() + clusters - 1) / clusters);
   }
-  if (chip_us > passes_us(cells, L, run, em, sms)) return HOM_OK;
+  return chip_us <= passes_us(sizes, L, run, em, sms);
+}
+
+}  // namespace
+
+bool resident2d_takes(const std::vector<int>& sizes, const std::vector<int>& stages, int L, int run, int nphase_cell, bool em) {
+  ResGroup by_size[4];
+  ResLaunch launch[4];
+  return res_launches(sizes, stages, L, run, nphase_cell, em, by_size, launch);
+}
+
+int resident2d_solve(const SolveArgs& A, const std::vector<CellDev>& cells, const std::vector<FastPlanDev>& plans, int L,
+                     int run, int* list, int nphase_cell, cudaStream_t st, int* count) {
+  *count = 0;
+  std::vector<int> sizes, stages, all;
+  for (const CellDev& c : cells) {
+    sizes.push_back(c.n);
+    stages.push_back(plans[c.fplan].run.m);
+  }
+  const bool em = A.scheme == HOM_SCHEME_EYRE_MILTON;
+  ResGroup by_size[4];
+  ResLaunch launch[4];
+  if (!res_launches(sizes, stages, L, run, nphase_cell, em, by_size, launch)) return HOM_OK;
+  for (int q = 3; q >= 0; --q) all.insert(all.end(), by_size[q].pairs.begin(), by_size[q].pairs.end());
   HOM_CUDA_TRY(cudaMemcpyAsync(list, all.data(), all.size() * sizeof(int), cudaMemcpyHostToDevice, st));
   const int* at = list;
   for (int q = 3; q >= 0; --q) {
     if (by_size[q].pairs.empty()) continue;
-    HOM_CUDA_TRY(cudaLaunchKernelEx(&cfg[q], kernel, A, at, priv_on_chip[q]));
+    launch[q].cfg.stream = st;
+    HOM_CUDA_TRY(cudaLaunchKernelEx(&launch[q].cfg, res_kernel(em), A, at, launch[q].priv_on_chip));
     at += by_size[q].pairs.size();
   }
   HOM_CUDA_TRY(cudaStreamSynchronize(st));  // the list's host copy goes out of scope

@@ -1219,8 +1219,38 @@ bool one_load_tasks(long long groups, int L, int dim, int run, int sms) {
   return dim == 3 ? groups <= slots : 2 * turns(groups * L) <= (L + 1) * turns(groups);
 }
 
+// Whether the FP32 passes with radices from a plan are the faster ones, for batches that do not run on chip.  They
+// keep a lane pair of lines per thread, with little per task; the generic ones hold many lines and radices up to 27
+// per task.  While the plan-read tasks fit the chip at once (two or three CTAs an SM in 2D, four or six in 3D, by
+// their registers) they win (325^2, 3 loads: 34 us an iteration against 45).  Beyond, they win where the generic
+// passes' lines fall on the same banks (512^2, 8 cells, 3 loads: 229 against 552; 208^2, 64 cells: 582 against 829;
+// 64^3, 6 loads: 232 against 381), on long lines (507^2, 8 cells: 276 against 306; 98^3: 679 against 946), and with
+// three stages of radices up to 9 (2D: 343^2, 8 cells: 136 against 148); and lose elsewhere (143^2, 64 cells, 3
+// loads: 362 against 174; 44^3, 6 loads: 149 against 96).  A batch goes as most of its voxels do.
+bool plan_reads_win(int dim, int n, int largest, int stages) {
+  if (dim == 2)
+    return n >= 455 || (n >= 128 && n % (n <= 256 || n >= 400 ? 16 : 32) == 0) ||
+           (n >= 243 && largest <= 9 && stages <= 3);
+  return (n >= 32 && n % 8 == 0) || (n >= 70 && (largest <= 9 || stages <= 2 || n >= 100));
+}
+bool plan_passes_faster(const std::vector<int>& sizes, const std::vector<int>& largest, const std::vector<int>& stages, int L,
+                        int dim, int run, int sms) {
+  long long tasks = 0;
+  double all = 0.0, good = 0.0;
+  for (size_t i = 0; i < sizes.size(); ++i) {
+    const int n = sizes[i];
+    const long long groups = (n + kFastRows - 1) / kFastRows;
+    tasks += L * groups * (dim == 2 ? 1 : n);
+    const double voxels = (double)n * n * (dim == 2 ? 1 : n);
+    all += voxels;
+    good += plan_reads_win(dim, n, largest[i], stages[i]) ? voxels : 0.0;
+  }
+  const long long slots = (long long)sms * (run > 9 ? 2 : 3) * (dim == 2 ? 1 : 2);
+  return tasks <= slots || 2.0 * good >= all;
+}
+
 int build_layout(const hom_cell* cells, int ncells, int L, int dim, size_t vsize, int max_radix, const double* c0,
-                 bool external, Layout& lay, bool em = false) {
+                 bool external, Layout& lay, bool em, bool chip) {
   const int nc = nc_of(dim);
   const size_t budget = kRowBudget;
   const size_t kMaxSmem = 227 * 1024;
@@ -1235,11 +1265,23 @@ int build_layout(const hom_cell* cells, int ncells, int L, int dim, size_t vsize
     }
     if (lay.run) {  // what the one-byte labels and their kernel cannot hold stays on the generic passes
       if (ncells > 65535) lay.fast = false;
+      size_t nph_max = 1;
       for (int ci = 0; ci < ncells && lay.fast; ++ci) {
         std::vector<int> ph{cells[ci].matrix_phase};
         for (int p = 0; p < cells[ci].nprim; ++p) ph.push_back(cells[ci].prims[p].phase);
         std::sort(ph.begin(), ph.end());
-        if (std::unique(ph.begin(), ph.end()) - ph.begin() > 254) lay.fast = false;
+        nph_max = std::max(nph_max, (size_t)(std::unique(ph.begin(), ph.end()) - ph.begin()));
+        if (nph_max > 254) lay.fast = false;
+      }
+      if (lay.fast) {
+        std::vector<int> sizes(ncells), largest(ncells), stages(ncells);
+        for (int ci = 0; ci < ncells; ++ci) {
+          sizes[ci] = cells[ci].n;
+          run_plan_shape(sizes[ci], &largest[ci], &stages[ci]);
+        }
+        const int run = *std::max_element(largest.begin(), largest.end());
+        if (!(chip && resident2d_takes(sizes, stages, L, run, (int)nph_max, em)))
+          lay.fast = plan_passes_faster(sizes, largest, stages, L, dim, run, sm_count());
       }
     }
     lay.run = lay.run && lay.fast;
@@ -1782,7 +1824,8 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
   lay.fast = std::is_same<T, float>::value && !cg && opts->passes != HOM_PASSES_GENERIC &&
              opts->green == HOM_GREEN_CONTINUOUS && !refine && !warm;
   lay.compact = ext && ext->compact;
-  int rc = build_layout(cells, ncells, L, DIM, sizeof(V), MAXR, c0, ext != nullptr, lay, em);
+  const bool chip = DIM == 2 && !adj && !out->stats && !lay.compact;  // the on-chip solver may run
+  int rc = build_layout(cells, ncells, L, DIM, sizeof(V), MAXR, c0, ext != nullptr, lay, em, chip);
   if (rc != HOM_OK) return rc;
   const int npairs = ncells * L;
   const bool want_fields = out->eps || out->sigma;
@@ -1864,7 +1907,7 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
     }
   }
   const size_t o_cphase = lay.fast ? take(cell_phases.size() * sizeof(int)) : 0;
-  const bool on_chip = lay.fast && DIM == 2 && !adj && !out->stats && !lay.compact;
+  const bool on_chip = lay.fast && chip;
   const size_t o_reslist = on_chip ? take((size_t)npairs * sizeof(int)) : 0;
   const size_t o_fplans = lay.fast ? take(lay.fplans.size() * sizeof(FastPlanDev)) : 0;
   const size_t o_stage_e = need_stage && out->eps && !eps_dev ? take(lay.fld_elems * sizeof(T)) : 0;

@@ -86,6 +86,24 @@ def test_batches_kept_in_the_passes(sizes, loads):
     _same(a, hom.hom_solve(mat, E, c0, tol=1e-4, max_iter=200, stats=True, **kw))
 
 
+@pytest.mark.parametrize("dim,sizes,loads,plan", [
+    (2, (143,) * 16, 3, False), (2, (150, 130, 121) * 20, 3, False), (2, (64,) * 64, 3, False), (2, (300,) * 8, 3, False),
+    (3, (44,), 6, False), (3, (26,) * 8, 6, False), (2, (325,), 3, True), (2, (208,) * 24, 3, True), (2, (512,) * 4, 3, True),
+    (2, (507, 45, 45), 3, True), (2, (343,) * 8, 3, True), (3, (64,), 6, True), (3, (49,), 1, True), (3, (98,), 2, True)],
+    ids=lambda v: "x".join(map(str, (v[0], len(v)))) if isinstance(v, tuple) else str(v))
+def test_plan_read_or_generic_passes(dim, sizes, loads, plan):
+    """Sizes without compiled radices take the plan-read passes where these were measured faster and the generic ones
+    elsewhere.  The same launches give the same bits; the other passes round differently."""
+    cells, mat, E, c0, kw = _problem(dim, sizes, loads, 0)
+    kw.update(tol=0.0, max_iter=5)
+    a, gen = hom.hom_solve(mat, E, c0, **kw), hom.hom_solve(mat, E, c0, passes=hom.HOM_PASSES_GENERIC, **kw)
+    if plan:
+        assert not torch.equal(a["eps"], gen["eps"])
+        _close(a, gen, cells, loads)
+    else:
+        _same(a, gen)
+
+
 @pytest.mark.parametrize("scheme", [0, 1], ids=["basic", "eyre-milton"])
 @pytest.mark.parametrize("dim,sizes,loads", [(2, (45, 135, 405), 3), (2, (45, 300, 77), 2), (3, (27,), 2), (3, (14, 22), 2)],
                          ids=["2d-compiled", "2d-plan", "3d-compiled", "3d-plan"])
