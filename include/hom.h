@@ -191,7 +191,7 @@ typedef struct hom_solve_opts {
                           /* observed contraction, enough for one correction to bring the */
                           /* error to tol / 5)                                            */
   int32_t scheme;         /* HOM_SCHEME_BASIC (0) or HOM_SCHEME_EYRE_MILTON: FP32 or FP64     */
-                          /* (specialised FP32 passes in 2D), continuous Green operator,    */
+                          /* (every kind of FP32 passes), continuous Green operator,        */
                           /* hom_solve only, no refine                                      */
   int32_t warm_start;     /* 1: hom_result.eps (device, field type) holds the initial strain */
                           /* field of every load case on entry (state in / out: the returned */
@@ -202,7 +202,10 @@ typedef struct hom_solve_opts {
 } hom_solve_opts;
 
 /* Per-kernel timing, filled when hom_result.stats is non-NULL (adds CUDA events around every
- * launch; the call then synchronises the stream before returning). */
+ * launch; the call then synchronises the stream before returning).  The times are those of passes,
+ * one launch per kernel: a batch of small 2D FP32 grids that would run on chip (the whole iteration in
+ * one launch, faster) is run in passes when they are asked for, and use_graph is ignored.  To time such
+ * a call as it runs, time it as a whole without stats. */
 #define HOM_NKERNEL 8
 #define HOM_K_FILTER 0   /* filter build (classification, sampling, rule)                */
 #define HOM_K_ROW 1      /* row pass: inverse x-FFT, constitutive, forward x-FFT          */
@@ -285,8 +288,8 @@ int hom_filter_build(const hom_cell* cells, int32_t ncells, const hom_phase* pha
  *   so a load case stops only when both its equilibrium error (opts->criterion) and its
  *   compatibility error e_c (hom_result.err_c) are below opts->tol.  Any positive-definite c0
  *   converges; the geometric means of the extreme phase moduli (bulk and shear) give the fastest
- *   contraction.  FP32 2D batches of specialised sizes run the specialised passes (as the basic
- *   scheme, unless opts->passes = HOM_PASSES_GENERIC), everything else the generic passes;
+ *   contraction.  FP32 batches run on chip or on the specialised passes where the basic scheme
+ *   does (unless opts->passes = HOM_PASSES_GENERIC), everything else on the generic passes;
  *   continuous Green operator; returns HOM_ERR_NOT_IMPL with opts->green = HOM_GREEN_ROTATED or
  *   opts->refine > 0. */
 int hom_solve(const hom_cell* cells, int32_t ncells, const hom_material* mat, const double* E, int32_t L,

@@ -329,7 +329,7 @@ def hom_solve(material: Material, E, c0, *, L: Optional[int] = None, precision: 
     c0: [ncells, 2] (or [2]) Lamé constants of the reference medium.
     Returns a dict with eps / sigma fields ([sum over cells of L*nc*n^dim], flat, cell-major),
     mean_sigma [ncells, L, nc], iterations / status / err / err_n / err_c [ncells, L] and the
-    kernel statistics when stats=True.
+    kernel statistics when stats=True (which runs small 2D FP32 batches in passes instead of on chip).
     eps0: warm start, a device tensor laid out like the returned eps (field precision); the solve
     reads it through the returned eps buffer, which starts as a copy of it.
     history=True adds "history" [ncells, L, max_iter + 1]: the stopping quantity of every

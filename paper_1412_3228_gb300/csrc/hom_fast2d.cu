@@ -1,5 +1,5 @@
-// Specialised FP32 row and Green passes of the 2D fixed-point scheme (section 2, eqs. 1-a, 1-b,
-// 2) for grid sizes n with a radix plan fixed at compile time.
+// Specialised FP32 row and Green passes of the 2D fixed-point and Eyre-Milton schemes (section 2, eqs. 1-a,
+// 1-b, 2), with the radices of a few grid sizes fixed at compile time and those of every other read from a plan.
 //
 // Lane pairs.  Shared memory holds one float4 per (position, pair): (re_A, re_B, im_A, im_B), the
 // same position of two complex lines A and B.  Every butterfly, the Green operator and the
@@ -13,7 +13,7 @@
 //
 // Transforms are the in-place mixed-radix DIF (natural -> digit-reversed) and DIT (digit-reversed
 // -> natural) of hom_common.cuh with the radices as template parameters: every index division is
-// by a compile-time constant.  The row pass works on x samples at digit-reversed positions and
+// by a compile-time constant (plan-read transforms: by multiplication, FastDiv).  The row pass works on x samples at digit-reversed positions and
 // reads one-byte labels permuted the same way (label8); the Green pass reads the wave number of each
 // position from a table.
 //
@@ -335,7 +335,7 @@ __global__ void __launch_bounds__(kT, 3) k_row_f2d(SolveArgs A, int ntasks, int 
 // up to 16 (lane pairs) take 128 registers, two CTAs per SM; batches whose plans stay at 9 and below run the
 // 80-register variant, three CTAs per SM.  Measured against the generic row pass, which keeps two real rows
 // per complex line and scalar arithmetic: 2 cells of 512^2, 3 loads: 72 us generic, 55 us with 128
-// registers, 39 us with 80; 143^2: 43 us generic, 20 us.
+// registers, 39 us with 80; 143^2: 43 us generic, 16 us (one load per task).
 template <bool OUT, bool SRC, bool EM, int MAXR>
 __global__ void __launch_bounds__(kT, MAXR > 9 ? 2 : 3) k_row_r2d(SolveArgs A, int ntasks, int ahead) {
   row_task<OUT, SRC, EM, MAXR>(A, ntasks, ahead);
@@ -599,7 +599,7 @@ __global__ void __launch_bounds__(kT, 3) k_green_f2d(SolveArgs A, int ntasks, in
   green_task<EM, 0>(A, ntasks, ahead);
 }
 // Radices read from a plan (see k_row_r2d): 2 cells of 512^2, 3 loads: 103 us generic, 45 us with 128
-// registers, 32 us with 80; 143^2: 42 us generic, 19 us.
+// registers, 33 us with 80; 143^2: 42 us generic, 14 us.
 template <bool EM, int MAXR>
 __global__ void __launch_bounds__(kT, MAXR > 9 ? 2 : 3) k_green_r2d(SolveArgs A, int ntasks, int ahead) {
   green_task<EM, MAXR>(A, ntasks, ahead);

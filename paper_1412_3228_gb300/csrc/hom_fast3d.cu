@@ -1,6 +1,6 @@
-// Specialised FP32 passes of the 3D fixed-point scheme (section 2, eqs. 1-a, 1-b, 2) for grid
-// sizes n with a compile-time radix plan (27, 45, 81, 135, 243).  Same lane-pair scheme as the 2D
-// passes (hom_fast2d.cu): shared memory holds float4 (re_A, re_B, im_A, im_B) per (position,
+// Specialised FP32 passes of the 3D fixed-point and Eyre-Milton schemes (section 2, eqs. 1-a, 1-b, 2), with the
+// radices of 27, 45, 81, 135 and 243 compiled in and those of every other size read from a plan.  Same lane-pair
+// scheme as the 2D passes (hom_fast2d.cu): shared memory holds float4 (re_A, re_B, im_A, im_B) per (position,
 // component), with the six Mandel components side by side; positions are 7 float4 apart in shared
 // memory (112 bytes: neighbouring threads' 16-byte accesses fall on distinct bank quads).
 //
@@ -440,7 +440,7 @@ __global__ void __launch_bounds__(kT3, kMinB3) k_row_f3d(SolveArgs A, int ntasks
 }
 // The same pass with radices read from a plan, for batches that hold a size without compiled ones (128
 // registers for radices up to 16, 80 up to 9).  Measured at 64^3, 6 loads: 112 us for the generic row pass,
-// 111 us with 128 registers, 101 us with 80.
+// 111 us with 128 registers, 80 us with 80.
 template <bool OUT, bool SRC, bool EM, int MAXR>
 __global__ void __launch_bounds__(kT3, MAXR > 9 ? kRunB3 : kMinB3) k_row_r3d(SolveArgs A, int ntasks, int ahead) {
   row3_task<OUT, SRC, EM, MAXR>(A, ntasks, ahead);
@@ -551,7 +551,7 @@ template <bool FWD>
 __global__ void __launch_bounds__(kT3, 1024 / kT3) k_ypass_f3d(SolveArgs A) {
   ypass3_task<FWD, 0>(A);
 }
-// radices read from a plan: 64^3, 6 loads: 115-120 us for the generic passes, 58 us with 128 registers, 44 us
+// radices read from a plan: 64^3, 6 loads: 115-120 us for the generic passes, 58 us with 128 registers, 45 us
 // with 80
 template <bool FWD, int MAXR>
 __global__ void __launch_bounds__(kT3, MAXR > 9 ? kRunB3 : kMinB3) k_ypass_r3d(SolveArgs A) {

@@ -16,8 +16,8 @@
 // to about 190, Eyre-Milton 170) and in the workspace otherwise: when iterate `it` passes, its own spectrum is
 // rebuilt from the state it was made with, and its rows are left where the output pass reads them.  The steps are those of the passes, so the iterates are too.
 //
-// Measured, 40 iterations, 3 loads (whole call): 45^2, one cell: 1.72 ms in passes, 0.69 ms here; 143^2, two
-// cells: 3.67 ms (generic passes), 1.10 ms.
+// Measured, 40 iterations, 3 loads (whole call): 45^2, one cell: 1.35 ms in passes, 0.69 ms here; 143^2, two
+// cells: 1.7 ms in passes, 1.11 ms.
 #define HOM_FILE_ID 4
 #include <cooperative_groups.h>
 

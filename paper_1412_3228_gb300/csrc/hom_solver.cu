@@ -1816,7 +1816,6 @@ int run_solve(const hom_cell* cells, int ncells, const hom_material* mat, const 
   // defect correction (FP32 with FP64 residuals) runs on the generic passes: FP32 and FP64 states
   // then share one layout
   const bool refine = std::is_same<T, float>::value && opts->refine > 0 && !cg && !adj && !ext;
-  // the Eyre-Milton scheme runs on the generic passes
   const bool em = opts->scheme == HOM_SCHEME_EYRE_MILTON && !cg && !adj && !ext;
   // a warm start converts the caller's real field on the generic passes' layout
   const bool warm = opts->warm_start != 0 && !cg && !adj && !ext;
