@@ -409,7 +409,7 @@ int hom_effective_stiffness(int32_t ncells, int32_t dim, const double* E, const 
 
 /* The autotuner's record.  The first FP32 hom_solve of a batch shape (device, dimension, load count,
  * Green operator, multiset of grid sizes) with opts->tune = 1 (passes = AUTO, max_radix = 0) times
- * four candidate plans on that batch -- the specialised passes and the generic passes with register
+ * four candidate plans on that batch -- the automatic choice ("specialised") and the generic passes with register
  * radices up to 15, 27 and 45 -- by the difference of calls of 8 and of 1 fixed iterations (after an
  * untimed one of 1), and every later solve of the shape runs the fastest.  Solves with refine or warm_start,
  * which run on the generic passes, have a record of their own, without the specialised candidate.
