@@ -413,8 +413,8 @@ int hom_effective_stiffness(int32_t ncells, int32_t dim, const double* E, const 
  * radices up to 15, 27 and 45 -- by the difference of calls of 8 and of 1 fixed iterations (after an
  * untimed one of 1), and every later solve of the shape runs the fastest.  Solves with refine or warm_start,
  * which run on the generic passes, have a record of their own, without the specialised candidate.
- * Writes one line per shape, "shape: timings (n trial iterations) -> choice", into buf (at most len bytes, NUL-terminated) and returns the full length.  The choice depends on
- * measured times, so two processes may pick different plans (results then differ by FP32 rounding). */
+ * Writes one line per shape, "shape: timings (n trial iterations) -> choice", into buf (at most len bytes,
+ * NUL-terminated) and returns the full length.  The choice depends on measured times, so two processes may pick different plans (results then differ by FP32 rounding). */
 int32_t hom_autotune_report(char* buf, int32_t len);
 
 /* Message of the last failed call on this host thread ("" if none). */

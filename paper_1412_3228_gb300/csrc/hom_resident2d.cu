@@ -14,7 +14,8 @@
 // Three cluster barriers an iteration, no launch and no trip through HBM.  The Green step's private state
 // (g, or u_hat of the Eyre-Milton scheme) has two buffers used in turn, in shared memory where they fit (n up
 // to about 190, Eyre-Milton 170) and in the workspace otherwise: when iterate `it` passes, its own spectrum is
-// rebuilt from the state it was made with, and its rows are left where the output pass reads them.  The steps are those of the passes, so the iterates are too.
+// rebuilt from the state it was made with, and its rows are left where the output pass reads them.  The steps are
+// those of the passes, so the iterates are too.
 //
 // Measured, 40 iterations, 3 loads (whole call): 45^2, one cell: 1.35 ms in passes, 0.69 ms here; 143^2, two
 // cells: 1.7 ms in passes, 1.11 ms.
